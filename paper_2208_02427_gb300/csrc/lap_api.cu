@@ -191,7 +191,6 @@ void check_params(const lap_params* p)
 // ---- line-solver tables --------------------------------------------------------------
 
 constexpr int LINE_MAX_N = 16383;
-constexpr int LINE_MIN_CHUNK = 16;
 
 // Thomas solve of tridiag(-alpha, delta, -alpha) x = rhs (size len) on the host.
 std::vector<double> host_thomas(int len, double alpha, double delta, const std::vector<double>& rhs)
@@ -206,9 +205,9 @@ std::vector<double> host_thomas(int len, double alpha, double delta, const std::
 }
 
 const LineTables& line_tables(lap_handle h, int N, double alpha, double delta, double wc,
-                              int max_chunks)
+                              int max_chunks, int min_chunk)
 {
-    auto key = std::make_tuple(N, alpha, delta, wc, max_chunks);
+    auto key = std::make_tuple(N, alpha, delta, wc, max_chunks, min_chunk);
     auto it = h->lines.find(key);
     if (it != h->lines.end()) return it->second.t;
     if (N > LINE_MAX_N) fail(LAP_EUNSUPPORTED, "line longer than 16383 unknowns");
@@ -220,18 +219,22 @@ const LineTables& line_tables(lap_handle h, int N, double alpha, double delta, d
     t.maxp = max_chunks;
     // P <= max_chunks chunks of L unknowns, each but the last followed by one separator unknown;
     // the last chunk holds the remaining 1..L unknowns (the line never ends on a separator)
-    if (N <= LINE_MIN_CHUNK) {
+    if (min_chunk == 0 && N <= max_chunks) {
+        // as many lanes as unknowns: all of them separators, the chunks empty
+        t.L = t.Ll = 0;
+        t.P = N + 1;
+    } else if (N <= min_chunk) {
         t.L = t.Ll = N;
         t.P = 1;
     } else {
-        t.L = std::max(LINE_MIN_CHUNK, (N - (max_chunks - 1) + max_chunks - 1) / max_chunks);
+        t.L = std::max(std::max(1, min_chunk), (N - (max_chunks - 1) + max_chunks - 1) / max_chunks);
         for (;; ++t.L) {
             t.P = (N + 1 + t.L) / (t.L + 1);  // ceil((N + 1) / (L + 1))
             t.Ll = N - (t.P - 1) * (t.L + 1);
             if (t.Ll >= 1) break;
         }
     }
-    if (t.Ll > t.L || t.P > max_chunks) fail(LAP_ECUDA, "internal: bad line partition");
+    if (t.Ll > t.L || (t.L > 0 && t.P > max_chunks)) fail(LAP_ECUDA, "internal: bad line partition");
     t.stride = (t.L + 1) | 1;
     const int L = t.L, S = t.P - 1;
     t.levels = 0;
@@ -246,10 +249,11 @@ const LineTables& line_tables(lap_handle h, int N, double alpha, double delta, d
         sc[q] = wc / den;
     }
     sc[L] = wc;
-    F[0] = alpha;
+    if (L > 0) F[0] = alpha;
     for (int q = 1; q < L; ++q) F[q] = F[q - 1] * e[q - 1];
     auto influence = [&](int len, bool left) {
         std::vector<double> rhs(len, 0.0);
+        if (len == 0) return rhs;
         rhs[left ? 0 : len - 1] = alpha;
         std::vector<double> g = host_thomas(len, alpha, delta, rhs);
         g.resize(L, 0.0);
@@ -276,7 +280,12 @@ const LineTables& line_tables(lap_handle h, int N, double alpha, double delta, d
     // separator p ends in y_last + x_{p-1} gL[L-1] + x_p gR[L-1], the chunk right of it starts in
     // y_first + x_p gL'[0] + x_{p+1} gR'[0] (the last chunk's vectors for p = S - 1)
     std::vector<double> a(S), b(S), c(S);
-    for (int p = 0; p < S; ++p) {
+    for (int p = 0; p < S && L == 0; ++p) {
+        a[p] = p >= 1 ? -alpha : 0.0;
+        b[p] = delta;
+        c[p] = p + 1 <= S - 1 ? -alpha : 0.0;
+    }
+    for (int p = 0; p < S && L > 0; ++p) {
         const bool right_last = p + 1 == t.P - 1;
         a[p] = p >= 1 ? -alpha * gL[L - 1] : 0.0;
         b[p] = delta - alpha * gR[L - 1] - alpha * (right_last ? gLl[0] : gL[0]);
@@ -350,6 +359,19 @@ double* line_scratch(lap_handle h, const LineTables& t, int64_t gp)
     return h->lscratch;
 }
 
+// The scalars of a half sweep with factor w (LineCoefs); returns the line matrix' off-diagonal.
+double line_coefs(const Coef& c, double w, int form, int direction, LineCoefs* k)
+{
+    const bool x = direction == 0;
+    const double off = x ? 1.0 : c.b2;    // coefficient along the line
+    const double cross = x ? c.b2 : 1.0;  // coefficient of the neighbouring lines
+    k->wc = w * cross;
+    k->bnd = off / cross;
+    k->c1 = form == LAP_FORM_B ? c.d * (1.0 - w) / k->wc : 0.0;
+    k->omw = 1.0 - w;
+    return form == LAP_FORM_A ? off : w * off;
+}
+
 // Tables, per-call coefficients and (y-lines) scratch of one zebra half sweep; allocates only
 // on the first use of a shape, so calling it before a graph capture prepares the capture.
 const LineTables& line_setup(lap_handle h, const Field& f, const Coef& c, double w, int form,
@@ -357,13 +379,7 @@ const LineTables& line_setup(lap_handle h, const Field& f, const Coef& c, double
 {
     const bool x = direction == 0;
     const int N = x ? f.m - 2 : f.n - 2;
-    const double off = x ? 1.0 : c.b2;    // coefficient along the line
-    const double cross = x ? c.b2 : 1.0;  // coefficient of the neighbouring lines
-    const double alpha = form == LAP_FORM_A ? off : w * off;
-    k->wc = w * cross;
-    k->bnd = off / cross;
-    k->c1 = form == LAP_FORM_B ? c.d * (1.0 - w) / k->wc : 0.0;
-    k->omw = 1.0 - w;
+    const double alpha = line_coefs(c, w, form, direction, k);
     // x-lines long enough for 64 chunks of at least 48 unknowns take the two-warp cut (at 4097^2:
     // 255 -> 242 us per half sweep); shorter chunks would spend most of their length in the
     // boundary layer (about 34 positions at beta = 1), so shorter lines keep 32 chunks
@@ -928,20 +944,55 @@ struct Solver {
         smooth(lv, p->nu2);
     }
 
-    // The whole solve in one CTA (solve_cta_kernel): point methods with the paper's stopping
-    // rule on grids whose sweeps cost less than the launches and host checks of the
-    // multi-CTA path (a block-wide max is order-free, so the test is the host loop's bit for
-    // bit). Red-black and Jacobi up to 4096 points: about the size where one SM sweeps as
-    // fast as two launches take; lexicographic grids always run on one SM.
-    bool solve_cta_ok() const
+    // The whole solve in one CTA: with the paper's stopping rule, on grids whose sweeps cost less
+    // than the launches and host checks of the multi-CTA path. Red-black, Jacobi and the line
+    // methods up to 4096 points: about the size where one SM sweeps as fast as two launches take
+    // (small_kernels.cu); lexicographic grids always run on one SM (solve_cta_kernel).
+    bool lex_cta() const
     {
-        if (p->norm != LAP_NORM_MAXDELTA) return false;
+        return p->norm == LAP_NORM_MAXDELTA && (p->method == LAP_GS_LEX || p->method == LAP_SOR_LEX);
+    }
+    // The point and line methods: runs the solve and returns true, or false where the multi-CTA
+    // path has to take it.
+    bool run_small(lap_result* out)
+    {
+        if (p->norm != LAP_NORM_MAXDELTA || p->max_iter < 1 || !small_points_ok(f.m, f.n)) return false;
         if (p->sum_order == LAP_SUM_DIAGONAL) return false;  // the one-CTA sweeps sum in paper order
-        if (p->method == LAP_GS_LEX || p->method == LAP_SOR_LEX) return true;
-        if (p->method == LAP_ADI || p->method == LAP_SLOR)
-            return (int64_t)f.m * f.n <= 4096 && solve_lines_cta_smem(f.m, f.n) <= 200 * 1024;
-        return (p->method == LAP_JACOBI || p->method == LAP_GS_RB || p->method == LAP_SOR_RB) &&
-               (int64_t)f.m * f.n <= 4096;
+        SmallReport* rep = reinterpret_cast<SmallReport*>(h->pinned);
+        static_assert(sizeof(SmallReport) <= 8 * sizeof(double), "pinned buffer holds 8 doubles");
+        if (p->method == LAP_JACOBI || p->method == LAP_GS_RB || p->method == LAP_SOR_RB) {
+            const bool gs = p->method == LAP_GS_RB;
+            ck(launch_small_point(f, c, p->method == LAP_JACOBI, gs, gs ? 1.0 : p->w, p->check_every,
+                                  p->max_iter, p->tol, rep, s),
+               "one-CTA solve kernel");
+        } else if (p->method == LAP_ADI || p->method == LAP_SLOR) {
+            const bool adi = p->method == LAP_ADI;
+            const int swx = small_line_lanes_log((f.n - 1) / 2, f.m - 2);
+            const int swy = small_line_lanes_log((f.m - 1) / 2, f.n - 2);
+            LineCoefs kx, ky;
+            const LineTables tx = small_line_setup(0, swx, &kx), ty = adi ? small_line_setup(1, swy, &ky) : tx;
+            if (!adi) ky = kx;
+            if (small_line_smem(f.m, f.n, tx, swx, ty, swy, adi) > 200 * 1024) return false;
+            ck(launch_small_line(f, c, adi, p->line_form == LAP_FORM_B ? 1 : 0, tx, kx, swx, ty, ky, swy,
+                                 p->check_every, p->max_iter, p->tol, rep, s),
+               "one-CTA line solve kernel");
+        } else {
+            return false;
+        }
+        ck(cudaStreamSynchronize(s), "stream sync");
+        out->status = rep->status;
+        out->iters = rep->k;
+        out->r0 = rep->r0;
+        out->r_final = rep->r_final;
+        out->last_check = rep->last_check;
+        return true;
+    }
+    // Tables and scalars of one direction for 2^sw lanes per line.
+    LineTables small_line_setup(int direction, int sw, LineCoefs* k)
+    {
+        const int N = direction == 0 ? f.m - 2 : f.n - 2;
+        const double alpha = line_coefs(c, p->w, p->line_form, direction, k);
+        return line_tables(h, N, alpha, c.d, k->wc, 1 << sw, 0);
     }
 
     // The iterations between two stopping tests, enqueued on stream s.
@@ -1182,6 +1233,7 @@ struct Solver {
 
     void run(lap_result* out)
     {
+        if (run_small(out)) return;
         out->status = LAP_MAXITER;
         out->iters = 0;
         out->last_check = NAN;
@@ -1250,8 +1302,8 @@ struct Solver {
         int64_t k = 0;
         double last_nr = r0;             // the L2 norm of the current iterate, when known
         bool last_is_current = p->method != LAP_MG_FP32;
-        if (out->status == LAP_MAXITER && p->max_iter > 0 && solve_cta_ok()) {
-            // small grid, the paper's stopping rule: the whole solve is one kernel
+        if (out->status == LAP_MAXITER && p->max_iter > 0 && lex_cta()) {
+            // lexicographic order, the paper's stopping rule: the whole solve is one kernel
             LoopState st{};
             st.k = 0;
             st.steps = p->check_every;
@@ -1263,15 +1315,7 @@ struct Solver {
             st.last_check = NAN;
             st.last_nr = r0;
             ck(cudaMemcpyAsync(w.loop, &st, sizeof st, cudaMemcpyHostToDevice, s), "upload loop state");
-            if (p->method == LAP_ADI || p->method == LAP_SLOR) {
-                ck(launch_solve_lines_cta(f, c, p->method == LAP_ADI, p->line_form == LAP_FORM_B,
-                                          w.wslot, w.loop, s),
-                   "one-CTA line solve kernel");
-            } else {
-                const int kind = p->method == LAP_JACOBI ? 0 : (p->method == LAP_GS_RB || p->method == LAP_SOR_RB ? 1 : 2);
-                const bool gs = p->method == LAP_GS_RB || p->method == LAP_GS_LEX;
-                ck(launch_solve_cta(f, c, kind, gs, w.wslot, w.loop, s), "one-CTA solve kernel");
-            }
+            ck(launch_solve_cta(f, c, p->method == LAP_GS_LEX, w.wslot, w.loop, s), "one-CTA solve kernel");
             ck(cudaMemcpyAsync(h->pinned, w.loop, sizeof st, cudaMemcpyDeviceToHost, s), "copy loop state");
             ck(cudaStreamSynchronize(s), "stream sync");
             std::memcpy(&st, h->pinned, sizeof st);

@@ -179,17 +179,11 @@ size_t lex_smem_bytes(int m, int n);
 cudaError_t prepare_lex_kernels(size_t smem);
 cudaError_t launch_lex_sweeps(const Field& f, const Coef& c, bool gs, double w, int nsweeps,
                               unsigned long long* maxd, cudaStream_t s);
-// A whole solve in one CTA with the stopping rule of Eq. 16 (max |change| <= tol, tested
-// after every st->steps iterations, up to st->max_iter): kind 0 Jacobi (2 m n doubles of
-// shared memory), 1 red-black, 2 lexicographic (m n doubles); gs or SOR with {w, 1 - w}
-// from wslot. Reads st->k, steps, max_iter, tol, last_check; writes k, status, last_check.
-// Zebra SLOR (adi = false) or ADI in one CTA with the field in shared memory, periods until
-// the stopping rule (MAXDELTA) holds; LoopState as for launch_solve_cta.
-size_t solve_lines_cta_smem(int m, int n);
-cudaError_t launch_solve_lines_cta(const Field& f, const Coef& c, bool adi, int form,
-                                   const double* wslot, LoopState* st, cudaStream_t s);
-cudaError_t launch_solve_cta(const Field& f, const Coef& c, int kind, bool gs, const double* wslot,
-                             LoopState* st, cudaStream_t s);
+// A whole lexicographic solve in one CTA with the stopping rule of Eq. 16 (max |change| <= tol,
+// tested after every st->steps iterations, up to st->max_iter); gs or SOR with {w, 1 - w} from
+// wslot. Reads st->k, steps, max_iter, tol, last_check; writes k, status, last_check.
+cudaError_t launch_solve_cta(const Field& f, const Coef& c, bool gs, const double* wslot, LoopState* st,
+                             cudaStream_t s);
 
 // ---- V-cycle over many grids (batch_kernels.cu) -------------------------------------
 // One level of one problem. Level 0 of the FP64 solve is the caller's field (q null).
@@ -337,9 +331,9 @@ constexpr int LINE_MAX_CHUNKS = 32;    // y-lines (one warp per line's separator
 constexpr int LINE_MAX_CHUNKS_X = 64;  // x-lines (two warps run a line's chunks)
 struct LineTables {
     int N;       // unknowns per line
-    int L;       // chunk length (full chunks)
+    int L;       // chunk length (full chunks; 0: every unknown is a separator, P = N + 1)
     int P;       // chunks (<= maxp); separators S = P - 1
-    int maxp;    // chunk cap of this partition (32 or 64): the row stride of k1 and k2
+    int maxp;    // chunk cap of this partition: the row stride of k1 and k2
     int Ll;      // length of the last chunk (1..L)
     int K0;      // F, gln, glnl are below 2^-64 of their first entry from position K0 on
     int levels;  // cyclic-reduction levels over the S separators
@@ -362,6 +356,43 @@ struct LineCoefs {
     double bnd, c1, omw, wc;
 };
 size_t line_smem_bytes(const LineTables& t);
+
+// ---- whole solves in one CTA (small_kernels.cu) -------------------------------------
+// What such a solve reports, written by the kernel (pinned host memory): iterations done,
+// lap_status, the last test's value (NaN: none), and the residual norms before and after.
+struct SmallReport {
+    long long k;
+    int status;
+    double last_check, r0, r_final;
+};
+// Jacobi or red-black Gauss-Seidel / SOR until max |change| (Eq. 16, tested every `every`
+// iterations) is <= tol, at most max_iter (>= 1) iterations; fields of at most 4096 points.
+bool small_points_ok(int m, int n);
+cudaError_t launch_small_point(const Field& f, const Coef& c, bool jacobi, bool gs, double w,
+                               int64_t every, int64_t max_iter, double tol, SmallReport* rep,
+                               cudaStream_t s);
+// Zebra SLOR (adi false) or ADI under the same rule. tx, ty: tables of the two directions (ty
+// unused by SLOR) for 2^swx and 2^swy lanes per line, see small_line_lanes_log.
+int small_line_lanes_log(int count, int N);  // count: lines of the larger zebra colour
+__host__ __device__ inline int small_line_table_doubles(const LineTables& t)
+{
+    return (int)(t.invb - t.e) + t.maxp;
+}
+// Work space: for every warp's worth of a colour's lines, 32 doubles per chunk position.
+__host__ __device__ inline int small_line_work_doubles(int m, int n, const LineTables& tx, int swx,
+                                                       const LineTables& ty, int swy, bool adi)
+{
+    const int gx = ((n - 1) / 2 + (32 >> swx) - 1) / (32 >> swx), gy = ((m - 1) / 2 + (32 >> swy) - 1) / (32 >> swy);
+    const int x = gx * 32 * (tx.L > 0 ? tx.L : 1), y = adi ? gy * 32 * (ty.L > 0 ? ty.L : 1) : 0;
+    return x > y ? x : y;
+}
+size_t small_line_smem(int m, int n, const LineTables& tx, int swx, const LineTables& ty, int swy, bool adi);
+cudaError_t launch_small_line(const Field& f, const Coef& c, bool adi, int form, const LineTables& tx,
+                              const LineCoefs& kx, int swx, const LineTables& ty, const LineCoefs& ky,
+                              int swy, int64_t every, int64_t max_iter, double tol, SmallReport* rep,
+                              cudaStream_t s);
+
+// ---- line relaxation, continued ------------------------------------------------------
 cudaError_t prepare_line_kernels(size_t smem);
 // x-lines: a whole zebra half sweep of the nlines interior rows (both colours) in one launch.
 // sync: line_x_sync_words(nlines) words of device memory; word 0 is an error word that the
