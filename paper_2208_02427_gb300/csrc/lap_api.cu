@@ -861,6 +861,14 @@ struct Solver {
     std::vector<BatchLevel<float>> hl32;  // FP32 level descriptors (host copy)
     bool fused32 = false;                 // descents/ascents as tile kernels
 
+    // Whether level l's descent and ascent run as row streams (stream32_kernels.cu): they need a
+    // zero ring, which level 0 of FP32 alone does not have. The shared-memory tiles take that level
+    // and the smoothing counts that the streams do not cover.
+    bool stream_level(int l) const
+    {
+        return stream32_supported(p->nu1, p->nu2) && (l > 0 || p->method == LAP_MG_MIXED);
+    }
+
     // The FP32 image of vcycle() on the correction equation. first: the first inner cycle
     // of an outer iteration (the level-0 correction starts at zero).
     void vcycle32(int l, bool first = false, bool fold = false)
@@ -880,9 +888,25 @@ struct Solver {
                "coarse solve kernel");
             return;
         }
+        const bool from_zero = l > 0 || first;
+        if (fused32 && l < L - 1 && stream_level(l)) {
+            const bool gs = p->smoother_w == 1.0;
+            if (from_zero)
+                ck(launch_stream_down(w.tl32, l, lv.u.m, lv.u.n, p->nu1, gs, p->smoother_w,
+                                      l + 1 == tail_first, s),
+                   "descent kernel");
+            else
+                ck(launch_down32(hl32[l], hl32[l + 1], p->nu1, p->nu2, false, gs, p->smoother_w, s),
+                   "descent kernel");
+            vcycle32(l + 1);
+            ck(launch_stream_up(w.tl32, l, lv.u.m, lv.u.n, p->nu2, gs, p->smoother_w, s,
+                                fold && l == 0 ? f.p : nullptr, f.pitch),
+               "ascent kernel");
+            return;
+        }
         if (fused32 && l < L - 1) {
             const bool gs = p->smoother_w == 1.0;
-            ck(launch_down32(hl32[l], hl32[l + 1], p->nu1, p->nu2, l > 0 || first, gs, p->smoother_w, s),
+            ck(launch_down32(hl32[l], hl32[l + 1], p->nu1, p->nu2, from_zero, gs, p->smoother_w, s),
                "descent kernel");
             vcycle32(l + 1);
             ck(launch_up32(hl32[l], hl32[l + 1], p->nu1, p->nu2, gs, p->smoother_w, s,

@@ -27,12 +27,12 @@ int tail_start(const BatchLevel<double>* lv, int nlev, int tail_size)
 void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJob>& jobs,
                  const std::vector<int>& who, const std::vector<int>& base,
                  const std::vector<int>& nlev, const std::vector<BatchLevel<double>>& lv,
-                 int tail_size, std::vector<TileItem>* tiles, int nu1, int nu2, int tile_variant,
-                 int item_points)
+                 int tail_size, std::vector<TileItem>* tiles, std::vector<StreamItem>* streams, int nu1,
+                 int nu2, int tile_variant, bool level0_tiles, int item_points)
 {
     L.fused = tiles != nullptr;
     L.tile_variant = tile_variant;
-    L.tiles.assign(0, {0, 0});
+    const bool rows = tile_variant == FUSED32_STREAMS;
     L.levels = 0;
     for (int q : who) L.levels = std::max(L.levels, nlev[q]);
     L.fine.assign(L.levels, {0, 0});
@@ -40,6 +40,8 @@ void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJ
     L.coarse.assign(L.levels, {0, 0});
     L.tail.assign(L.levels, {0, 0});
     L.tiles.assign(L.levels, {0, 0});
+    L.sdown.assign(L.levels, {0, 0});
+    L.sup.assign(L.levels, {0, 0});
     std::vector<int> t(who.size());
     for (size_t k = 0; k < who.size(); ++k) t[k] = tail_start(&lv[base[who[k]]], nlev[who[k]], tail_size);
     for (int l = 0; l < L.levels; ++l) {
@@ -50,14 +52,36 @@ void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJ
                 add_items(items, base[q] + l, lv[base[q] + l].m, lv[base[q] + l].n, item_points);
         }
         L.fine[l] = {f0, (int)items.size() - f0};
-        if (tiles) {
+        if (tiles && rows) {
+            // strips as long as the level's share of about three waves of warps allows: short ones
+            // spend their steps on halo rows, long ones leave multiprocessors idle at the end
+            int64_t points = 0;
+            for (size_t k = 0; k < who.size(); ++k)
+                if (nlev[who[k]] - 1 > l && l < t[k])
+                    points += (int64_t)lv[base[who[k]] + l].m * lv[base[who[k]] + l].n;
+            const int64_t budget = 3 * 16 * (int64_t)device_sms();
+            std::vector<StreamItem> dn, up;
+            for (size_t k = 0; k < who.size(); ++k) {
+                const int q = who[k];
+                if (!(nlev[q] - 1 > l && l < t[k])) continue;
+                const BatchLevel<double>& d = lv[base[q] + l];
+                const int64_t share = std::max<int64_t>(1, budget * ((int64_t)d.m * d.n) / points);
+                stream32_items(base[q] + l, d.m, d.n, nu1, nu2, share, &dn, &up);
+            }
+            L.sdown[l] = {(int)streams->size(), (int)dn.size()};
+            streams->insert(streams->end(), dn.begin(), dn.end());
+            L.sup[l] = {(int)streams->size(), (int)up.size()};
+            streams->insert(streams->end(), up.begin(), up.end());
+        }
+        if (tiles && (!rows || (l == 0 && level0_tiles))) {
+            const int variant = rows ? 1 : tile_variant;
             const int t0 = (int)tiles->size();
             for (size_t k = 0; k < who.size(); ++k) {
                 const int q = who[k];
                 if (!(nlev[q] - 1 > l && l < t[k])) continue;
                 const BatchLevel<double>& d = lv[base[q] + l];
                 int tx, ty, ntx, nty;
-                fused32_tile_variant(tile_variant, d.m, d.n, nu1, nu2, &tx, &ty, &ntx, &nty);
+                fused32_tile_variant(variant, d.m, d.n, nu1, nu2, &tx, &ty, &ntx, &nty);
                 for (int by = 0; by < nty; ++by)
                     for (int bx = 0; bx < ntx; ++bx)
                         tiles->push_back(TileItem{base[q] + l, 1 + bx * tx, 1 + by * ty, tx, ty});
@@ -125,6 +149,7 @@ struct CandPlan {
     BatchItem* items = nullptr;
     TailJob* jobs = nullptr;
     TileItem* tiles = nullptr;
+    StreamItem* streams = nullptr;
     void* dev = nullptr;
     size_t bytes = 0;
     cudaGraphExec_t exec = nullptr;
@@ -217,10 +242,16 @@ void tuner_values(const lap_params* p, std::vector<int>* tails, std::vector<int>
     *tails = tail_candidates(true, mixed, p->tail_size);
     tilings->clear();
     if (mixed && !p->unfused && fused32_supported(p->nu1, p->nu2) && p->tiling >= 0) {
-        for (int v = 1; v <= FUSED32_VARIANTS; ++v)
-            if ((p->tiling == 0 || p->tiling == v) && fused32_variant_supported(v, p->nu1, p->nu2))
-                tilings->push_back(v);
-        if (p->tiling == 0) tilings->push_back(0);
+        // row streams where they cover the smoothing counts (the tiles and the per-pass kernels were
+        // never faster in any batch measured); else the tile variants and one kernel per pass
+        if (p->tiling == 0 && stream32_supported(p->nu1, p->nu2)) {
+            tilings->push_back(FUSED32_STREAMS);
+        } else {
+            for (int v = 1; v <= FUSED32_VARIANTS; ++v)
+                if ((p->tiling == 0 || p->tiling == v) && fused32_variant_supported(v, p->nu1, p->nu2))
+                    tilings->push_back(v);
+            if (p->tiling == 0) tilings->push_back(0);
+        }
     }
     if (tilings->empty()) tilings->push_back(0);  // one kernel per pass
     if (p->item_points > 0) *items = {p->item_points};
@@ -353,26 +384,32 @@ CandPlan& ensure_candidate(BatchCache& C, int c, const BatchConfig& cfg, const l
     std::vector<BatchItem> items;
     std::vector<TailJob> jobs;
     std::vector<TileItem> tiles;
+    std::vector<StreamItem> streams;
     build_lists(K.L, items, jobs, all_problems, P.base, P.nlev, P.lv64, cfg.tail,
-                cfg.tiles > 0 ? &tiles : nullptr, p->nu1, p->nu2, std::max(1, cfg.tiles), cfg.item);
+                cfg.tiles > 0 ? &tiles : nullptr, &streams, p->nu1, p->nu2, std::max(1, cfg.tiles),
+                p->inner_cycles > 1, cfg.item);
     K.L.claim = cfg.persist != 0 ? C.claim : nullptr;
-    // one allocation: items, jobs, tiles (each 256-byte aligned)
+    // one allocation: items, jobs, tiles, streams (each 256-byte aligned)
     Sizer sz;
     sz.take<BatchItem>(std::max<size_t>(1, items.size()));
     sz.take<TailJob>(std::max<size_t>(1, jobs.size()));
     sz.take<TileItem>(std::max<size_t>(1, tiles.size()));
+    sz.take<StreamItem>(std::max<size_t>(1, streams.size()));
     K.bytes = sz.off;
     K.dev = dev_alloc(C.h, K.bytes);
     Carver cv(K.dev);
     K.items = cv.take<BatchItem>(std::max<size_t>(1, items.size()));
     K.jobs = cv.take<TailJob>(std::max<size_t>(1, jobs.size()));
     K.tiles = cv.take<TileItem>(std::max<size_t>(1, tiles.size()));
+    K.streams = cv.take<StreamItem>(std::max<size_t>(1, streams.size()));
     if (!items.empty())
         ck(cudaMemcpy(K.items, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice), "upload items");
     if (!jobs.empty())
         ck(cudaMemcpy(K.jobs, jobs.data(), jobs.size() * sizeof(TailJob), cudaMemcpyHostToDevice), "upload jobs");
     if (!tiles.empty())
         ck(cudaMemcpy(K.tiles, tiles.data(), tiles.size() * sizeof(TileItem), cudaMemcpyHostToDevice), "upload tiles");
+    if (!streams.empty())
+        ck(cudaMemcpy(K.streams, streams.data(), streams.size() * sizeof(StreamItem), cudaMemcpyHostToDevice), "upload streams");
     return K;
 }
 
@@ -450,7 +487,7 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
                 if (mixed) {
                     for (int k = 0; k < p->inner_cycles; ++k) {
                         if (L.fused)
-                            enqueue_vcycle32_fused(list, L, lv32, active, K.jobs, K.tiles, *p, p->smoother_w,
+                            enqueue_vcycle32_fused(list, L, lv32, active, K.jobs, K.tiles, K.streams, *p, p->smoother_w,
                                                    k == 0, st, k == p->inner_cycles - 1 ? lv64 : nullptr);
                         else
                             enqueue_vcycle(list, L, lv32, active, K.jobs, *p, p->smoother_w, st);

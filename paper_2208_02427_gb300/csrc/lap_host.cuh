@@ -69,7 +69,7 @@ struct BatchConfig {
     int tail;   // small-level tail size (-1: none; see TailTuner)
     int tiles;  // FP32 levels of the mixed solver: 0 = one kernel per pass (temporal depth 1),
                 // 1..FUSED32_VARIANTS = a level's whole descent / ascent per tile load (depth nu)
-                // with that tile variant (CTA size and region rows)
+                // with that tile variant (CTA size and region rows), FUSED32_STREAMS = row streams
     int item;   // interior points per work item of the per-pass kernels
     int persist;  // 1: every phase a persistent launch (resident CTAs claim its items), 0: one CTA per item
     bool operator==(const BatchConfig& o) const
@@ -317,9 +317,10 @@ void add_items(std::vector<BatchItem>& items, int level_index, int m, int n,
 struct LevelLists {
     std::vector<std::pair<int, int>> fine, all, coarse, tail;
     std::vector<std::pair<int, int>> tiles;  // FP32 tile items of the fine lists (fused cycle)
+    std::vector<std::pair<int, int>> sdown, sup;  // the same as pieces of row streams
     std::pair<int, int> upd0{0, 0};  // fused: level-0 items of the problems without level-0 tiles
     bool fused = false;
-    int tile_variant = 1;  // the fused FP32 levels' tile variant
+    int tile_variant = 1;  // the fused FP32 levels' tile variant, or FUSED32_STREAMS
     unsigned* claim = nullptr;  // non-null: every launch persistent, claiming items here (BatchList)
     int levels = 0;
     int max_coarse = 0;
@@ -331,12 +332,15 @@ int tail_start(const BatchLevel<double>* lv, int nlev, int tail_size);
 
 // Lists of one V-cycle over problems `who`: problem q owns levels base[q] .. base[q] +
 // nlev[q] - 1 of lv. Levels above a problem's tail go through item lists, the tail is one job.
-// With tiles, the fine levels also get the tile items of the fused FP32 descent/ascent.
+// With tiles and streams, the fine levels also get the items of the fused FP32 descent/ascent: tile
+// items, or with tile_variant FUSED32_STREAMS pieces of row streams (and level-0 tile items too when
+// level0_tiles: the descents of a later inner cycle do not start from zero).
 void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJob>& jobs,
                  const std::vector<int>& who, const std::vector<int>& base,
                  const std::vector<int>& nlev, const std::vector<BatchLevel<double>>& lv,
-                 int tail_size, std::vector<TileItem>* tiles = nullptr, int nu1 = 0, int nu2 = 0,
-                 int tile_variant = 1, int item_points = BATCH_ITEM_POINTS);
+                 int tail_size, std::vector<TileItem>* tiles = nullptr,
+                 std::vector<StreamItem>* streams = nullptr, int nu1 = 0, int nu2 = 0,
+                 int tile_variant = 1, bool level0_tiles = false, int item_points = BATCH_ITEM_POINTS);
 
 // One V-cycle over every active problem of L: descend (coarsest solves and tails start when
 // the descent reaches a problem's coarsest or tail level), then ascend; each problem sees
@@ -366,30 +370,42 @@ void enqueue_vcycle(ListFn list, const LevelLists& L, const BatchLevel<T>* lv, c
     }
 }
 
-// The FP32 V-cycle with each fine level's descent and ascent as one tile launch over all
-// problems (first: the level-0 corrections start at zero).
+// The FP32 V-cycle with each fine level's descent and ascent as one launch of tiles or row streams
+// over all problems (first: the level-0 corrections start at zero).
 // fold64 (nullable): the level-0 ascent adds its result to these FP64 fields (psi += e).
 template <class ListFn>
 void enqueue_vcycle32_fused(ListFn list, const LevelLists& L, const BatchLevel<float>* lv,
                             const int* active, const TailJob* jobs, const TileItem* tiles,
-                            const lap_params& p, double smoother_w, bool first, cudaStream_t st,
-                            const BatchLevel<double>* fold64 = nullptr)
+                            const StreamItem* streams, const lap_params& p, double smoother_w, bool first,
+                            cudaStream_t st, const BatchLevel<double>* fold64 = nullptr)
 {
-    const bool gs = smoother_w == 1.0;
+    const bool gs = smoother_w == 1.0, rows = L.tile_variant == FUSED32_STREAMS;
+    const int variant = rows ? 1 : L.tile_variant;
     for (int l = 0; l < L.levels; ++l) {
         ck(launch_b_coarse(list(L.coarse[l]), lv, active, L.max_coarse, st), "batched coarse");
         ck(launch_b_tail(jobs + L.tail[l].first, L.tail[l].second, lv, active, p.nu1, p.nu2, gs,
                          smoother_w, L.max_coarse, st, false, L.claim),
            "batched tail");
         if (l == L.levels - 1) break;
-        ck(launch_b_down32(tiles + L.tiles[l].first, L.tiles[l].second, lv, active, p.nu1,
-                           l > 0 || first, gs, smoother_w, st, L.tile_variant, L.claim),
-           "batched descent");
+        if (rows && (l > 0 || first))
+            ck(launch_b_stream_down(streams + L.sdown[l].first, L.sdown[l].second, lv, active, p.nu1, gs,
+                                    smoother_w, st),
+               "batched descent");
+        else
+            ck(launch_b_down32(tiles + L.tiles[l].first, L.tiles[l].second, lv, active, p.nu1,
+                               l > 0 || first, gs, smoother_w, st, variant, L.claim),
+               "batched descent");
     }
-    for (int l = L.levels - 2; l >= 0; --l)
-        ck(launch_b_up32(tiles + L.tiles[l].first, L.tiles[l].second, lv, active, p.nu2, gs,
-                         smoother_w, st, l == 0 ? fold64 : nullptr, L.tile_variant, L.claim),
-           "batched ascent");
+    for (int l = L.levels - 2; l >= 0; --l) {
+        if (rows)
+            ck(launch_b_stream_up(streams + L.sup[l].first, L.sup[l].second, lv, active, p.nu2, gs, smoother_w,
+                                  st, l == 0 ? fold64 : nullptr),
+               "batched ascent");
+        else
+            ck(launch_b_up32(tiles + L.tiles[l].first, L.tiles[l].second, lv, active, p.nu2, gs,
+                             smoother_w, st, l == 0 ? fold64 : nullptr, variant, L.claim),
+               "batched ascent");
+    }
 }
 
 }  // namespace lap

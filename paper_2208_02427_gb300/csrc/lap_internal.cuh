@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <atomic>
 #include <cstdint>
+#include <vector>
 
 namespace lap {
 
@@ -319,6 +320,51 @@ cudaError_t launch_b_up32(const TileItem* items, int count, const BatchLevel<flo
                           const int* active, int nu2, bool gs, double w, cudaStream_t s,
                           const BatchLevel<double>* lv64 = nullptr, int variant = 1,
                           unsigned* claim = nullptr);
+
+// ---- the FP32 cycle's levels as row streams (stream32_kernels.cu) ------------------
+// A warp's piece of level `level`: columns from gx0 on (4 per lane), of which it stores [x0, x1);
+// the warp's 32 lanes in segments of 2^sw_log, segment s storing rows y0 + s rows .. + rows - 1.
+struct StreamItem {
+    int level, gx0, x0, x1, y0, rows, sw_log;
+};
+// How a level of m x n is cut into such pieces: nb column blocks side by side (halos of hl and hr
+// columns between them), strips of `rows` rows in each segment.
+struct StreamCut {
+    int level, m, n, nb, strips, rows, sw_log, hl, hr;
+};
+__host__ __device__ inline StreamItem stream_piece(const StreamCut& c, int index)
+{
+    StreamItem it;
+    const int b = index % c.nb, s = index / c.nb, width = 4 << c.sw_log;
+    it.level = c.level;
+    it.x0 = b == 0 ? 0 : (width - c.hr) + (b - 1) * (width - c.hl - c.hr);
+    it.gx0 = b == 0 ? 0 : it.x0 - c.hl;
+    it.x1 = b == c.nb - 1 ? it.gx0 + width : (width - c.hr) + b * (width - c.hl - c.hr);
+    it.y0 = s * c.rows * (32 >> c.sw_log);
+    it.rows = c.rows;
+    it.sw_log = c.sw_log;
+    return it;
+}
+
+// Whether the streams cover V(nu1, nu2).
+bool stream32_supported(int nu1, int nu2);
+// The descent of level `level` (m x n, lv[level] and lv[level + 1] on the device) from u = 0: nu
+// sweeps, F.r := the smoothed u, C.q := restricted residual, C.u := 0 when zero_c. The ascent:
+// F.u := smoothed (F.r + P C.u) after nu sweeps, or psi += it. Every level buffer's ring must be zero.
+cudaError_t launch_stream_down(const BatchLevel<float>* lv, int level, int m, int n, int nu, bool gs, double w,
+                               bool zero_c, cudaStream_t s);
+cudaError_t launch_stream_up(const BatchLevel<float>* lv, int level, int m, int n, int nu, bool gs, double w,
+                             cudaStream_t s, double* psi = nullptr, int64_t psi_pitch = 0);
+// The same over pieces of many problems' levels; the descent always zeroes C.u. lv64 (nullable):
+// the items' FP64 fields (same level indices) take psi += result instead.
+constexpr int FUSED32_STREAMS = FUSED32_VARIANTS + 1;  // the batched tiling that stands for streams
+void stream32_items(int level, int m, int n, int nu1, int nu2, int64_t warps, std::vector<StreamItem>* down_items,
+                    std::vector<StreamItem>* up_items);
+cudaError_t launch_b_stream_down(const StreamItem* items, int count, const BatchLevel<float>* lv,
+                                 const int* active, int nu, bool gs, double w, cudaStream_t s);
+cudaError_t launch_b_stream_up(const StreamItem* items, int count, const BatchLevel<float>* lv,
+                               const int* active, int nu, bool gs, double w, cudaStream_t s,
+                               const BatchLevel<double>* lv64 = nullptr);
 
 // ---- line relaxation (line_kernels.cu) --------------------------------------------
 // Constant-coefficient tridiagonal systems -alpha x_{k-1} + delta x_k - alpha x_{k+1} = b_k,

@@ -149,6 +149,7 @@ struct SrvPlan {
     std::vector<BatchItem> items;
     std::vector<TailJob> jobs;
     std::vector<TileItem> tiles;
+    std::vector<StreamItem> streams;
     LevelLists mg64, mg32;
     std::pair<int, int> sor, update, init, norm;
     std::vector<int> first_init, first_norm;
@@ -323,7 +324,8 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
             const bool fused = method == LAP_MG_MIXED && !S->mg.unfused &&
                                fused32_supported(S->mg.nu1, S->mg.nu2);
             build_lists(L, P.items, P.jobs, who, base, nlev, P.lv64, ts, fused ? &P.tiles : nullptr,
-                        S->mg.nu1, S->mg.nu2);
+                        &P.streams, S->mg.nu1, S->mg.nu2,
+                        stream32_supported(S->mg.nu1, S->mg.nu2) ? FUSED32_STREAMS : 1, S->mg.inner_cycles > 1);
         };
         mg_lists(LAP_MG, P.mg64);
         mg_lists(LAP_MG_MIXED, P.mg32);
@@ -382,6 +384,7 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
             auto* items = cv.template take<BatchItem>(std::max<size_t>(1, P.items.size()));
             auto* jobs = cv.template take<TailJob>(std::max<size_t>(1, P.jobs.size()));
             auto* tiles = cv.template take<TileItem>(std::max<size_t>(1, P.tiles.size()));
+            auto* streams = cv.template take<StreamItem>(std::max<size_t>(1, P.streams.size()));
             auto* fi = cv.template take<int>(P.first_init.size());
             auto* fn = cv.template take<int>(P.first_norm.size());
             auto* active = cv.template take<int>(R);
@@ -396,7 +399,7 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
             auto* pnorm = cv.template take<double>(std::max(1, P.norm.second));
             auto* done = cv.template take<Completion>(R);
             auto* ndone = cv.template take<int>(1);
-            return std::make_tuple(lv64, lv32, items, jobs, tiles, fi, fn, active, status, remaining,
+            return std::make_tuple(lv64, lv32, items, jobs, tiles, streams, fi, fn, active, status, remaining,
                                    iters, maxit, dr0, rnow, dtol, pinit, pnorm, done, ndone);
         };
         Sizer sz;
@@ -416,11 +419,12 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
         BatchItem* items;
         TailJob* jobs;
         TileItem* tiles;
+        StreamItem* streams;
         int *fi, *fn, *active, *status, *remaining, *ndone;
         long long *iters, *maxit;
         double *dr0, *rnow, *dtol, *pinit, *pnorm;
         Completion* done;
-        std::tie(lv64, lv32, items, jobs, tiles, fi, fn, active, status, remaining, iters, maxit, dr0,
+        std::tie(lv64, lv32, items, jobs, tiles, streams, fi, fn, active, status, remaining, iters, maxit, dr0,
                  rnow, dtol, pinit, pnorm, done, ndone) = carve_stage(cv);
         auto up = [&](void* dst, const void* src, size_t bytes) {
             if (bytes) ck(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st), "upload plan");
@@ -430,6 +434,7 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
         up(items, P.items.data(), P.items.size() * sizeof(BatchItem));
         up(jobs, P.jobs.data(), P.jobs.size() * sizeof(TailJob));
         up(tiles, P.tiles.data(), P.tiles.size() * sizeof(TileItem));
+        up(streams, P.streams.data(), P.streams.size() * sizeof(StreamItem));
         if (P.mg32.fused) ck(prepare_fused32(), "tile kernel attributes");
         up(fi, P.first_init.data(), P.first_init.size() * sizeof(int));
         up(fn, P.first_norm.data(), P.first_norm.size() * sizeof(int));
@@ -449,7 +454,7 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
         enqueue_vcycle(list, P.mg64, lv64, active, jobs, S->mg, S->mg.smoother_w, st);
         for (int k = 0; k < S->mg.inner_cycles && P.mg32.levels; ++k) {
             if (P.mg32.fused)
-                enqueue_vcycle32_fused(list, P.mg32, lv32, active, jobs, tiles, S->mg, S->mg.smoother_w,
+                enqueue_vcycle32_fused(list, P.mg32, lv32, active, jobs, tiles, streams, S->mg, S->mg.smoother_w,
                                        k == 0, st, k == S->mg.inner_cycles - 1 ? lv64 : nullptr);
             else
                 enqueue_vcycle(list, P.mg32, lv32, active, jobs, S->mg, S->mg.smoother_w, st);
