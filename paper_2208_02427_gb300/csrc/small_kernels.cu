@@ -499,11 +499,12 @@ cudaError_t launch_small_point(const Field& f, const Coef& c, bool jacobi, bool 
                                int64_t every, int64_t max_iter, double tol, SmallReport* rep,
                                cudaStream_t s)
 {
-    static std::atomic<size_t> set[24][ATTR_DEVICES];
-    // as many warps as one colour fills (at least 2, at most 16): a warp with idle lanes costs
-    // the FP64 pipe as much as a full one
+    static std::atomic<size_t> set[36][ATTR_DEVICES];
+    // as many warps as one colour fills with 1, 2 or 4 points per thread (at least 2): a warp with
+    // idle lanes, or a point per thread too many, costs the FP64 pipe as much as a full one
     const int per_pass = ((f.m - 2) * (f.n - 2) + 1) / 2;
-    const int threads = std::min(SP_THREADS, std::max(64, (per_pass + 31) / 32 * 32));
+    const int each = per_pass <= SP_THREADS ? 1 : (per_pass <= 2 * SP_THREADS ? 2 : 4);
+    const int threads = std::max(64, ((per_pass + each - 1) / each + 31) / 32 * 32);
     const size_t smem = (jacobi ? 2 : 1) * sizeof(double) * (size_t)f.m * f.n;
     const bool p2 = c.inv_d_shift > 0;
     cudaError_t e = cudaSuccess;
@@ -527,7 +528,9 @@ cudaError_t launch_small_point(const Field& f, const Coef& c, bool jacobi, bool 
             if (p2) LAP_SP(N, false, true, SLOT + 6); else LAP_SP(N, false, false, SLOT + 9); \
         }                                                                                \
     } while (0)
-    if (per_pass <= SP_THREADS) LAP_SPN(1, 0); else LAP_SPN(4, 12);
+    if (each == 1) LAP_SPN(1, 0);
+    else if (each == 2) LAP_SPN(2, 12);
+    else LAP_SPN(4, 24);
 #undef LAP_SPN
 #undef LAP_SP
     note_launch();
