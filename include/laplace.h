@@ -127,11 +127,11 @@ typedef struct {
     int32_t line_form;    /* LAP_ADI, LAP_SLOR: lap_line_form */
     int32_t inner_cycles; /* LAP_MG_MIXED: FP32 V-cycles per FP64 correction (>= 1) */
     int32_t tail_size;    /* LAP_MG, LAP_MG_MIXED, batched: the levels whose sides are all
-                             <= tail_size run as one single-CTA kernel per V-cycle (the
-                             small-level tail: a CTA barrier per phase instead of a launch;
-                             the same arithmetic, so the same iterates bit for bit).
-                             0 = chosen by timing the first cycles of a shape (cached in the
-                             handle), -1 = never; otherwise >= 3 */
+                             <= tail_size run as one kernel per V-cycle (the small-level
+                             tail, on one CTA or a thread-block cluster: a barrier per phase
+                             instead of a launch; the same arithmetic, so the same iterates
+                             bit for bit). 0 = chosen (one grid: by the levels' sizes; a
+                             batch: by timing its first cycles), -1 = never; otherwise >= 3 */
     int32_t unfused;      /* LAP_MG_MIXED: 0 = each FP32 level's descent (smoothing, residual,
                              restriction) and ascent (interpolation, smoothing) run as one
                              shared-memory tile kernel each; non-zero = one kernel per pass

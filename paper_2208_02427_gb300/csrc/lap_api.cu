@@ -516,13 +516,12 @@ int mg_level_count(int m, int n, int coarsest_min, int max_levels)
     return levels;
 }
 
-// Tail sizes worth timing for a batch of V-cycles (one CTA per problem runs the levels at or
-// below the size) and for one grid (one CTA in all).
-std::vector<int> tail_candidates(bool batched, bool fp32, int tail_size)
+// Tail sizes worth timing for a batch of V-cycles (one CTA per problem runs the levels at or below
+// the size).
+std::vector<int> tail_candidates(int tail_size)
 {
     if (tail_size != 0) return {tail_size};
-    if (batched) return {-1, 33, 65, 129, 257};
-    return fp32 ? std::vector<int>{-1, 33, 65, 129, 257} : std::vector<int>{-1, 17, 33, 65};
+    return {-1, 33, 65, 129, 257};
 }
 
 std::string tuner_key(char kind, const lap_params* p, const std::vector<int>& shape)
@@ -767,20 +766,31 @@ struct Solver {
         }
     }
 
-    // First level of the small-level tail in vcycle()/vcycle32() (-1: none), see set_tail.
+    // First level of the small-level tail in vcycle()/vcycle32() (-1: none), see set_tail, and how
+    // it lies in shared memory (bytes 0: not at all, b_tail_kernel).
     int tail_first = -1;
+    SmemTail tail_plan;
 
-    // Run the levels whose sides are both <= S (S > 0) as the tail; -1 = no tail.
+    // The levels that run as the tail: those whose sides are both <= S, none for S = -1, and for S = 0
+    // all from the first one of at most TAIL_POINTS points that fits shared memory. Measured per cycle
+    // with the tail from one level up or down: FP64 257x129 61 us in the tail and 64 us with its two
+    // largest levels outside, 257x257 (66,000 points) 120 us in and 102 us out; mixed 46 and 51 us,
+    // 73 and 71 us.
+    static constexpr int64_t TAIL_POINTS = 40000;
     void set_tail(int S)
     {
         tail_first = -1;
-        if (S <= 0) return;
+        if (S < 0) return;
         const int L = p->method == LAP_MG ? (int)w.levels.size() : (int)w.levels32.size();
         int m = f.m, n = f.n;
         for (int l = 0; l < L; ++l) {
-            if (m <= S && n <= S) {
-                tail_first = l;
-                return;
+            if (S == 0 ? (int64_t)m * n <= TAIL_POINTS : m <= S && n <= S) {
+                tail_plan = p->method == LAP_MG ? plan_smem_tail<double>(m, n, L - l, true)
+                                                : plan_smem_tail<float>(m, n, L - l, true);
+                if (S > 0 || tail_plan.bytes) {
+                    tail_first = l;
+                    return;
+                }
             }
             m = (m - 1) / 2 + 1;
             n = (n - 1) / 2 + 1;
@@ -875,6 +885,12 @@ struct Solver {
     {
         Level32& lv = w.levels32[l];
         const int L = (int)w.levels32.size();
+        if (l == tail_first && tail_plan.bytes) {
+            ck(launch_smem_tail(w.tjob + l, 1, w.tl32, nullptr, p->nu1, p->nu2, p->smoother_w == 1.0, p->smoother_w,
+                                tail_plan, s),
+               "tail kernel");
+            return;
+        }
         if (l == tail_first) {
             ck(launch_b_tail(w.tjob + l, 1, w.tl32, nullptr, p->nu1, p->nu2, p->smoother_w == 1.0,
                              p->smoother_w, coarsest_unknowns(), s),
@@ -947,6 +963,12 @@ struct Solver {
     {
         Level& lv = w.levels[l];
         const int L = (int)w.levels.size();
+        if (l == tail_first && tail_plan.bytes) {
+            ck(launch_smem_tail(w.tjob + l, 1, w.tl64, nullptr, p->nu1, p->nu2, p->smoother_w == 1.0, p->smoother_w,
+                                tail_plan, s),
+               "tail kernel");
+            return;
+        }
         if (l == tail_first) {
             ck(launch_b_tail(w.tjob + l, 1, w.tl64, nullptr, p->nu1, p->nu2, p->smoother_w == 1.0,
                              p->smoother_w, coarsest_unknowns(), s),
@@ -1086,14 +1108,12 @@ struct Solver {
     }
 
     // A period as one CUDA graph: captured once on the handle's own stream, replayed on s.
-    // Returns true when this call captured the graph (its first use).
-    bool run_period(int64_t steps, bool maxdelta, bool fused_maxd)
+    void run_period(int64_t steps, bool maxdelta, bool fused_maxd)
     {
         if (!h->use_graphs) {
             period(steps, maxdelta, fused_maxd);
-            return false;
+            return;
         }
-        bool captured = false;
         const std::string key = graph_key(steps, maxdelta, fused_maxd);
         auto it = h->graphs.find(key);
         if (it == h->graphs.end()) {
@@ -1128,12 +1148,10 @@ struct Solver {
             it = h->graphs.emplace(key, std::make_pair(exec, kernels)).first;
             jac_cur = cur0;  // the host-side ping-pong state advances on replay below
             jac_other = other0;
-            captured = true;
         }
         ck(cudaGraphLaunch(it->second.first, s), "launch graph");
         add_launches(it->second.second);
         if (p->method == LAP_JACOBI && (steps & 1)) std::swap(jac_cur, jac_other);
-        return captured;
     }
 
     // The norm of the stopping test, enqueued on s (the kernels of the host check).
@@ -1155,12 +1173,10 @@ struct Solver {
 
     // Device-resident loop: whole check periods, each followed by the stopping test on the
     // device, as the body of a conditional (while) node of one CUDA graph, so that the host
-    // waits once per solve instead of once per period. Used once the small-level tail is
-    // chosen, for full periods (Jacobi: even periods, whose buffer roles repeat).
-    bool device_loop_ok(int64_t k, int64_t steps, const TailTuner* tuner) const
+    // waits once per solve instead of once per period. For full periods (Jacobi: even periods, whose buffer roles repeat).
+    bool device_loop_ok(int64_t k, int64_t steps) const
     {
         if (!h->use_graphs || steps != p->check_every || k + steps > p->max_iter) return false;
-        if (tuner && !tuner->done) return false;
         if (p->method == LAP_JACOBI && (steps & 1)) return false;
         return true;
     }
@@ -1301,16 +1317,13 @@ struct Solver {
                 ck(launch_defect32_sumsq(l0.u, l0.q, c, w.partials, s), "residual kernel");
             }
         }
-        TailTuner* tuner = nullptr;
         const bool fp32_norm = p->method == LAP_MG_MIXED || p->method == LAP_MG_FP32;
         if (p->method == LAP_MG || fp32_norm) {
             upload_tail();
             if (p->method == LAP_MG_MIXED)
                 ck(launch_zero_rings32(w.tl32, (int)w.levels32.size(), std::max(f.m, f.n), s),
                    "ring kernel");
-            const char kind = p->method == LAP_MG ? 'S' : (p->method == LAP_MG_MIXED ? 'M' : 'F');
-            tuner = &h->tail_tuners[tuner_key(kind, p, {f.m, f.n})];
-            if (tuner->cand.empty()) tuner->init(tail_candidates(false, kind != 'S', p->tail_size));
+            set_tail(p->tail_size);
         }
         // the mixed iteration ends with the FP64 residual's partial sums; FP32 alone with
         // its FP32 residual's
@@ -1354,8 +1367,7 @@ struct Solver {
             const bool fused_maxd = maxdelta && (p->method == LAP_JACOBI || p->method == LAP_GS_RB ||
                                                  p->method == LAP_SOR_RB || p->method == LAP_GS_LEX ||
                                                  p->method == LAP_SOR_LEX);
-            if (tuner && tuner->done) set_tail(tuner->cand[tuner->best]);
-            if (device_loop_ok(k, steps, tuner)) {
+            if (device_loop_ok(k, steps)) {
                 const LoopState st = device_loop(k, r0, last_nr, maxdelta, fused_maxd);
                 k = st.k;
                 out->last_check = st.last_check;
@@ -1368,25 +1380,7 @@ struct Solver {
                 }
                 continue;
             }
-            if (tuner) {
-                // the tail size of this period: the next untried candidate while tuning; a
-                // period that captures its graph is not timed
-                const int cidx = tuner->next();
-                set_tail(tuner->cand[cidx]);
-                if (tuner->done) {
-                    run_period(steps, maxdelta, fused_maxd);
-                } else {
-                    ck(cudaEventRecord(tuner_event(h, 0), s), "record event");
-                    const bool captured = run_period(steps, maxdelta, fused_maxd);
-                    ck(cudaEventRecord(tuner_event(h, 1), s), "record event");
-                    ck(cudaEventSynchronize(tuner_event(h, 1)), "event sync");
-                    float ms = 0.f;
-                    ck(cudaEventElapsedTime(&ms, tuner_event(h, 0), tuner_event(h, 1)), "event time");
-                    if (!captured) tuner->record(cidx, ms / (double)steps);
-                }
-            } else {
-                run_period(steps, maxdelta, fused_maxd);
-            }
+            run_period(steps, maxdelta, fused_maxd);
             k += steps;
             double val;
             bool conv;

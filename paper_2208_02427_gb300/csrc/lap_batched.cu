@@ -42,6 +42,8 @@ void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJ
     L.tiles.assign(L.levels, {0, 0});
     L.sdown.assign(L.levels, {0, 0});
     L.sup.assign(L.levels, {0, 0});
+    L.tail64.assign(L.levels, 0);
+    L.tail32.assign(L.levels, 0);
     std::vector<int> t(who.size());
     for (size_t k = 0; k < who.size(); ++k) t[k] = tail_start(&lv[base[who[k]]], nlev[who[k]], tail_size);
     for (int l = 0; l < L.levels; ++l) {
@@ -106,15 +108,25 @@ void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJ
         }
         L.coarse[l] = {c0, (int)items.size() - c0};
         const int j0 = (int)jobs.size();
+        bool fits64 = true, fits32 = true;
         for (size_t k = 0; k < who.size(); ++k) {
             const int q = who[k];
             if (t[k] == l && l < nlev[q]) {
+                const BatchLevel<double>& f = lv[base[q] + l];
+                const size_t b64 = plan_smem_tail<double>(f.m, f.n, nlev[q] - l, false).bytes;
+                const size_t b32 = plan_smem_tail<float>(f.m, f.n, nlev[q] - l, false).bytes;
+                fits64 = fits64 && b64;
+                fits32 = fits32 && b32;
+                L.tail64[l] = std::max(L.tail64[l], b64);
+                L.tail32[l] = std::max(L.tail32[l], b32);
                 jobs.push_back(TailJob{base[q] + l, base[q] + nlev[q] - 1});
                 const BatchLevel<double>& d = lv[base[q] + nlev[q] - 1];
                 L.max_coarse = std::max(L.max_coarse, (d.m - 2) * (d.n - 2));
             }
         }
         L.tail[l] = {j0, (int)jobs.size() - j0};
+        if (!fits64) L.tail64[l] = 0;
+        if (!fits32) L.tail32[l] = 0;
     }
     if (tiles) {
         const int u0 = (int)items.size();
@@ -239,7 +251,7 @@ void tuner_values(const lap_params* p, std::vector<int>* tails, std::vector<int>
                   std::vector<int>* items, std::vector<int>* persists)
 {
     const bool mixed = p->method == LAP_MG_MIXED;
-    *tails = tail_candidates(true, mixed, p->tail_size);
+    *tails = tail_candidates(p->tail_size);
     tilings->clear();
     if (mixed && !p->unfused && fused32_supported(p->nu1, p->nu2) && p->tiling >= 0) {
         // row streams where they cover the smoothing counts (the tiles and the per-pass kernels were

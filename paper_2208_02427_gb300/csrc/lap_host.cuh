@@ -27,46 +27,9 @@ namespace lap {
 int64_t launches_now();
 void add_launches(int64_t k);
 
-// Chooses the small-level tail size of one shape by timing. The tail changes how a V-cycle
-// is launched and nothing else (every candidate gives the same iterates bit for bit), so
-// the candidates are tried on the first cycles of real solves: each cycle (or check
-// period) runs with the next untried candidate, its device time per cycle is recorded,
-// and once every candidate has been timed the fastest is kept for the handle's lifetime.
-struct TailTuner {
-    std::vector<int> cand;  // tail sizes; -1 = no tail
-    std::vector<double> ms; // best time per cycle seen, +inf = not tried yet
-    int best = 0;
-    bool done = false;
-    void init(std::vector<int> c)
-    {
-        cand = std::move(c);
-        ms.assign(cand.size(), HUGE_VAL);
-        best = 0;
-        done = cand.size() <= 1;
-    }
-    int next() const
-    {
-        if (done) return best;
-        for (size_t i = 0; i < cand.size(); ++i)
-            if (ms[i] == HUGE_VAL) return (int)i;
-        return best;
-    }
-    void record(int i, double v)
-    {
-        if (done || i < 0 || i >= (int)cand.size() || !(v > 0.0)) return;
-        ms[i] = std::min(ms[i], v);
-        bool all = true;
-        for (size_t k = 0; k < cand.size(); ++k) {
-            if (ms[k] == HUGE_VAL) all = false;
-            else if (ms[k] < ms[best] || ms[best] == HUGE_VAL) best = (int)k;
-        }
-        done = all;
-    }
-};
-
 // One launch configuration of a batched V-cycle; none of its choices changes a computed value.
 struct BatchConfig {
-    int tail;   // small-level tail size (-1: none; see TailTuner)
+    int tail;   // small-level tail size (-1: none)
     int tiles;  // FP32 levels of the mixed solver: 0 = one kernel per pass (temporal depth 1),
                 // 1..FUSED32_VARIANTS = a level's whole descent / ascent per tile load (depth nu)
                 // with that tile variant (CTA size and region rows), FUSED32_STREAMS = row streams
@@ -227,8 +190,6 @@ struct lap_handle_s {
     bool use_graphs = true;
     cudaStream_t capture = nullptr;
     std::map<std::string, std::pair<cudaGraphExec_t, int64_t>> graphs;  // exec, kernels
-    // Small-level tail sizes chosen by timing, per shape (see TailTuner)
-    std::map<std::string, lap::TailTuner> tail_tuners;
     std::map<std::string, lap::BatchTuner> batch_tuners;  // batched solves' configurations
     lap::BatchConfig last_batch{0, 0, 0, 0};  // the configuration the last batched cycle ran
     bool last_batch_tuned = false;         // whether its tuner had finished
@@ -299,8 +260,8 @@ constexpr int COARSE_MAX_UNKNOWNS = 1024;
 const double* coarse_inverse(lap_handle h, int m, int n, double b2, double d);
 int mg_level_count(int m, int n, int coarsest_min, int max_levels);
 
-// the timing-based choice of the small-level tail
-std::vector<int> tail_candidates(bool batched, bool fp32, int tail_size);
+// the timing-based choice of a batched solve's configuration
+std::vector<int> tail_candidates(int tail_size);
 std::string tuner_key(char kind, const lap_params* p, const std::vector<int>& shape);
 cudaEvent_t tuner_event(lap_handle h, int k);
 
@@ -324,6 +285,9 @@ struct LevelLists {
     unsigned* claim = nullptr;  // non-null: every launch persistent, claiming items here (BatchList)
     int levels = 0;
     int max_coarse = 0;
+    // shared memory of the tail jobs of a level in FP64 and FP32 (smem_tail_kernel; 0: some job does
+    // not fit, b_tail_kernel)
+    std::vector<size_t> tail64, tail32;
 };
 
 // First level of a problem that the small-level tail runs (both sides <= tail_size), or
@@ -342,6 +306,24 @@ void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJ
                  std::vector<StreamItem>* streams = nullptr, int nu1 = 0, int nu2 = 0,
                  int tile_variant = 1, bool level0_tiles = false, int item_points = BATCH_ITEM_POINTS);
 
+// The tail jobs of level l.
+template <class T>
+void enqueue_tail(const LevelLists& L, int l, const BatchLevel<T>* lv, const int* active, const TailJob* jobs,
+                  const lap_params& p, double smoother_w, cudaStream_t st)
+{
+    const bool gs = smoother_w == 1.0;
+    SmemTail plan;
+    plan.bytes = (sizeof(T) == 8 ? L.tail64 : L.tail32)[l];
+    if (plan.bytes)
+        ck(launch_smem_tail(jobs + L.tail[l].first, L.tail[l].second, lv, active, p.nu1, p.nu2, gs, smoother_w, plan,
+                            st, false, L.claim),
+           "batched tail");
+    else
+        ck(launch_b_tail(jobs + L.tail[l].first, L.tail[l].second, lv, active, p.nu1, p.nu2, gs, smoother_w,
+                         L.max_coarse, st, false, L.claim),
+           "batched tail");
+}
+
 // One V-cycle over every active problem of L: descend (coarsest solves and tails start when
 // the descent reaches a problem's coarsest or tail level), then ascend; each problem sees
 // its own V-cycle.
@@ -352,9 +334,7 @@ void enqueue_vcycle(ListFn list, const LevelLists& L, const BatchLevel<T>* lv, c
     const bool gs = smoother_w == 1.0;
     for (int l = 0; l < L.levels; ++l) {
         ck(launch_b_coarse(list(L.coarse[l]), lv, active, L.max_coarse, st), "batched coarse");
-        ck(launch_b_tail(jobs + L.tail[l].first, L.tail[l].second, lv, active, p.nu1, p.nu2, gs,
-                         smoother_w, L.max_coarse, st, false, L.claim),
-           "batched tail");
+        enqueue_tail(L, l, lv, active, jobs, p, smoother_w, st);
         if (l == L.levels - 1) break;
         for (int k = 0; k < p.nu1; ++k)
             for (int colour = 0; colour < 2; ++colour)
@@ -383,9 +363,7 @@ void enqueue_vcycle32_fused(ListFn list, const LevelLists& L, const BatchLevel<f
     const int variant = rows ? 1 : L.tile_variant;
     for (int l = 0; l < L.levels; ++l) {
         ck(launch_b_coarse(list(L.coarse[l]), lv, active, L.max_coarse, st), "batched coarse");
-        ck(launch_b_tail(jobs + L.tail[l].first, L.tail[l].second, lv, active, p.nu1, p.nu2, gs,
-                         smoother_w, L.max_coarse, st, false, L.claim),
-           "batched tail");
+        enqueue_tail(L, l, lv, active, jobs, p, smoother_w, st);
         if (l == L.levels - 1) break;
         if (rows && (l > 0 || first))
             ck(launch_b_stream_down(streams + L.sdown[l].first, L.sdown[l].second, lv, active, p.nu1, gs,

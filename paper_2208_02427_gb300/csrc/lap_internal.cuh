@@ -259,6 +259,21 @@ template <class T>
 cudaError_t launch_b_tail(const TailJob* jobs, int count, const BatchLevel<T>* lv, const int* active,
                           int nu1, int nu2, bool gs, double w, int max_unknowns, cudaStream_t s,
                           bool per_level_w = false, unsigned* claim = nullptr);
+// The same with every level's u and q in shared memory (tail_kernels.cu): nc = 1 one CTA per job, or
+// one job on a cluster of nc CTAs that split its first ncl levels by rows. bytes = 0: the levels do
+// not fit.
+constexpr int SMEM_TAIL_THREADS = 512;
+struct SmemTail {
+    int nc = 1, ncl = 0;
+    size_t bytes = 0;
+};
+// The plan for the nl levels from an m x n one down (cluster: more than one CTA allowed).
+template <class T>
+SmemTail plan_smem_tail(int m, int n, int nl, bool cluster);
+template <class T>
+cudaError_t launch_smem_tail(const TailJob* jobs, int count, const BatchLevel<T>* lv, const int* active, int nu1,
+                             int nu2, bool gs, double w, const SmemTail& plan, cudaStream_t s,
+                             bool per_level_w = false, unsigned* claim = nullptr);
 // per-item FP64 sum of squares of the residual; with lv32 also r32 := residual, e32 := 0;
 // with r0 (per problem) the mixed problems sum their squares in FP32 after an exact
 // power-of-two scaling from r0 (the partials are stored descaled)
