@@ -573,6 +573,7 @@ struct Work {
     double* nrm = nullptr;       // [sum, sqrt]
     float* nscale = nullptr;     // the mixed solver's norm scale (power of two near 1/||r0||)
     LoopState* loop = nullptr;   // device-resident solve loop state
+    unsigned* done = nullptr;    // blocks of a norm kernel that have finished (NormEnd)
     unsigned long long* maxd = nullptr;
     double* aux = nullptr;       // Jacobi second buffer, or previous iterate for max|delta|
     std::vector<Level> levels;
@@ -591,6 +592,7 @@ void carve(C& cv, Work& w, const lap_grid* g, const lap_params* p)
     w.nrm = cv.template take<double>(2);
     w.nscale = cv.template take<float>(1);
     w.loop = cv.template take<LoopState>(1);
+    w.done = cv.template take<unsigned>(1);
     w.maxd = cv.template take<unsigned long long>(1);
     const size_t field = (size_t)g->n * (size_t)g->pitch;
     const bool need_aux =
@@ -656,31 +658,40 @@ struct Solver {
     const lap_params* p;
     Work w;
 
-    double residual(const Field& u, const double* q)
+    NormEnd sum_only() const
     {
-        ck(launch_defect_sumsq(u, q, c, w.partials, s), "residual kernel");
-        ck(launch_sum_partials(w.partials, norm_blocks(u), w.nrm, s), "sum kernel");
+        NormEnd e;
+        e.nrm = w.nrm;
+        e.done = w.done;
+        return e;
+    }
+
+    double read_norm()
+    {
         ck(cudaMemcpyAsync(h->pinned, w.nrm + 1, sizeof(double), cudaMemcpyDeviceToHost, s),
            "copy norm");
         ck(cudaStreamSynchronize(s), "stream sync");
         return h->pinned[0];
     }
 
-    // Norm from partial sums already written by the last FP64 residual pass (squares of
-    // norm_sc r when scaled).
-    double partial_norm(const Field& u, bool scaled = false)
+    double residual(const Field& u, const double* q)
     {
-        ck(launch_sum_partials(w.partials, mixed_norm_blocks(u.m, u.n), w.nrm, s), "sum kernel");
-        ck(cudaMemcpyAsync(h->pinned, w.nrm + 1, sizeof(double), cudaMemcpyDeviceToHost, s),
-           "copy norm");
-        ck(cudaStreamSynchronize(s), "stream sync");
-        return scaled ? h->pinned[0] / norm_sc : h->pinned[0];
+        ck(launch_defect_sumsq(u, q, c, w.partials, s, sum_only()), "residual kernel");
+        return read_norm();
+    }
+
+    // The norm that the last residual pass of the mixed or FP32 solver left in w.nrm (of norm_sc r
+    // when scaled).
+    double left_norm(bool scaled = false)
+    {
+        const double v = read_norm();
+        return scaled ? v / norm_sc : v;
     }
 
     // The mixed solver sums its iterations' residual squares in FP32 once r0 is known:
     // scale = 2^-e with r0 = f 2^e (so the scaled values stay in FP32's range).
     double norm_sc = 0.0;
-    void set_norm_scale(double r0)
+    void set_norm_scale(double r0, bool upload = true)
     {
         norm_sc = 0.0;
         if (!(r0 > 0.0) || !std::isfinite(r0)) return;
@@ -688,6 +699,7 @@ struct Solver {
         if (e < -100 || e > 100) return;
         norm_sc = std::ldexp(1.0, -e);
         const float v = (float)norm_sc;  // exact: a power of two in FP32's range
+        if (!upload) return;
         // pageable source: staged by the copy before it returns
         ck(cudaMemcpyAsync(w.nscale, &v, sizeof v, cudaMemcpyHostToDevice, s), "upload norm scale");
     }
@@ -715,7 +727,8 @@ struct Solver {
     double* jac_cur = nullptr;  // Jacobi: buffer holding the current iterate
     double* jac_other = nullptr;
 
-    void iterate(bool want_maxd)
+    // norm: what the mixed iteration's closing residual does with its sums
+    void iterate(bool want_maxd, const NormEnd& norm)
     {
         unsigned long long* md = want_maxd ? w.maxd : nullptr;
         const bool gs = p->method == LAP_GS_RB;
@@ -759,7 +772,7 @@ struct Solver {
             // the tiles' first level-0 descent treats e as zero: no need to clear it
             const bool keep_e = fused32 && tail_first != 0 && w.levels32.size() > 1;
             ck(launch_defect64_to32(f, c, l0.q, keep_e ? nullptr : l0.u.p, l0.u.pitch, w.partials, s,
-                                    norm_sc > 0.0 ? w.nscale : nullptr),
+                                    norm_sc > 0.0 ? w.nscale : nullptr, norm),
                "mixed residual kernel");
             break;
         }
@@ -808,64 +821,30 @@ struct Solver {
         return (m - 2) * (n - 2);
     }
 
-    // Level descriptors and tail jobs of this call (level 0 is the caller's field, or the
-    // FP32 correction), uploaded before any period runs.
-    void upload_tail()
+    // Level descriptors of this call (level 0 is the caller's field, or the FP32 correction).
+    template <class T, class LevelOf>
+    std::vector<BatchLevel<T>> describe(int L, LevelOf&& of)
     {
-        const bool mixed = p->method == LAP_MG_MIXED || p->method == LAP_MG_FP32;
-        const int L = mixed ? (int)w.levels32.size() : (int)w.levels.size();
-        std::vector<BatchLevel<double>> d(L);
-        std::vector<BatchLevel<float>> g(L);
-        std::vector<TailJob> jobs(L);
+        std::vector<BatchLevel<T>> d(L);
         int m = f.m, n = f.n;
         for (int l = 0; l < L; ++l) {
-            BatchLevel<double> a{};
+            BatchLevel<T>& a = d[l];
+            of(l, a);
             a.m = m;
             a.n = n;
             a.problem = 0;
             a.unit_beta = c.unit_beta;
+            a.inv_d_shift = sizeof(T) == 8 ? c.inv_d_shift : 0;
             a.b2 = c.b2;
             a.d = c.d;
             a.inv_d = c.inv_d;
             a.w = p->smoother_w;
             a.omw = 1.0 - p->smoother_w;
             a.ainv_t = l == L - 1 ? coarse_inverse(h, m, n, c.b2, c.d) : nullptr;
-            if (mixed) {
-                BatchLevel<float> b{};
-                b.u = w.levels32[l].u.p;
-                b.q = w.levels32[l].q;
-                b.r = w.levels32[l].r;
-                b.m = m;
-                b.n = n;
-                b.pitch = w.levels32[l].u.pitch;
-                b.unit_beta = a.unit_beta;
-                b.inv_d_shift = 0;
-                b.b2 = a.b2;
-                b.d = a.d;
-                b.inv_d = a.inv_d;
-                b.w = a.w;
-                b.omw = a.omw;
-                b.ainv_t = a.ainv_t;
-                g[l] = b;
-            } else {
-                a.u = w.levels[l].u.p;
-                a.q = w.levels[l].q;
-                a.r = w.levels[l].r;
-                a.pitch = w.levels[l].u.pitch;
-                a.inv_d_shift = c.inv_d_shift;
-                d[l] = a;
-            }
-            jobs[l] = TailJob{l, L - 1};
             m = (m - 1) / 2 + 1;
             n = (n - 1) / 2 + 1;
         }
-        // pageable sources: the copies are staged before the calls return
-        if (mixed) hl32 = g;
-        if (mixed)
-            ck(cudaMemcpyAsync(w.tl32, g.data(), L * sizeof(g[0]), cudaMemcpyHostToDevice, s), "upload levels");
-        else
-            ck(cudaMemcpyAsync(w.tl64, d.data(), L * sizeof(d[0]), cudaMemcpyHostToDevice, s), "upload levels");
-        ck(cudaMemcpyAsync(w.tjob, jobs.data(), L * sizeof(TailJob), cudaMemcpyHostToDevice, s), "upload jobs");
+        return d;
     }
 
     std::vector<BatchLevel<float>> hl32;  // FP32 level descriptors (host copy)
@@ -1042,7 +1021,8 @@ struct Solver {
     }
 
     // The iterations between two stopping tests, enqueued on stream s.
-    void period(int64_t steps, bool maxdelta, bool fused_maxd)
+    // norm: the end of the period's last residual (mixed solver)
+    void period(int64_t steps, bool maxdelta, bool fused_maxd, const NormEnd& norm)
     {
         if (p->method == LAP_GS_LEX || p->method == LAP_SOR_LEX) {
             // the whole period in one launch (the field stays in shared memory)
@@ -1064,7 +1044,7 @@ struct Solver {
                 ck(cudaMemsetAsync(w.maxd, 0, 8, s), "zero max delta");
                 if (!fused_maxd) copy_field(w.aux, f.p);
             }
-            iterate(last && fused_maxd);
+            iterate(last && fused_maxd, last ? norm : NormEnd{});
         }
     }
 
@@ -1111,7 +1091,7 @@ struct Solver {
     void run_period(int64_t steps, bool maxdelta, bool fused_maxd)
     {
         if (!h->use_graphs) {
-            period(steps, maxdelta, fused_maxd);
+            period(steps, maxdelta, fused_maxd, sum_only());
             return;
         }
         const std::string key = graph_key(steps, maxdelta, fused_maxd);
@@ -1129,7 +1109,7 @@ struct Solver {
             s = h->capture;
             cudaGraph_t g = nullptr;
             try {
-                period(steps, maxdelta, fused_maxd);
+                period(steps, maxdelta, fused_maxd, sum_only());
             } catch (...) {
                 s = caller;
                 cudaStreamEndCapture(h->capture, &g);
@@ -1154,20 +1134,30 @@ struct Solver {
         if (p->method == LAP_JACOBI && (steps & 1)) std::swap(jac_cur, jac_other);
     }
 
-    // The norm of the stopping test, enqueued on s (the kernels of the host check).
-    void enqueue_norm(bool maxdelta, bool fused_maxd, const Field& cur)
+    // The residual norm of the current iterate with `end`, enqueued on s. (The mixed iteration's own
+    // residual takes it.)
+    void enqueue_norm(const Field& cur, const NormEnd& end)
     {
-        if (maxdelta) {
-            if (!fused_maxd) ck(launch_maxdelta(f, w.aux, w.maxd, s), "max delta kernel");
+        if (p->method == LAP_MG_FP32)
+            ck(launch_defect32_sumsq(w.levels32[0].u, w.levels32[0].q, c, w.partials, s, end), "residual kernel");
+        else if (p->method != LAP_MG_MIXED)
+            ck(launch_defect_sumsq(cur, nullptr, c, w.partials, s, end), "residual kernel");
+    }
+
+    // The first residual of a solve: the mixed and the FP32 solver's first right-hand side and field too.
+    void enqueue_first(const NormEnd& end)
+    {
+        if (p->method == LAP_MG_MIXED) {
+            const Level32& l0 = w.levels32[0];
+            ck(launch_defect64_to32(f, c, l0.q, l0.u.p, l0.u.pitch, w.partials, s, nullptr, end),
+               "mixed residual kernel");
         } else if (p->method == LAP_MG_FP32) {
-            ck(launch_defect32_sumsq(w.levels32[0].u, w.levels32[0].q, c, w.partials, s),
-               "residual kernel");
-            ck(launch_sum_partials(w.partials, mixed_norm_blocks(f.m, f.n), w.nrm, s), "sum kernel");
-        } else if (p->method == LAP_MG_MIXED) {
-            ck(launch_sum_partials(w.partials, mixed_norm_blocks(f.m, f.n), w.nrm, s), "sum kernel");
+            // FP32 alone: psi (ring included) rounded into level 0's two buffers, q = 0
+            const Level32& l0 = w.levels32[0];
+            ck(launch_to32(f, l0.u.p, l0.r, l0.u.pitch, s), "conversion kernel");
+            ck(launch_defect32_sumsq(l0.u, l0.q, c, w.partials, s, end), "residual kernel");
         } else {
-            ck(launch_defect_sumsq(cur, nullptr, c, w.partials, s), "residual kernel");
-            ck(launch_sum_partials(w.partials, norm_blocks(cur), w.nrm, s), "sum kernel");
+            ck(launch_defect_sumsq(f, nullptr, c, w.partials, s, end), "residual kernel");
         }
     }
 
@@ -1182,12 +1172,16 @@ struct Solver {
     }
 
     // Runs periods on the device until the stopping rule holds or the next period would pass
-    // max_iter; returns the loop state read back.
-    LoopState device_loop(int64_t k, double r0, double last_nr, bool maxdelta, bool fused_maxd)
+    // max_iter; returns the loop state read back. first: the graph starts with the solve's first
+    // residual, which decides whether the loop runs at all (the state is in place, see setup()); else
+    // the loop goes on from iteration k.
+    LoopState device_loop(bool first, int64_t k, double r0, double last_nr, bool maxdelta, bool fused_maxd)
     {
         const int64_t steps = p->check_every;
-        const bool scaled = p->method == LAP_MG_MIXED && norm_sc > 0.0;
-        const std::string key = graph_key(steps, maxdelta, fused_maxd) + (scaled ? "|loop-scaled" : "|loop");
+        const bool mixed = p->method == LAP_MG_MIXED;
+        if (first && mixed) norm_sc = 1.0;  // the iterations read their scale from w.nscale
+        const bool scaled = mixed && norm_sc > 0.0;
+        const std::string key = graph_key(steps, maxdelta, fused_maxd) + (first ? "|solve" : "|loop");
         auto it = h->graphs.find(key);
         if (it == h->graphs.end()) {
             prepare();
@@ -1201,31 +1195,20 @@ struct Solver {
             cudaStream_t caller = s;
             double* cur0 = jac_cur;
             double* other0 = jac_other;
-            try {
-                cudaGraphConditionalHandle hnd;
-                ck(cudaGraphConditionalHandleCreate(&hnd, g, 1, cudaGraphCondAssignDefault),
-                   "conditional handle");
-                // zero-initialised node parameters (the struct's union has no default constructor)
-                alignas(cudaGraphNodeParams) unsigned char raw[sizeof(cudaGraphNodeParams)] = {};
-                cudaGraphNodeParams* np = reinterpret_cast<cudaGraphNodeParams*>(raw);
-                np->type = cudaGraphNodeTypeConditional;
-                np->conditional.handle = hnd;
-                np->conditional.type = cudaGraphCondTypeWhile;
-                np->conditional.size = 1;
-                cudaGraphNode_t node;
-                ck(cudaGraphAddNode(&node, g, nullptr, nullptr, 0, np), "conditional node");
-                cudaGraph_t body = np->conditional.phGraph_out[0];
-                const int64_t before = launches_now();
-                ck(cudaStreamBeginCaptureToGraph(h->capture, body, nullptr, nullptr, 0,
+            // f's launches as nodes of graph `into`; returns the last one
+            auto captured = [&](cudaGraph_t into, auto&& body) {
+                ck(cudaStreamBeginCaptureToGraph(h->capture, into, nullptr, nullptr, 0,
                                                  cudaStreamCaptureModeThreadLocal),
                    "begin capture");
                 s = h->capture;
+                cudaGraphNode_t last = nullptr;
                 try {
-                    period(steps, maxdelta, fused_maxd);
-                    const Field cur{p->method == LAP_JACOBI ? jac_cur : f.p, f.m, f.n, f.pitch};
-                    enqueue_norm(maxdelta, fused_maxd, cur);
-                    ck(launch_loop_decide(w.loop, w.nrm, w.maxd, scaled ? w.nscale : nullptr, hnd, s),
-                       "loop test kernel");
+                    body();
+                    cudaStreamCaptureStatus status;
+                    const cudaGraphNode_t* deps = nullptr;
+                    size_t count = 0;
+                    ck(cudaStreamGetCaptureInfo(s, &status, nullptr, nullptr, &deps, nullptr, &count), "capture info");
+                    if (count == 1) last = deps[0];
                 } catch (...) {
                     s = caller;
                     cudaGraph_t junk = nullptr;
@@ -1234,8 +1217,47 @@ struct Solver {
                     throw;
                 }
                 s = caller;
-                cudaGraph_t body_out = nullptr;
-                ck(cudaStreamEndCapture(h->capture, &body_out), "end capture");
+                cudaGraph_t out = nullptr;
+                ck(cudaStreamEndCapture(h->capture, &out), "end capture");
+                return last;
+            };
+            try {
+                cudaGraphConditionalHandle hnd;
+                ck(cudaGraphConditionalHandleCreate(&hnd, g, 1, cudaGraphCondAssignDefault),
+                   "conditional handle");
+                NormEnd end = sum_only();
+                end.loop = w.loop;
+                end.handle = hnd;
+                const int64_t before = launches_now();
+                cudaGraphNode_t head = nullptr;
+                if (first) {
+                    NormEnd start = end;
+                    start.first = true;
+                    start.scale_out = mixed ? w.nscale : nullptr;
+                    head = captured(g, [&] { enqueue_first(start); });
+                    if (!head) fail(LAP_ECUDA, "internal: the first residual is not one chain of nodes");
+                    add_launches(before - launches_now());
+                }
+                // zero-initialised node parameters (the struct's union has no default constructor)
+                alignas(cudaGraphNodeParams) unsigned char raw[sizeof(cudaGraphNodeParams)] = {};
+                cudaGraphNodeParams* np = reinterpret_cast<cudaGraphNodeParams*>(raw);
+                np->type = cudaGraphNodeTypeConditional;
+                np->conditional.handle = hnd;
+                np->conditional.type = cudaGraphCondTypeWhile;
+                np->conditional.size = 1;
+                cudaGraphNode_t node;
+                ck(cudaGraphAddNode(&node, g, first ? &head : nullptr, nullptr, first ? 1 : 0, np),
+                   "conditional node");
+                captured(np->conditional.phGraph_out[0], [&] {
+                    end.scale = scaled ? w.nscale : nullptr;
+                    period(steps, maxdelta, fused_maxd, end);
+                    if (maxdelta) {
+                        if (!fused_maxd) ck(launch_maxdelta(f, w.aux, w.maxd, s), "max delta kernel");
+                        ck(launch_loop_decide(w.loop, w.maxd, hnd, s), "loop test kernel");
+                    } else {
+                        enqueue_norm(Field{p->method == LAP_JACOBI ? jac_cur : f.p, f.m, f.n, f.pitch}, end);
+                    }
+                });
                 kernels = launches_now() - before;
                 add_launches(-kernels);
                 ck(cudaGraphInstantiate(&exec, g, 0), "instantiate graph");
@@ -1251,24 +1273,54 @@ struct Solver {
             jac_other = other0;
             it = h->graphs.emplace(key, std::make_pair(exec, kernels)).first;
         }
-        LoopState st{};
-        st.k = k;
-        st.steps = steps;
-        st.max_iter = p->max_iter;
-        st.mode = maxdelta ? 2 : (p->norm == LAP_NORM_L2_REL ? 0 : 1);
-        st.status = LAP_MAXITER;
-        st.r0 = r0;
-        st.tol = p->tol;
-        st.last_check = NAN;
-        st.last_nr = last_nr;
+        LoopState st = start_state();
         static_assert(sizeof(LoopState) <= 8 * sizeof(double), "pinned buffer holds 8 doubles");
-        ck(cudaMemcpyAsync(w.loop, &st, sizeof st, cudaMemcpyHostToDevice, s), "upload loop state");
+        if (!first) {
+            st.k = k;
+            st.r0 = r0;
+            st.last_nr = last_nr;
+            ck(cudaMemcpyAsync(w.loop, &st, sizeof st, cudaMemcpyHostToDevice, s), "upload loop state");
+        }
         ck(cudaGraphLaunch(it->second.first, s), "launch graph");
         ck(cudaMemcpyAsync(h->pinned, w.loop, sizeof st, cudaMemcpyDeviceToHost, s), "copy loop state");
         ck(cudaStreamSynchronize(s), "stream sync");
         std::memcpy(&st, h->pinned, sizeof st);
-        add_launches(it->second.second * ((st.k - k) / steps));
+        add_launches(it->second.second * ((st.k - k) / steps) + (first ? 1 : 0));
         return st;
+    }
+
+    // The loop state of a solve that has not begun.
+    LoopState start_state() const
+    {
+        LoopState st{};
+        st.steps = p->check_every;
+        st.max_iter = p->max_iter;
+        st.mode = p->norm == LAP_NORM_MAXDELTA ? 2 : (p->norm == LAP_NORM_L2_REL ? 0 : 1);
+        st.status = LAP_MAXITER;
+        st.tol = p->tol;
+        st.last_check = NAN;
+        return st;
+    }
+
+    // The solve's small state on the device, and the multigrid levels' (level 0 is the caller's field,
+    // or the FP32 correction): one launch before anything else.
+    template <class T>
+    void setup(double wv, int levels, int rings, BatchLevel<T>* lv, const std::vector<BatchLevel<T>>& level)
+    {
+        if (levels > SETUP_LEVELS) fail(LAP_EUNSUPPORTED, "more than 24 multigrid levels");
+        SolveSetup<T> a{};
+        a.w = wv;
+        a.omw = 1.0 - wv;
+        a.state = start_state();
+        a.wslot = w.wslot;
+        a.loop = w.loop;
+        a.done = w.done;
+        a.levels = levels;
+        a.rings = rings;
+        a.lv = lv;
+        a.jobs = w.tjob;
+        std::copy(level.begin(), level.end(), a.level);
+        ck(launch_setup(a, s), "setup kernel");
     }
 
     void run(lap_result* out)
@@ -1277,68 +1329,79 @@ struct Solver {
         out->status = LAP_MAXITER;
         out->iters = 0;
         out->last_check = NAN;
-        {
-            const double wv = p->method == LAP_MG ? p->smoother_w : p->w;
-            const double pair[2] = {wv, 1.0 - wv};  // staged by the copy before it returns
-            ck(cudaMemcpyAsync(w.wslot, pair, sizeof pair, cudaMemcpyHostToDevice, s), "upload w");
-        }
         if (p->method == LAP_ADI || p->method == LAP_SLOR) prepare();  // tables, scratch: before any capture
         if (p->method == LAP_JACOBI) {
             copy_field(w.aux, f.p);  // ring + initial interior in both buffers
             jac_cur = f.p;
             jac_other = w.aux;
         }
+        const bool fp32_norm = p->method == LAP_MG_MIXED || p->method == LAP_MG_FP32;
         if (p->method == LAP_MG) {
+            // interiors of the levels below are written before they are read; their rings stay zero
             w.levels[0].u.p = f.p;
-            for (size_t l = 1; l < w.levels.size(); ++l) {
-                const Field& u = w.levels[l].u;
-                ck(cudaMemsetAsync(u.p, 0, (size_t)u.n * u.pitch * 8, s), "zero coarse level");
-                ck(cudaMemsetAsync(w.levels[l].q, 0, (size_t)u.n * u.pitch * 8, s), "zero source");
-            }
-        }
-        if (p->method == LAP_MG_MIXED || p->method == LAP_MG_FP32) {
+            const auto d = describe<double>((int)w.levels.size(), [&](int l, BatchLevel<double>& a) {
+                a.u = w.levels[l].u.p;
+                a.q = w.levels[l].q;
+                a.r = w.levels[l].r;
+                a.pitch = w.levels[l].u.pitch;
+            });
+            setup<double>(p->smoother_w, (int)d.size(), 1, w.tl64, d);
+            set_tail(p->tail_size);
+        } else if (fp32_norm) {
+            hl32 = describe<float>((int)w.levels32.size(), [&](int l, BatchLevel<float>& a) {
+                a.u = w.levels32[l].u.p;
+                a.q = w.levels32[l].q;
+                a.r = w.levels32[l].r;
+                a.pitch = w.levels32[l].u.pitch;
+            });
             // FP32 alone needs its level-0 source zero; the mixed solver writes every interior
-            // before reading it and needs only the rings zero (after upload_tail, below)
+            // before reading it
             if (p->method == LAP_MG_FP32)
                 for (const Level32& lv : w.levels32) {
                     ck(cudaMemsetAsync(lv.u.p, 0, (size_t)lv.u.n * lv.u.pitch * 4, s), "zero level");
                     ck(cudaMemsetAsync(lv.q, 0, (size_t)lv.u.n * lv.u.pitch * 4, s), "zero source");
                     if (lv.r) ck(cudaMemsetAsync(lv.r, 0, (size_t)lv.u.n * lv.u.pitch * 4, s), "zero level");
                 }
+            setup<float>(p->w, (int)hl32.size(), 0, w.tl32, hl32);
+            set_tail(p->tail_size);
             fused32 = !p->unfused && fused32_supported(p->nu1, p->nu2);
             if (fused32) ck(prepare_fused32(), "tile kernel attributes");
-            const Level32& l0 = w.levels32[0];
-            if (p->method == LAP_MG_MIXED) {
-                ck(launch_defect64_to32(f, c, l0.q, l0.u.p, l0.u.pitch, w.partials, s),
-                   "mixed residual kernel");
-            } else {
-                // FP32 alone: psi (ring included) rounded into level 0's two buffers, q = 0
-                ck(launch_to32(f, l0.u.p, l0.r, l0.u.pitch, s), "conversion kernel");
-                ck(launch_defect32_sumsq(l0.u, l0.q, c, w.partials, s), "residual kernel");
+        } else {
+            setup<double>(p->w, 0, 0, nullptr, {});
+        }
+        const bool maxdelta = p->norm == LAP_NORM_MAXDELTA;
+        const bool fused_maxd = maxdelta && (p->method == LAP_JACOBI || p->method == LAP_GS_RB ||
+                                             p->method == LAP_SOR_RB || p->method == LAP_GS_LEX ||
+                                             p->method == LAP_SOR_LEX);
+        int64_t k = 0;
+        double r0, last_nr;
+        bool last_is_current = p->method != LAP_MG_FP32;  // last_nr: the L2 norm of the current iterate
+        // the whole solve on the device, its first residual included (FP32 alone starts with more than
+        // one kernel; Eq. 16 needs no more than the norm r0 from it, and lexicographic grids no graph)
+        const bool whole = p->max_iter > 0 && device_loop_ok(0, p->check_every) && !lex_cta() &&
+                           p->method != LAP_MG_FP32;
+        if (whole) {
+            const LoopState st = device_loop(true, 0, 0.0, 0.0, maxdelta, fused_maxd);
+            r0 = st.r0;
+            last_nr = st.last_nr;
+            k = st.k;
+            if (maxdelta && k > 0) last_is_current = false;
+            out->r0 = r0;
+            out->status = st.status == LOOP_NO_SCALE ? (int)LAP_MAXITER : st.status;
+            out->last_check = st.last_check;
+            if (p->method == LAP_MG_MIXED) set_norm_scale(r0, false);
+        } else {
+            enqueue_first(sum_only());
+            r0 = last_nr = read_norm();
+            out->r0 = r0;
+            if (p->method == LAP_MG_MIXED) set_norm_scale(r0);
+            if (!std::isfinite(r0)) {
+                out->status = LAP_DIVERGED;
+            } else if ((p->norm == LAP_NORM_L2_REL && r0 == 0.0) ||
+                       (p->norm == LAP_NORM_L2_ABS && r0 <= p->tol)) {
+                out->status = LAP_CONVERGED;
             }
         }
-        const bool fp32_norm = p->method == LAP_MG_MIXED || p->method == LAP_MG_FP32;
-        if (p->method == LAP_MG || fp32_norm) {
-            upload_tail();
-            if (p->method == LAP_MG_MIXED)
-                ck(launch_zero_rings32(w.tl32, (int)w.levels32.size(), std::max(f.m, f.n), s),
-                   "ring kernel");
-            set_tail(p->tail_size);
-        }
-        // the mixed iteration ends with the FP64 residual's partial sums; FP32 alone with
-        // its FP32 residual's
-        const double r0 = fp32_norm ? partial_norm(f) : residual(f, nullptr);
-        out->r0 = r0;
-        if (p->method == LAP_MG_MIXED) set_norm_scale(r0);
-        if (!std::isfinite(r0)) {
-            out->status = LAP_DIVERGED;
-        } else if ((p->norm == LAP_NORM_L2_REL && r0 == 0.0) ||
-                   (p->norm == LAP_NORM_L2_ABS && r0 <= p->tol)) {
-            out->status = LAP_CONVERGED;
-        }
-        int64_t k = 0;
-        double last_nr = r0;             // the L2 norm of the current iterate, when known
-        bool last_is_current = p->method != LAP_MG_FP32;
         if (out->status == LAP_MAXITER && p->max_iter > 0 && lex_cta()) {
             // lexicographic order, the paper's stopping rule: the whole solve is one kernel
             LoopState st{};
@@ -1363,12 +1426,8 @@ struct Solver {
         }
         while (out->status == LAP_MAXITER && k < p->max_iter) {
             const int64_t steps = std::min<int64_t>(p->check_every - (k % p->check_every), p->max_iter - k);
-            const bool maxdelta = p->norm == LAP_NORM_MAXDELTA;
-            const bool fused_maxd = maxdelta && (p->method == LAP_JACOBI || p->method == LAP_GS_RB ||
-                                                 p->method == LAP_SOR_RB || p->method == LAP_GS_LEX ||
-                                                 p->method == LAP_SOR_LEX);
             if (device_loop_ok(k, steps)) {
-                const LoopState st = device_loop(k, r0, last_nr, maxdelta, fused_maxd);
+                const LoopState st = device_loop(false, k, r0, last_nr, maxdelta, fused_maxd);
                 k = st.k;
                 out->last_check = st.last_check;
                 out->status = st.status;
@@ -1391,12 +1450,8 @@ struct Solver {
                 conv = val <= p->tol;
                 last_is_current = false;
             } else {
-                const Field cur{p->method == LAP_JACOBI ? jac_cur : f.p, f.m, f.n, f.pitch};
-                if (p->method == LAP_MG_FP32)
-                    ck(launch_defect32_sumsq(w.levels32[0].u, w.levels32[0].q, c, w.partials, s),
-                       "residual kernel");
-                const double nr = fp32_norm ? partial_norm(f, p->method == LAP_MG_MIXED && norm_sc > 0.0)
-                                            : residual(cur, nullptr);
+                enqueue_norm(Field{p->method == LAP_JACOBI ? jac_cur : f.p, f.m, f.n, f.pitch}, sum_only());
+                const double nr = left_norm(p->method == LAP_MG_MIXED && norm_sc > 0.0);
                 val = p->norm == LAP_NORM_L2_REL ? nr / r0 : nr;
                 conv = p->norm == LAP_NORM_L2_REL ? nr <= p->tol * r0 : nr <= p->tol;
                 last_nr = nr;

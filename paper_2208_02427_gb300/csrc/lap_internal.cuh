@@ -87,6 +87,31 @@ cudaError_t launch_defect(const Field& f, const double* q, double* r, const Coef
 int device_sms();
 // The most partial sums a norm kernel writes: its solve-scratch buffers hold this many.
 constexpr int NORM_PARTIALS_MAX = 2046;
+// State of a device-resident solve loop (host-written before launch, read back after).
+struct LoopState {
+    long long k;         // iterations done
+    long long steps;     // iterations per period
+    long long max_iter;
+    int mode;            // 0 L2_REL, 1 L2_ABS, 2 MAXDELTA
+    int status;          // lap_status of the last test
+    double r0, tol;
+    double last_check;   // the last test's value
+    double last_nr;      // the L2 norm at the last test
+};
+constexpr int LOOP_NO_SCALE = 3;  // LoopState::status, see norm_end.cuh
+// What the last block of a norm kernel does with the blocks' sums (norm_end.cuh): nothing (done null);
+// nrm[0] := their sum, nrm[1] := its square root; and with loop the stopping test of a device-resident
+// solve (or, first, the test of its initial residual, and the mixed solver's norm scale to scale_out),
+// which sets the loop's condition `handle`. done: a zeroed word, left zero.
+struct NormEnd {
+    double* nrm = nullptr;
+    unsigned* done = nullptr;
+    LoopState* loop = nullptr;
+    const float* scale = nullptr;  // the norm is of scaled values (divided by *scale)
+    float* scale_out = nullptr;
+    cudaGraphConditionalHandle handle = 0;
+    bool first = false;
+};
 // sum of squares of the residual into per-block partials; partials[nblocks].
 // Blocks of the norm kernels (256 threads, a grid-stride walk over the interior): one per 256
 // interior points, at least 1 and at most 6 per multiprocessor of the current device, all
@@ -101,7 +126,7 @@ inline int norm_blocks_for(int m, int n)
 }
 int norm_blocks(const Field& f);
 cudaError_t launch_defect_sumsq(const Field& f, const double* q, const Coef& c, double* partials,
-                                cudaStream_t s);
+                                cudaStream_t s, const NormEnd& end = NormEnd{});
 // out[0] = sum(partials[0..count)), fixed order; out[1] = sqrt(out[0]).
 cudaError_t launch_sum_partials(const double* partials, int count, double* out, cudaStream_t s);
 // FP64 fma issue-rate probe: blocks x 256 threads, `iters` steps of 8 independent fma chains
@@ -111,21 +136,9 @@ int64_t launch_fp64_rate(int blocks, long long iters, double* sink, cudaStream_t
 // *bad += mismatches of the integer-pipe FP64 -> FP32 rounding against the instruction.
 cudaError_t launch_check_rounding(long long count, unsigned long long seed, unsigned long long* bad,
                                   cudaStream_t s);
-// State of a device-resident solve loop (host-written before launch, read back after).
-struct LoopState {
-    long long k;         // iterations done
-    long long steps;     // iterations per period
-    long long max_iter;
-    int mode;            // 0 L2_REL, 1 L2_ABS, 2 MAXDELTA
-    int status;          // lap_status of the last test
-    double r0, tol;
-    double last_check;   // the last test's value
-    double last_nr;      // the L2 norm at the last test
-};
-// k += steps; test nrm[1] (divided by *scale when scale is set) or *maxd (MAXDELTA);
-// cudaGraphSetConditional(h, keep going).
-cudaError_t launch_loop_decide(LoopState* st, const double* nrm, const unsigned long long* maxd,
-                               const float* scale, cudaGraphConditionalHandle h, cudaStream_t s);
+// The stopping test of a loop on *maxd (MAXDELTA): cudaGraphSetConditional(h, keep going).
+cudaError_t launch_loop_decide(LoopState* st, const unsigned long long* maxd, cudaGraphConditionalHandle h,
+                               cudaStream_t s);
 // Batched solves: st[0] += 1 (cycles done), then the loop's condition := some problem still
 // running (*remaining > 0) and st[0] < st[1] (the cycle cap).
 cudaError_t launch_batch_loop_decide(long long* st, const int* remaining, cudaGraphConditionalHandle h,
@@ -162,13 +175,13 @@ cudaError_t launch_coarse32(const Field32& u, const float* q, const double* ainv
 // e32 nullable: leave the correction alone.
 cudaError_t launch_defect64_to32(const Field& psi, const Coef& c, float* r32, float* e32,
                                  int64_t pitch32, double* partials, cudaStream_t s,
-                                 const float* norm_scale = nullptr);
+                                 const float* norm_scale = nullptr, const NormEnd& end = NormEnd{});
 // FP32 alone: a (and b, nullable) := psi rounded to FP32 on every node; psi interior :=
 // (double) u; per-block FP64 sums of the squared FP32 residual (mixed_norm_blocks blocks).
 cudaError_t launch_to32(const Field& psi, float* a, float* b, int64_t pitch32, cudaStream_t s);
 cudaError_t launch_to64(const Field& psi, const float* u, int64_t pitch32, cudaStream_t s);
 cudaError_t launch_defect32_sumsq(const Field32& f, const float* q, const Coef& c, double* partials,
-                                  cudaStream_t s);
+                                  cudaStream_t s, const NormEnd& end = NormEnd{});
 // psi += (double) e32 on interior nodes.
 cudaError_t launch_update64(const Field& psi, const float* e32, int64_t pitch32, cudaStream_t s);
 
@@ -230,9 +243,24 @@ inline int batch_grid(const void* kernel, int threads, size_t smem, int count, b
 struct TailJob {
     int first, last;
 };
-// The Dirichlet ring of the u, q and r buffers of FP32 levels lv[0 .. count) (device
-// descriptors) set to zero; max_side >= every level's m and n.
-cudaError_t launch_zero_rings32(const BatchLevel<float>* lv, int count, int max_side, cudaStream_t s);
+// What a solve needs on the device before its first kernel, in one launch: w and 1 - w of the point
+// sweeps, the loop's state, a zero norm counter, and with levels their descriptors, tail jobs (level l
+// down to the last) and zero rings in the u, q and r buffers of the levels from `rings` on.
+constexpr int SETUP_LEVELS = 24;
+template <class T>
+struct SolveSetup {
+    double w, omw;
+    LoopState state;
+    double* wslot;
+    LoopState* loop;
+    unsigned* done;
+    int levels, rings;
+    BatchLevel<T>* lv;
+    TailJob* jobs;
+    BatchLevel<T> level[SETUP_LEVELS];
+};
+template <class T>
+cudaError_t launch_setup(const SolveSetup<T>& a, cudaStream_t s);
 // per_level_w: Eq. 7 with each level's own w (BatchLevel::w) instead of the argument
 template <class T>
 cudaError_t launch_b_rb(const BatchList& l, const BatchLevel<T>* lv, const int* active, int colour,

@@ -1,45 +1,60 @@
 // loop_kernels.cu -- the device-side stopping test of a solve loop, and a self-check.
 //
 // loop_decide_kernel runs inside the body of a conditional CUDA graph node: after each check
-// period it applies the host loop's stopping rule (Eq. 16 or the L2 rules) and sets the
-// loop's condition. check_rounding_kernel compares the residual kernels' integer-pipe
+// period it applies the host loop's stopping rule of Eq. 16 and sets the loop's condition.
+// setup_kernel puts a solve's small state on the device. check_rounding_kernel compares the residual kernels' integer-pipe
 // FP64 -> FP32 rounding with the conversion instruction. fp64_rate_kernel measures the FP64
 // fused multiply-add issue rate, the peak that the FP64-bound kernels are measured against.
+#include <algorithm>
+
 #include "lap_device.cuh"
 #include "lap_internal.cuh"
+#include "norm_end.cuh"
 
 namespace lap {
 
 namespace {
 
-// The stopping test of a device-resident solve loop (Eq. 16 or the L2 rules), run after each
-// period inside the loop body of a conditional CUDA graph: the same arithmetic as the host's
-// test; clears the loop's condition when the solve stops or the next period would pass
-// max_iter.
-__global__ void loop_decide_kernel(LoopState* st, const double* __restrict__ nrm,
-                                   const unsigned long long* __restrict__ maxd,
-                                   const float* __restrict__ scale, cudaGraphConditionalHandle h)
+// The stopping test of Eq. 16 in a device-resident solve loop, after each period inside the body of a
+// conditional CUDA graph (the L2 rules are taken at the end of the norm kernels, norm_end.cuh).
+__global__ void loop_decide_kernel(LoopState* st, const unsigned long long* __restrict__ maxd,
+                                   cudaGraphConditionalHandle h)
 {
     if (threadIdx.x != 0) return;
-    st->k += st->steps;
-    double val, nr = st->last_nr;
-    bool conv;
-    if (st->mode == 2) {
-        val = __longlong_as_double((long long)*maxd);
-        conv = val <= st->tol;
-    } else {
-        nr = nrm[1];
-        if (scale) nr = nr / (double)*scale;
-        val = st->mode == 0 ? nr / st->r0 : nr;
-        conv = st->mode == 0 ? nr <= st->tol * st->r0 : nr <= st->tol;
+    const bool on = loop_test(st, st->last_nr, __longlong_as_double((long long)*maxd));
+    cudaGraphSetConditional(h, on ? 1u : 0u);
+}
+
+// SolveSetup: block row l takes the ring of level l (row 0, row n - 1, columns 0 and m - 1).
+template <class T>
+__global__ void setup_kernel(const SolveSetup<T> a)
+{
+    if (blockIdx.x == 0 && blockIdx.y == 0) {
+        if (threadIdx.x == 0) {
+            a.wslot[0] = a.w;
+            a.wslot[1] = a.omw;
+            *a.loop = a.state;
+            *a.done = 0u;
+        }
+        for (int l = threadIdx.x; l < a.levels; l += blockDim.x) {
+            a.lv[l] = a.level[l];
+            a.jobs[l] = TailJob{l, a.levels - 1};
+        }
     }
-    st->last_check = val;
-    st->last_nr = nr;
-    int status = 1;  // LAP_MAXITER
-    if (!isfinite(val)) status = 2;  // LAP_DIVERGED
-    else if (conv) status = 0;       // LAP_CONVERGED
-    st->status = status;
-    cudaGraphSetConditional(h, status == 1 && st->k + st->steps <= st->max_iter ? 1u : 0u);
+    const int l = blockIdx.y;
+    if (l >= a.levels || l < a.rings) return;
+    const BatchLevel<T>& V = a.level[l];
+    const int m = V.m, n = V.n;
+    for (int64_t k = blockIdx.x * blockDim.x + threadIdx.x; k < 2 * ((int64_t)m + n); k += gridDim.x * blockDim.x) {
+        int64_t at;
+        if (k < m) at = k;
+        else if (k < 2 * (int64_t)m) at = (int64_t)(n - 1) * V.pitch + (k - m);
+        else if (k < 2 * (int64_t)m + n) at = (k - 2 * (int64_t)m) * V.pitch;
+        else at = (k - 2 * (int64_t)m - n) * V.pitch + (m - 1);
+        V.u[at] = (T)0;
+        if (V.q) V.q[at] = (T)0;
+        if (V.r) V.r[at] = (T)0;
+    }
 }
 
 // The loop test of a device-resident batched solve, run after each cycle inside the body of
@@ -159,12 +174,25 @@ cudaError_t launch_batch_loop_decide(long long* st, const int* remaining, cudaGr
     return cudaGetLastError();
 }
 
-cudaError_t launch_loop_decide(LoopState* st, const double* nrm, const unsigned long long* maxd,
-                               const float* scale, cudaGraphConditionalHandle h, cudaStream_t s)
+cudaError_t launch_loop_decide(LoopState* st, const unsigned long long* maxd, cudaGraphConditionalHandle h,
+                               cudaStream_t s)
 {
-    loop_decide_kernel<<<1, 32, 0, s>>>(st, nrm, maxd, scale, h);
+    loop_decide_kernel<<<1, 32, 0, s>>>(st, maxd, h);
     note_launch();
     return cudaGetLastError();
 }
+
+template <class T>
+cudaError_t launch_setup(const SolveSetup<T>& a, cudaStream_t s)
+{
+    int64_t side = 0;
+    for (int l = a.rings; l < a.levels; ++l) side = std::max<int64_t>(side, (int64_t)a.level[l].m + a.level[l].n);
+    const int x = (int)std::min<int64_t>(64, std::max<int64_t>(1, (2 * side + 255) / 256));
+    setup_kernel<T><<<dim3(x, std::max(1, a.levels)), 256, 0, s>>>(a);
+    note_launch();
+    return cudaGetLastError();
+}
+template cudaError_t launch_setup<double>(const SolveSetup<double>&, cudaStream_t);
+template cudaError_t launch_setup<float>(const SolveSetup<float>&, cudaStream_t);
 
 }  // namespace lap

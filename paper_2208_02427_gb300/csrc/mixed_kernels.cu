@@ -12,6 +12,7 @@
 // by arithmetic; the FP64 work per outer iteration is two passes over the fine grid.
 #include "lap_device.cuh"
 #include "lap_internal.cuh"
+#include "norm_end.cuh"
 
 namespace lap {
 
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
     defect64_to32_kernel(const double* __restrict__ psi, int m, int n, int64_t pitch, double b2,
                          double d, float* __restrict__ r32, float* __restrict__ e32,
                          int64_t pitch32, double* __restrict__ partials,
-                         const float* __restrict__ sc)
+                         const float* __restrict__ sc, const NormEnd end)
 {
     const FmaOps o = load_fma_ops();
     if (!UNIT) b2 = in_reg(o, b2);
@@ -178,11 +179,9 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
     acc = warp_sum(acc);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double v = threadIdx.x < NORM_THREADS / 32 ? red[threadIdx.x] : 0.0;
-        v = warp_sum(v);
-        if (threadIdx.x == 0) partials[blockIdx.x] = v;
-    }
+    double v = 0.0;
+    if (threadIdx.x < 32) v = warp_sum(threadIdx.x < NORM_THREADS / 32 ? red[threadIdx.x] : 0.0);
+    norm_end(end, v, partials, red);
 }
 
 __global__ void __launch_bounds__(PX* PY)
@@ -227,7 +226,7 @@ __global__ void __launch_bounds__(PX* PY)
 template <bool UNIT>
 __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
     defect32_sumsq_kernel(const float* __restrict__ u, const float* __restrict__ q, int m, int n,
-                          int64_t pitch, float b2, float d, double* __restrict__ partials)
+                          int64_t pitch, float b2, float d, double* __restrict__ partials, const NormEnd end)
 {
     double acc = 0.0;
     for (StrideWalk<NORM_THREADS> p(m, n); p.left > 0; p.next()) {
@@ -241,41 +240,12 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
     acc = warp_sum(acc);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double v = threadIdx.x < NORM_THREADS / 32 ? red[threadIdx.x] : 0.0;
-        v = warp_sum(v);
-        if (threadIdx.x == 0) partials[blockIdx.x] = v;
-    }
-}
-
-// The ring of every FP32 level buffer (u, q, r) of levels 0 .. count - 1 set to zero: thread k
-// of block row l takes point k of level l's ring (row 0, row n - 1, column 0, column m - 1).
-__global__ void zero_rings32_kernel(const BatchLevel<float>* __restrict__ lv)
-{
-    const BatchLevel<float> V = lv[blockIdx.y];
-    const int m = V.m, n = V.n;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 2 * m + 2 * n; k += gridDim.x * blockDim.x) {
-        int64_t at;
-        if (k < m) at = k;
-        else if (k < 2 * m) at = (int64_t)(n - 1) * V.pitch + (k - m);
-        else if (k < 2 * m + n) at = (int64_t)(k - 2 * m) * V.pitch;
-        else at = (int64_t)(k - 2 * m - n) * V.pitch + (m - 1);
-        V.u[at] = 0.0f;
-        if (V.q) V.q[at] = 0.0f;
-        if (V.r) V.r[at] = 0.0f;
-    }
+    double v = 0.0;
+    if (threadIdx.x < 32) v = warp_sum(threadIdx.x < NORM_THREADS / 32 ? red[threadIdx.x] : 0.0);
+    norm_end(end, v, partials, red);
 }
 
 }  // namespace
-
-cudaError_t launch_zero_rings32(const BatchLevel<float>* lv, int count, int max_side, cudaStream_t s)
-{
-    if (count <= 0) return cudaSuccess;
-    const int per = 4 * max_side;
-    zero_rings32_kernel<<<dim3((per + 255) / 256, count), 256, 0, s>>>(lv);
-    note_launch();
-    return cudaGetLastError();
-}
 
 cudaError_t launch_to32(const Field& psi, float* a, float* b, int64_t pitch32, cudaStream_t s)
 {
@@ -294,13 +264,13 @@ cudaError_t launch_to64(const Field& psi, const float* u, int64_t pitch32, cudaS
 }
 
 cudaError_t launch_defect32_sumsq(const Field32& f, const float* q, const Coef& c, double* partials,
-                                  cudaStream_t s)
+                                  cudaStream_t s, const NormEnd& end)
 {
     const int blocks = mixed_norm_blocks(f.m, f.n);
     if (c.unit_beta)
-        defect32_sumsq_kernel<true><<<blocks, NORM_THREADS, 0, s>>>(f.p, q, f.m, f.n, f.pitch, (float)c.b2, (float)c.d, partials);
+        defect32_sumsq_kernel<true><<<blocks, NORM_THREADS, 0, s>>>(f.p, q, f.m, f.n, f.pitch, (float)c.b2, (float)c.d, partials, end);
     else
-        defect32_sumsq_kernel<false><<<blocks, NORM_THREADS, 0, s>>>(f.p, q, f.m, f.n, f.pitch, (float)c.b2, (float)c.d, partials);
+        defect32_sumsq_kernel<false><<<blocks, NORM_THREADS, 0, s>>>(f.p, q, f.m, f.n, f.pitch, (float)c.b2, (float)c.d, partials, end);
     note_launch();
     return cudaGetLastError();
 }
@@ -370,13 +340,13 @@ cudaError_t launch_coarse32(const Field32& u, const float* q, const double* ainv
 
 cudaError_t launch_defect64_to32(const Field& psi, const Coef& c, float* r32, float* e32,
                                  int64_t pitch32, double* partials, cudaStream_t s,
-                                 const float* norm_scale)
+                                 const float* norm_scale, const NormEnd& end)
 {
     const int blocks = mixed_norm_blocks(psi.m, psi.n);
 #define LAP_D64(U, F)                                                                            \
     defect64_to32_kernel<U, F><<<blocks, NORM_THREADS, 0, s>>>(psi.p, psi.m, psi.n, psi.pitch, c.b2, \
                                                                c.d, r32, e32, pitch32, partials, \
-                                                               norm_scale)
+                                                               norm_scale, end)
     if (c.unit_beta) {
         if (norm_scale) LAP_D64(true, true); else LAP_D64(true, false);
     } else {

@@ -12,6 +12,7 @@
 // pipe when 1/d is a power of two, and one multiply plus one fma for the SOR blend.
 #include "lap_device.cuh"
 #include "lap_internal.cuh"
+#include "norm_end.cuh"
 
 namespace lap {
 
@@ -242,7 +243,8 @@ __global__ void __launch_bounds__(JA_BX* JA_BY)
 template <bool UNIT_BETA, bool HAS_Q>
 __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
     defect_sumsq_kernel(const double* __restrict__ u, const double* __restrict__ q, int m, int n,
-                        int64_t pitch, double b2, double d, double* __restrict__ partials)
+                        int64_t pitch, double b2, double d, double* __restrict__ partials,
+                        const NormEnd end)
 {
     const FmaOps o = load_fma_ops();
     if (!UNIT_BETA) b2 = in_reg(o, b2);
@@ -270,29 +272,19 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
     acc = warp_sum(acc);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double v = threadIdx.x < NORM_THREADS / 32 ? red[threadIdx.x] : 0.0;
-        v = warp_sum(v);
-        if (threadIdx.x == 0) partials[blockIdx.x] = v;
-    }
+    double v = 0.0;
+    if (threadIdx.x < 32) v = warp_sum(threadIdx.x < NORM_THREADS / 32 ? red[threadIdx.x] : 0.0);
+    norm_end(end, v, partials, red);
 }
 
 __global__ void __launch_bounds__(NORM_THREADS)
     sum_partials_kernel(const double* __restrict__ partials, int count, double* __restrict__ out)
 {
-    double acc = 0.0;
-    for (int k = threadIdx.x; k < count; k += NORM_THREADS) acc = __dadd_rn(acc, partials[k]);
     __shared__ double red[NORM_THREADS / 32];
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double v = threadIdx.x < NORM_THREADS / 32 ? red[threadIdx.x] : 0.0;
-        v = warp_sum(v);
-        if (threadIdx.x == 0) {
-            out[0] = v;
-            out[1] = sqrt(v);
-        }
+    const double v = sum_partials_256(partials, count, red);
+    if (threadIdx.x == 0) {
+        out[0] = v;
+        out[1] = sqrt(v);
     }
 }
 
@@ -390,12 +382,12 @@ cudaError_t launch_defect(const Field& f, const double* q, double* r, const Coef
 int norm_blocks(const Field& f) { return norm_blocks_for(f.m, f.n); }
 
 cudaError_t launch_defect_sumsq(const Field& f, const double* q, const Coef& c, double* partials,
-                                cudaStream_t s)
+                                cudaStream_t s, const NormEnd& end)
 {
     const int blocks = norm_blocks(f);
     LAP_DISPATCH_BOOL(c.unit_beta, UB, LAP_DISPATCH_BOOL(q != nullptr, HQ,
         defect_sumsq_kernel<UB, HQ><<<blocks, NORM_THREADS, 0, s>>>(f.p, q, f.m, f.n, f.pitch, c.b2,
-                                                                    c.d, partials)));
+                                                                    c.d, partials, end)));
     note_launch();
     return cudaGetLastError();
 }
