@@ -12,6 +12,7 @@
 //
 // The level data are generic in T: double for the FP64 V-cycle, float for the inner cycle
 // of the mixed-precision solver (FP32 inside FP64 defect correction).
+#include "gs_restrict.cuh"
 #include "lap_device.cuh"
 #include "lap_internal.cuh"
 #include "vcycle_arith.cuh"
@@ -83,10 +84,11 @@ __device__ __forceinline__ void on_rb_flags(const BatchLevel<T>& L, bool gs, F&&
 }
 
 // Coarse point (I, J): qc = 0.25 ((4 c + 2 edges) + corners) of the fine residual; the
-// coarse correction starts at zero.
+// coarse correction starts at zero, or with red (Gauss-Seidel) after its first red pass, which leaves
+// the black points alone.
 template <class T>
 __device__ __forceinline__ void restrict_point(const Arith<T>& A, const BatchLevel<T>& C,
-                                               const BatchLevel<T>& F, int I, int J)
+                                               const BatchLevel<T>& F, int I, int J, bool red = false)
 {
     const int64_t pf = F.pitch;
     const T* c = F.r + (int64_t)(2 * J) * pf + 2 * I;
@@ -95,8 +97,13 @@ __device__ __forceinline__ void restrict_point(const Arith<T>& A, const BatchLev
     const T two = A.two();
     const T t = A.fma(two, c[0], edges);
     const int64_t at = (int64_t)J * C.pitch + I;
-    C.q[at] = A.quarter(A.fma(two, t, corners));
-    C.u[at] = (T)0;
+    const T v = A.quarter(A.fma(two, t, corners));
+    C.q[at] = v;
+    if (!red) C.u[at] = (T)0;
+    else if (((I + J) & 1) == 0) {
+        const T s = A.add((T)0, v);
+        C.u[at] = C.inv_d_shift > 0 ? A.template inv_d<true>(s, C) : A.template inv_d<false>(s, C);
+    }
 }
 
 // Fine row j, coarse column I: bilinear interpolation added to fine points 2I and 2I + 1.
@@ -118,6 +125,18 @@ __device__ __forceinline__ void prolong_pair(const Arith<T>& A, const BatchLevel
             row[i1] = A.add(row[i1], A.quarter(s));
         }
     }
+}
+
+// The black one of the two points alone (prolong_black_kernel).
+template <class T>
+__device__ __forceinline__ void prolong_black(const Arith<T>& A, const BatchLevel<T>& F,
+                                              const BatchLevel<T>& C, int I, int j)
+{
+    const int odd = j & 1;
+    if (odd && I == 0) return;
+    const T* a = C.u + (int64_t)(j >> 1) * C.pitch + I;
+    T* x = F.u + (int64_t)j * F.pitch + 2 * I + (odd ? 0 : 1);
+    *x = A.add(*x, A.half(A.add(a[0], a[odd ? C.pitch : 1])));
 }
 
 // One smoother colour pass (Eq. 6 when gs, Eq. 7 otherwise) over the rows of each item.
@@ -150,7 +169,7 @@ __global__ void __launch_bounds__(BT)
 template <class T>
 __global__ void __launch_bounds__(BT)
     b_defect_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim,
-                    const BatchLevel<T>* __restrict__ lv, const int* __restrict__ active)
+                    const BatchLevel<T>* __restrict__ lv, const int* __restrict__ active, int gs)
 {
     const Arith<T> A = arith<T>();
     const ItemClaim ic{claim, count};
@@ -158,6 +177,7 @@ __global__ void __launch_bounds__(BT)
         const BatchItem it = items[b];
         const BatchLevel<T> L = lv[it.level];
         if (!active[L.problem]) continue;
+        if (sizeof(T) == 8 && gs && L.unit_beta) continue;  // the restriction takes the residual
         const int wdt = L.m - 2;
         on_flag(L.unit_beta != 0, [&](auto U) {
             on_flag(L.q != nullptr, [&](auto Q) {
@@ -172,9 +192,9 @@ __global__ void __launch_bounds__(BT)
 // Items of the coarse level: qc from the fine residual (the level before it in lv), and the
 // coarse correction zeroed.
 template <class T>
-__global__ void __launch_bounds__(BT)
+__global__ void __launch_bounds__(BT, 4)
     b_restrict_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim,
-                      const BatchLevel<T>* __restrict__ lv, const int* __restrict__ active)
+                      const BatchLevel<T>* __restrict__ lv, const int* __restrict__ active, int gs)
 {
     const Arith<T> A = arith<T>();
     const ItemClaim ic{claim, count};
@@ -183,8 +203,24 @@ __global__ void __launch_bounds__(BT)
         const BatchLevel<T> C = lv[it.level];
         if (!active[C.problem]) continue;
         const BatchLevel<T> F = lv[it.level - 1];
+        const bool red = gs && it.red;
+        if constexpr (sizeof(T) == 8) {
+            if (gs && F.unit_beta) {
+                // the item's rows in runs of four for the warps (a run computes one corner row more)
+                const int segs = (C.m - 2 + 30) / 31, nw = BT / 32, wid = threadIdx.x >> 5;
+                const int runs = (it.rows + 3) / 4, per = (it.rows + runs - 1) / runs;
+                for (int k = wid; k < segs * runs; k += nw) {
+                    const int run = k / segs, J0 = it.row0 + run * per, J1 = min(J0 + per, it.row0 + it.rows);
+                    if (F.q)
+                        gs_restrict_run<true>(A.o, F.u, F.q, F.m, F.pitch, C.q, C.u, C.pitch, k - run * segs, J0, J1, red);
+                    else
+                        gs_restrict_run<false>(A.o, F.u, nullptr, F.m, F.pitch, C.q, C.u, C.pitch, k - run * segs, J0, J1, red);
+                }
+                continue;
+            }
+        }
         const int wdt = C.m - 2;
-        for (Walk k(wdt); k.r < it.rows; k.next()) restrict_point(A, C, F, 1 + k.c, it.row0 + k.r);
+        for (Walk k(wdt); k.r < it.rows; k.next()) restrict_point(A, C, F, 1 + k.c, it.row0 + k.r, red);
     }
     ic.finish();
 }
@@ -193,7 +229,7 @@ __global__ void __launch_bounds__(BT)
 template <class T>
 __global__ void __launch_bounds__(BT)
     b_prolong_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim,
-                     const BatchLevel<T>* __restrict__ lv, const int* __restrict__ active)
+                     const BatchLevel<T>* __restrict__ lv, const int* __restrict__ active, int gs)
 {
     const Arith<T> A = arith<T>();
     const ItemClaim ic{claim, count};
@@ -203,7 +239,10 @@ __global__ void __launch_bounds__(BT)
         if (!active[F.problem]) continue;
         const BatchLevel<T> C = lv[it.level + 1];
         const int pairs = (F.m - 1) / 2;  // coarse columns 0 .. mc-2
-        for (Walk k(pairs); k.r < it.rows; k.next()) prolong_pair(A, F, C, k.c, it.row0 + k.r);
+        if (gs)
+            for (Walk k(pairs); k.r < it.rows; k.next()) prolong_black(A, F, C, k.c, it.row0 + k.r);
+        else
+            for (Walk k(pairs); k.r < it.rows; k.next()) prolong_pair(A, F, C, k.c, it.row0 + k.r);
     }
     ic.finish();
 }
@@ -401,12 +440,41 @@ __device__ __forceinline__ double sumsq_item(const BatchItem& it, const BatchLev
     return acc;
 }
 
+// The same after Gauss-Seidel smoothing with beta = 1: the red points, and the black ones that are not
+// known to have a zero residual (gs_norm_kernel).
+__device__ __forceinline__ double gs_sumsq_item(const BatchItem& it, const BatchLevel<double>& L)
+{
+    const Arith<double> A = arith<double>();
+    const double nd = -in_reg(A.o, 4.0);
+    double acc = 0.0;
+    auto point = [&](const Stencil5& x, int64_t at, int i) {
+        const double r = __fma_rn(nd, x.c, A.template nsum<true>(x.w, x.e, x.s, x.n, 1.0));
+        acc = __fma_rn(r, r, acc);
+        if (i + 1 <= L.m - 2 && irregular(x.e)) acc = black_square(L.u + at + 1, L.pitch, A.o.one, A.o.nzero, acc);
+        if (i == 2 && irregular(x.w)) acc = black_square(L.u + at - 1, L.pitch, A.o.one, A.o.nzero, acc);
+    };
+    Walk k((L.m - 1) / 2);
+    while (k.r < it.rows) {
+        const int j0 = it.row0 + k.r, i0 = 1 + ((1 + j0) & 1) + 2 * k.c;
+        k.next();
+        const bool two = k.r < it.rows;
+        const int j1 = two ? it.row0 + k.r : j0, i1 = two ? 1 + ((1 + j1) & 1) + 2 * k.c : i0;
+        if (two) k.next();
+        const bool in0 = i0 <= L.m - 2, in1 = two && i1 <= L.m - 2;
+        const int64_t a0 = (int64_t)j0 * L.pitch + (in0 ? i0 : 1), a1 = (int64_t)j1 * L.pitch + (in1 ? i1 : 1);
+        const Stencil5 x0 = load5(L.u + a0, L.pitch), x1 = load5(L.u + a1, L.pitch);
+        if (in0) point(x0, a0, i0);
+        if (in1) point(x1, a1, i1);
+    }
+    return acc;
+}
+
 // Item ib's partial sum of squares (see b_sumsq_kernel) by the whole CTA into partials[ib].
 __device__ __forceinline__ void sumsq_block(const BatchItem* __restrict__ items, int ib,
                                             const BatchLevel<double>* __restrict__ lv,
                                             const int* __restrict__ active, double* __restrict__ partials,
                                             const BatchLevel<float>* __restrict__ lv32,
-                                            const double* __restrict__ r0)
+                                            const double* __restrict__ r0, bool gs)
 {
     const BatchItem it = items[ib];
     const BatchLevel<double> L = lv[it.level];
@@ -424,7 +492,9 @@ __device__ __forceinline__ void sumsq_block(const BatchItem* __restrict__ items,
     double acc = 0.0;
     // the FP32 or the FP64 sum of squares, chosen per block (as a per-point choice the
     // compiler would issue the FP64 fma for every point)
-    on_flag(L.unit_beta != 0, [&](auto U) {
+    // an FP64 multigrid problem with more than one level has a residual scratch
+    if (gs && !mixed && L.r && L.unit_beta) acc = gs_sumsq_item(it, L);
+    else on_flag(L.unit_beta != 0, [&](auto U) {
         if (!mixed)
             acc = sumsq_item<false, decltype(U)::value, false>(it, L, lv32, 0.0f);
         else
@@ -451,15 +521,15 @@ __global__ void __launch_bounds__(BT, 5)
     b_sumsq_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim,
                    const BatchLevel<double>* __restrict__ lv, const int* __restrict__ active,
                    double* __restrict__ partials, const BatchLevel<float>* __restrict__ lv32,
-                   const double* __restrict__ r0)
+                   const double* __restrict__ r0, int gs)
 {
     if (!CLAIM) {
-        sumsq_block(items, blockIdx.x, lv, active, partials, lv32, r0);
+        sumsq_block(items, blockIdx.x, lv, active, partials, lv32, r0, gs != 0);
         return;
     }
     const ItemClaim ic{claim, count};
     for (int b = ic.take(-1); b < count; b = ic.take(b))
-        sumsq_block(items, b, lv, active, partials, lv32, r0);
+        sumsq_block(items, b, lv, active, partials, lv32, r0, gs != 0);
     ic.finish();
 }
 
@@ -549,31 +619,31 @@ cudaError_t launch_b_rb(const BatchList& l, const BatchLevel<T>* lv, const int* 
 }
 template <class T>
 cudaError_t launch_b_defect(const BatchList& l, const BatchLevel<T>* lv, const int* active,
-                            cudaStream_t s)
+                            cudaStream_t s, bool gs)
 {
     if (l.count == 0) return cudaSuccess;
     const int grid = batch_grid((const void*)b_defect_kernel<T>, BT, 0, l.count, l.claim != nullptr);
-    b_defect_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active);
+    b_defect_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, gs ? 1 : 0);
     note_launch();
     return cudaGetLastError();
 }
 template <class T>
 cudaError_t launch_b_restrict(const BatchList& l, const BatchLevel<T>* lv, const int* active,
-                              cudaStream_t s)
+                              cudaStream_t s, bool gs)
 {
     if (l.count == 0) return cudaSuccess;
     const int grid = batch_grid((const void*)b_restrict_kernel<T>, BT, 0, l.count, l.claim != nullptr);
-    b_restrict_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active);
+    b_restrict_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, gs ? 1 : 0);
     note_launch();
     return cudaGetLastError();
 }
 template <class T>
 cudaError_t launch_b_prolong(const BatchList& l, const BatchLevel<T>* lv, const int* active,
-                             cudaStream_t s)
+                             cudaStream_t s, bool gs)
 {
     if (l.count == 0) return cudaSuccess;
     const int grid = batch_grid((const void*)b_prolong_kernel<T>, BT, 0, l.count, l.claim != nullptr);
-    b_prolong_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active);
+    b_prolong_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, gs ? 1 : 0);
     note_launch();
     return cudaGetLastError();
 }
@@ -593,12 +663,12 @@ cudaError_t launch_b_coarse(const BatchList& l, const BatchLevel<T>* lv, const i
 
 template cudaError_t launch_b_rb<double>(const BatchList&, const BatchLevel<double>*, const int*, int, bool, double, cudaStream_t, bool);
 template cudaError_t launch_b_rb<float>(const BatchList&, const BatchLevel<float>*, const int*, int, bool, double, cudaStream_t, bool);
-template cudaError_t launch_b_defect<double>(const BatchList&, const BatchLevel<double>*, const int*, cudaStream_t);
-template cudaError_t launch_b_defect<float>(const BatchList&, const BatchLevel<float>*, const int*, cudaStream_t);
-template cudaError_t launch_b_restrict<double>(const BatchList&, const BatchLevel<double>*, const int*, cudaStream_t);
-template cudaError_t launch_b_restrict<float>(const BatchList&, const BatchLevel<float>*, const int*, cudaStream_t);
-template cudaError_t launch_b_prolong<double>(const BatchList&, const BatchLevel<double>*, const int*, cudaStream_t);
-template cudaError_t launch_b_prolong<float>(const BatchList&, const BatchLevel<float>*, const int*, cudaStream_t);
+template cudaError_t launch_b_defect<double>(const BatchList&, const BatchLevel<double>*, const int*, cudaStream_t, bool);
+template cudaError_t launch_b_defect<float>(const BatchList&, const BatchLevel<float>*, const int*, cudaStream_t, bool);
+template cudaError_t launch_b_restrict<double>(const BatchList&, const BatchLevel<double>*, const int*, cudaStream_t, bool);
+template cudaError_t launch_b_restrict<float>(const BatchList&, const BatchLevel<float>*, const int*, cudaStream_t, bool);
+template cudaError_t launch_b_prolong<double>(const BatchList&, const BatchLevel<double>*, const int*, cudaStream_t, bool);
+template cudaError_t launch_b_prolong<float>(const BatchList&, const BatchLevel<float>*, const int*, cudaStream_t, bool);
 template cudaError_t launch_b_coarse<double>(const BatchList&, const BatchLevel<double>*, const int*, int, cudaStream_t);
 template cudaError_t launch_b_coarse<float>(const BatchList&, const BatchLevel<float>*, const int*, int, cudaStream_t);
 
@@ -620,15 +690,15 @@ template cudaError_t launch_b_tail<float>(const TailJob*, int, const BatchLevel<
 
 cudaError_t launch_b_sumsq(const BatchList& l, const BatchLevel<double>* lv, const int* active,
                            double* partials, const BatchLevel<float>* lv32, cudaStream_t s,
-                           const double* r0)
+                           const double* r0, bool gs)
 {
     if (l.count == 0) return cudaSuccess;
     if (l.claim) {
         const int grid = batch_grid((const void*)b_sumsq_kernel<true>, BT, 0, l.count, true);
-        b_sumsq_kernel<true><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, partials, lv32, r0);
+        b_sumsq_kernel<true><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, partials, lv32, r0, gs ? 1 : 0);
     } else {
         b_sumsq_kernel<false><<<l.count, BT, 0, s>>>(l.items, l.count, nullptr, lv, active, partials, lv32,
-                                                     r0);
+                                                     r0, gs ? 1 : 0);
     }
     note_launch();
     return cudaGetLastError();

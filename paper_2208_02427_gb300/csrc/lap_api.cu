@@ -929,16 +929,19 @@ struct Solver {
                 ck(launch_rb32(lv.u, lv.q, c, gs, p->smoother_w, colour, s), "smoother kernel");
     }
 
-    void smooth(const Level& lv, int sweeps)
+    // red_done: the first red pass has been done (by the restriction into the level)
+    void smooth(const Level& lv, int sweeps, bool red_done = false)
     {
         const bool gs = p->smoother_w == 1.0;
-        for (int k = 0; k < sweeps; ++k)
-            for (int colour = 0; colour < 2; ++colour)
-                ck(launch_rb_colour(lv.u, lv.q, c, gs, p->smoother_w, colour, nullptr, s, w.wslot),
-                   "smoother kernel");
+        for (int k = red_done ? 1 : 0; k < 2 * sweeps; ++k)
+            ck(launch_rb_colour(lv.u, lv.q, c, gs, p->smoother_w, k & 1, nullptr, s, w.wslot), "smoother kernel");
     }
 
-    void vcycle(int l)
+    // Gauss-Seidel smoothing with beta = 1 leaves black residuals that are exactly zero.
+    bool exact_blacks() const { return p->smoother_w == 1.0 && c.unit_beta; }
+
+    // red_done: see smooth()
+    void vcycle(int l, bool red_done = false)
     {
         Level& lv = w.levels[l];
         const int L = (int)w.levels.size();
@@ -959,13 +962,21 @@ struct Solver {
             ck(launch_coarse_solve(lv.u, lv.q, c, ainv, s), "coarse solve kernel");
             return;
         }
-        smooth(lv, p->nu1);
+        smooth(lv, p->nu1, red_done);
         Level& cv = w.levels[l + 1];
-        ck(launch_defect(lv.u, lv.q, lv.r, c, s), "defect kernel");
-        ck(launch_restrict(Field{lv.r, lv.u.m, lv.u.n, lv.u.pitch}, cv.q, cv.u.p, cv.u.pitch, s),
-           "restrict kernel");
-        vcycle(l + 1);
-        ck(launch_prolong_add(lv.u, cv.u.p, cv.u.pitch, s), "prolong kernel");
+        const bool gs = p->smoother_w == 1.0;
+        // the next level's first red pass: where it is smoothed by kernels of its own
+        const bool red = gs && p->nu1 > 0 && l + 1 != tail_first && l + 1 != L - 1;
+        if (exact_blacks() && p->nu1 > 0) {
+            ck(launch_gs_restrict(lv.u, lv.q, cv.q, cv.u.p, cv.u.pitch, red, s), "restrict kernel");
+        } else {
+            ck(launch_defect(lv.u, lv.q, lv.r, c, s), "defect kernel");
+            ck(launch_restrict(Field{lv.r, lv.u.m, lv.u.n, lv.u.pitch}, cv.q, cv.u.p, cv.u.pitch, s, red ? &c : nullptr),
+               "restrict kernel");
+        }
+        vcycle(l + 1, red);
+        if (gs && p->nu2 > 0) ck(launch_prolong_black(lv.u, cv.u.p, cv.u.pitch, s), "prolong kernel");
+        else ck(launch_prolong_add(lv.u, cv.u.p, cv.u.pitch, s), "prolong kernel");
         smooth(lv, p->nu2);
     }
 
@@ -1140,6 +1151,8 @@ struct Solver {
     {
         if (p->method == LAP_MG_FP32)
             ck(launch_defect32_sumsq(w.levels32[0].u, w.levels32[0].q, c, w.partials, s, end), "residual kernel");
+        else if (p->method == LAP_MG && exact_blacks() && p->nu2 > 0 && w.levels.size() > 1)
+            ck(launch_gs_norm(cur, w.partials, s, end), "residual kernel");
         else if (p->method != LAP_MG_MIXED)
             ck(launch_defect_sumsq(cur, nullptr, c, w.partials, s, end), "residual kernel");
     }

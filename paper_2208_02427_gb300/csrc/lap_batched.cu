@@ -5,10 +5,10 @@
 
 namespace lap {
 
-void add_items(std::vector<BatchItem>& items, int level_index, int m, int n, int points)
+void add_items(std::vector<BatchItem>& items, int level_index, int m, int n, int points, bool red)
 {
     const int per = std::max(1, points / std::max(1, m - 2));
-    for (int r = 1; r <= n - 2; r += per) items.push_back(BatchItem{level_index, r, std::min(per, n - 1 - r)});
+    for (int r = 1; r <= n - 2; r += per) items.push_back(BatchItem{level_index, r, std::min(per, n - 1 - r), red ? 1 : 0});
 }
 
 // First level of a problem that the small-level tail runs (both sides <= tail_size), or
@@ -94,7 +94,8 @@ void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJ
         for (size_t k = 0; k < who.size(); ++k) {
             const int q = who[k];
             if (nlev[q] > l && l <= t[k])
-                add_items(items, base[q] + l, lv[base[q] + l].m, lv[base[q] + l].n, item_points);
+                add_items(items, base[q] + l, lv[base[q] + l].m, lv[base[q] + l].n, item_points,
+                          nlev[q] - 1 > l && l < t[k]);
         }
         L.all[l] = {a0, (int)items.size() - a0};
         const int c0 = (int)items.size();
@@ -102,7 +103,7 @@ void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJ
             const int q = who[k];
             if (nlev[q] - 1 == l && t[k] == nlev[q]) {
                 const BatchLevel<double>& d = lv[base[q] + l];
-                items.push_back(BatchItem{base[q] + l, 1, d.n - 2});
+                items.push_back(BatchItem{base[q] + l, 1, d.n - 2, 0});
                 L.max_coarse = std::max(L.max_coarse, (d.m - 2) * (d.n - 2));
             }
         }
@@ -510,7 +511,9 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
                     ck(launch_b_sumsq(norms, lv64, active, partials, lv32, st, r0), "batched residual");
                 } else {
                     enqueue_vcycle(list, L, lv64, active, K.jobs, *p, p->smoother_w, st);
-                    ck(launch_b_sumsq(norms, lv64, active, partials, nullptr, st), "batched residual");
+                    ck(launch_b_sumsq(norms, lv64, active, partials, nullptr, st, nullptr,
+                                      p->smoother_w == 1.0 && p->nu2 > 0),
+                       "batched residual");
                 }
                 ck(launch_b_converge(partials, first, count, active, r0, rnow, iters, status, remaining,
                                      1, rel, p->tol, st), "batched convergence");

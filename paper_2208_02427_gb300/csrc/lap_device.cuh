@@ -126,6 +126,21 @@ __device__ __forceinline__ double scale_down_pow2(const FmaOps& o, double x, int
     return fmul_rare(x, two_pow_minus_k, o.nzero);
 }
 
+// 0 + x on the integer pipe: x, but +0 for -0 (the neighbour sum of a point whose neighbours are zero).
+__device__ __forceinline__ double plus_zero(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return b == (long long)0x8000000000000000ull ? 0.0 : x;
+}
+
+// Whether a Gauss-Seidel point psi = s 2^-k may differ from s 2^-k before rounding (or is not a
+// number): zero, subnormal, infinite or NaN. Elsewhere its residual fma(-d, psi, s) is exactly 0.
+__device__ __forceinline__ bool irregular(double x)
+{
+    const int e = (__double2hiint(x) >> 20) & 0x7ff;
+    return e == 0 || e == 0x7ff;
+}
+
 // Multiply by 1/d: the integer-pipe path when 1/d is an exact power of two.
 template <bool POW2>
 __device__ __forceinline__ double times_inv_d(const FmaOps& o, double s, double inv_d, int shift)

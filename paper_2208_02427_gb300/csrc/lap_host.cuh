@@ -271,7 +271,7 @@ cudaEvent_t tuner_event(lap_handle h, int k);
 // points, the mixed solver 74 / 71 / 69 / 68 ms; 8192 for both.
 constexpr int BATCH_ITEM_POINTS = 8192;
 void add_items(std::vector<BatchItem>& items, int level_index, int m, int n,
-               int points = BATCH_ITEM_POINTS);
+               int points = BATCH_ITEM_POINTS, bool red = false);
 
 // Per-level work lists of one V-cycle over a set of problems: [first, count) into the items
 // (fine, all, coarse) or into the tail jobs (tail).
@@ -336,14 +336,15 @@ void enqueue_vcycle(ListFn list, const LevelLists& L, const BatchLevel<T>* lv, c
         ck(launch_b_coarse(list(L.coarse[l]), lv, active, L.max_coarse, st), "batched coarse");
         enqueue_tail(L, l, lv, active, jobs, p, smoother_w, st);
         if (l == L.levels - 1) break;
-        for (int k = 0; k < p.nu1; ++k)
-            for (int colour = 0; colour < 2; ++colour)
-                ck(launch_b_rb(list(L.fine[l]), lv, active, colour, gs, smoother_w, st), "batched smoother");
-        ck(launch_b_defect(list(L.fine[l]), lv, active, st), "batched defect");
-        ck(launch_b_restrict(list(L.all[l + 1]), lv, active, st), "batched restrict");
+        // below level 0 the restriction has done the first red pass
+        for (int k = l > 0 && gs ? 1 : 0; k < 2 * p.nu1; ++k)
+            ck(launch_b_rb(list(L.fine[l]), lv, active, k & 1, gs, smoother_w, st), "batched smoother");
+        const bool after_gs = gs && p.nu1 > 0;
+        ck(launch_b_defect(list(L.fine[l]), lv, active, st, after_gs), "batched defect");
+        ck(launch_b_restrict(list(L.all[l + 1]), lv, active, st, after_gs), "batched restrict");
     }
     for (int l = L.levels - 2; l >= 0; --l) {
-        ck(launch_b_prolong(list(L.fine[l]), lv, active, st), "batched prolong");
+        ck(launch_b_prolong(list(L.fine[l]), lv, active, st, gs && p.nu2 > 0), "batched prolong");
         for (int k = 0; k < p.nu2; ++k)
             for (int colour = 0; colour < 2; ++colour)
                 ck(launch_b_rb(list(L.fine[l]), lv, active, colour, gs, smoother_w, st), "batched smoother");

@@ -125,6 +125,10 @@ inline int norm_blocks_for(int m, int n)
     return b < cap ? (int)b : cap;
 }
 int norm_blocks(const Field& f);
+// The same norm of a field whose last update was a Gauss-Seidel black pass with beta = 1 (no source):
+// black residuals are zero where the value is regular, so only red points are summed (in a walk of
+// their own), and the others' black neighbours.
+cudaError_t launch_gs_norm(const Field& f, double* partials, cudaStream_t s, const NormEnd& end);
 cudaError_t launch_defect_sumsq(const Field& f, const double* q, const Coef& c, double* partials,
                                 cudaStream_t s, const NormEnd& end = NormEnd{});
 // out[0] = sum(partials[0..count)), fixed order; out[1] = sqrt(out[0]).
@@ -148,9 +152,15 @@ cudaError_t launch_maxdelta(const Field& a, const double* b, unsigned long long*
                             cudaStream_t s);
 
 // ---- multigrid transfer kernels (mg_kernels.cu) ----------------------------------
-// qc (coarse interior) := 0.25 ((4 r_c + 2 edges) + corners); ec (nullable) := 0 in the interior.
+// qc (coarse interior) := 0.25 ((4 r_c + 2 edges) + corners); ec (nullable) := 0 in the interior, or
+// with `red` (the coefficients) the first red pass of Gauss-Seidel from zero, black points untouched.
 cudaError_t launch_restrict(const Field& fine_r, double* qc, double* ec, int64_t pitch_c,
-                            cudaStream_t s);
+                            cudaStream_t s, const Coef* red = nullptr);
+// The same from u itself (f) after a Gauss-Seidel black pass, beta = 1.
+cudaError_t launch_gs_restrict(const Field& f, const double* q, double* qc, double* ec, int64_t pitch_c, bool red,
+                               cudaStream_t s);
+// u (black fine interior points) += bilinear interpolation of ec.
+cudaError_t launch_prolong_black(const Field& fine_u, const double* ec, int64_t pitch_c, cudaStream_t s);
 // u (fine interior) += bilinear interpolation of ec.
 cudaError_t launch_prolong_add(const Field& fine_u, const double* ec, int64_t pitch_c,
                                cudaStream_t s);
@@ -219,6 +229,7 @@ struct BatchItem {
     int level;  // index into the level array
     int row0;   // first interior row
     int rows;   // rows in this item
+    int red;    // restriction: the level is smoothed next (its first red pass can be done with it)
 };
 // A work list of one launch. claim (nullable): two words of device memory, zero between
 // launches; with it the launch is persistent -- as many CTAs as fit the device at once, each
@@ -265,17 +276,21 @@ cudaError_t launch_setup(const SolveSetup<T>& a, cudaStream_t s);
 template <class T>
 cudaError_t launch_b_rb(const BatchList& l, const BatchLevel<T>* lv, const int* active, int colour,
                         bool gs, double w, cudaStream_t s, bool per_level_w = false);
+// gs: the levels have just been smoothed by Gauss-Seidel. Then FP64 problems with beta = 1 need no
+// residual pass (their restriction takes it, gs_restrict.cuh), and the restriction into a level that
+// is smoothed next does its first red pass.
 template <class T>
 cudaError_t launch_b_defect(const BatchList& l, const BatchLevel<T>* lv, const int* active,
-                            cudaStream_t s);
+                            cudaStream_t s, bool gs = false);
 // items of the coarse level; the fine level is the preceding entry of lv
 template <class T>
 cudaError_t launch_b_restrict(const BatchList& l, const BatchLevel<T>* lv, const int* active,
-                              cudaStream_t s);
-// items of the fine level; the coarse level is the following entry of lv
+                              cudaStream_t s, bool gs = false);
+// items of the fine level; the coarse level is the following entry of lv. gs: Gauss-Seidel smoothing
+// follows, whose first red pass does not read the red points (black ones only)
 template <class T>
 cudaError_t launch_b_prolong(const BatchList& l, const BatchLevel<T>* lv, const int* active,
-                             cudaStream_t s);
+                             cudaStream_t s, bool gs = false);
 template <class T>
 cudaError_t launch_b_coarse(const BatchList& l, const BatchLevel<T>* lv, const int* active,
                             int max_unknowns, cudaStream_t s);
@@ -305,9 +320,11 @@ cudaError_t launch_smem_tail(const TailJob* jobs, int count, const BatchLevel<T>
 // per-item FP64 sum of squares of the residual; with lv32 also r32 := residual, e32 := 0;
 // with r0 (per problem) the mixed problems sum their squares in FP32 after an exact
 // power-of-two scaling from r0 (the partials are stored descaled)
+// gs: FP64 multigrid problems come from Gauss-Seidel smoothing (with beta = 1 only their red points
+// are summed, see launch_gs_norm)
 cudaError_t launch_b_sumsq(const BatchList& l, const BatchLevel<double>* lv, const int* active,
                            double* partials, const BatchLevel<float>* lv32, cudaStream_t s,
-                           const double* r0 = nullptr);
+                           const double* r0 = nullptr, bool gs = false);
 cudaError_t launch_b_update(const BatchList& l, const BatchLevel<double>* lv, const int* active,
                             const BatchLevel<float>* lv32, cudaStream_t s);
 // A problem that left the batch in a convergence test: its index, lap_status, cycles run and

@@ -467,7 +467,9 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
             for (int colour = 0; colour < 2; ++colour)
                 ck(launch_b_rb(list(swept), lv64, active, colour, false, 1.0, st, true), "server sweep");
         }
-        ck(launch_b_sumsq(list(P.norm), lv64, active, pnorm, lv32, st, dr0), "server residual");
+        ck(launch_b_sumsq(list(P.norm), lv64, active, pnorm, lv32, st, dr0,
+                          S->mg.smoother_w == 1.0 && S->mg.nu2 > 0),
+           "server residual");
         ck(launch_b_converge(pnorm, fn, R, active, dr0, rnow, iters, status, remaining, 1, true, 0.0,
                              st, dtol, maxit, done, ndone), "server convergence");
         // ---- the step's completion list (written by the convergence tests), read once ----

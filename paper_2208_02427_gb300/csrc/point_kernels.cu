@@ -10,6 +10,7 @@
 // sweeps; the kernels spend the minimum number of FP64 operations per point: 3 adds for
 // the neighbour sum (one more fma when beta != 1), the multiply by 1/d on the integer
 // pipe when 1/d is a power of two, and one multiply plus one fma for the SOR blend.
+#include "gs_restrict.cuh"
 #include "lap_device.cuh"
 #include "lap_internal.cuh"
 #include "norm_end.cuh"
@@ -277,6 +278,60 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
     norm_end(end, v, partials, red);
 }
 
+// The norm after Gauss-Seidel smoothing with beta = 1: a black point's residual is exactly zero where
+// its value is regular (mg_kernels.cu), so the red points are summed alone: 2.5 FP64 operations per
+// point instead of 5. 4097^2: 145 -> 91 us. A red point also looks at the black point to its east (the first one of a row
+// at the one to its west too), so that every black point is looked at once.
+__global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
+    gs_norm_kernel(const double* __restrict__ u, int m, int n, int64_t pitch, double* __restrict__ partials,
+                   const NormEnd end)
+{
+    const FmaOps o = load_fma_ops();
+    const double d = in_reg(o, 4.0);
+    double acc = 0.0;
+    auto blacks = [&](const Stencil5& x, int64_t at, int i) {
+        if (i + 1 <= m - 2 && irregular(x.e)) acc = black_square(u + at + 1, pitch, o.one, o.nzero, acc);
+        if (i == 2 && irregular(x.w)) acc = black_square(u + at - 1, pitch, o.one, o.nzero, acc);
+    };
+    // the walk's column t = 1, 2, .. of row j is red point i = 1 + (1 + j & 1) + 2 (t - 1)
+    StrideWalk<NORM_THREADS> p((m - 1) / 2 + 2, n);
+    auto column = [&] { return 1 + ((1 + p.j) & 1) + 2 * (p.i - 1); };
+    while (p.left >= 2) {
+        const int i0 = column(), j0 = p.j;
+        p.next();
+        const int i1 = column(), j1 = p.j;
+        p.next();
+        const bool in0 = i0 <= m - 2, in1 = i1 <= m - 2;
+        const int64_t a0 = (int64_t)j0 * pitch + (in0 ? i0 : 1), a1 = (int64_t)j1 * pitch + (in1 ? i1 : 1);
+        const Stencil5 x0 = load5(u + a0, pitch), x1 = load5(u + a1, pitch);
+        const double r0 = defect5<true, false>(o, x0, 0.0, 1.0, d);
+        const double r1 = defect5<true, false>(o, x1, 0.0, 1.0, d);
+        if (in0) {
+            acc = __fma_rn(r0, r0, acc);
+            blacks(x0, a0, i0);
+        }
+        if (in1) {
+            acc = __fma_rn(r1, r1, acc);
+            blacks(x1, a1, i1);
+        }
+    }
+    if (p.left > 0 && column() <= m - 2) {
+        const int i = column();
+        const int64_t at = (int64_t)p.j * pitch + i;
+        const Stencil5 x = load5(u + at, pitch);
+        const double r = defect5<true, false>(o, x, 0.0, 1.0, d);
+        acc = __fma_rn(r, r, acc);
+        blacks(x, at, i);
+    }
+    __shared__ double red[NORM_THREADS / 32];
+    acc = warp_sum(acc);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    double v = 0.0;
+    if (threadIdx.x < 32) v = warp_sum(threadIdx.x < NORM_THREADS / 32 ? red[threadIdx.x] : 0.0);
+    norm_end(end, v, partials, red);
+}
+
 __global__ void __launch_bounds__(NORM_THREADS)
     sum_partials_kernel(const double* __restrict__ partials, int count, double* __restrict__ out)
 {
@@ -388,6 +443,14 @@ cudaError_t launch_defect_sumsq(const Field& f, const double* q, const Coef& c, 
     LAP_DISPATCH_BOOL(c.unit_beta, UB, LAP_DISPATCH_BOOL(q != nullptr, HQ,
         defect_sumsq_kernel<UB, HQ><<<blocks, NORM_THREADS, 0, s>>>(f.p, q, f.m, f.n, f.pitch, c.b2,
                                                                     c.d, partials, end)));
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gs_norm(const Field& f, double* partials, cudaStream_t s, const NormEnd& end)
+{
+    const int blocks = norm_blocks_for((f.m - 1) / 2 + 2, f.n);
+    gs_norm_kernel<<<blocks, NORM_THREADS, 0, s>>>(f.p, f.m, f.n, f.pitch, partials, end);
     note_launch();
     return cudaGetLastError();
 }

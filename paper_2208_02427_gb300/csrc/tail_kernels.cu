@@ -176,14 +176,6 @@ __device__ __forceinline__ void tail_pass(const Tail<T>& t, const TailLevel& g, 
     }
 }
 
-// A value whose residual may be other than zero after a Gauss-Seidel update with 1/d = 2^-k: zero,
-// subnormal, infinite or NaN.
-__device__ __forceinline__ bool irregular(double x)
-{
-    const int e = (__double2hiint(x) >> 20) & 0x7ff;
-    return e == 0 || e == 0x7ff;
-}
-
 // Takes the restricted residual v of coarse point (I, J): C.q, and the first red pass there (the
 // correction starts at zero: s = 0 + q) for a red point. dst: the arrays that hold the coarse level,
 // cb0 the row of their slot 1. first: there is a red pass to do.
