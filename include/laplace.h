@@ -130,23 +130,24 @@ typedef struct {
                              <= tail_size run as one kernel per V-cycle (the small-level
                              tail, on one CTA or a thread-block cluster: a barrier per phase
                              instead of a launch; the same arithmetic, so the same iterates
-                             bit for bit). 0 = chosen (one grid: by the levels' sizes; a
-                             batch: by timing its first cycles), -1 = never; otherwise >= 3 */
+                             bit for bit). 0 = chosen by the levels' sizes (a batch: its size),
+                             -1 = never; otherwise >= 3 */
     int32_t unfused;      /* LAP_MG_MIXED: 0 = each FP32 level's descent (smoothing, residual,
                              restriction) and ascent (interpolation, smoothing) run as one
                              shared-memory tile kernel each; non-zero = one kernel per pass
                              (the same values bit for bit; the reference for the tiles) */
     int32_t tiling;       /* batched LAP_MG_MIXED with unfused == 0: how the FP32 levels run.
-                             0 = chosen by timing (see lap_solve_batched), -1 = one kernel per
+                             0 = chosen (see lap_solve_batched), -1 = one kernel per
                              pass, 1..3 = tiles of one variant (1: 512 threads over 128 x 64
                              regions, 2: 1024 threads over 128 x 64, 3: 512 threads over
                              128 x 32). Every choice gives the same values bit for bit */
     int32_t item_points;  /* batched solves: interior points per work item of the per-pass
-                             kernels (>= 32), 0 = chosen by timing. No effect on the values */
+                             kernels (>= 32), 0 = chosen by the batch's size. No effect on
+                             the values */
     int32_t persistent;   /* batched solves: how a phase's work items map to CTAs. -1 = one
                              CTA per item, 1 = persistent: as many CTAs as fit the device at
                              once, each claiming the next unclaimed item until none is left;
-                             0 = chosen by timing. No effect on the values */
+                             0 = one CTA per item. No effect on the values */
     int32_t sum_order;    /* lap_sum_order (default LAP_SUM_PAPER). LAP_SUM_DIAGONAL with any
                              other method: LAP_EINVAL; with dx != dy: LAP_EUNSUPPORTED */
 } lap_params;
@@ -207,17 +208,14 @@ int lap_solve_host(lap_handle h, const lap_grid* g, double* psi_host, int64_t ho
  * Every phase of a cycle is one launch over all problems that take part in it; each
  * problem gets exactly the arithmetic of its own lap_solve (per problem the iterates are
  * the same), stops on its own (convergence is decided on the device) and reports in
- * results[k] (host). While the launch configuration is still being chosen (below), the
- * host polls the number of problems still running every p->check_every cycles; once it is
- * chosen (and graphs are on), the remaining cycles run on the device as one conditional CUDA
+ * results[k] (host). With graphs on, the cycles run on the device as one conditional CUDA
  * graph that stops itself when no problem is left or p->max_iter cycles are done, and the host
- * waits once. Synchronises `stream` before returning.
- * The launch configuration -- the small-level tail size (p->tail_size), the FP32 levels'
- * temporal blocking and tile shape (p->tiling), the per-pass kernels' work-item size
- * (p->item_points) and persistent or one-CTA-per-item launches (p->persistent) -- is chosen
- * by timing where a parameter leaves it open (0): the first
- * cycles of a batch shape each run a different candidate, one knob at a time, the fastest
- * is kept in the handle for that shape. No choice changes a value.
+ * waits once; without, the host polls the number of problems still running every
+ * p->check_every cycles. Synchronises `stream` before returning.
+ * Where a parameter leaves the launch configuration open (0) it follows from the batch: a
+ * small-level tail for a small FP64 batch only, the FP32 levels as row streams (tiling 4 in lap_last_batch_config; as tiles
+ * of variant 1 where the smoothing counts are outside 1..3), work items of 1024 to 4096 points,
+ * one CTA per item. No choice changes a value.
  * The plan of a call (level descriptors, work lists, the captured cycle graphs) stays in the
  * handle: a following call with the same grids, field addresses and multigrid parameters
  * reuses it, unless another call of the handle has used its scratch memory in between. */
@@ -226,10 +224,9 @@ int lap_solve_batched(lap_handle h, int count, const lap_grid* grids, double* co
 
 /* The launch configuration of the last cycle of the last lap_solve_batched call on h (no
  * counterpart in the paper; for reports): *tail_size (-1 = no tail), *tiling (-1 = one kernel
- * per pass, 1..3 = tile variant; see lap_params), *item_points, *persistent (1 = persistent
- * launches, -1 = one CTA per item), and *tuned = 1 if the choice by timing had finished for
- * that batch shape (0 while candidates were still being timed). Any pointer may be NULL. All
- * zero before the first batched solve. */
+ * per pass, 1..3 = tile variant, 4 = row streams; see lap_params), *item_points, *persistent (1 = persistent
+ * launches, -1 = one CTA per item), and *tuned = 1 (the choice
+ * takes no timing). Any pointer may be NULL. All zero before the first batched solve. */
 int lap_last_batch_config(lap_handle h, int32_t* tail_size, int32_t* tiling, int32_t* item_points,
                           int32_t* persistent, int32_t* tuned);
 

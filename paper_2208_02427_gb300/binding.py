@@ -272,8 +272,8 @@ class Laplace:
                  "r_final": r.r_final, "last_check": r.last_check} for r in res]
 
     def last_batch_config(self) -> dict:
-        """The launch configuration the last batched cycle ran, and whether the choice by timing
-        had finished (see lap_last_batch_config)."""
+        """The launch configuration the last batched cycle ran; tuned is true once there was one
+        (see lap_last_batch_config)."""
         v = [c_int32(0) for _ in range(5)]
         _check(self._lib.lap_last_batch_config(self._h, *[C.byref(x) for x in v]))
         return {"tail_size": v[0].value, "tiling": v[1].value, "item_points": v[2].value,

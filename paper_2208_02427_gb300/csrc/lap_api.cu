@@ -516,35 +516,6 @@ int mg_level_count(int m, int n, int coarsest_min, int max_levels)
     return levels;
 }
 
-// Tail sizes worth timing for a batch of V-cycles (one CTA per problem runs the levels at or below
-// the size).
-std::vector<int> tail_candidates(int tail_size)
-{
-    if (tail_size != 0) return {tail_size};
-    return {-1, 33, 65, 129, 257};
-}
-
-std::string tuner_key(char kind, const lap_params* p, const std::vector<int>& shape)
-{
-    uint64_t hsh = 1469598103934665603ull;  // FNV-1a over the shapes
-    for (int v : shape) {
-        hsh ^= (uint32_t)v;
-        hsh *= 1099511628211ull;
-    }
-    char buf[240];
-    std::snprintf(buf, sizeof buf, "%c %d %d %d %d %d %.17g %d %d %d %d %d %d %zu %llx", kind,
-                  p->method, p->nu1, p->nu2, p->coarsest_min, p->max_levels, p->smoother_w,
-                  p->inner_cycles, p->tail_size, p->unfused, p->tiling, p->item_points,
-                  p->persistent, shape.size(), (unsigned long long)hsh);
-    return buf;
-}
-
-cudaEvent_t tuner_event(lap_handle h, int k)
-{
-    if (!h->ev[k]) ck(cudaEventCreate(&h->ev[k]), "create event");
-    return h->ev[k];
-}
-
 }  // namespace lap
 
 using namespace lap;
@@ -1541,8 +1512,6 @@ void lap_destroy(lap_handle h)
     for (auto& kv : h->coarse) dev_free(h, kv.second.dev, kv.second.bytes);
     drop_graphs(h);
     if (h->capture) cudaStreamDestroy(h->capture);
-    for (cudaEvent_t e : h->ev)
-        if (e) cudaEventDestroy(e);
     dev_free(h, h->lscratch, h->lscratch_bytes);
     dev_free(h, h->hfield, h->hfield_bytes);
     dev_free(h, h->lsync, h->lsync_bytes);

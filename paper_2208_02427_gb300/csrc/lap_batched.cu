@@ -155,9 +155,9 @@ struct BatchPlan {
     int levels = 0;
 };
 
-// The work lists of one tuner candidate (a BatchConfig), on the device in one allocation, and
-// the cycle graph captured with them.
-struct CandPlan {
+// The work lists of a configuration, on the device in one allocation, and the cycle graphs captured
+// with them.
+struct CyclePlan {
     LevelLists L;
     BatchItem* items = nullptr;
     TailJob* jobs = nullptr;
@@ -165,8 +165,6 @@ struct CandPlan {
     StreamItem* streams = nullptr;
     void* dev = nullptr;
     size_t bytes = 0;
-    cudaGraphExec_t exec = nullptr;
-    int64_t kernels = 0;  // kernels one replay of exec launches
     // the device-resident loop: cycle after cycle as the body of a conditional (while) node
     cudaGraphExec_t loop_exec = nullptr;
     int64_t loop_kernels = 0;  // kernels one iteration of the loop launches
@@ -203,7 +201,6 @@ struct BatchCache : BatchCacheBase {
     BatchKey key;
     BatchPlan P;
     uint64_t epoch = 0;
-    size_t level_bytes = 0;
     BatchLevel<double>* lv64 = nullptr;
     BatchLevel<float>* lv32 = nullptr;
     BatchItem* norm_items = nullptr;
@@ -212,14 +209,11 @@ struct BatchCache : BatchCacheBase {
     double *r0 = nullptr, *rnow = nullptr, *partials = nullptr;
     unsigned* claim = nullptr;  // item counter of the persistent launches (two words, zero between launches)
     long long* loop = nullptr;  // device-resident loop: cycles done, cycle cap
-    std::vector<CandPlan> cands;  // indexed like the tuner's candidates
+    CyclePlan plan;
     ~BatchCache() override
     {
-        for (CandPlan& c : cands) {
-            if (c.exec) cudaGraphExecDestroy(c.exec);
-            if (c.loop_exec) cudaGraphExecDestroy(c.loop_exec);
-            dev_free(h, c.dev, c.bytes);
-        }
+        if (plan.loop_exec) cudaGraphExecDestroy(plan.loop_exec);
+        dev_free(h, plan.dev, plan.bytes);
     }
 };
 
@@ -245,32 +239,28 @@ BatchKey make_key(int count, const lap_grid* grids, double* const* psi_devs, con
     return k;
 }
 
-// The configurations a batched solve of these parameters tries (first = the default of each
-// knob): tail sizes, FP32 tilings (mixed solver, tiles allowed: the tile variants and one
-// kernel per pass), work-item sizes, one CTA per item or persistent launches.
-void tuner_values(const lap_params* p, std::vector<int>* tails, std::vector<int>* tilings,
-                  std::vector<int>* items, std::vector<int>* persists)
+// The configuration of a batched solve where its parameters leave it open, for `points` level-0 points
+// in all: none changes a value. Tail: FP64 levels up to 33 points wide as one CTA per problem while the
+// batch is below about 10M points (whole solves without / with it: 24 grids up to 129^2 1650 / 1400 us, 256 up
+// to 257^2 3680 / 3500, 64 up to 513^2 3420 / 3440); above, and for the row streams of the mixed solver, whose
+// small levels are two launches each, it gains nothing (1024 grids up to 513^2: 22.6 / 23.1 ms, mixed 8.0 /
+// 8.6 ms). FP32 levels: row streams where they cover the smoothing counts, else the first tile variant. Work items: about 16 per
+// multiprocessor, so that the last wave is a small part of a pass, between 1024 points (below, a CTA's
+// start outweighs its work) and 4096 (above, nothing is gained). One CTA per item: the block
+// scheduler hands out uniform items as well as a claim counter does.
+BatchConfig batch_config(const lap_params* p, int64_t points)
 {
-    const bool mixed = p->method == LAP_MG_MIXED;
-    *tails = tail_candidates(p->tail_size);
-    tilings->clear();
-    if (mixed && !p->unfused && fused32_supported(p->nu1, p->nu2) && p->tiling >= 0) {
-        // row streams where they cover the smoothing counts (the tiles and the per-pass kernels were
-        // never faster in any batch measured); else the tile variants and one kernel per pass
-        if (p->tiling == 0 && stream32_supported(p->nu1, p->nu2)) {
-            tilings->push_back(FUSED32_STREAMS);
-        } else {
-            for (int v = 1; v <= FUSED32_VARIANTS; ++v)
-                if ((p->tiling == 0 || p->tiling == v) && fused32_variant_supported(v, p->nu1, p->nu2))
-                    tilings->push_back(v);
-            if (p->tiling == 0) tilings->push_back(0);
-        }
+    BatchConfig c;
+    const int64_t per = points / (16 * (int64_t)device_sms());
+    c.tail = p->tail_size != 0 ? p->tail_size : p->method == LAP_MG && per < 4096 ? 33 : -1;
+    c.tiles = 0;
+    if (p->method == LAP_MG_MIXED && !p->unfused && p->tiling >= 0 && fused32_supported(p->nu1, p->nu2)) {
+        if (p->tiling == 0 && stream32_supported(p->nu1, p->nu2)) c.tiles = FUSED32_STREAMS;
+        else c.tiles = fused32_variant_supported(std::max(1, p->tiling), p->nu1, p->nu2) ? std::max(1, p->tiling) : 0;
     }
-    if (tilings->empty()) tilings->push_back(0);  // one kernel per pass
-    if (p->item_points > 0) *items = {p->item_points};
-    else *items = {BATCH_ITEM_POINTS, 2048, 32768};
-    if (p->persistent != 0) *persists = {p->persistent > 0 ? 1 : 0};
-    else *persists = {0, 1};
+    c.item = p->item_points > 0 ? p->item_points : (int)std::min<int64_t>(4096, std::max<int64_t>(1024, per));
+    c.persist = p->persistent > 0 ? 1 : 0;
+    return c;
 }
 
 // The level descriptors, the norm list, the arena carved for them (level buffers first) and
@@ -373,7 +363,6 @@ std::unique_ptr<BatchCache> build_plan(lap_handle h, int count, const lap_grid* 
     Carver cv(arena(h, sz.off));
     carve_all(cv);
     C->epoch = h->arena_epoch;
-    C->level_bytes = (size_t)((char*)C->lv64 - (char*)h->arena);
     ck(cudaMemcpyAsync(C->lv64, P.lv64.data(), P.lv64.size() * sizeof(P.lv64[0]), cudaMemcpyHostToDevice, s), "upload levels");
     ck(cudaMemcpyAsync(C->lv32, P.lv32.data(), P.lv32.size() * sizeof(P.lv32[0]), cudaMemcpyHostToDevice, s), "upload levels");
     ck(cudaMemcpyAsync(C->norm_items, P.norm_items.data(), P.norm_items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, s), "upload items");
@@ -383,13 +372,11 @@ std::unique_ptr<BatchCache> build_plan(lap_handle h, int count, const lap_grid* 
     return C;
 }
 
-// The lists of candidate c (configuration cfg), built and uploaded on first use; called
-// outside graph capture (it allocates and copies synchronously).
-CandPlan& ensure_candidate(BatchCache& C, int c, const BatchConfig& cfg, const lap_params* p,
-                           int count)
+// The lists of configuration cfg, built and uploaded on first use; called outside graph capture (it
+// allocates and copies synchronously).
+CyclePlan& ensure_plan(BatchCache& C, const BatchConfig& cfg, const lap_params* p, int count)
 {
-    if ((int)C.cands.size() <= c) C.cands.resize(c + 1);
-    CandPlan& K = C.cands[c];
+    CyclePlan& K = C.plan;
     if (K.dev) return K;
     const BatchPlan& P = C.P;
     std::vector<int> all_problems(count);
@@ -446,17 +433,9 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
         }
         const bool mixed = p->method == LAP_MG_MIXED;
         cudaStream_t s = (cudaStream_t)stream;
-        std::vector<int> shape;
-        for (int q = 0; q < count; ++q) {
-            shape.push_back(grids[q].m);
-            shape.push_back(grids[q].n);
-        }
-        BatchTuner& tuner = h->batch_tuners[tuner_key('B', p, shape)];
-        if (tuner.cand.empty()) {
-            std::vector<int> tails, tilings, items, persists;
-            tuner_values(p, &tails, &tilings, &items, &persists);
-            tuner.init(tails, tilings, items, persists);
-        }
+        int64_t points = 0;
+        for (int q = 0; q < count; ++q) points += (int64_t)grids[q].m * grids[q].n;
+        const BatchConfig cfg = batch_config(p, points);
         if (mixed && !p->unfused && fused32_supported(p->nu1, p->nu2))
             ck(prepare_fused32(), "tile kernel attributes");
         // the plan of the previous call, if it was this batch and nothing has carved the arena
@@ -469,9 +448,10 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
         }
         try {
             const BatchPlan& P = C->P;
-            // per call: every level buffer zeroed (rings of corrections stay zero), every
-            // problem active, no cycles done
-            if (C->level_bytes) ck(cudaMemsetAsync(h->arena, 0, C->level_bytes, s), "zero levels");
+            // per call: zero rings (interiors are written before they are read), every problem
+            // active, no cycles done
+            if (mixed) ck(launch_zero_rings(C->lv32, (int)P.lv32.size(), s), "zero rings");
+            else ck(launch_zero_rings(C->lv64, (int)P.lv64.size(), s), "zero rings");
             std::vector<int> ones(count, 1);
             const int cnt = count;
             ck(cudaMemcpyAsync(C->active, ones.data(), count * sizeof(int), cudaMemcpyHostToDevice, s), "upload flags");
@@ -491,7 +471,7 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
             const BatchList norm_list{C->norm_items, (int)P.norm_items.size()};
             const bool rel = p->norm == LAP_NORM_L2_REL;
             // ---- one cycle (V-cycle(s) and stopping test) with candidate c's lists ----
-            auto cycle = [&](const CandPlan& K, cudaStream_t st) {
+            auto cycle = [&](const CyclePlan& K, cudaStream_t st) {
                 const LevelLists& L = K.L;
                 auto list = [&](std::pair<int, int> r) {
                     return BatchList{K.items + r.first, r.second, L.claim};
@@ -522,47 +502,12 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
             ck(launch_b_sumsq(norm_list, lv64, active, partials, mixed ? lv32 : nullptr, s), "batched residual");
             ck(launch_b_converge(partials, first, count, active, r0, rnow, iters, status, remaining, 0,
                                  rel, p->tol, s), "batched convergence");
-            // one cycle of candidate c as a graph, captured on the handle's stream when first
-            // used (kept with the plan for later calls) and replayed on the caller's
-            auto launch_cycle = [&](int c) {
-                CandPlan& K = ensure_candidate(*C, c, tuner.cand[c], p, count);
-                h->last_batch = tuner.cand[c];
-                h->last_batch_tuned = tuner.done;
-                if (!h->use_graphs) {
-                    cycle(K, s);
-                    return;
-                }
-                if (!K.exec) {
-                    if (!h->capture)
-                        ck(cudaStreamCreateWithFlags(&h->capture, cudaStreamNonBlocking), "capture stream");
-                    const int64_t before = launches_now();
-                    ck(cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal), "begin capture");
-                    cudaGraph_t g = nullptr;
-                    try {
-                        cycle(K, h->capture);
-                    } catch (...) {
-                        cudaStreamEndCapture(h->capture, &g);
-                        if (g) cudaGraphDestroy(g);
-                        cudaGetLastError();
-                        throw;
-                    }
-                    ck(cudaStreamEndCapture(h->capture, &g), "end capture");
-                    K.kernels = launches_now() - before;
-                    add_launches(-K.kernels);
-                    const cudaError_t e = cudaGraphInstantiate(&K.exec, g, 0);
-                    cudaGraphDestroy(g);
-                    ck(e, "instantiate graph");
-                }
-                ck(cudaGraphLaunch(K.exec, s), "launch graph");
-                add_launches(K.kernels);
-            };
-            // once the configuration is chosen: the remaining cycles on the device, each followed
-            // by the loop test, as one conditional graph replayed on the caller's stream until no
-            // problem is left or max_iter cycles are done; the host waits once
-            auto device_loop = [&](int c, int64_t done) {
-                CandPlan& K = ensure_candidate(*C, c, tuner.cand[c], p, count);
-                h->last_batch = tuner.cand[c];
-                h->last_batch_tuned = true;
+            CyclePlan& K = ensure_plan(*C, cfg, p, count);
+            h->last_batch = cfg;
+            // the cycles on the device, each followed by the loop test, as one conditional graph
+            // replayed on the caller's stream until no problem is left or max_iter cycles are done; the
+            // host waits once
+            auto device_loop = [&](int64_t done) {
                 if (!K.loop_exec) {
                     if (!h->capture)
                         ck(cudaStreamCreateWithFlags(&h->capture, cudaStreamNonBlocking), "capture stream");
@@ -578,8 +523,23 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
                         np->conditional.handle = hnd;
                         np->conditional.type = cudaGraphCondTypeWhile;
                         np->conditional.size = 1;
-                        cudaGraphNode_t node;
-                        ck(cudaGraphAddNode(&node, g, nullptr, nullptr, 0, np), "conditional node");
+                        // the test before the loop: nothing runs when every problem is already solved
+                        cudaGraphNode_t head = nullptr, node;
+                        ck(cudaStreamBeginCaptureToGraph(h->capture, g, nullptr, nullptr, 0,
+                                                         cudaStreamCaptureModeThreadLocal),
+                           "begin capture");
+                        cudaGraph_t junk = nullptr;
+                        const cudaError_t he = launch_batch_loop_decide(C->loop, remaining, hnd, true, h->capture);
+                        cudaStreamCaptureStatus cs;
+                        const cudaGraphNode_t* deps = nullptr;
+                        size_t nd = 0;
+                        const cudaError_t ie = cudaStreamGetCaptureInfo(h->capture, &cs, nullptr, nullptr, &deps, nullptr, &nd);
+                        if (ie == cudaSuccess && nd == 1) head = deps[0];
+                        ck(cudaStreamEndCapture(h->capture, &junk), "end capture");
+                        ck(he, "batched loop test");
+                        if (!head) fail(LAP_ECUDA, "internal: the loop's first test is not a node");
+                        add_launches(-1);
+                        ck(cudaGraphAddNode(&node, g, &head, nullptr, 1, np), "conditional node");
                         cudaGraph_t body = np->conditional.phGraph_out[0];
                         const int64_t before = launches_now();
                         ck(cudaStreamBeginCaptureToGraph(h->capture, body, nullptr, nullptr, 0,
@@ -587,7 +547,7 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
                            "begin capture");
                         try {
                             cycle(K, h->capture);
-                            ck(launch_batch_loop_decide(C->loop, remaining, hnd, h->capture),
+                            ck(launch_batch_loop_decide(C->loop, remaining, hnd, false, h->capture),
                                "batched loop test");
                         } catch (...) {
                             cudaGraph_t junk = nullptr;
@@ -613,48 +573,18 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
                 ck(cudaMemcpyAsync(h->pinned, C->loop, sizeof st, cudaMemcpyDeviceToHost, s), "copy loop state");
                 ck(cudaStreamSynchronize(s), "stream sync");
                 std::memcpy(st, h->pinned, sizeof st);
-                add_launches(K.loop_kernels * (st[0] - (long long)done));
+                add_launches(K.loop_kernels * (st[0] - (long long)done) + 1);
                 return (int64_t)st[0];
             };
-            int64_t done = 0;
-            int left = count;
-            while (done < p->max_iter) {
+            if (h->use_graphs && p->max_iter > 0) device_loop(0);
+            for (int64_t done = 0; !h->use_graphs && done < p->max_iter;) {
+                int left = 0;
                 ck(cudaMemcpyAsync(h->pinned, remaining, sizeof(int), cudaMemcpyDeviceToHost, s), "copy count");
                 ck(cudaStreamSynchronize(s), "stream sync");
                 std::memcpy(&left, h->pinned, sizeof(int));
                 if (left == 0) break;
-                if (tuner.done && h->use_graphs) {
-                    done = device_loop(tuner.best, done);
-                    continue;
-                }
                 const int64_t steps = std::min<int64_t>(p->check_every, p->max_iter - done);
-                for (int64_t k = 0; k < steps; ++k) {
-                    const int c = tuner.next();
-                    if (tuner.done) {
-                        launch_cycle(c);
-                        continue;
-                    }
-                    if (left < count) {
-                        // problems already converged make the cycle cheaper: its time is not
-                        // comparable, so the best configuration so far runs untimed
-                        launch_cycle(tuner.best);
-                        continue;
-                    }
-                    // not tuned yet: time this cycle (candidate c's graph captured before e0)
-                    const bool fresh = c >= (int)C->cands.size() || !C->cands[c].dev || !C->cands[c].exec;
-                    if (h->use_graphs && fresh) {
-                        launch_cycle(c);  // first use builds, captures and runs it once
-                        ck(cudaStreamSynchronize(s), "stream sync");
-                        continue;
-                    }
-                    ck(cudaEventRecord(tuner_event(h, 0), s), "record event");
-                    launch_cycle(c);
-                    ck(cudaEventRecord(tuner_event(h, 1), s), "record event");
-                    ck(cudaEventSynchronize(tuner_event(h, 1)), "event sync");
-                    float ms = 0.f;
-                    ck(cudaEventElapsedTime(&ms, tuner_event(h, 0), tuner_event(h, 1)), "event time");
-                    tuner.record(c, ms);
-                }
+                for (int64_t k = 0; k < steps; ++k) cycle(K, s);
                 done += steps;
             }
             // ---- results ----
@@ -689,6 +619,6 @@ extern "C" int lap_last_batch_config(lap_handle h, int32_t* tail_size, int32_t* 
         if (tiling) *tiling = h->last_batch.tiles == 0 ? -1 : h->last_batch.tiles;
         if (item_points) *item_points = h->last_batch.item;
         if (persistent) *persistent = h->last_batch.item == 0 ? 0 : (h->last_batch.persist ? 1 : -1);
-        if (tuned) *tuned = h->last_batch_tuned ? 1 : 0;
+        if (tuned) *tuned = h->last_batch.item == 0 ? 0 : 1;
     });
 }

@@ -41,85 +41,6 @@ struct BatchConfig {
     }
 };
 
-// Chooses a batched solve's configuration by timing real cycles, one knob at a time (a
-// coordinate search): stage 0 the small-level tail (the level-to-CTA mapping), stage 1 the
-// FP32 levels' temporal blocking and tile shape (mixed solver), stage 2 the work-item size of
-// the per-pass kernels (when some run), stage 3 one CTA per work item or persistent launches
-// (resident CTAs claiming items from a counter). A stage's candidates are the best configuration so far
-// with that one knob changed; each is timed on one cycle in which every problem still runs
-// (the graph of a candidate is captured on an earlier cycle), and the fastest is kept. The
-// cycles being timed are real cycles of the solve, and all candidates give the same iterates.
-struct BatchTuner {
-    std::vector<BatchConfig> cand;
-    std::vector<double> ms;  // time per cycle, +inf = not timed yet
-    int best = 0;
-    int stage = 0;
-    int stage_begin = 0;
-    bool done = false;
-    std::vector<int> tails, tilings, items, persists;  // the values each stage tries
-    void init(std::vector<int> tail_values, std::vector<int> tiling_values, std::vector<int> item_values,
-              std::vector<int> persist_values)
-    {
-        tails = std::move(tail_values);
-        tilings = std::move(tiling_values);
-        items = std::move(item_values);
-        persists = std::move(persist_values);
-        cand.clear();
-        ms.clear();
-        best = stage = stage_begin = 0;
-        done = false;
-        for (int t : tails) add(BatchConfig{t, tilings.front(), items.front(), persists.front()});
-        if (cand.size() <= 1) advance();
-    }
-    void add(BatchConfig c)
-    {
-        for (const BatchConfig& k : cand)
-            if (k == c) return;
-        cand.push_back(c);
-        ms.push_back(HUGE_VAL);
-    }
-    int next() const
-    {
-        if (done) return best;
-        for (size_t i = stage_begin; i < cand.size(); ++i)
-            if (ms[i] == HUGE_VAL) return (int)i;
-        return best;
-    }
-    void record(int i, double v)
-    {
-        if (done || i < 0 || i >= (int)cand.size() || !(v > 0.0)) return;
-        ms[i] = std::min(ms[i], v);
-        if (ms[best] == HUGE_VAL || ms[i] < ms[best]) best = i;
-        for (size_t k = stage_begin; k < cand.size(); ++k)
-            if (ms[k] == HUGE_VAL) return;
-        advance();
-    }
-    // The next stage with more than the current best to try, or done.
-    void advance()
-    {
-        while (stage < 3) {
-            ++stage;
-            stage_begin = (int)cand.size();
-            const BatchConfig b = cand[best];
-            const std::vector<int>& values = stage == 1 ? tilings : stage == 2 ? items : persists;
-            for (int v : values) {
-                BatchConfig c = b;
-                if (stage == 1) c.tiles = v;
-                else if (stage == 2) c.item = v;
-                else c.persist = v;
-                if (c == b) continue;
-                if (stage == 2 && b.tiles != 0 && c.item != b.item) {
-                    // with tiles the per-pass kernels only serve the tail's neighbours: skip
-                    continue;
-                }
-                add(c);
-            }
-            if ((int)cand.size() > stage_begin) return;
-        }
-        done = true;
-    }
-};
-
 extern thread_local std::string t_last_error;
 
 struct Error {
@@ -190,10 +111,7 @@ struct lap_handle_s {
     bool use_graphs = true;
     cudaStream_t capture = nullptr;
     std::map<std::string, std::pair<cudaGraphExec_t, int64_t>> graphs;  // exec, kernels
-    std::map<std::string, lap::BatchTuner> batch_tuners;  // batched solves' configurations
     lap::BatchConfig last_batch{0, 0, 0, 0};  // the configuration the last batched cycle ran
-    bool last_batch_tuned = false;         // whether its tuner had finished
-    cudaEvent_t ev[2] = {nullptr, nullptr};
     // y-line scratch of line relaxation: forward-elimination values and chunk ends (grown on
     // demand)
     double* lscratch = nullptr;
@@ -260,10 +178,6 @@ constexpr int COARSE_MAX_UNKNOWNS = 1024;
 const double* coarse_inverse(lap_handle h, int m, int n, double b2, double d);
 int mg_level_count(int m, int n, int coarsest_min, int max_levels);
 
-// the timing-based choice of a batched solve's configuration
-std::vector<int> tail_candidates(int tail_size);
-std::string tuner_key(char kind, const lap_params* p, const std::vector<int>& shape);
-cudaEvent_t tuner_event(lap_handle h, int k);
 
 // ---- V-cycles over many problems (lap_batched.cu, lap_server.cu) ----
 // Interior points per work item (rows are not split). Measured on the 4096-grid batch (sides

@@ -143,10 +143,10 @@ cudaError_t launch_check_rounding(long long count, unsigned long long seed, unsi
 // The stopping test of a loop on *maxd (MAXDELTA): cudaGraphSetConditional(h, keep going).
 cudaError_t launch_loop_decide(LoopState* st, const unsigned long long* maxd, cudaGraphConditionalHandle h,
                                cudaStream_t s);
-// Batched solves: st[0] += 1 (cycles done), then the loop's condition := some problem still
-// running (*remaining > 0) and st[0] < st[1] (the cycle cap).
+// Batched solves: st[0] += 1 (cycles done; not before the loop, first), then the loop's condition :=
+// some problem still running (*remaining > 0) and st[0] < st[1] (the cycle cap).
 cudaError_t launch_batch_loop_decide(long long* st, const int* remaining, cudaGraphConditionalHandle h,
-                                     cudaStream_t s);
+                                     bool first, cudaStream_t s);
 // maxd := max |a - b| over interior nodes (bit pattern), a and b share f's shape/pitch.
 cudaError_t launch_maxdelta(const Field& a, const double* b, unsigned long long* maxd,
                             cudaStream_t s);
@@ -272,6 +272,9 @@ struct SolveSetup {
 };
 template <class T>
 cudaError_t launch_setup(const SolveSetup<T>& a, cudaStream_t s);
+// Zero rings in the u, q and r buffers of a batch's levels lv[0 .. count).
+template <class T>
+cudaError_t launch_zero_rings(const BatchLevel<T>* lv, int count, cudaStream_t s);
 // per_level_w: Eq. 7 with each level's own w (BatchLevel::w) instead of the argument
 template <class T>
 cudaError_t launch_b_rb(const BatchList& l, const BatchLevel<T>* lv, const int* active, int colour,

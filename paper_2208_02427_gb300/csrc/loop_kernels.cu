@@ -57,17 +57,37 @@ __global__ void setup_kernel(const SolveSetup<T> a)
     }
 }
 
-// The loop test of a device-resident batched solve, run after each cycle inside the body of
-// a conditional CUDA graph: st[0] counts the cycles, st[1] is the cap; the loop goes on while
-// some problem is still running (the convergence kernel counts them down) and the cap is not
+// The loop test of a device-resident batched solve, run before the loop (first) and after each cycle
+// inside the body of a conditional CUDA graph: st[0] counts the cycles, st[1] is the cap; the loop goes
+// on while some problem is still running (the convergence kernel counts them down) and the cap is not
 // reached.
 __global__ void batch_loop_decide_kernel(long long* st, const int* __restrict__ remaining,
-                                         cudaGraphConditionalHandle h)
+                                         cudaGraphConditionalHandle h, int first)
 {
     if (threadIdx.x != 0) return;
-    const long long k = st[0] + 1;
+    const long long k = st[0] + (first ? 0 : 1);
     st[0] = k;
     cudaGraphSetConditional(h, *remaining > 0 && k < st[1] ? 1u : 0u);
+}
+
+// The rings of the u, q and r buffers of a batch's levels set to zero, a block per level (level 0 of
+// an FP64 problem, the caller's field, has no q and is left alone).
+template <class T>
+__global__ void zero_rings_kernel(const BatchLevel<T>* __restrict__ lv)
+{
+    const BatchLevel<T> V = lv[blockIdx.x];
+    if (!V.q) return;
+    const int64_t m = V.m, n = V.n;
+    for (int64_t k = threadIdx.x; k < 2 * (m + n); k += blockDim.x) {
+        int64_t at;
+        if (k < m) at = k;
+        else if (k < 2 * m) at = (n - 1) * V.pitch + (k - m);
+        else if (k < 2 * m + n) at = (k - 2 * m) * V.pitch;
+        else at = (k - 2 * m - n) * V.pitch + (m - 1);
+        V.u[at] = (T)0;
+        V.q[at] = (T)0;
+        if (V.r) V.r[at] = (T)0;
+    }
 }
 
 }  // namespace
@@ -167,12 +187,23 @@ cudaError_t launch_check_rounding(long long count, unsigned long long seed, unsi
 }
 
 cudaError_t launch_batch_loop_decide(long long* st, const int* remaining, cudaGraphConditionalHandle h,
-                                     cudaStream_t s)
+                                     bool first, cudaStream_t s)
 {
-    batch_loop_decide_kernel<<<1, 32, 0, s>>>(st, remaining, h);
+    batch_loop_decide_kernel<<<1, 32, 0, s>>>(st, remaining, h, first ? 1 : 0);
     note_launch();
     return cudaGetLastError();
 }
+
+template <class T>
+cudaError_t launch_zero_rings(const BatchLevel<T>* lv, int count, cudaStream_t s)
+{
+    if (count <= 0) return cudaSuccess;
+    zero_rings_kernel<T><<<count, 256, 0, s>>>(lv);
+    note_launch();
+    return cudaGetLastError();
+}
+template cudaError_t launch_zero_rings<double>(const BatchLevel<double>*, int, cudaStream_t);
+template cudaError_t launch_zero_rings<float>(const BatchLevel<float>*, int, cudaStream_t);
 
 cudaError_t launch_loop_decide(LoopState* st, const unsigned long long* maxd, cudaGraphConditionalHandle h,
                                cudaStream_t s)
