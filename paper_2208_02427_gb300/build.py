@@ -21,7 +21,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["lap_api.cu", "lap_batched.cu", "lap_server.cu", "point_kernels.cu", "line_kernels.cu", "mg_kernels.cu",
            "mixed_kernels.cu", "lex_kernels.cu", "batch_kernels.cu", "fused32_kernels.cu",
            "loop_kernels.cu", "small_kernels.cu",
-           "stream32_kernels.cu", "tail_kernels.cu"]
+           "stream32_kernels.cu", "tail_kernels.cu", "sweep_tiles.cu"]
 HEADERS = ["lap_internal.cuh", "lap_device.cuh", "lap_host.cuh", "vcycle_arith.cuh",
            "norm_end.cuh", "gs_restrict.cuh"]
 

@@ -70,13 +70,30 @@ Coef make_coef(double dx, double dy)
 
 void set_device(lap_handle h) { ck(cudaSetDevice(h->device), "cudaSetDevice"); }
 
+// Gives the spare buffer back (and the graphs that use it); false if there is none. It is used inside
+// lap_solve alone, which ends synchronised, so nothing in flight reads it.
+static bool drop_spare(lap_handle h)
+{
+    if (!h->spare) return false;
+    drop_graphs(h);
+    dev_free(h, h->spare, h->spare_bytes);
+    h->spare = nullptr;
+    h->spare_bytes = 0;
+    return true;
+}
+
 void* dev_alloc(lap_handle h, size_t bytes)
 {
+    if (h->budget && h->held + bytes > h->budget) drop_spare(h);
     if (h->budget && h->held + bytes > h->budget)
         fail(LAP_ENOMEM, "HBM budget of the handle exceeded (" + std::to_string(h->held + bytes) +
                              " > " + std::to_string(h->budget) + " bytes)");
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation && drop_spare(h)) {
+        cudaGetLastError();
+        e = cudaMalloc(&p, bytes);
+    }
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         fail(LAP_ENOMEM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
@@ -114,6 +131,24 @@ double* arena(lap_handle h, size_t bytes)
         h->arena_bytes = bytes;
     }
     return h->arena;
+}
+
+double* spare(lap_handle h, size_t bytes)
+{
+    bytes = (size_t)round_up((int64_t)bytes, 1 << 20);
+    if (bytes > h->spare_bytes) {
+        drop_spare(h);
+        if (h->budget && h->held + bytes > h->budget) return nullptr;
+        void* p = nullptr;
+        if (cudaMalloc(&p, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        h->spare = p;
+        h->spare_bytes = bytes;
+        h->held += bytes;
+    }
+    return (double*)h->spare;
 }
 
 void check_grid(const lap_grid* g)
@@ -698,6 +733,56 @@ struct Solver {
     double* jac_cur = nullptr;  // Jacobi: buffer holding the current iterate
     double* jac_other = nullptr;
 
+    // ---- several sweeps per launch (sweep_tiles.cu) ----
+    SweepTiles tiles;                // sweeps = 0: one pass per launch
+    double* tiles_other = nullptr;   // the second field
+    int sweep_kind() const
+    {
+        return p->method == LAP_JACOBI ? SWEEP_JACOBI : p->method == LAP_GS_RB ? SWEEP_GS : SWEEP_SOR;
+    }
+    bool tiles_diag() const { return p->method != LAP_JACOBI && p->sum_order == LAP_SUM_DIAGONAL; }
+
+    // Takes the tiles where they pay and their second field is to be had.
+    void choose_tiles()
+    {
+        tiles = SweepTiles{};
+        if (p->method != LAP_JACOBI && p->method != LAP_GS_RB && p->method != LAP_SOR_RB) return;
+        if (p->check_every < 2 || p->max_iter < 2) return;
+        tiles = plan_sweep_tiles(f.m, f.n, c, sweep_kind(), tiles_diag(), device_sms());
+        if (!tiles.sweeps) return;
+        tiles_other = p->method == LAP_JACOBI ? w.aux : spare(h, (size_t)f.n * f.pitch * sizeof(double));
+        if (!tiles_other) tiles = SweepTiles{};
+        else ck(prepare_sweep_tiles(c, sweep_kind(), tiles_diag()), "tile sweep attributes");
+    }
+
+    // The sweeps of a period that run on tiles. One whose largest change is asked for runs pass by pass
+    // (Jacobi: two at the end of an even period, so that its buffers keep their roles).
+    int64_t tiled_count(int64_t steps, bool maxdelta) const
+    {
+        if (!tiles.sweeps) return 0;
+        const int64_t count = steps - (!maxdelta ? 0 : p->method == LAP_JACOBI && !(steps & 1) ? 2 : 1);
+        return count >= 2 ? count : 0;
+    }
+    // Whether a period leaves Jacobi's iterate in the other buffer.
+    bool flips(int64_t steps, bool maxdelta) const
+    {
+        return p->method == LAP_JACOBI && ((steps - tiled_count(steps, maxdelta)) & 1);
+    }
+
+    // `count` >= 2 sweeps in an even number of launches, so that the iterate ends where it was.
+    void tiled_sweeps(int64_t count)
+    {
+        const int64_t launches = 2 * ((count + 2 * tiles.sweeps - 1) / (2 * tiles.sweeps));
+        double* a = p->method == LAP_JACOBI ? jac_cur : f.p;
+        double* b = p->method == LAP_JACOBI ? jac_other : tiles_other;
+        for (int64_t k = 0; k < launches; ++k) {
+            const int sweeps = (int)(count / launches + (k < count % launches ? 1 : 0));
+            ck(launch_sweep_tiles(Field{a, f.m, f.n, f.pitch}, b, c, tiles, sweep_kind(), tiles_diag(), sweeps, w.wslot, s),
+               "tile sweeps");
+            std::swap(a, b);
+        }
+    }
+
     // norm: what the mixed iteration's closing residual does with its sums
     void iterate(bool want_maxd, const NormEnd& norm)
     {
@@ -1020,7 +1105,9 @@ struct Solver {
             }
             return;
         }
-        for (int64_t st = 0; st < steps; ++st) {
+        const int64_t tiled = tiled_count(steps, maxdelta);
+        if (tiled) tiled_sweeps(tiled);
+        for (int64_t st = tiled; st < steps; ++st) {
             const bool last = st == steps - 1;
             if (last && maxdelta) {
                 ck(cudaMemsetAsync(w.maxd, 0, 8, s), "zero max delta");
@@ -1060,9 +1147,9 @@ struct Solver {
                                 p->nu1, p->nu2, p->coarsest_min, p->max_levels, p->line_form,
                                 (int64_t)w.levels.size(), p->inner_cycles,
                                 (int64_t)w.levels32.size(), tail_first, fused32, norm_sc > 0.0,
-                                p->sum_order};
+                                p->sum_order, tiles.sweeps, tiles.tx, tiles.ty};
         const double dbl[] = {c.b2, c.d, c.inv_d, p->w, p->smoother_w};
-        const void* ptrs[] = {f.p, jac_cur, jac_other, w.aux, w.maxd, h->arena, h->lscratch};
+        const void* ptrs[] = {f.p, jac_cur, jac_other, w.aux, w.maxd, h->arena, h->lscratch, tiles_other};
         put(ints, sizeof ints);
         put(dbl, sizeof dbl);
         put(ptrs, sizeof ptrs);
@@ -1113,7 +1200,7 @@ struct Solver {
         }
         ck(cudaGraphLaunch(it->second.first, s), "launch graph");
         add_launches(it->second.second);
-        if (p->method == LAP_JACOBI && (steps & 1)) std::swap(jac_cur, jac_other);
+        if (flips(steps, maxdelta)) std::swap(jac_cur, jac_other);
     }
 
     // The residual norm of the current iterate with `end`, enqueued on s. (The mixed iteration's own
@@ -1147,12 +1234,12 @@ struct Solver {
 
     // Device-resident loop: whole check periods, each followed by the stopping test on the
     // device, as the body of a conditional (while) node of one CUDA graph, so that the host
-    // waits once per solve instead of once per period. For full periods (Jacobi: even periods, whose buffer roles repeat).
+    // waits once per solve instead of once per period. For full periods (Jacobi: those that
+    // leave its buffers' roles).
     bool device_loop_ok(int64_t k, int64_t steps) const
     {
         if (!h->use_graphs || steps != p->check_every || k + steps > p->max_iter) return false;
-        if (p->method == LAP_JACOBI && (steps & 1)) return false;
-        return true;
+        return !flips(steps, p->norm == LAP_NORM_MAXDELTA);
     }
 
     // Runs periods on the device until the stopping rule holds or the next period would pass
@@ -1253,7 +1340,7 @@ struct Solver {
                 throw;
             }
             cudaGraphDestroy(g);
-            jac_cur = cur0;  // even periods: the buffer roles are the same after each
+            jac_cur = cur0;  // the buffer roles are the same after each period
             jac_other = other0;
             it = h->graphs.emplace(key, std::make_pair(exec, kernels)).first;
         }
@@ -1314,8 +1401,10 @@ struct Solver {
         out->iters = 0;
         out->last_check = NAN;
         if (p->method == LAP_ADI || p->method == LAP_SLOR) prepare();  // tables, scratch: before any capture
+        choose_tiles();
         if (p->method == LAP_JACOBI) {
-            copy_field(w.aux, f.p);  // ring + initial interior in both buffers
+            // a sweep writes every interior point of the other buffer, and reads none of it before
+            ck(launch_copy_ring(w.aux, f, s), "ring copy");
             jac_cur = f.p;
             jac_other = w.aux;
         }
@@ -1512,6 +1601,7 @@ void lap_destroy(lap_handle h)
     for (auto& kv : h->coarse) dev_free(h, kv.second.dev, kv.second.bytes);
     drop_graphs(h);
     if (h->capture) cudaStreamDestroy(h->capture);
+    dev_free(h, h->spare, h->spare_bytes);
     dev_free(h, h->lscratch, h->lscratch_bytes);
     dev_free(h, h->hfield, h->hfield_bytes);
     dev_free(h, h->lsync, h->lsync_bytes);

@@ -116,6 +116,8 @@ struct lap_handle_s {
     // demand)
     double* lscratch = nullptr;
     size_t lscratch_bytes = 0;
+    void* spare = nullptr;  // second field of the tiled sweeps; given back when memory is short
+    size_t spare_bytes = 0;
     // x-line sweeps: error word, item counter and row flags; one block of at least 1 MiB,
     // allocated on first use and grown only for more than 262,140 lines
     unsigned* lsync = nullptr;
@@ -133,6 +135,9 @@ void dev_free(lap_handle h, void* p, size_t bytes);
 void drop_graphs(lap_handle h);
 // Scratch for one call: grows (never shrinks) the handle's arena.
 double* arena(lap_handle h, size_t bytes);
+// The handle's spare buffer of at least `bytes`, or null where the budget or the device has no room for
+// it: a call that can do without takes its other path.
+double* spare(lap_handle h, size_t bytes);
 
 // Carves aligned sub-buffers out of a byte range.
 struct Carver {

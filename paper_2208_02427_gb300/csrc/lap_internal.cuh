@@ -54,6 +54,19 @@ struct Field32 {
 // Every kernel launch of the library goes through this counter.
 void note_launch();
 
+// Several sweeps in one launch, on tiles in shared memory (sweep_tiles.cu): in -> out, the same values
+// as as many one-pass sweeps leave. diag: neighbour sums paired along diagonals (beta = 1). sweeps = 0 in the
+// plan: the one-pass kernels are as fast.
+enum { SWEEP_JACOBI = 0, SWEEP_SOR = 1, SWEEP_GS = 2 };
+struct SweepTiles {
+    int sweeps = 0;  // at most this many in a launch
+    int tx = 0, ty = 0;
+};
+SweepTiles plan_sweep_tiles(int m, int n, const Coef& c, int kind, bool diag, int sms);
+cudaError_t prepare_sweep_tiles(const Coef& c, int kind, bool diag);
+cudaError_t launch_sweep_tiles(const Field& in, double* out, const Coef& c, const SweepTiles& t, int kind, bool diag,
+                               int sweeps, const double* wslot, cudaStream_t s);
+
 // ---- point kernels (point_kernels.cu) -------------------------------------------
 // One colour of a red-black sweep, in place: Gauss-Seidel (Eq. 6) when gs is true,
 // SOR (Eq. 7) otherwise; q may be null. maxd (nullable) accumulates max|new - old| as
@@ -272,6 +285,8 @@ struct SolveSetup {
 };
 template <class T>
 cudaError_t launch_setup(const SolveSetup<T>& a, cudaStream_t s);
+// dst's ring (src's size and pitch) := src's.
+cudaError_t launch_copy_ring(double* dst, const Field& src, cudaStream_t s);
 // Zero rings in the u, q and r buffers of a batch's levels lv[0 .. count).
 template <class T>
 cudaError_t launch_zero_rings(const BatchLevel<T>* lv, int count, cudaStream_t s);

@@ -70,6 +70,19 @@ __global__ void batch_loop_decide_kernel(long long* st, const int* __restrict__ 
     cudaGraphSetConditional(h, *remaining > 0 && k < st[1] ? 1u : 0u);
 }
 
+// dst's ring := src's.
+__global__ void copy_ring_kernel(double* __restrict__ dst, const double* __restrict__ src, int m, int n, int64_t pitch)
+{
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= 2 * ((int64_t)m + n)) return;
+    int64_t at;
+    if (k < m) at = k;
+    else if (k < 2 * (int64_t)m) at = (n - 1) * pitch + (k - m);
+    else if (k < 2 * (int64_t)m + n) at = (k - 2 * (int64_t)m) * pitch;
+    else at = (k - 2 * (int64_t)m - n) * pitch + (m - 1);
+    dst[at] = src[at];
+}
+
 // The rings of the u, q and r buffers of a batch's levels set to zero, a block per level (level 0 of
 // an FP64 problem, the caller's field, has no q and is left alone).
 template <class T>
@@ -190,6 +203,14 @@ cudaError_t launch_batch_loop_decide(long long* st, const int* remaining, cudaGr
                                      bool first, cudaStream_t s)
 {
     batch_loop_decide_kernel<<<1, 32, 0, s>>>(st, remaining, h, first ? 1 : 0);
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_copy_ring(double* dst, const Field& src, cudaStream_t s)
+{
+    const int64_t points = 2 * ((int64_t)src.m + src.n);
+    copy_ring_kernel<<<(unsigned)((points + 255) / 256), 256, 0, s>>>(dst, src.p, src.m, src.n, src.pitch);
     note_launch();
     return cudaGetLastError();
 }

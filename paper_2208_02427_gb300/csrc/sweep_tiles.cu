@@ -1,0 +1,238 @@
+// sweep_tiles.cu -- several point sweeps in one launch, on tiles in shared memory.
+//
+// A small grid is bound by launches, not by its sweeps: a colour pass over 513 x 385 points is 0.8 us of
+// FP64 arithmetic in a launch of 2.3 us. Here a CTA loads its tile with a halo of one
+// point per pass, runs the passes of `sweeps` sweeps in shared memory with a CTA barrier between them,
+// and writes its own points to the other buffer. Each pass covers one halo point less than the one
+// before, so every value is the one that the passes over the whole grid would have left: the same
+// expression of the same operands, bit for bit. The halo costs arithmetic (a 37 x 39 tile does 1.3 times its
+// own points over three red-black sweeps), so the number of sweeps and the tile follow from the grid
+// (plan_sweep_tiles). What is left beside the FP64 work: a launch and the window's load and store, 1.7 us
+// or more, and about 0.4 us a pass (a point's chain of FP64 operations of 71 cycles each, the barrier, the
+// warps' uneven last round).
+#include <algorithm>
+#include <cmath>
+
+#include "lap_device.cuh"
+#include "lap_internal.cuh"
+
+namespace lap {
+
+namespace {
+
+constexpr int ST_THREADS = 512;
+constexpr size_t ST_SMEM_MAX = 224 * 1024;
+// The cost model of plan_sweep_tiles, in SM cycles beside the FP64 work: a one-pass launch (the walks along
+// diagonals take longer to drain), a tile launch, a window point's load and store, and a pass's latency,
+// barrier and uneven last round. Fitted to times per sweep from 65^2 to 4097^2 points.
+constexpr double PASS_CYCLES = 2900, DIAG_PASS_CYCLES = 5000;
+constexpr double TILE_CYCLES = 3500, TILE_POINT_CYCLES = 0.4, TILE_PASS_CYCLES = 900;
+
+__device__ __forceinline__ void copy8(double* smem, const double* global)
+{
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(global) : "memory");
+}
+
+struct SweepCoef {
+    double b2, inv_d;
+    int shift;
+    double w, omw;
+};
+
+// One point from the tile `a` (row pitch W): the expression of the one-pass kernels.
+template <int KIND, bool UNIT, bool POW2, bool DIAG>
+__device__ __forceinline__ double swept(const FmaOps& o, const double* c, int W, const SweepCoef& k)
+{
+    const double s = DIAG ? fadd(o, fadd(o, c[-1], c[-W]), fadd(o, c[1], c[W]))
+                          : neighbour_sum<UNIT>(o, c[-1], c[1], c[-W], c[W], k.b2);
+    const double g = times_inv_d<POW2>(o, s, k.inv_d, k.shift);
+    return KIND == SWEEP_SOR ? __fma_rn(k.w, g, fmul(o, k.omw, *c)) : g;
+}
+
+// The tile of interior columns [x0, x1) and rows [y0, y1) through `passes` passes (two colours a sweep, or
+// one for Jacobi), in -> out. The ring points beside the tile are copied along, so that `out` needs no
+// preparation. sm: (x1 - x0 + 2 passes) (y1 - y0 + 2 passes) doubles, twice that for Jacobi.
+template <int KIND, bool UNIT, bool POW2, bool DIAG>
+__device__ __forceinline__ void sweep_tile(const FmaOps& o, const double* __restrict__ in, double* __restrict__ out,
+                                           int m, int n, int64_t pitch, int x0, int x1, int y0, int y1, int passes,
+                                           const SweepCoef& k, double* sm)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int X0 = max(0, x0 - passes), X1 = min(m, x1 + passes);
+    const int Y0 = max(0, y0 - passes), Y1 = min(n, y1 + passes);
+    const int W = X1 - X0, H = Y1 - Y0;
+    for (int r = wid; r < H; r += nw) {
+        const double* src = in + (int64_t)(Y0 + r) * pitch + X0;
+        for (int c = lane; c < W; c += 32) copy8(sm + r * W + c, src + c);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    double* a = sm;
+    double* b = sm + W * H;
+    if (KIND == SWEEP_JACOBI) {
+        // the ring, which no pass writes, in the second buffer too
+        for (int t = threadIdx.x; t < W; t += blockDim.x) {
+            b[t] = a[t];
+            b[(H - 1) * W + t] = a[(H - 1) * W + t];
+        }
+        for (int t = threadIdx.x; t < H; t += blockDim.x) {
+            b[t * W] = a[t * W];
+            b[t * W + W - 1] = a[t * W + W - 1];
+        }
+        __syncthreads();
+    }
+    // A pass's region [ia, ib) x [ja, jb) of the window, `per` of its points to a row; thread t takes points
+    // t, t + blockDim, .. row by row: first (r, c), then (dr, dc) on. The quotients from the FP32 divide are
+    // exact: (t + 1/2) / per is at least 1 / (2 per) away from a whole number. Taken before the barrier that
+    // ends the pass before, so that this arithmetic runs beside that pass's FP64 chains.
+    int ia, ib, ja, rows, per, r, c, dr, dc;
+    auto region = [&](int p) {
+        ia = X0 == 0 ? 1 : p + 1;
+        ib = W - (X1 == m ? 1 : p + 1);
+        ja = Y0 == 0 ? 1 : p + 1;
+        rows = H - (Y1 == n ? 1 : p + 1) - ja;
+        per = KIND == SWEEP_JACOBI ? ib - ia : (ib - ia + 1) / 2;
+        const float inv = __fdividef(1.0f, (float)per);
+        r = (int)(((float)threadIdx.x + 0.5f) * inv);
+        c = threadIdx.x - r * per;
+        dr = (int)(((float)blockDim.x + 0.5f) * inv);
+        dc = blockDim.x - dr * per;
+    };
+    region(0);
+    for (int p = 0; p < passes; ++p) {
+        double* dst = KIND == SWEEP_JACOBI ? b : a;
+        while (r < rows) {
+            const int j = ja + r;
+            const int i = ia + (KIND == SWEEP_JACOBI ? c : ((ia + X0 + j + Y0 + p) & 1) + 2 * c);
+            const int at = j * W + i;
+            if (KIND == SWEEP_JACOBI || i < ib) dst[at] = swept<KIND, UNIT, POW2, DIAG>(o, a + at, W, k);
+            c += dc;
+            r += dr;
+            if (c >= per) {
+                c -= per;
+                ++r;
+            }
+        }
+        region(p + 1 < passes ? p + 1 : p);
+        __syncthreads();
+        if (KIND == SWEEP_JACOBI) {
+            double* t = a;
+            a = b;
+            b = t;
+        }
+    }
+    const int sx0 = x0 == 1 ? 0 : x0, sx1 = x1 == m - 1 ? m : x1;
+    const int sy0 = y0 == 1 ? 0 : y0, sy1 = y1 == n - 1 ? n : y1;
+    for (int j = sy0 + wid; j < sy1; j += nw)
+        for (int i = sx0 + lane; i < sx1; i += 32) out[(int64_t)j * pitch + i] = a[(j - Y0) * W + (i - X0)];
+}
+
+// Tile (blockIdx.x, blockIdx.y) of gridDim.x x gridDim.y equal parts of the interior.
+template <int KIND, bool UNIT, bool POW2, bool DIAG>
+__global__ void __launch_bounds__(ST_THREADS)
+    sweep_tiles_kernel(const double* __restrict__ in, double* __restrict__ out, int m, int n, int64_t pitch,
+                       int passes, SweepCoef k, const double* __restrict__ wslot)
+{
+    extern __shared__ double sm[];
+    const FmaOps o = load_fma_ops();
+    if (KIND == SWEEP_SOR) {
+        k.w = wslot[0];
+        k.omw = wslot[1];
+    }
+    if (!UNIT) k.b2 = in_reg(o, k.b2);
+    if (!POW2) k.inv_d = in_reg(o, k.inv_d);
+    const int x0 = 1 + (int)((int64_t)blockIdx.x * (m - 2) / gridDim.x);
+    const int x1 = 1 + (int)((int64_t)(blockIdx.x + 1) * (m - 2) / gridDim.x);
+    const int y0 = 1 + (int)((int64_t)blockIdx.y * (n - 2) / gridDim.y);
+    const int y1 = 1 + (int)((int64_t)(blockIdx.y + 1) * (n - 2) / gridDim.y);
+    sweep_tile<KIND, UNIT, POW2, DIAG>(o, in, out, m, n, pitch, x0, x1, y0, y1, passes, k, sm);
+}
+
+template <class F>
+cudaError_t on_sweep_kernel(const Coef& c, int kind, bool diag, F&& f)
+{
+    const bool pow2 = c.inv_d_shift > 0;
+    if (kind == SWEEP_JACOBI) {
+        if (c.unit_beta) return pow2 ? f(sweep_tiles_kernel<SWEEP_JACOBI, true, true, false>)
+                                     : f(sweep_tiles_kernel<SWEEP_JACOBI, true, false, false>);
+        return pow2 ? f(sweep_tiles_kernel<SWEEP_JACOBI, false, true, false>)
+                    : f(sweep_tiles_kernel<SWEEP_JACOBI, false, false, false>);
+    }
+    if (kind == SWEEP_SOR) {
+        if (diag) return f(sweep_tiles_kernel<SWEEP_SOR, true, true, true>);
+        if (c.unit_beta) return pow2 ? f(sweep_tiles_kernel<SWEEP_SOR, true, true, false>)
+                                     : f(sweep_tiles_kernel<SWEEP_SOR, true, false, false>);
+        return pow2 ? f(sweep_tiles_kernel<SWEEP_SOR, false, true, false>)
+                    : f(sweep_tiles_kernel<SWEEP_SOR, false, false, false>);
+    }
+    if (diag) return f(sweep_tiles_kernel<SWEEP_GS, true, true, true>);
+    if (c.unit_beta) return pow2 ? f(sweep_tiles_kernel<SWEEP_GS, true, true, false>)
+                                 : f(sweep_tiles_kernel<SWEEP_GS, true, false, false>);
+    return pow2 ? f(sweep_tiles_kernel<SWEEP_GS, false, true, false>)
+                : f(sweep_tiles_kernel<SWEEP_GS, false, false, false>);
+}
+
+int halo(int kind, int sweeps) { return kind == SWEEP_JACOBI ? sweeps : 2 * sweeps; }
+
+}  // namespace
+
+// At most one tile per multiprocessor, nearly square, and as many sweeps per launch as cost least; none
+// where the one-pass kernels are within 5%. Measured per sweep (one pass per launch / tiles), SOR in the
+// paper's order: 65^2 3.06 / 1.8 us, 257^2 3.44 / 2.5, 513 x 385 4.8 / 4.0, 700^2 7.4 / 6.8, 1000^2 equal;
+// paired along diagonals 5.4 / 1.8, 5.9 / 2.5, 6.2 / 4.0, 8.4 / 6.8, equal; Jacobi 1.60 / 1.02, 1.91 / 1.57,
+// from 513 x 385 on equal. Two or three smaller tiles per multiprocessor hide a tile's load but have more
+// halo: equal or slower.
+SweepTiles plan_sweep_tiles(int m, int n, const Coef& c, int kind, bool diag, int sms)
+{
+    SweepTiles best;
+    const int colours = kind == SWEEP_JACOBI ? 1 : 2;
+    const double ops = 3.0 + (c.inv_d_shift > 0 ? 0 : 1) + (kind == SWEEP_SOR ? 2 : 0);
+    // per sweep; an FP64 operation takes half a cycle of an SM
+    double least = colours * (diag ? DIAG_PASS_CYCLES : PASS_CYCLES) +
+                   1.07 * (m - 2) * (double)(n - 2) * (ops - (diag ? 1 : 0)) / 2 / sms;
+    least *= 0.95;
+    const int near = (int)std::min(std::sqrt((double)sms * (m - 2) / (n - 2)), (double)sms);
+    for (int sweeps = 1; sweeps <= 8; ++sweeps) {
+        const int h = halo(kind, sweeps);
+        for (int tx = std::max(1, near - 2); tx <= std::min({sms, m - 2, near + 3}); ++tx) {
+            const int ty = std::min(sms / tx, n - 2);
+            const int64_t tw = (m - 2 + tx - 1) / tx, th = (n - 2 + ty - 1) / ty;
+            const int64_t window = (tw + 2 * h) * (th + 2 * h);
+            if (window * 8 * (kind == SWEEP_JACOBI ? 2 : 1) > (int64_t)ST_SMEM_MAX) continue;
+            // points of the h passes: (tw + 2a)(th + 2a) for a = 0 .. h - 1, one colour of them
+            const double sum = (double)h * tw * th + (double)(tw + th) * h * (h - 1) + 2.0 / 3.0 * h * (h - 1) * (2 * h - 1);
+            const double cost =
+                (TILE_CYCLES + window * TILE_POINT_CYCLES + h * TILE_PASS_CYCLES + sum / colours * ops / 2) / sweeps;
+            if (cost < least) {
+                least = cost;
+                best = SweepTiles{sweeps, tx, ty};
+            }
+        }
+    }
+    return best;
+}
+
+cudaError_t prepare_sweep_tiles(const Coef& c, int kind, bool diag)
+{
+    return on_sweep_kernel(c, kind, diag, [](auto* kernel) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ST_SMEM_MAX);
+    });
+}
+
+cudaError_t launch_sweep_tiles(const Field& in, double* out, const Coef& c, const SweepTiles& t, int kind, bool diag,
+                               int sweeps, const double* wslot, cudaStream_t s)
+{
+    const int h = halo(kind, sweeps);
+    const int tw = (in.m - 2 + t.tx - 1) / t.tx, th = (in.n - 2 + t.ty - 1) / t.ty;
+    const size_t bytes = (size_t)(tw + 2 * h) * (th + 2 * h) * 8 * (kind == SWEEP_JACOBI ? 2 : 1);
+    const SweepCoef k{c.b2, c.inv_d, c.inv_d_shift, 1.0, 0.0};
+    const cudaError_t e = on_sweep_kernel(c, kind, diag, [&](auto* kernel) {
+        kernel<<<dim3(t.tx, t.ty), ST_THREADS, bytes, s>>>(in.p, out, in.m, in.n, in.pitch, h, k, wslot);
+        return cudaGetLastError();
+    });
+    note_launch();
+    return e;
+}
+
+}  // namespace lap

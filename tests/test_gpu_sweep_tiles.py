@@ -1,0 +1,67 @@
+"""Several point sweeps per launch on shared-memory tiles against the one-pass kernels, bit for bit:
+sizes on both sides of the rule, uneven tiles, periods that leave every remainder of sweeps per launch,
+a pitch wider than the rows, and the stopping rule that needs the last sweep's largest change."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2208_02427_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(65, 65), (97, 70), (70, 301), (513, 385), (1000, 67), (67, 1000), (641, 479), (1531, 1021), (3, 4000)]
+METHODS = [("jacobi", 1.0, "paper"), ("sor", 1.7, "paper"), ("gs", 1.0, "paper"), ("sor", 1.7, "diagonal"),
+           ("gs", 1.0, "diagonal")]
+
+
+@pytest.fixture(scope="module")
+def b():
+    from paper_2208_02427_gb300 import binding
+    binding.load()
+    return binding
+
+
+def run(b, lap, psi, method, w, order, dx, every, sweeps, norm="l2_rel"):
+    t = b.to_field(psi)
+    r = lap.solve(t, dx, 1.0, method=method, w=w, sum_order=order, tol=0.0, check_every=every, max_iter=sweeps,
+                  norm=norm)
+    torch.cuda.synchronize()
+    return t.cpu().numpy(), r
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("method,w,order", METHODS)
+def test_tiles_equal_single_passes(b, shape, method, w, order):
+    m, n = shape
+    psi = wl.random_interior(wl.random_ring(m, n, 3), 4, 1.0)
+    lap = b.Laplace()
+    for dx in (1.0,) if order == "diagonal" else (1.0, 0.7):
+        want, r1 = run(b, lap, psi, method, w, order, dx, 1, 34)
+        for every in (2, 5, 17, 32, 34):
+            got, r2 = run(b, lap, psi, method, w, order, dx, every, 34)
+            assert np.array_equal(got, want), every
+            assert r1["r_final"] == r2["r_final"]
+    lap.close()
+
+
+@pytest.mark.parametrize("method,w,order", METHODS)
+@pytest.mark.parametrize("norm", ["l2_abs", "maxdelta"])
+def test_norms_graphs_and_budgets(b, method, w, order, norm):
+    m, n = 257, 193
+    psi = wl.random_interior(wl.random_ring(m, n, 5), 6, 1.0)
+    field = b.to_field(psi)
+    bytes_ = field.stride(0) * n * 8
+    outs = []
+    for graphs, budget in ((True, 0), (False, 0), (True, bytes_ + (2 << 20)), (True, (2 << 20))):
+        if method == "jacobi" and budget == (2 << 20) and bytes_ > budget:
+            continue
+        lap = b.Laplace(hbm_budget=budget)
+        lap.set_graphs(graphs)
+        outs.append(run(b, lap, psi, method, w, order, 1.0, 7, 30, norm))
+        lap.close()
+    lap = b.Laplace()
+    want, r = run(b, lap, psi, method, w, order, 1.0, 1, 30, norm)
+    lap.close()
+    for got, q in outs:
+        assert np.array_equal(got, want)
+        assert (q["iters"], q["last_check"], q["r_final"]) == (r["iters"], r["last_check"], r["r_final"])
