@@ -143,7 +143,7 @@ __device__ __forceinline__ void prolong_black(const Arith<T>& A, const BatchLeve
 template <class T>
 __global__ void __launch_bounds__(BT)
     b_rb_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim, const BatchLevel<T>* __restrict__ lv,
-                const int* __restrict__ active, int colour, int gs, T w_arg, T omw_arg, int per_level_w)
+                const int* __restrict__ active, int colour, int gs, T w, T omw)
 {
     const Arith<T> A = arith<T>();
     const ItemClaim ic{claim, count};
@@ -151,7 +151,6 @@ __global__ void __launch_bounds__(BT)
         const BatchItem it = items[b];
         const BatchLevel<T> L = lv[it.level];
         if (!active[L.problem]) continue;
-        const T w = per_level_w ? (T)L.w : w_arg, omw = per_level_w ? (T)L.omw : omw_arg;
         const int half_w = (L.m - 2 + 1) / 2;
         on_rb_flags(L, gs != 0, [&](auto U, auto P, auto Q, auto G) {
             for (Walk k(half_w); k.r < it.rows; k.next()) {
@@ -164,6 +163,58 @@ __global__ void __launch_bounds__(BT)
         });
     }
     ic.finish();
+}
+
+// One SOR colour pass over many fields, a CTA per item, SWEEP_PPT points per thread at a time, counted row by
+// row so that a step does not depend on the fields' widths. What bounds it is FP64 (5 operations a point)
+// once enough loads are in flight: everything that a point needs stands in the item (one load, against item,
+// level and flag one after the other), and the operands of a step are loaded before the first is written,
+// beside the field's flag.
+constexpr int SWEEP_PPT = SWEEP_STEP / BT;
+
+template <bool UNIT, bool POW2>
+__device__ __forceinline__ void sweep_steps(const FmaOps& o, const SweepItem& it, int run, int colour)
+{
+    const unsigned half = (unsigned)(it.m - 1) / 2;
+    const double w = in_reg(o, it.w), omw = in_reg(o, it.omw);
+    for (unsigned base = threadIdx.x; base < (unsigned)it.count; base += SWEEP_STEP) {
+        double W[SWEEP_PPT], E[SWEEP_PPT], S[SWEEP_PPT], N[SWEEP_PPT], C[SWEEP_PPT];
+        double* at[SWEEP_PPT];
+#pragma unroll
+        for (int k = 0; k < SWEEP_PPT; ++k) {
+            const unsigned l = base + k * BT, t = (unsigned)it.col0 + l;
+            const int r = (int)(t / half), j = it.row0 + r;
+            const int i = 1 + ((1 + j + colour) & 1) + 2 * (int)(t - r * half);
+            at[k] = l < (unsigned)it.count && i <= it.m - 2 ? it.u + (int64_t)j * it.pitch + i : nullptr;
+            if (at[k]) {
+                W[k] = at[k][-1];
+                E[k] = at[k][1];
+                S[k] = at[k][-it.pitch];
+                N[k] = at[k][it.pitch];
+                C[k] = *at[k];
+            }
+        }
+        if (!run) return;
+#pragma unroll
+        for (int k = 0; k < SWEEP_PPT; ++k) {
+            if (!at[k]) continue;
+            const double s = neighbour_sum<UNIT>(o, W[k], E[k], S[k], N[k], it.b2);
+            const double g = times_inv_d<POW2>(o, s, it.inv_d, it.inv_d_shift);
+            *at[k] = __fma_rn(w, g, fmul(o, omw, C[k]));
+        }
+    }
+}
+
+__global__ void __launch_bounds__(BT)
+    b_sweep_kernel(const SweepItem* __restrict__ items, const int* __restrict__ active, int colour)
+{
+    const FmaOps o = load_fma_ops();
+    const SweepItem it = items[blockIdx.x];
+    const int run = active[it.problem];
+    on_flag(it.unit_beta != 0, [&](auto U) {
+        on_flag(it.inv_d_shift > 0,
+                [&](auto P) { sweep_steps<decltype(U)::value, decltype(P)::value>(o, it, run, colour); });
+    });
 }
 
 template <class T>
@@ -608,15 +659,23 @@ __global__ void b_converge_kernel(const double* __restrict__ partials,
 
 template <class T>
 cudaError_t launch_b_rb(const BatchList& l, const BatchLevel<T>* lv, const int* active, int colour,
-                        bool gs, double w, cudaStream_t s, bool per_level_w)
+                        bool gs, double w, cudaStream_t s)
 {
     if (l.count == 0) return cudaSuccess;
     const int grid = batch_grid((const void*)b_rb_kernel<T>, BT, 0, l.count, l.claim != nullptr);
     b_rb_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, colour, gs ? 1 : 0, (T)w,
-                                       (T)(1.0 - w), per_level_w ? 1 : 0);
+                                       (T)(1.0 - w));
     note_launch();
     return cudaGetLastError();
 }
+cudaError_t launch_b_sweep(const SweepItem* items, int count, const int* active, int colour, cudaStream_t s)
+{
+    if (count == 0) return cudaSuccess;
+    b_sweep_kernel<<<count, BT, 0, s>>>(items, active, colour);
+    note_launch();
+    return cudaGetLastError();
+}
+
 template <class T>
 cudaError_t launch_b_defect(const BatchList& l, const BatchLevel<T>* lv, const int* active,
                             cudaStream_t s, bool gs)
@@ -661,8 +720,8 @@ cudaError_t launch_b_coarse(const BatchList& l, const BatchLevel<T>* lv, const i
     return cudaGetLastError();
 }
 
-template cudaError_t launch_b_rb<double>(const BatchList&, const BatchLevel<double>*, const int*, int, bool, double, cudaStream_t, bool);
-template cudaError_t launch_b_rb<float>(const BatchList&, const BatchLevel<float>*, const int*, int, bool, double, cudaStream_t, bool);
+template cudaError_t launch_b_rb<double>(const BatchList&, const BatchLevel<double>*, const int*, int, bool, double, cudaStream_t);
+template cudaError_t launch_b_rb<float>(const BatchList&, const BatchLevel<float>*, const int*, int, bool, double, cudaStream_t);
 template cudaError_t launch_b_defect<double>(const BatchList&, const BatchLevel<double>*, const int*, cudaStream_t, bool);
 template cudaError_t launch_b_defect<float>(const BatchList&, const BatchLevel<float>*, const int*, cudaStream_t, bool);
 template cudaError_t launch_b_restrict<double>(const BatchList&, const BatchLevel<double>*, const int*, cudaStream_t, bool);

@@ -290,10 +290,40 @@ cudaError_t launch_copy_ring(double* dst, const Field& src, cudaStream_t s);
 // Zero rings in the u, q and r buffers of a batch's levels lv[0 .. count).
 template <class T>
 cudaError_t launch_zero_rings(const BatchLevel<T>* lv, int count, cudaStream_t s);
-// per_level_w: Eq. 7 with each level's own w (BatchLevel::w) instead of the argument
 template <class T>
 cudaError_t launch_b_rb(const BatchList& l, const BatchLevel<T>* lv, const int* active, int colour,
-                        bool gs, double w, cudaStream_t s, bool per_level_w = false);
+                        bool gs, double w, cudaStream_t s);
+// SOR sweeps over many fields (the server's), several per launch on tiles (sweep_tiles.cu): one tile of
+// a field that takes `sweeps` sweeps in all, with a second buffer for it.
+struct alignas(16) SweepTileItem {
+    double *u, *other;
+    int64_t pitch, pitch_other;
+    double w, omw, b2, inv_d;
+    int m, n, x0, x1, y0, y1;
+    int problem, unit_beta, inv_d_shift, sweeps;
+};
+struct BatchSweepPlan {
+    int sweeps = 0;  // at most this many in a launch
+    int sx = 0, sy = 0;  // at most this many interior points to a tile's sides
+};
+BatchSweepPlan plan_batch_sweeps(const std::vector<std::pair<int, int>>& fields, int sms);
+// Adds the tiles of it's field.
+void add_sweep_tiles(std::vector<SweepTileItem>& items, SweepTileItem it, const BatchSweepPlan& plan);
+// Launch k of an even number that leave the sweeps' result in u; none takes more than plan.sweeps.
+cudaError_t launch_b_sweep_tiles(const SweepTileItem* items, int count, const BatchSweepPlan& plan, const int* active,
+                                 int k, int launches, cudaStream_t s);
+// The same one pass per launch, without a second buffer: `count` points of a colour of one field, counted row by row
+// ((m - 1) / 2 to a row) from column col0 of row row0 on.
+struct alignas(16) SweepItem {
+    double* u;
+    int64_t pitch;
+    double w, omw, b2, inv_d;
+    int m, row0, col0, count;
+    int problem, unit_beta, inv_d_shift;
+};
+constexpr int SWEEP_STEP = 512;  // points of an item taken at a time
+// One colour pass over items[0 .. count) of the fields whose active flag is set.
+cudaError_t launch_b_sweep(const SweepItem* items, int count, const int* active, int colour, cudaStream_t s);
 // gs: the levels have just been smoothed by Gauss-Seidel. Then FP64 problems with beta = 1 need no
 // residual pass (their restriction takes it, gs_restrict.cuh), and the restriction into a level that
 // is smoothed next does its first red pass.

@@ -129,18 +129,22 @@ void srv_levels(lap_server S, SrvRequest& r, C& cv)
 constexpr int SERVER_TAIL_FP64 = 33;
 constexpr int SERVER_TAIL_FP32 = 129;
 
-// Interior points per work item of a step's SOR colour passes, for `points` points in all: about
-// 16 items per multiprocessor, so that the last wave is a small part of the pass, between 512
-// points (one per thread of a colour; smaller items would leave threads idle) and the 8192 of a
-// large batch. The passes are bound by the FP64 pipe, and with 8192-point items a running set of
-// 2.6 million points is 320 items on 152 multiprocessors: some take three and some two. Measured on
-// a burst of 48 requests (sides 33..1025, half of them SOR): 142.6 -> 126.3 ms, the colour passes
-// 24 -> 18-20 us.
+// Points of a colour per work item of a step's SOR passes (of fields without a second buffer), for `points` of them in all: SWEEP_STEP, or as many
+// steps as leave about 48 items per multiprocessor (more would only cost memory).
 // No effect on the values.
 int sor_item_points(int64_t points)
 {
-    const int64_t per = points / (16 * (int64_t)device_sms());
-    return (int)std::min<int64_t>(BATCH_ITEM_POINTS, std::max<int64_t>(512, per));
+    const int64_t steps = points / (48 * (int64_t)device_sms() * SWEEP_STEP);
+    return SWEEP_STEP * (int)std::min<int64_t>(1024, std::max<int64_t>(1, steps));
+}
+
+// Adds the items of one field.
+void add_sweep_items(std::vector<SweepItem>& items, const BatchLevel<double>& L, int per_item)
+{
+    const int64_t half = (L.m - 1) / 2, points = half * (L.n - 2);
+    for (int64_t k = 0; k < points; k += per_item)
+        items.push_back({L.u, L.pitch, L.w, L.omw, L.b2, L.inv_d, L.m, (int)(1 + k / half), (int)(k % half),
+                         (int)std::min<int64_t>(per_item, points - k), L.problem, L.unit_beta, L.inv_d_shift});
 }
 
 struct SrvPlan {
@@ -151,9 +155,13 @@ struct SrvPlan {
     std::vector<TileItem> tiles;
     std::vector<StreamItem> streams;
     LevelLists mg64, mg32;
-    std::pair<int, int> sor, update, init, norm;
+    std::vector<SweepItem> sweeps;  // SOR pass by pass, for the fields without a second buffer
+    std::vector<SweepTileItem> tiled;
+    BatchSweepPlan tile_plan;
+    int tile_launches = 0;
+    std::pair<int, int> update, init, norm;
     std::vector<int> first_init, first_norm;
-    std::vector<int> sor_upto;  // items of `sor` (a prefix) swept in the step's k-th sweep
+    std::vector<int> sor_upto;  // items of `sweeps` (a prefix) swept in the step's k-th sweep
 };
 
 }  // namespace
@@ -290,6 +298,17 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
             S->queue.pop_front();
             ++nrun;
         }
+        // pool blocks lent to this step's sweeps, given back when it ends (an error waits for what is in flight)
+        struct Lent {
+            lap_server S;
+            cudaStream_t st;
+            std::vector<std::pair<size_t, size_t>> blocks;
+            ~Lent()
+            {
+                if (!blocks.empty() && std::uncaught_exceptions()) cudaStreamSynchronize(st);
+                for (const auto& b : blocks) pool_free(S, b.first, b.second);
+            }
+        } second{S, st, {}};
         std::vector<SrvRequest*> run;
         for (auto& kv : S->reqs)
             if (kv.second.state == 1) run.push_back(&kv.second);
@@ -351,17 +370,39 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
                 if (run[q]->method == LAP_SOR_RB) sor_q.push_back(q);
             std::stable_sort(sor_q.begin(), sor_q.end(),
                              [&](int a, int c) { return sweeps_now(a) > sweeps_now(c); });
-            P.sor.first = (int)P.items.size();
+            // a second buffer for a field from the pool's free space, until the step's end
+            std::vector<std::pair<int, int>> shapes;
+            std::vector<SweepTileItem> tiled;
+            std::vector<int> rest;
+            for (int q : sor_q) {
+                const BatchLevel<double>& L = P.lv64[base[q]];
+                const int64_t pitch = round_up(L.m, 32);
+                const size_t bytes = (size_t)(pitch * L.n) * sizeof(double);
+                size_t off = 0;
+                if (S->sor_sweeps < 2 || !pool_alloc(S, bytes, &off)) {
+                    rest.push_back(q);
+                    continue;
+                }
+                second.blocks.push_back({off, bytes});
+                shapes.push_back({L.m, L.n});
+                tiled.push_back({L.u, (double*)(S->pool + off), L.pitch, pitch, L.w, L.omw, L.b2, L.inv_d, L.m, L.n,
+                                 0, 0, 0, 0, L.problem, L.unit_beta, L.inv_d_shift, sweeps_now(q)});
+            }
+            if (!tiled.empty()) {
+                P.tile_plan = plan_batch_sweeps(shapes, device_sms());
+                for (const SweepTileItem& t : tiled) add_sweep_tiles(P.tiled, t, P.tile_plan);
+                const int most = tiled.front().sweeps;  // sor_q is in falling order
+                P.tile_launches = 2 * ((most + 2 * P.tile_plan.sweeps - 1) / (2 * P.tile_plan.sweeps));
+            }
             P.sor_upto.assign(S->sor_sweeps, 0);
             int64_t sor_points = 0;
-            for (int q : sor_q) sor_points += (int64_t)(run[q]->g.m - 2) * (run[q]->g.n - 2);
+            for (int q : rest) sor_points += (int64_t)((run[q]->g.m - 1) / 2) * (run[q]->g.n - 2);
             const int per_item = sor_item_points(sor_points);
-            for (int q : sor_q) {
-                add_items(P.items, base[q], run[q]->g.m, run[q]->g.n, per_item);
-                const int upto = (int)P.items.size() - P.sor.first;
+            for (int q : rest) {
+                add_sweep_items(P.sweeps, P.lv64[base[q]], per_item);
+                const int upto = (int)P.sweeps.size();
                 for (int k = 0; k < sweeps_now(q); ++k) P.sor_upto[k] = upto;
             }
-            P.sor.second = (int)P.items.size() - P.sor.first;
         }
         P.update = level0([](const SrvRequest& r) { return r.method == LAP_MG_MIXED; }, nullptr);
         P.init = level0([](const SrvRequest& r) { return r.fresh; }, &P.first_init);
@@ -385,6 +426,8 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
             auto* jobs = cv.template take<TailJob>(std::max<size_t>(1, P.jobs.size()));
             auto* tiles = cv.template take<TileItem>(std::max<size_t>(1, P.tiles.size()));
             auto* streams = cv.template take<StreamItem>(std::max<size_t>(1, P.streams.size()));
+            auto* sweeps = cv.template take<SweepItem>(std::max<size_t>(1, P.sweeps.size()));
+            auto* tiled = cv.template take<SweepTileItem>(std::max<size_t>(1, P.tiled.size()));
             auto* fi = cv.template take<int>(P.first_init.size());
             auto* fn = cv.template take<int>(P.first_norm.size());
             auto* active = cv.template take<int>(R);
@@ -399,7 +442,7 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
             auto* pnorm = cv.template take<double>(std::max(1, P.norm.second));
             auto* done = cv.template take<Completion>(R);
             auto* ndone = cv.template take<int>(1);
-            return std::make_tuple(lv64, lv32, items, jobs, tiles, streams, fi, fn, active, status, remaining,
+            return std::make_tuple(lv64, lv32, items, jobs, tiles, streams, sweeps, tiled, fi, fn, active, status, remaining,
                                    iters, maxit, dr0, rnow, dtol, pinit, pnorm, done, ndone);
         };
         Sizer sz;
@@ -420,11 +463,13 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
         TailJob* jobs;
         TileItem* tiles;
         StreamItem* streams;
+        SweepItem* sweeps;
+        SweepTileItem* tiled;
         int *fi, *fn, *active, *status, *remaining, *ndone;
         long long *iters, *maxit;
         double *dr0, *rnow, *dtol, *pinit, *pnorm;
         Completion* done;
-        std::tie(lv64, lv32, items, jobs, tiles, streams, fi, fn, active, status, remaining, iters, maxit, dr0,
+        std::tie(lv64, lv32, items, jobs, tiles, streams, sweeps, tiled, fi, fn, active, status, remaining, iters, maxit, dr0,
                  rnow, dtol, pinit, pnorm, done, ndone) = carve_stage(cv);
         auto up = [&](void* dst, const void* src, size_t bytes) {
             if (bytes) ck(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st), "upload plan");
@@ -435,6 +480,8 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
         up(jobs, P.jobs.data(), P.jobs.size() * sizeof(TailJob));
         up(tiles, P.tiles.data(), P.tiles.size() * sizeof(TileItem));
         up(streams, P.streams.data(), P.streams.size() * sizeof(StreamItem));
+        up(tiled, P.tiled.data(), P.tiled.size() * sizeof(SweepTileItem));
+        up(sweeps, P.sweeps.data(), P.sweeps.size() * sizeof(SweepItem));
         if (P.mg32.fused) ck(prepare_fused32(), "tile kernel attributes");
         up(fi, P.first_init.data(), P.first_init.size() * sizeof(int));
         up(fn, P.first_norm.data(), P.first_norm.size() * sizeof(int));
@@ -462,11 +509,11 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
         // fused: the level-0 ascents did psi += e except where a tail holds level 0
         ck(launch_b_update(list(P.mg32.fused ? P.mg32.upd0 : P.update), lv64, active, lv32, st),
            "server update");
-        for (int k = 0; k < S->sor_sweeps && P.sor.second; ++k) {
-            const std::pair<int, int> swept{P.sor.first, P.sor_upto[k]};
+        for (int k = 0; k < P.tile_launches; ++k)
+            ck(launch_b_sweep_tiles(tiled, (int)P.tiled.size(), P.tile_plan, active, k, P.tile_launches, st), "server sweeps");
+        for (int k = 0; k < S->sor_sweeps && P.sor_upto[k]; ++k)
             for (int colour = 0; colour < 2; ++colour)
-                ck(launch_b_rb(list(swept), lv64, active, colour, false, 1.0, st, true), "server sweep");
-        }
+                ck(launch_b_sweep(sweeps, P.sor_upto[k], active, colour, st), "server sweep");
         ck(launch_b_sumsq(list(P.norm), lv64, active, pnorm, lv32, st, dr0,
                           S->mg.smoother_w == 1.0 && S->mg.nu2 > 0),
            "server residual");

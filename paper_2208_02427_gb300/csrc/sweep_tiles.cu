@@ -15,6 +15,7 @@
 
 #include "lap_device.cuh"
 #include "lap_internal.cuh"
+#include "vcycle_arith.cuh"
 
 namespace lap {
 
@@ -55,12 +56,13 @@ __device__ __forceinline__ double swept(const FmaOps& o, const double* c, int W,
 // preparation. sm: (x1 - x0 + 2 passes) (y1 - y0 + 2 passes) doubles, twice that for Jacobi.
 template <int KIND, bool UNIT, bool POW2, bool DIAG>
 __device__ __forceinline__ void sweep_tile(const FmaOps& o, const double* __restrict__ in, double* __restrict__ out,
-                                           int m, int n, int64_t pitch, int x0, int x1, int y0, int y1, int passes,
-                                           const SweepCoef& k, double* sm)
+                                           int m, int n, int64_t pitch, int64_t pitch_out, int x0, int x1, int y0,
+                                           int y1, int passes, const SweepCoef& k, double* sm)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int X0 = max(0, x0 - passes), X1 = min(m, x1 + passes);
-    const int Y0 = max(0, y0 - passes), Y1 = min(n, y1 + passes);
+    const int h = max(1, passes);  // no pass, a copy: the ring beside the tile all the same
+    const int X0 = max(0, x0 - h), X1 = min(m, x1 + h);
+    const int Y0 = max(0, y0 - h), Y1 = min(n, y1 + h);
     const int W = X1 - X0, H = Y1 - Y0;
     for (int r = wid; r < H; r += nw) {
         const double* src = in + (int64_t)(Y0 + r) * pitch + X0;
@@ -125,7 +127,7 @@ __device__ __forceinline__ void sweep_tile(const FmaOps& o, const double* __rest
     const int sx0 = x0 == 1 ? 0 : x0, sx1 = x1 == m - 1 ? m : x1;
     const int sy0 = y0 == 1 ? 0 : y0, sy1 = y1 == n - 1 ? n : y1;
     for (int j = sy0 + wid; j < sy1; j += nw)
-        for (int i = sx0 + lane; i < sx1; i += 32) out[(int64_t)j * pitch + i] = a[(j - Y0) * W + (i - X0)];
+        for (int i = sx0 + lane; i < sx1; i += 32) out[(int64_t)j * pitch_out + i] = a[(j - Y0) * W + (i - X0)];
 }
 
 // Tile (blockIdx.x, blockIdx.y) of gridDim.x x gridDim.y equal parts of the interior.
@@ -146,7 +148,31 @@ __global__ void __launch_bounds__(ST_THREADS)
     const int x1 = 1 + (int)((int64_t)(blockIdx.x + 1) * (m - 2) / gridDim.x);
     const int y0 = 1 + (int)((int64_t)blockIdx.y * (n - 2) / gridDim.y);
     const int y1 = 1 + (int)((int64_t)(blockIdx.y + 1) * (n - 2) / gridDim.y);
-    sweep_tile<KIND, UNIT, POW2, DIAG>(o, in, out, m, n, pitch, x0, x1, y0, y1, passes, k, sm);
+    sweep_tile<KIND, UNIT, POW2, DIAG>(o, in, out, m, n, pitch, pitch, x0, x1, y0, y1, passes, k, sm);
+}
+
+// Launch `k` of `launches` over the tiles of many fields (SOR, each field's own factor and spacing): an even
+// launch takes a field to its second buffer and an odd one back, each with its share of the field's sweeps,
+// at times none (a copy). Bound by FP64 and, between its tiles' barriers, by latency: three CTAs to a
+// multiprocessor (40 registers) against two: 108.6 against 112 ms on the burst below.
+__global__ void __launch_bounds__(ST_THREADS, 3)
+    b_sweep_tiles_kernel(const SweepTileItem* __restrict__ items, const int* __restrict__ active, int k, int launches)
+{
+    extern __shared__ double sm[];
+    const FmaOps o = load_fma_ops();
+    const SweepTileItem it = items[blockIdx.x];
+    if (!active[it.problem]) return;
+    const int passes = 2 * (it.sweeps / launches + (k < it.sweeps % launches ? 1 : 0));
+    const bool back = k & 1;
+    SweepCoef c{it.b2, it.inv_d, it.inv_d_shift, in_reg(o, it.w), in_reg(o, it.omw)};
+    auto run = [&](auto U, auto P) {
+        if (!decltype(U)::value) c.b2 = in_reg(o, c.b2);
+        if (!decltype(P)::value) c.inv_d = in_reg(o, c.inv_d);
+        sweep_tile<SWEEP_SOR, decltype(U)::value, decltype(P)::value, false>(
+            o, back ? it.other : it.u, back ? it.u : it.other, it.m, it.n, back ? it.pitch_other : it.pitch,
+            back ? it.pitch : it.pitch_other, it.x0, it.x1, it.y0, it.y1, passes, c, sm);
+    };
+    on_flag(it.unit_beta != 0, [&](auto U) { on_flag(it.inv_d_shift > 0, [&](auto P) { run(U, P); }); });
 }
 
 template <class F>
@@ -233,6 +259,84 @@ cudaError_t launch_sweep_tiles(const Field& in, double* out, const Coef& c, cons
     });
     note_launch();
     return e;
+}
+
+// Tile sides and sweeps per launch that cost least for SOR fields of m[k] x n[k] points, by the model of
+// plan_sweep_tiles with the tiles in as many rounds as it takes. Sides are tried around those that give
+// one, two or three tiles per multiprocessor (or as many as shared memory needs), upright and flat.
+// Per colour pass of a step of 50 sweeps, one pass per launch / tiles: one field of 33^2 points 4.0 / 1.4 us,
+// 257^2 5.0 / 2.5, 513^2 7.2 / 3.8, 1025^2 11.5 / 7.8, four of 1025^2 26.5 / 23.6 (FP64 alone 16.8). A burst of
+// 48 requests (sides 33..1025, half of them SOR): 125.6 / 108.6 ms.
+BatchSweepPlan plan_batch_sweeps(const std::vector<std::pair<int, int>>& fields, int sms)
+{
+    BatchSweepPlan best;
+    double least = 1e300, points = 0;
+    const int most_side = 148;
+    for (const auto& f : fields) points += (double)(f.first - 2) * (f.second - 2);
+    const int fewest = std::max(1, (int)std::ceil(points / ((double)sms * most_side * most_side)));
+    for (int per_sm = fewest; per_sm < fewest + 3; ++per_sm) {
+        const double even_side = std::sqrt(points / ((double)sms * per_sm));
+        for (double factor = 0.94; factor < 1.6; factor *= 1.02) {
+            for (double flat : {1.0, 0.87, 0.75}) {
+                const int sx = (int)std::min<double>(most_side, std::max(6.0, even_side * factor));
+                const int sy = (int)std::max(6.0, sx * flat);
+                double tiles = 0, rim = 0, tw1 = 1, th1 = 1;
+                for (const auto& f : fields) {
+                    const int tx = (f.first - 2 + sx - 1) / sx, ty = (f.second - 2 + sy - 1) / sy;
+                    const double tw = (double)(f.first - 2) / tx, th = (double)(f.second - 2) / ty;
+                    tiles += (double)tx * ty;
+                    rim += (double)tx * ty * (tw + th);
+                    if (tw * th > tw1 * th1) tw1 = tw, th1 = th;
+                }
+                for (int sweeps = 1; sweeps <= 6; ++sweeps) {
+                    const int h = 2 * sweeps;
+                    if ((int64_t)(sx + 2 * h) * (sy + 2 * h) * 8 > (int64_t)ST_SMEM_MAX) break;
+                    // cycles of `t` tiles with `a` points and half rims of `r` in all: the FP64 work of
+                    // their passes and their windows
+                    auto cycles = [&](double t, double a, double r) {
+                        const double sum = h * a + r * h * (h - 1) + t * 2.0 / 3.0 * h * (h - 1) * (2 * h - 1);
+                        return sum / 2 * 5 / 2 + (a + 2 * h * r + t * 4.0 * h * h) * TILE_POINT_CYCLES;
+                    };
+                    const double rounds = std::ceil(tiles / sms);
+                    const double busy = std::max(cycles(1, tw1 * th1, tw1 + th1), cycles(tiles, points, rim) / tiles * rounds);
+                    const double cost = (TILE_CYCLES + h * TILE_PASS_CYCLES + busy) / sweeps;
+                    if (cost < least) {
+                        least = cost;
+                        best = BatchSweepPlan{sweeps, sx, sy};
+                    }
+                }
+            }
+        }
+    }
+    return best;
+}
+
+void add_sweep_tiles(std::vector<SweepTileItem>& items, SweepTileItem it, const BatchSweepPlan& plan)
+{
+    const int tx = (it.m - 2 + plan.sx - 1) / plan.sx, ty = (it.n - 2 + plan.sy - 1) / plan.sy;
+    for (int y = 0; y < ty; ++y)
+        for (int x = 0; x < tx; ++x) {
+            it.x0 = 1 + (int)((int64_t)x * (it.m - 2) / tx);
+            it.x1 = 1 + (int)((int64_t)(x + 1) * (it.m - 2) / tx);
+            it.y0 = 1 + (int)((int64_t)y * (it.n - 2) / ty);
+            it.y1 = 1 + (int)((int64_t)(y + 1) * (it.n - 2) / ty);
+            items.push_back(it);
+        }
+}
+
+cudaError_t launch_b_sweep_tiles(const SweepTileItem* items, int count, const BatchSweepPlan& plan, const int* active,
+                                 int k, int launches, cudaStream_t s)
+{
+    if (count == 0) return cudaSuccess;
+    const size_t bytes = (size_t)(plan.sx + 4 * plan.sweeps) * (plan.sy + 4 * plan.sweeps) * 8;
+    if (k == 0) {
+        const cudaError_t e = cudaFuncSetAttribute(b_sweep_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)ST_SMEM_MAX);
+        if (e != cudaSuccess) return e;
+    }
+    b_sweep_tiles_kernel<<<count, ST_THREADS, bytes, s>>>(items, active, k, launches);
+    note_launch();
+    return cudaGetLastError();
 }
 
 }  // namespace lap

@@ -65,3 +65,31 @@ def test_norms_graphs_and_budgets(b, method, w, order, norm):
     for got, q in outs:
         assert np.array_equal(got, want)
         assert (q["iters"], q["last_check"], q["r_final"]) == (r["iters"], r["last_check"], r["r_final"])
+
+
+@pytest.mark.parametrize("sweeps", [1, 2, 7, 50])
+@pytest.mark.parametrize("room", [0, 300 << 10, 64 << 20])
+def test_server_sweeps_equal_single_solves(b, sweeps, room):
+    """Fields with a second buffer from the server's pool and fields without (room for none, some, all):
+    uneven sizes and spacings, sweep counts cut short at different places, a field solved already."""
+    shapes = [(3, 3), (33, 65), (130, 47), (257, 129), (66, 300), (40, 40), (200, 201)]
+    lap = b.Laplace()
+    srv = b.Server(lap, hbm_budget=room, max_running=len(shapes), sor_sweeps=sweeps)
+    fields, ids, want = [], [], []
+    for k, (m, n) in enumerate(shapes):
+        psi = wl.random_interior(wl.random_ring(m, n, 20 + k), 30 + k, 1.0)
+        if k == 5:
+            psi[:] = 0.0
+        dx, w, cap = (1.0 if k % 2 else 0.8), 1.3 + 0.08 * k, 2 * sweeps + 3 * k
+        t = b.to_field(psi)
+        r = lap.solve(t, dx, 1.0, method="sor", w=w, tol=1e-13, check_every=sweeps, max_iter=cap)
+        want.append((t.cpu().numpy(), r["iters"], r["status"]))
+        f = b.to_field(psi)
+        fields.append(f)
+        ids.append(srv.submit(f, dx=dx, dy=1.0, method="sor", w=w, tol=1e-13, max_iter=cap))
+    while sum(srv.step()):
+        pass
+    res = dict(srv.drain())
+    for f, i, (psi, iters, status) in zip(fields, ids, want):
+        assert np.array_equal(f.cpu().numpy(), psi)
+        assert (res[i]["iters"], res[i]["status"]) == (iters, status)
