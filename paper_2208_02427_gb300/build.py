@@ -23,7 +23,7 @@ SOURCES = ["lap_api.cu", "lap_batched.cu", "lap_server.cu", "point_kernels.cu", 
            "loop_kernels.cu", "small_kernels.cu",
            "stream32_kernels.cu", "tail_kernels.cu", "sweep_tiles.cu"]
 HEADERS = ["lap_internal.cuh", "lap_device.cuh", "lap_host.cuh", "vcycle_arith.cuh",
-           "norm_end.cuh", "gs_restrict.cuh"]
+           "norm_end.cuh", "gs_restrict.cuh", "residual32.cuh"]
 
 
 def nvcc() -> str:

@@ -15,6 +15,7 @@
 #include "gs_restrict.cuh"
 #include "lap_device.cuh"
 #include "lap_internal.cuh"
+#include "residual32.cuh"
 #include "vcycle_arith.cuh"
 
 namespace lap {
@@ -525,33 +526,22 @@ __device__ __forceinline__ void sumsq_block(const BatchItem* __restrict__ items,
                                             const BatchLevel<double>* __restrict__ lv,
                                             const int* __restrict__ active, double* __restrict__ partials,
                                             const BatchLevel<float>* __restrict__ lv32,
-                                            const double* __restrict__ r0, bool gs)
+                                            int skip32, bool gs)
 {
     const BatchItem it = items[ib];
     const BatchLevel<double> L = lv[it.level];
     if (!active[L.problem]) return;
-    // problems solved by the FP32 inner cycle have an FP32 level 0
+    // problems solved by the FP32 inner cycle have an FP32 level 0; after their cycles
+    // b_residual32_kernel takes them
     const bool mixed = lv32 && lv32[it.level].q;
-    float sc = 0.0f;
-    if (mixed && r0) {
-        const double z = r0[L.problem];
-        if (z > 0.0 && isfinite(z)) {
-            const int e = ilogb(z);
-            if (e >= -100 && e <= 100) sc = ldexpf(1.0f, -e);
-        }
-    }
+    if (mixed && skip32) return;
     double acc = 0.0;
-    // the FP32 or the FP64 sum of squares, chosen per block (as a per-point choice the
-    // compiler would issue the FP64 fma for every point)
     // an FP64 multigrid problem with more than one level has a residual scratch
     if (gs && !mixed && L.r && L.unit_beta) acc = gs_sumsq_item(it, L);
     else on_flag(L.unit_beta != 0, [&](auto U) {
-        if (!mixed)
-            acc = sumsq_item<false, decltype(U)::value, false>(it, L, lv32, 0.0f);
-        else
-            on_flag(sc > 0.0f, [&](auto SC) {
-                acc = sumsq_item<true, decltype(U)::value, decltype(SC)::value>(it, L, lv32, sc);
-            });
+        on_flag(mixed, [&](auto M) {
+            acc = sumsq_item<decltype(M)::value, decltype(U)::value, false>(it, L, lv32, 0.0f);
+        });
     });
     __shared__ double red[BT / 32];  // a persistent CTA's next claim waits for the reads below
     acc = warp_sum(acc);
@@ -560,9 +550,79 @@ __device__ __forceinline__ void sumsq_block(const BatchItem* __restrict__ items,
     if (threadIdx.x < 32) {
         double v = threadIdx.x < BT / 32 ? red[threadIdx.x] : 0.0;
         v = warp_sum(v);
-        if (threadIdx.x == 0)
-            partials[ib] = sc > 0.0f ? v / ((double)sc * (double)sc) : v;  // exact
+        if (threadIdx.x == 0) partials[ib] = v;
     }
+}
+
+// The mixed problems' residuals after a cycle, and their sums of squares by item: with beta = 1 on the
+// integer pipe (residual32.cuh; the items' rows are whole runs), else as sumsq_item, the squares in FP32
+// scaled by a power of two near 1 / r0 where that is in range (chosen per block: as a per-point choice the
+// compiler would issue the FP64 fma for every point). clear_e: the FP32 corrections start from zero.
+template <bool SCALED>
+static __device__ __noinline__ double sumsq_item_rare(const BatchItem& it, const BatchLevel<double>& L,
+                                                      const BatchLevel<float>* __restrict__ lv32, float sc)
+{
+    double acc = 0.0;
+    on_flag(L.unit_beta != 0, [&](auto U) { acc = sumsq_item<true, decltype(U)::value, SCALED>(it, L, lv32, sc); });
+    return acc;
+}
+
+__device__ __forceinline__ void residual32_block(const BatchItem* __restrict__ items, int ib,
+                                                 const BatchLevel<double>* __restrict__ lv,
+                                                 const int* __restrict__ active, double* __restrict__ partials,
+                                                 const BatchLevel<float>* __restrict__ lv32,
+                                                 const double* __restrict__ r0, int clear_e)
+{
+    const BatchItem it = items[ib];
+    const BatchLevel<double> L = lv[it.level];
+    const BatchLevel<float> E = lv32[it.level];
+    if (!active[L.problem] || !E.q) return;
+    float sc = 0.0f;
+    const double z = r0[L.problem];
+    if (z > 0.0 && isfinite(z)) {
+        const int e = ilogb(z);
+        if (e >= -100 && e <= 100) sc = ldexpf(1.0f, -e);
+    }
+    double acc = 0.0;
+    if (sc > 0.0f && L.unit_beta) {
+        const bool vec = (L.pitch & 1) == 0 && ((uintptr_t)L.u & 15) == 0;
+        const ResidualRuns R{L.u, L.pitch, E.q, clear_e ? E.u : nullptr, E.pitch, L.m, L.n, vec};
+        const int strips = run_strips(L.m), b0 = (it.row0 - 1) / RUN_ROWS;
+        const int runs = strips * ((it.rows + RUN_ROWS - 1) / RUN_ROWS);
+        float acc32 = 0.0f;
+        for (int k = threadIdx.x >> 5; k < runs; k += BT / 32) {
+            const int b = k / strips;
+            acc32 = residual_run(R, k - b * strips, b0 + b, sc, acc32);
+        }
+        acc = (double)acc32;
+    } else {
+        acc = sc > 0.0f ? sumsq_item_rare<true>(it, L, lv32, sc) : sumsq_item_rare<false>(it, L, lv32, 0.0f);
+    }
+    __shared__ double red[BT / 32];  // a persistent CTA's next claim waits for the reads below
+    acc = warp_sum(acc);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const double v = warp_sum(threadIdx.x < BT / 32 ? red[threadIdx.x] : 0.0);
+        if (threadIdx.x == 0) partials[ib] = sc > 0.0f ? v / ((double)sc * (double)sc) : v;  // exact
+    }
+}
+
+template <bool CLAIM>
+__global__ void __launch_bounds__(BT, 3)
+    b_residual32_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim,
+                        const BatchLevel<double>* __restrict__ lv, const int* __restrict__ active,
+                        double* __restrict__ partials, const BatchLevel<float>* __restrict__ lv32,
+                        const double* __restrict__ r0, int clear_e)
+{
+    if (!CLAIM) {
+        residual32_block(items, blockIdx.x, lv, active, partials, lv32, r0, clear_e);
+        return;
+    }
+    const ItemClaim ic{claim, count};
+    for (int b = ic.take(-1); b < count; b = ic.take(b))
+        residual32_block(items, b, lv, active, partials, lv32, r0, clear_e);
+    ic.finish();
 }
 
 // CLAIM: a persistent launch (compiled apart: the one-item form keeps its registers free of
@@ -572,15 +632,15 @@ __global__ void __launch_bounds__(BT, 5)
     b_sumsq_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim,
                    const BatchLevel<double>* __restrict__ lv, const int* __restrict__ active,
                    double* __restrict__ partials, const BatchLevel<float>* __restrict__ lv32,
-                   const double* __restrict__ r0, int gs)
+                   int skip32, int gs)
 {
     if (!CLAIM) {
-        sumsq_block(items, blockIdx.x, lv, active, partials, lv32, r0, gs != 0);
+        sumsq_block(items, blockIdx.x, lv, active, partials, lv32, skip32, gs != 0);
         return;
     }
     const ItemClaim ic{claim, count};
     for (int b = ic.take(-1); b < count; b = ic.take(b))
-        sumsq_block(items, b, lv, active, partials, lv32, r0, gs != 0);
+        sumsq_block(items, b, lv, active, partials, lv32, skip32, gs != 0);
     ic.finish();
 }
 
@@ -749,15 +809,30 @@ template cudaError_t launch_b_tail<float>(const TailJob*, int, const BatchLevel<
 
 cudaError_t launch_b_sumsq(const BatchList& l, const BatchLevel<double>* lv, const int* active,
                            double* partials, const BatchLevel<float>* lv32, cudaStream_t s,
-                           const double* r0, bool gs)
+                           bool skip32, bool gs)
 {
     if (l.count == 0) return cudaSuccess;
     if (l.claim) {
         const int grid = batch_grid((const void*)b_sumsq_kernel<true>, BT, 0, l.count, true);
-        b_sumsq_kernel<true><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, partials, lv32, r0, gs ? 1 : 0);
+        b_sumsq_kernel<true><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, partials, lv32, skip32 ? 1 : 0, gs ? 1 : 0);
     } else {
         b_sumsq_kernel<false><<<l.count, BT, 0, s>>>(l.items, l.count, nullptr, lv, active, partials, lv32,
-                                                     r0, gs ? 1 : 0);
+                                                     skip32 ? 1 : 0, gs ? 1 : 0);
+    }
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_b_residual32(const BatchList& l, const BatchLevel<double>* lv, const int* active,
+                                double* partials, const BatchLevel<float>* lv32, const double* r0, bool clear_e,
+                                cudaStream_t s)
+{
+    if (l.count == 0) return cudaSuccess;
+    if (l.claim) {
+        const int grid = batch_grid((const void*)b_residual32_kernel<true>, BT, 0, l.count, true);
+        b_residual32_kernel<true><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, partials, lv32, r0, clear_e ? 1 : 0);
+    } else {
+        b_residual32_kernel<false><<<l.count, BT, 0, s>>>(l.items, l.count, nullptr, lv, active, partials, lv32, r0, clear_e ? 1 : 0);
     }
     note_launch();
     return cudaGetLastError();

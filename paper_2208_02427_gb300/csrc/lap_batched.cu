@@ -5,9 +5,9 @@
 
 namespace lap {
 
-void add_items(std::vector<BatchItem>& items, int level_index, int m, int n, int points, bool red)
+void add_items(std::vector<BatchItem>& items, int level_index, int m, int n, int points, bool red, int unit)
 {
-    const int per = std::max(1, points / std::max(1, m - 2));
+    const int per = (int)round_up(std::max(1, points / std::max(1, m - 2)), unit);
     for (int r = 1; r <= n - 2; r += per) items.push_back(BatchItem{level_index, r, std::min(per, n - 1 - r), red ? 1 : 0});
 }
 
@@ -318,7 +318,7 @@ std::unique_ptr<BatchCache> build_plan(lap_handle h, int count, const lap_grid* 
     }
     for (int q = 0; q < count; ++q) {
         P.first_item.push_back((int)P.norm_items.size());
-        add_items(P.norm_items, P.base[q], grids[q].m, grids[q].n);
+        add_items(P.norm_items, P.base[q], grids[q].m, grids[q].n, BATCH_ITEM_POINTS, false, mixed ? RUN_ROWS : 1);
     }
     P.first_item.push_back((int)P.norm_items.size());
     auto carve_all = [&](auto& cv) {
@@ -488,10 +488,12 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
                     // fused: the level-0 ascents did psi += e except where a tail holds level 0
                     ck(launch_b_update(L.fused ? list(L.upd0) : norms, lv64, active, lv32, st),
                        "batched update");
-                    ck(launch_b_sumsq(norms, lv64, active, partials, lv32, st, r0), "batched residual");
+                    // fused level-0 descents start from zero and do not read e
+                    ck(launch_b_residual32(norms, lv64, active, partials, lv32, r0, !L.fused || L.upd0.second > 0, st),
+                       "batched residual");
                 } else {
                     enqueue_vcycle(list, L, lv64, active, K.jobs, *p, p->smoother_w, st);
-                    ck(launch_b_sumsq(norms, lv64, active, partials, nullptr, st, nullptr,
+                    ck(launch_b_sumsq(norms, lv64, active, partials, nullptr, st, false,
                                       p->smoother_w == 1.0 && p->nu2 > 0),
                        "batched residual");
                 }

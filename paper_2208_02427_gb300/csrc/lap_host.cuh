@@ -190,7 +190,7 @@ int mg_level_count(int m, int n, int coarsest_min, int max_levels);
 // points, the mixed solver 74 / 71 / 69 / 68 ms; 8192 for both.
 constexpr int BATCH_ITEM_POINTS = 8192;
 void add_items(std::vector<BatchItem>& items, int level_index, int m, int n,
-               int points = BATCH_ITEM_POINTS, bool red = false);
+               int points = BATCH_ITEM_POINTS, bool red = false, int unit = 1);
 
 // Per-level work lists of one V-cycle over a set of problems: [first, count) into the items
 // (fine, all, coarse) or into the tail jobs (tail).

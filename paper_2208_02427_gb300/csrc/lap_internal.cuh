@@ -366,13 +366,19 @@ cudaError_t launch_smem_tail(const TailJob* jobs, int count, const BatchLevel<T>
                              int nu2, bool gs, double w, const SmemTail& plan, cudaStream_t s,
                              bool per_level_w = false, unsigned* claim = nullptr);
 // per-item FP64 sum of squares of the residual; with lv32 also r32 := residual, e32 := 0;
-// with r0 (per problem) the mixed problems sum their squares in FP32 after an exact
-// power-of-two scaling from r0 (the partials are stored descaled)
+// skip32: the mixed problems are left to launch_b_residual32
 // gs: FP64 multigrid problems come from Gauss-Seidel smoothing (with beta = 1 only their red points
 // are summed, see launch_gs_norm)
 cudaError_t launch_b_sumsq(const BatchList& l, const BatchLevel<double>* lv, const int* active,
                            double* partials, const BatchLevel<float>* lv32, cudaStream_t s,
-                           const double* r0 = nullptr, bool gs = false);
+                           bool skip32 = false, bool gs = false);
+// The mixed problems of the list after a cycle: r32 := residual, with clear_e e32 := 0, per-item sums of
+// squares (taken in FP32 after an exact power-of-two scaling from r0 where that is in range; stored
+// descaled). The items' rows are whole runs (RUN_ROWS).
+constexpr int RUN_ROWS = 8;
+cudaError_t launch_b_residual32(const BatchList& l, const BatchLevel<double>* lv, const int* active,
+                                double* partials, const BatchLevel<float>* lv32, const double* r0, bool clear_e,
+                                cudaStream_t s);
 cudaError_t launch_b_update(const BatchList& l, const BatchLevel<double>* lv, const int* active,
                             const BatchLevel<float>* lv32, cudaStream_t s);
 // A problem that left the batch in a convergence test: its index, lap_status, cycles run and

@@ -352,7 +352,8 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
             const int i0 = (int)P.items.size();
             for (int q = 0; q < R; ++q) {
                 if (first) first->push_back((int)P.items.size() - i0);
-                if (pred(*run[q])) add_items(P.items, base[q], run[q]->g.m, run[q]->g.n);
+                if (pred(*run[q]))
+                    add_items(P.items, base[q], run[q]->g.m, run[q]->g.n, BATCH_ITEM_POINTS, false, RUN_ROWS);
             }
             if (first) first->push_back((int)P.items.size() - i0);
             return std::make_pair(i0, (int)P.items.size() - i0);
@@ -514,9 +515,14 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
         for (int k = 0; k < S->sor_sweeps && P.sor_upto[k]; ++k)
             for (int colour = 0; colour < 2; ++colour)
                 ck(launch_b_sweep(sweeps, P.sor_upto[k], active, colour, st), "server sweep");
-        ck(launch_b_sumsq(list(P.norm), lv64, active, pnorm, lv32, st, dr0,
-                          S->mg.smoother_w == 1.0 && S->mg.nu2 > 0),
-           "server residual");
+        int mixed = 0;
+        for (const SrvRequest* r : run) mixed += r->method == LAP_MG_MIXED;
+        if (mixed)
+            ck(launch_b_residual32(list(P.norm), lv64, active, pnorm, lv32, dr0, !P.mg32.fused || P.mg32.upd0.second > 0, st),
+               "server residual");
+        if (mixed < R)
+            ck(launch_b_sumsq(list(P.norm), lv64, active, pnorm, lv32, st, true, S->mg.smoother_w == 1.0 && S->mg.nu2 > 0),
+               "server residual");
         ck(launch_b_converge(pnorm, fn, R, active, dr0, rnow, iters, status, remaining, 1, true, 0.0,
                              st, dtol, maxit, done, ndone), "server convergence");
         // ---- the step's completion list (written by the convergence tests), read once ----

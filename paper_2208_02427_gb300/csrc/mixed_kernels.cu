@@ -10,9 +10,12 @@
 //   3. psi += e in FP64.
 // FP32 runs 62x faster than FP64 on GB300, so the inner cycle is bound by memory, not
 // by arithmetic; the FP64 work per outer iteration is two passes over the fine grid.
+#include <algorithm>
+
 #include "lap_device.cuh"
 #include "lap_internal.cuh"
 #include "norm_end.cuh"
+#include "residual32.cuh"
 
 namespace lap {
 
@@ -184,6 +187,28 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
     norm_end(end, v, partials, red);
 }
 
+// The same with beta = 1 and a norm scale, on the integer pipe (residual32.cuh), a warp per run.
+constexpr int RUN_BLOCKS_PER_SM = 3;  // 80 registers; with two blocks of 102, 194 us at 8193^2 against 178
+__global__ void __launch_bounds__(NORM_THREADS, RUN_BLOCKS_PER_SM)
+    residual32_kernel(const ResidualRuns R, double* __restrict__ partials, const float* __restrict__ sc, const NormEnd end)
+{
+    const float scale = *sc;
+    const int strips = run_strips(R.m), warps = gridDim.x * (NORM_THREADS / 32);
+    const int64_t runs = (int64_t)strips * run_blocks(R.n);
+    float acc32 = 0.0f;
+    for (int64_t k = (int64_t)blockIdx.x * (NORM_THREADS / 32) + (threadIdx.x >> 5); k < runs; k += warps) {
+        const int b = (int)(k / strips);
+        acc32 = residual_run(R, (int)(k - (int64_t)b * strips), b, scale, acc32);
+    }
+    __shared__ double red[NORM_THREADS / 32];
+    const double acc = warp_sum((double)acc32);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    double v = 0.0;
+    if (threadIdx.x < 32) v = warp_sum(threadIdx.x < NORM_THREADS / 32 ? red[threadIdx.x] : 0.0);
+    norm_end(end, v, partials, red);
+}
+
 __global__ void __launch_bounds__(PX* PY)
     update64_kernel(double* __restrict__ psi, int m, int n, int64_t pitch,
                     const float* __restrict__ e32, int64_t pitch32)
@@ -342,13 +367,23 @@ cudaError_t launch_defect64_to32(const Field& psi, const Coef& c, float* r32, fl
                                  int64_t pitch32, double* partials, cudaStream_t s,
                                  const float* norm_scale, const NormEnd& end)
 {
+    if (c.unit_beta && norm_scale) {
+        const int64_t runs = (int64_t)run_strips(psi.m) * run_blocks(psi.n);
+        const int grid = (int)std::min<int64_t>((runs + NORM_THREADS / 32 - 1) / (NORM_THREADS / 32),
+                                                std::min(RUN_BLOCKS_PER_SM * device_sms(), NORM_PARTIALS_MAX));
+        const bool vec = (psi.pitch & 1) == 0 && ((uintptr_t)psi.p & 15) == 0;
+        residual32_kernel<<<grid, NORM_THREADS, 0, s>>>(
+            ResidualRuns{psi.p, psi.pitch, r32, e32, pitch32, psi.m, psi.n, vec}, partials, norm_scale, end);
+        note_launch();
+        return cudaGetLastError();
+    }
     const int blocks = mixed_norm_blocks(psi.m, psi.n);
 #define LAP_D64(U, F)                                                                            \
     defect64_to32_kernel<U, F><<<blocks, NORM_THREADS, 0, s>>>(psi.p, psi.m, psi.n, psi.pitch, c.b2, \
                                                                c.d, r32, e32, pitch32, partials, \
                                                                norm_scale, end)
     if (c.unit_beta) {
-        if (norm_scale) LAP_D64(true, true); else LAP_D64(true, false);
+        LAP_D64(true, false);
     } else {
         if (norm_scale) LAP_D64(false, true); else LAP_D64(false, false);
     }
