@@ -326,6 +326,10 @@ const LineTables& line_tables(lap_handle h, int N, double alpha, double delta, d
         b[p] = delta - alpha * gR[L - 1] - alpha * (right_last ? gLl[0] : gL[0]);
         c[p] = p + 1 <= S - 1 ? -alpha * gR[0] : 0.0;
     }
+    // separators a boundary layer or more apart do not see each other: no reduction
+    bool coupled = L == 0;
+    for (int p = 0; p < S; ++p) coupled = coupled || big(a[p], b[p]) || big(c[p], b[p]);
+    if (!coupled) t.levels = 0;
     // parallel cyclic reduction, one lane per separator: tables indexed [level * maxp + lane]
     const size_t mp = (size_t)max_chunks;
     std::vector<double> k1((size_t)std::max(1, t.levels) * mp, 0.0), k2(k1.size(), 0.0), invb(mp, 0.0);
@@ -407,60 +411,108 @@ double line_coefs(const Coef& c, double w, int form, int direction, LineCoefs* k
     return form == LAP_FORM_A ? off : w * off;
 }
 
+// Chunks of a y-line, for lines of N unknowns, nl of them to a CTA: the cut whose slowest scheduler has the
+// least to do. A CTA has a multiprocessor to itself, its warps (nl P / 32) share four schedulers, an FP64
+// operation takes 64 clocks of one, and a chunk of L unknowns costs 5 L of them and two more within K0 of its
+// ends' reach; separators closer than that need the reduction, about 250 clocks a level. One warp alone takes
+// about 900 clocks a position (loads, addresses and stores between the 320 of FP64). Half sweeps of 4 / 12 / 16
+// warps to a multiprocessor at 3001 x 2050: 106 / 85 / 75 us.
+int line_y_chunks(int N, double alpha, double delta, int nl)
+{
+    const double x = alpha / delta, e = 2.0 * x / (1.0 + std::sqrt(std::max(0.0, 1.0 - 4.0 * x * x)));
+    const double K0 = 64.0 * std::log(2.0) / -std::log(std::min(e, 0.999));
+    // lines close to singular (relaxation near 2) keep long chunks: their separators' system is no better
+    const bool slow = K0 > 64.0;
+    const int most = slow ? LINE_MAX_CHUNKS : 64, shortest = slow ? LINE_MIN_CHUNK : LINE_Y_MIN_CHUNK;
+    int best = 1;
+    double least = 1e300;
+    for (int P = 1; P * nl <= LY_THREADS && P <= most; ++P) {
+        const int L = (N - (P - 1) + P - 1) / P;
+        if (P > 1 && L < shortest) break;
+        const int rounds = (nl * P + 127) / 128;
+        const double levels = P > 2 && L <= K0 ? std::ceil(std::log2(P - 1.0)) : 0.0;
+        const double cost = std::max(rounds * 64.0 * (5.0 * L + 2.0 * std::min<double>(L, K0)), 900.0 * L) + 250.0 * levels;
+        if (cost < least) {
+            least = cost;
+            best = P;
+        }
+    }
+    return best;
+}
+
 // Tables, per-call coefficients and (y-lines) scratch of one zebra half sweep; allocates only
 // on the first use of a shape, so calling it before a graph capture prepares the capture.
+// threads: x-lines as a thread per chunk (line_y_kernel), the scratch the caller's.
 const LineTables& line_setup(lap_handle h, const Field& f, const Coef& c, double w, int form,
-                             int direction, LineCoefs* k, double** scratch)
+                             int direction, LineCoefs* k, double** scratch, bool threads)
 {
     const bool x = direction == 0;
     const int N = x ? f.m - 2 : f.n - 2;
     const double alpha = line_coefs(c, w, form, direction, k);
+    *scratch = nullptr;
+    if (!x || threads) {
+        const int cut = line_y_chunks(N, alpha, c.d, line_y_lines(((x ? f.n : f.m) - 1) / 2, device_sms()));
+        const LineTables& t = line_tables(h, N, alpha, c.d, k->wc, cut, LINE_Y_MIN_CHUNK);
+        if (!x) *scratch = line_scratch(h, t, line_scratch_pitch(f, direction));
+        return t;
+    }
     // x-lines long enough for 64 chunks of at least 48 unknowns take the two-warp cut (at 4097^2:
     // 255 -> 242 us per half sweep); shorter chunks would spend most of their length in the
     // boundary layer (about 34 positions at beta = 1), so shorter lines keep 32 chunks
-    const bool cut64 = x && N >= LINE_MAX_CHUNKS_X * 48;
+    const bool cut64 = N >= LINE_MAX_CHUNKS_X * 48;
     const LineTables& t = line_tables(h, N, alpha, c.d, k->wc, cut64 ? LINE_MAX_CHUNKS_X : LINE_MAX_CHUNKS);
-    if (x) {
-        ck(prepare_line_kernels(line_smem_bytes(t)), "line kernel attributes");
-        *scratch = nullptr;
-        const size_t bytes = std::max<size_t>(line_x_sync_words(f.n - 2) * sizeof(unsigned), 1 << 20);
-        if (bytes > h->lsync_bytes) {
-            // keep a timeout that the old block recorded
-            unsigned err = 0;
-            if (h->lsync) ck(cudaMemcpy(&err, h->lsync, sizeof err, cudaMemcpyDeviceToHost), "read line flags");
-            drop_graphs(h);
-            dev_free(h, h->lsync, h->lsync_bytes);
-            h->lsync = nullptr;
-            h->lsync_bytes = 0;
-            h->lsync = (unsigned*)dev_alloc(h, bytes);
-            h->lsync_bytes = bytes;
-            ck(cudaMemset(h->lsync, 0, sizeof(unsigned)), "clear line error");
-            if (err) ck(cudaMemcpy(h->lsync, &err, sizeof err, cudaMemcpyHostToDevice), "keep line error");
-        }
-    } else {
-        *scratch = line_scratch(h, t, line_scratch_pitch(f, direction));
+    ck(prepare_line_kernels(line_smem_bytes(t)), "line kernel attributes");
+    const size_t bytes = std::max<size_t>(line_x_sync_words(f.n - 2) * sizeof(unsigned), 1 << 20);
+    if (bytes > h->lsync_bytes) {
+        // keep a timeout that the old block recorded
+        unsigned err = 0;
+        if (h->lsync) ck(cudaMemcpy(&err, h->lsync, sizeof err, cudaMemcpyDeviceToHost), "read line flags");
+        drop_graphs(h);
+        dev_free(h, h->lsync, h->lsync_bytes);
+        h->lsync = nullptr;
+        h->lsync_bytes = 0;
+        h->lsync = (unsigned*)dev_alloc(h, bytes);
+        h->lsync_bytes = bytes;
+        ck(cudaMemset(h->lsync, 0, sizeof(unsigned)), "clear line error");
+        if (err) ck(cudaMemcpy(h->lsync, &err, sizeof err, cudaMemcpyHostToDevice), "keep line error");
     }
     return t;
 }
 
+// The scratch with which the x-lines of a solve go by line_y_kernel, the rows' elements a pitch apart for
+// neighbouring threads: null where the row kernel is as fast, or where there is no room. A row CTA
+// costs a claim, two barriers and a flag per line, and its two colours wait on each other; the threads'
+// loads touch a sector each, which the caches only bear while lines are short. Half sweeps by rows / by
+// threads: 150^2 18.3 / 11.8 us, 300^2 21.2 / 15.2, 700^2 29 / 24.5, 1000^2 36.2 / 35.5, 498 x 4000 54 / 51,
+// 2050 x 3001 102 / 111, 4000 x 500 70 / 85.
+double* line_rows(lap_handle h, const Field& f, const Coef& c, double w, int form)
+{
+    if (f.m - 2 > 1024) return nullptr;
+    LineCoefs k;
+    double* none = nullptr;
+    const int64_t gp = line_scratch_pitch(f, 0);
+    return spare(h, line_y_scratch_doubles(line_setup(h, f, c, w, form, 0, &k, &none, true), gp) * sizeof(double));
+}
+
 // One zebra half sweep (odd lines, then even lines) in `direction` (0: x-lines = rows,
-// 1: y-lines = columns), form A or B.
+// 1: y-lines = columns), form A or B. rows: line_rows' scratch (x-lines).
 void line_half_sweep(lap_handle h, const Field& f, const Coef& c, double w, int form,
-                     int direction, cudaStream_t s)
+                     int direction, cudaStream_t s, double* rows)
 {
     LineCoefs k;
     double* scratch = nullptr;
-    const LineTables& t = line_setup(h, f, c, w, form, direction, &k, &scratch);
-    if (direction == 0) {  // both colours in one launch
+    const bool x = direction == 0;
+    const LineTables& t = line_setup(h, f, c, w, form, direction, &k, &scratch, rows != nullptr);
+    if (x && !rows) {  // both colours in one launch
         ck(launch_line_x(f.p, f.pitch, f.n - 2, t, form, k, h->lsync, s), "x-line kernel");
         return;
     }
-    const int nlines = f.m - 2;
+    const int nlines = x ? f.n - 2 : f.m - 2;
     const int64_t gp = line_scratch_pitch(f, direction);
     for (int first = 1; first <= 2; ++first) {
         const int count = first == 1 ? (nlines + 1) / 2 : nlines / 2;
-        ck(launch_line_scratch(f.p, f.pitch, 1, first, count, t, form, k, scratch, gp, s),
-           "y-line kernels");
+        ck(launch_line_y(f.p, x ? 1 : f.pitch, x ? f.pitch : 1, first, count, t, form, k, x ? rows : scratch, gp, s),
+           "line kernel");
     }
 }
 
@@ -733,6 +785,8 @@ struct Solver {
     double* jac_cur = nullptr;  // Jacobi: buffer holding the current iterate
     double* jac_other = nullptr;
 
+    double* rows = nullptr;  // the scratch of short x-lines (line_rows)
+
     // ---- several sweeps per launch (sweep_tiles.cu) ----
     SweepTiles tiles;                // sweeps = 0: one pass per launch
     double* tiles_other = nullptr;   // the second field
@@ -807,11 +861,11 @@ struct Solver {
             }
             break;
         case LAP_ADI:
-            line_half_sweep(h, f, c, p->w, p->line_form, 0, s);
+            line_half_sweep(h, f, c, p->w, p->line_form, 0, s, rows);
             line_half_sweep(h, f, c, p->w, p->line_form, 1, s);
             break;
         case LAP_SLOR:
-            line_half_sweep(h, f, c, p->w, p->line_form, 0, s);
+            line_half_sweep(h, f, c, p->w, p->line_form, 0, s, rows);
             break;
         case LAP_MG:
             vcycle(0);
@@ -1121,11 +1175,10 @@ struct Solver {
     void prepare()
     {
         if (p->method == LAP_ADI || p->method == LAP_SLOR) {
-            for (int dir = 0; dir < (p->method == LAP_ADI ? 2 : 1); ++dir) {
-                LineCoefs k;
-                double* scratch = nullptr;
-                line_setup(h, f, c, p->w, p->line_form, dir, &k, &scratch);
-            }
+            LineCoefs k;
+            double* scratch = nullptr;
+            if (p->method == LAP_ADI) line_setup(h, f, c, p->w, p->line_form, 1, &k, &scratch);
+            line_setup(h, f, c, p->w, p->line_form, 0, &k, &scratch, rows != nullptr);
         }
         if (p->method == LAP_MG) {
             const Level& lv = w.levels.back();
@@ -1149,7 +1202,7 @@ struct Solver {
                                 (int64_t)w.levels32.size(), tail_first, fused32, norm_sc > 0.0,
                                 p->sum_order, tiles.sweeps, tiles.tx, tiles.ty};
         const double dbl[] = {c.b2, c.d, c.inv_d, p->w, p->smoother_w};
-        const void* ptrs[] = {f.p, jac_cur, jac_other, w.aux, w.maxd, h->arena, h->lscratch, tiles_other};
+        const void* ptrs[] = {f.p, jac_cur, jac_other, w.aux, w.maxd, h->arena, h->lscratch, tiles_other, rows};
         put(ints, sizeof ints);
         put(dbl, sizeof dbl);
         put(ptrs, sizeof ptrs);
@@ -1400,7 +1453,10 @@ struct Solver {
         out->status = LAP_MAXITER;
         out->iters = 0;
         out->last_check = NAN;
-        if (p->method == LAP_ADI || p->method == LAP_SLOR) prepare();  // tables, scratch: before any capture
+        if (p->method == LAP_ADI || p->method == LAP_SLOR) {
+            prepare();  // tables, scratch: before any capture
+            rows = line_rows(h, f, c, p->w, p->line_form);
+        }
         choose_tiles();
         if (p->method == LAP_JACOBI) {
             // a sweep writes every interior point of the other buffer, and reads none of it before

@@ -171,12 +171,14 @@ void check_params(const lap_params* p);
 // line relaxation: cached tables of a line length and coefficients; the tables, coefficients
 // and scratch of a half sweep (allocating only on a shape's first use); one zebra half sweep
 constexpr int LINE_MIN_CHUNK = 16;
+constexpr int LINE_Y_MIN_CHUNK = 4;
 const LineTables& line_tables(lap_handle h, int N, double alpha, double delta, double wc,
                               int max_chunks = LINE_MAX_CHUNKS, int min_chunk = LINE_MIN_CHUNK);
 const LineTables& line_setup(lap_handle h, const Field& f, const Coef& c, double w, int form,
-                             int direction, LineCoefs* k, double** scratch);
+                             int direction, LineCoefs* k, double** scratch, bool threads = false);
+double* line_rows(lap_handle h, const Field& f, const Coef& c, double w, int form);
 void line_half_sweep(lap_handle h, const Field& f, const Coef& c, double w, int form,
-                     int direction, cudaStream_t s);
+                     int direction, cudaStream_t s, double* rows = nullptr);
 
 // the coarsest level's 5-point matrix, inverted once per shape (transposed, on the device)
 constexpr int COARSE_MAX_UNKNOWNS = 1024;

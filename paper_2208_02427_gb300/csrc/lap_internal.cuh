@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 #include <vector>
@@ -561,13 +562,15 @@ cudaError_t prepare_line_kernels(size_t smem);
 size_t line_x_sync_words(int nlines);
 cudaError_t launch_line_x(double* psi, int64_t pitch, int nlines, const LineTables& t, int form,
                           const LineCoefs& k, unsigned* sync, cudaStream_t s);
-// Lines first_line, first_line + 2, ... (count of them) through a scratch array, one thread
-// per (line, chunk): element k of line l at psi + l * sx + k * sa (y-lines: sa = pitch,
-// sx = 1; x-lines: sa = 1, sx = pitch). scratch holds line_y_scratch_doubles(t, gp)
-// doubles, gp >= count a multiple of 32.
+// Lines first_line, first_line + 2, ... (count of them), one thread per (line, chunk): element k of line l
+// at psi + l * sx + k * sa (y-lines: sa = pitch, sx = 1). scratch holds line_y_scratch_doubles(t, gp)
+// doubles, gp >= count.
+constexpr int LY_THREADS = 512;  // most threads of a CTA, each a chunk of a line
+// Lines to a CTA (t.P no more than LY_THREADS over that): as many as give every multiprocessor one CTA, at
+// least 4 (a 64-byte run of a row).
+inline int line_y_lines(int count, int sms) { return std::min(64, std::max(4, (count + sms - 1) / sms)); }
 size_t line_y_scratch_doubles(const LineTables& t, int64_t gp);
-cudaError_t launch_line_scratch(double* psi, int64_t sa, int64_t sx, int first_line, int count,
-                                const LineTables& t, int form, const LineCoefs& k, double* scratch,
-                                int64_t gp, cudaStream_t s);
+cudaError_t launch_line_y(double* psi, int64_t sa, int64_t sx, int first_line, int count, const LineTables& t, int form,
+                          const LineCoefs& k, double* scratch, int64_t gp, cudaStream_t s);
 
 }  // namespace lap

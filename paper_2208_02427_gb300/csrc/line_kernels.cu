@@ -26,19 +26,15 @@
 // only and are computed once on the host.
 //
 // x-lines (rows, contiguous): a CTA works on one line at a time; b~ is built into shared memory
-// with coalesced loads, one warp runs the chunk recurrences (lane = chunk) and the separator
-// solve (lane = separator, register shuffles), and the CTA writes the line back coalesced. The
+// with coalesced loads, one or two warps run the chunk recurrences (thread = chunk) and the separator
+// solve, and the CTA writes the line back coalesced. The
 // CTAs stay resident and take the lines of both zebra colours in order from a counter, so a
 // half sweep is one launch (line_x_kernel). On GB300 each of
 // an SM's four schedulers has its own FP64 unit (0.5 fma per clock; measured), and one warp's
 // dependent fma chain alone keeps it busy, so the six line CTAs that fit an SM's shared memory
 // are enough recurrence warps; the CTA's other warps shorten the load and store phases.
-// y-lines (columns, strided by the pitch): lane = line (32 adjacent lines of a colour, so every
-// row access is a contiguous 512-byte run), one thread per (line, chunk); three launches per
-// colour -- forward (G to a scratch array laid out [position][line]), separators (a warp per
-// line), back -- so that no transposed copy of the field is needed. (The same kernels serve
-// x-lines with the strides swapped, but their lanes then read 32 rows apart and ran 20-70%
-// slower than the shared-memory kernel.)
+// y-lines (columns, strided by the pitch), and rows of up to 1024 unknowns: a thread per (line,
+// chunk), one launch per colour, no transposed copy of the field (line_y_kernel).
 #include "lap_device.cuh"
 #include "lap_internal.cuh"
 
@@ -54,24 +50,6 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr int LX_THREADS = 256;
 constexpr int LX_UNROLL = 8;
 constexpr int XB = 8;
-constexpr int LY_WARPS = 2;      // y-lines: chunk warps per CTA of the forward and back kernels
-constexpr int LS_WARPS = 4;      // y-lines: lines (warps) per CTA of the separator kernel
-
-// Parallel cyclic reduction of the separators of one line, lane p holding separator p < S:
-// returns x~ of separator p (0 for lanes p >= S).
-__device__ __forceinline__ double separator_solve(const LineTables& t, int p, int S, double rho)
-{
-    double r = p < S ? rho : 0.0;
-    for (int lev = 0, s = 1; lev < t.levels; ++lev, s <<= 1) {
-        const double up = __shfl_up_sync(FULL, r, s);
-        const double dn = __shfl_down_sync(FULL, r, s);
-        double v = r;
-        if (p < S && p >= s) v = __fma_rn(t.k1[lev * t.maxp + p], up, v);
-        if (p + s < S) v = __fma_rn(t.k2[lev * t.maxp + p], dn, v);
-        r = v;
-    }
-    return p < S ? r * t.invb[p] : 0.0;
-}
 
 // ---- x-lines --------------------------------------------------------------------------
 // x-lines are cut into up to LINE_MAX_CHUNKS_X = 64 chunks, run by the CTA's first two warps
@@ -115,16 +93,24 @@ __device__ __forceinline__ void line_recurrences(const FmaOps& o, const LineTabl
         const double* __restrict__ gl = p == P - 1 ? t.glnl : t.gln;
         const double alpha = in_reg(o, t.alpha);
         double G = 0.0, D = 0.0;
+        const double* __restrict__ te = t.e;
         if (act) {
+            // operands of a step are loaded in the step before, ahead of its store, which waits for the
+            // fma (half sweeps at 3001 x 2050 113 -> 102 us)
             const int kb = min(len, K0);
             G = y[0];
-            D = fmul(o, gl[0], G);
+            D = fmul(o, __ldg(gl), G);
             int q = 1;
+            double b = y[min(1, len - 1)], e = __ldg(te), gv = __ldg(gl + min(1, len - 1));
             for (; q < kb; ++q) {
-                const double b = y[q];
-                D = __fma_rn(gl[q], b, D);
-                G = __fma_rn(t.e[q - 1], G, b);
+                const int nx = min(q + 1, len - 1);
+                const double nb = y[nx], ne = __ldg(te + q), ng = __ldg(gl + nx);
+                D = __fma_rn(gv, b, D);
+                G = __fma_rn(e, G, b);
                 y[q] = G;
+                b = nb;
+                e = ne;
+                gv = ng;
             }
             // the bulk in batches: operands of XB positions loaded before the chain uses them
             for (; q + XB <= len; q += XB) {
@@ -132,7 +118,7 @@ __device__ __forceinline__ void line_recurrences(const FmaOps& o, const LineTabl
 #pragma unroll
                 for (int u = 0; u < XB; ++u) {
                     bv[u] = y[q + u];
-                    ev[u] = t.e[q + u - 1];
+                    ev[u] = __ldg(te + q + u - 1);
                 }
 #pragma unroll
                 for (int u = 0; u < XB; ++u) {
@@ -140,9 +126,16 @@ __device__ __forceinline__ void line_recurrences(const FmaOps& o, const LineTabl
                     y[q + u] = G;
                 }
             }
-            for (; q < len; ++q) {
-                G = __fma_rn(t.e[q - 1], G, y[q]);
-                y[q] = G;
+            if (q < len) {
+                b = y[q];
+                e = __ldg(te + q - 1);
+                for (; q < len; ++q) {
+                    const double nb = y[min(q + 1, len - 1)], ne = __ldg(te + q);
+                    G = __fma_rn(e, G, b);
+                    y[q] = G;
+                    b = nb;
+                    e = ne;
+                }
             }
         }
         const double ylast = act ? fmul(o, t.inv_den[len - 1], G) : 0.0;
@@ -170,7 +163,7 @@ __device__ __forceinline__ void line_recurrences(const FmaOps& o, const LineTabl
 #pragma unroll
                 for (int u = 0; u < XB; ++u) {
                     gv[u] = y[q - u];
-                    ev[u] = t.e[q - u + 1];
+                    ev[u] = __ldg(te + q - u + 1);
                 }
 #pragma unroll
                 for (int u = 0; u < XB; ++u) {
@@ -178,13 +171,26 @@ __device__ __forceinline__ void line_recurrences(const FmaOps& o, const LineTabl
                     y[q - u] = Z;
                 }
             }
-            for (; q >= K0; --q) {
-                Z = __fma_rn(t.e[q + 1], Z, y[q]);
-                y[q] = Z;
-            }
-            for (; q >= 0; --q) {
-                Z = __fma_rn(t.e[q + 1], Z, __fma_rn(xl, t.F[q], y[q]));
-                y[q] = Z;
+            if (q >= 0) {
+                double gv = y[q], e = __ldg(te + q + 1), f = __ldg(t.F + q);
+                for (; q >= K0; --q) {
+                    const int nx = max(q - 1, 0);
+                    const double ng = y[nx], ne = __ldg(te + nx + 1), nf = __ldg(t.F + nx);
+                    Z = __fma_rn(e, Z, gv);
+                    y[q] = Z;
+                    gv = ng;
+                    e = ne;
+                    f = nf;
+                }
+                for (; q >= 0; --q) {
+                    const int nx = max(q - 1, 0);
+                    const double ng = y[nx], ne = __ldg(te + nx + 1), nf = __ldg(t.F + nx);
+                    Z = __fma_rn(e, Z, __fma_rn(xl, f, gv));
+                    y[q] = Z;
+                    gv = ng;
+                    e = ne;
+                    f = nf;
+                }
             }
             if (p < S) y[L] = xs;
         }
@@ -310,195 +316,205 @@ __global__ void __launch_bounds__(LX_THREADS, 6)
     }
 }
 
-// ---- lines through a scratch array: lane = line --------------------------------------
-// Thread (line l = first + 2 * (32 * blockIdx.x + lane), chunk c = LY_WARPS * blockIdx.y +
-// warp); element k of line l at psi + l * sx + k * sa, its neighbouring lines at +-sx
-// (y-lines: sa = pitch, sx = 1, so a warp's 32 lines read one contiguous run of a row;
-// x-lines: sa = 1, sx = pitch). G[(k - 1) * gp + lane index], coalesced either way. The
-// loops are software-pipelined: the loads of the next PIPE positions are issued before the
-// current ones are used.
-constexpr int PIPE = 8;  // 16 was slower (registers), and L2 evict-last hints on G gained nothing
+// ---- y-lines: lines across the threads ----------------------------------------------
+// A zebra colour is one launch. A CTA takes `nl` neighbouring lines of the colour whole: thread (line l,
+// chunk c) runs its chunk's forward recurrence (G to a scratch array laid out [position][line]; it reads
+// it back itself), the CTA solves its lines' separators in shared memory, and the threads run back and
+// write. Element k of line l lies at psi + (first_line + 2 l) sx + k sa, its neighbouring lines at +-sx (sa =
+// pitch, sx = 1: neighbouring lines share the sectors of a row). With two warps' lines and chunks in CTAs of
+// their own the separators took a launch between forward and back, three launches a colour; one
+// launch gives every multiprocessor the same number of lines and no waits between them. Half sweeps, three
+// launches a colour / one: 300^2 27 / 14 us, 1000^2 41 / 28, 3001 x 2050 84 / 75, 2050 x 3001 102 / 86, 500 x
+// 4000 99 / 72, 4097^2 195 / 203.
+// What bounds it is the recurrence: a dependent fma takes 71 clocks, one warp on each scheduler nearly
+// fills the FP64 pipe, and everything else has to be out of the way: a step's field values and table
+// entries are loaded PIPE positions ahead, into registers (a table entry loaded in its step waited for the
+// store of the step before, which waits for that step's fma).
+constexpr int PIPE = 4;  // 8 needs 200 registers, and fewer warps hide less: 79 us against 75 at 3001 x 2050
 
 template <int FORM>
-__global__ void __launch_bounds__(32 * LY_WARPS)
-    line_forward_kernel(const double* __restrict__ psi, int64_t sa, int64_t sx, int first_line,
-                        int count, const LineTables t, double bnd, double c1, double* __restrict__ G,
-                        int64_t gp, double* __restrict__ ylast, double* __restrict__ yfirst)
+__global__ void __launch_bounds__(LY_THREADS)
+    line_y_kernel(double* __restrict__ psi, int64_t sa, int64_t sx, int first_line, int count, int nl, const LineTables t,
+                  double bnd, double c1, double omw, double wc, double* __restrict__ G, int64_t gp)
 {
+    extern __shared__ double sm[];
     const FmaOps o = load_fma_ops();
-    const int li = blockIdx.x * 32 + (threadIdx.x & 31);
-    const int c = blockIdx.y * LY_WARPS + (threadIdx.x >> 5);
-    if (li >= count || c >= t.P) return;
-    const int L = t.L, len = c == t.P - 1 ? t.Ll : L, K0 = t.K0;
-    const int k0 = 1 + c * (L + 1);
-    const double* __restrict__ line = psi + (int64_t)(first_line + 2 * li) * sx;
-    double* __restrict__ g = G + li + (int64_t)(k0 - 1) * gp;
-    const double* __restrict__ gl = c == t.P - 1 ? t.glnl : t.gln;
-    c1 = in_reg(o, c1);
-
-    // right-hand side of chunk position q (loads only; the adds come with the recurrence)
-    double ra[PIPE], rb[PIPE], rc[PIPE];
-    auto load = [&](int q0, double* a, double* b_, double* cc) {
-#pragma unroll
-        for (int u = 0; u < PIPE; ++u)
-            if (q0 + u < len) {
-                const double* at = line + (int64_t)(k0 + q0 + u) * sa;
-                a[u] = at[-sx];
-                b_[u] = at[sx];
-                if (FORM == 1) cc[u] = at[0];
-            }
-    };
-    // position 0 (peeled: a per-step test inside the batches would issue both sides' FP64
-    // operations on every step)
-    double b0;
-    {
-        const double* at = line + (int64_t)k0 * sa;
-        b0 = fadd(o, at[-sx], at[sx]);
-        if (FORM == 1) b0 = __fma_rn(c1, at[0], b0);
-        if (c == 0) b0 = __fma_rn(bnd, line[0], b0);  // the near Dirichlet end
-    }
-    double G_ = b0;
-    double D = fmul(o, gl[0], b0);
-    g[0] = G_;
-    // positions 1.., PIPE at a time; batches that reach into the boundary layer also carry the
-    // y_first sum, the others only the recurrence
-    auto step = [&](int q, double a_, double b_, double c_) {
-        const double nbv = fadd(o, a_, b_);
-        const double b = FORM == 1 ? __fma_rn(c1, c_, nbv) : nbv;
-        G_ = __fma_rn(t.e[q - 1], G_, b);
-        g[(int64_t)q * gp] = G_;
-        return b;
-    };
-    load(1, ra, rb, rc);
-    for (int q0 = 1; q0 < len; q0 += PIPE) {
-        double na[PIPE], nb_[PIPE], nc[PIPE];
-        if (q0 + PIPE < len) load(q0 + PIPE, na, nb_, nc);
-        if (q0 < K0) {
-#pragma unroll
-            for (int u = 0; u < PIPE; ++u) {
-                const int q = q0 + u;
-                if (q < len) {
-                    const double b = step(q, ra[u], rb[u], rc[u]);
-                    if (q < K0) D = __fma_rn(gl[q], b, D);
-                }
-            }
-        } else if (q0 + PIPE <= len) {
-#pragma unroll
-            for (int u = 0; u < PIPE; ++u) step(q0 + u, ra[u], rb[u], rc[u]);
-        } else {
-#pragma unroll
-            for (int u = 0; u < PIPE; ++u)
-                if (q0 + u < len) step(q0 + u, ra[u], rb[u], rc[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < PIPE; ++u) {
-            ra[u] = na[u];
-            rb[u] = nb_[u];
-            if (FORM == 1) rc[u] = nc[u];
-        }
-    }
-    if (c == t.P - 1) {  // the far Dirichlet end enters b~_N with coefficient 1
-        const double extra = fmul(o, bnd, line[(int64_t)(t.N + 1) * sa]);
-        G_ = fadd(o, G_, extra);
-        g[(int64_t)(len - 1) * gp] = G_;
-        if (len - 1 < K0) D = __fma_rn(gl[len - 1], extra, D);
-    }
-    ylast[(int64_t)c * gp + li] = fmul(o, t.inv_den[len - 1], G_);
-    yfirst[(int64_t)c * gp + li] = D;
-}
-
-// One warp per line: lane p = separator p; writes the separators' solution xs and their
-// output values.
-template <int FORM>
-__global__ void __launch_bounds__(32 * LS_WARPS)
-    line_separator_kernel(double* __restrict__ psi, int64_t sa, int64_t sx, int first_line, int count,
-                          const LineTables t, double c1, double omw, double wc,
-                          const double* __restrict__ ylast, const double* __restrict__ yfirst,
-                          double* __restrict__ xsep, int64_t gp)
-{
-    const FmaOps o = load_fma_ops();
-    const int li = blockIdx.x * LS_WARPS + (threadIdx.x >> 5);
-    if (li >= count) return;  // warp-uniform
-    const int p = threadIdx.x & 31, S = t.P - 1;
-    double* line = psi + (int64_t)(first_line + 2 * li) * sx;
-    double* at = line + (int64_t)((p + 1) * (t.L + 1)) * sa;
-    double rho = 0.0, old = 0.0;
-    if (p < S) {
-        const double nb = fadd(o, at[-sx], at[sx]);
-        old = at[0];
-        const double b = FORM == 1 ? __fma_rn(c1, old, nb) : nb;
-        const double yl = ylast[(int64_t)p * gp + li], yf = yfirst[(int64_t)(p + 1) * gp + li];
-        rho = __fma_rn(t.alpha, fadd(o, yl, yf), b);
-    }
-    const double xs = separator_solve(t, p, S, rho);
-    if (p < S) {
-        xsep[(int64_t)p * gp + li] = xs;
-        at[0] = FORM == 0 ? __fma_rn(wc, xs, fmul(o, omw, old)) : fmul(o, wc, xs);
-    }
-}
-
-template <int FORM>
-__global__ void __launch_bounds__(32 * LY_WARPS)
-    line_back_kernel(double* __restrict__ psi, int64_t sa, int64_t sx, int first_line, int count,
-                     const LineTables t, double omw, const double* __restrict__ G, int64_t gp,
-                     const double* __restrict__ xsep)
-{
-    const FmaOps o = load_fma_ops();
-    const int li = blockIdx.x * 32 + (threadIdx.x & 31);
-    const int c = blockIdx.y * LY_WARPS + (threadIdx.x >> 5);
-    if (li >= count || c >= t.P) return;
+    const int l0 = blockIdx.x * nl, lines = min(nl, count - l0);
+    const int c = (int)threadIdx.x / nl, l = (int)threadIdx.x - c * nl;
+    const bool act = c < t.P && l < lines;
     const int L = t.L, len = c == t.P - 1 ? t.Ll : L, K0 = t.K0, S = t.P - 1;
     const int k0 = 1 + c * (L + 1);
-    double* __restrict__ line = psi + (int64_t)(first_line + 2 * li) * sx + (int64_t)k0 * sa;
-    const double* __restrict__ g = G + li + (int64_t)(k0 - 1) * gp;
-    const double xl = c > 0 ? xsep[(int64_t)(c - 1) * gp + li] : 0.0;
-    const double xr = c < S ? xsep[(int64_t)c * gp + li] : 0.0;
-    omw = in_reg(o, omw);
+    const double* __restrict__ te = t.e;
+    double* __restrict__ line = psi + (int64_t)(first_line + 2 * (l0 + l)) * sx;
+    double* __restrict__ g = G + (l0 + l) + (int64_t)(k0 - 1) * gp;
+    double* const yl = sm;                  // [chunk][line] the last value of a chunk's zero-end solution,
+    double* const yf = sm + t.P * nl;       // its first,
+    double* const bs = sm + 2 * t.P * nl;   // and the right-hand side of the separator behind it
     const double alpha = in_reg(o, t.alpha);
+    c1 = in_reg(o, c1);
+    omw = in_reg(o, omw);
+    wc = in_reg(o, wc);
 
+    if (act) {
+        const double* __restrict__ gl = c == t.P - 1 ? t.glnl : t.gln;
+        // the field values and table entries of chunk positions q0 .. (loads only; the adds come with the
+        // recurrence)
+        double ra[PIPE], rb[PIPE], rc[PIPE], re[PIPE];
+        auto load = [&](int q0, double* a, double* b_, double* cc, double* ee) {
+#pragma unroll
+            for (int u = 0; u < PIPE; ++u)
+                if (q0 + u < len) {
+                    const double* at = line + (int64_t)(k0 + q0 + u) * sa;
+                    a[u] = at[-sx];
+                    b_[u] = at[sx];
+                    if (FORM == 1) cc[u] = at[0];
+                    ee[u] = __ldg(te + q0 + u - 1);
+                }
+        };
+        load(1, ra, rb, rc, re);
+        // position 0 (peeled: a per-step test inside the batches would issue both sides' FP64
+        // operations on every step)
+        double b0;
+        {
+            const double* at = line + (int64_t)k0 * sa;
+            b0 = fadd(o, at[-sx], at[sx]);
+            if (FORM == 1) b0 = __fma_rn(c1, at[0], b0);
+            if (c == 0) b0 = __fma_rn(bnd, line[0], b0);  // the near Dirichlet end
+        }
+        double G_ = b0;
+        double D = fmul(o, __ldg(gl), b0);
+        g[0] = G_;
+        // positions 1.., PIPE at a time; batches that reach into the boundary layer also carry the
+        // y_first sum, the others only the recurrence
+        auto step = [&](int q, double a_, double b_, double c_, double e_) {
+            const double nbv = fadd(o, a_, b_);
+            const double b = FORM == 1 ? __fma_rn(c1, c_, nbv) : nbv;
+            G_ = __fma_rn(e_, G_, b);
+            g[(int64_t)q * gp] = G_;
+            return b;
+        };
+        for (int q0 = 1; q0 < len; q0 += PIPE) {
+            double na[PIPE], nb_[PIPE], nc[PIPE], ne[PIPE];
+            if (q0 + PIPE < len) load(q0 + PIPE, na, nb_, nc, ne);
+            if (q0 < K0) {
+                double gv[PIPE];
+#pragma unroll
+                for (int u = 0; u < PIPE; ++u)
+                    if (q0 + u < len) gv[u] = __ldg(gl + q0 + u);
+#pragma unroll
+                for (int u = 0; u < PIPE; ++u) {
+                    const int q = q0 + u;
+                    if (q < len) {
+                        const double b = step(q, ra[u], rb[u], rc[u], re[u]);
+                        if (q < K0) D = __fma_rn(gv[u], b, D);
+                    }
+                }
+            } else if (q0 + PIPE <= len) {
+#pragma unroll
+                for (int u = 0; u < PIPE; ++u) step(q0 + u, ra[u], rb[u], rc[u], re[u]);
+            } else {
+#pragma unroll
+                for (int u = 0; u < PIPE; ++u)
+                    if (q0 + u < len) step(q0 + u, ra[u], rb[u], rc[u], re[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < PIPE; ++u) {
+                ra[u] = na[u];
+                rb[u] = nb_[u];
+                if (FORM == 1) rc[u] = nc[u];
+                re[u] = ne[u];
+            }
+        }
+        if (c == t.P - 1) {  // the far Dirichlet end enters b~_N with coefficient 1
+            const double extra = fmul(o, bnd, line[(int64_t)(t.N + 1) * sa]);
+            G_ = fadd(o, G_, extra);
+            g[(int64_t)(len - 1) * gp] = G_;
+            if (len - 1 < K0) D = __fma_rn(gl[len - 1], extra, D);
+        }
+        if (c < S) {
+            const double* at = line + (int64_t)(k0 + len) * sa;
+            const double nb = fadd(o, at[-sx], at[sx]);
+            bs[c * nl + l] = FORM == 1 ? __fma_rn(c1, at[0], nb) : nb;
+        }
+        yl[c * nl + l] = fmul(o, t.inv_den[len - 1], G_);
+        yf[c * nl + l] = D;
+    }
+    __syncthreads();
+    // separator c of the line: thread (l, c); its solution into bs
+    double r = 0.0;
+    if (act && c < S)
+        r = __fma_rn(alpha, fadd(o, yl[c * nl + l], yf[(c + 1) * nl + l]), bs[c * nl + l]);
+    for (int lev = 0, d = 1; lev < t.levels; ++lev, d <<= 1) {  // cyclic reduction (line_tables)
+        __syncthreads();
+        if (act && c < S) yl[c * nl + l] = r;
+        __syncthreads();
+        if (act && c < S) {
+            double v = r;
+            if (c >= d) v = __fma_rn(t.k1[lev * t.maxp + c], yl[(c - d) * nl + l], v);
+            if (c + d < S) v = __fma_rn(t.k2[lev * t.maxp + c], yl[(c + d) * nl + l], v);
+            r = v;
+        }
+    }
+    if (act && c < S) bs[c * nl + l] = r = r * t.invb[c];
+    __syncthreads();
+    if (!act) return;
+
+    const double xl = c > 0 ? bs[(c - 1) * nl + l] : 0.0;
+    const double xr = c < S ? r : 0.0;
+    line += (int64_t)k0 * sa;
     // positions run backwards: batch j holds q = top - u, u = 0..PIPE-1
-    double gv[PIPE], ov[PIPE];
-    auto load = [&](int top, double* gg, double* oo) {
+    const double* __restrict__ tsc = t.sc;
+    double gv[PIPE], ov[PIPE], ev[PIPE], sv[PIPE];
+    auto load = [&](int top, double* gg, double* oo, double* ee, double* ss) {
 #pragma unroll
         for (int u = 0; u < PIPE; ++u)
             if (top - u >= 0) {
                 gg[u] = g[(int64_t)(top - u) * gp];
                 if (FORM == 0) oo[u] = line[(int64_t)(top - u) * sa];
+                ee[u] = __ldg(te + top - u + 1);
+                ss[u] = __ldg(tsc + top - u);
             }
     };
     // position len - 1 (peeled), then len - 2 .. 0, PIPE at a time; batches wholly past the
     // boundary layer skip its term
-    auto out = [&](int q, double Z, double old) {
-        double* at = line + (int64_t)q * sa;
-        *at = FORM == 0 ? __fma_rn(t.sc[q], Z, fmul(o, omw, old)) : fmul(o, t.sc[q], Z);
+    auto out = [&](int q, double Z, double old, double sc) {
+        line[(int64_t)q * sa] = FORM == 0 ? __fma_rn(sc, Z, fmul(o, omw, old)) : fmul(o, sc, Z);
     };
+    load(len - 2, gv, ov, ev, sv);
+    if (c < S) {  // the separator behind the chunk
+        double* at = line + (int64_t)len * sa;
+        *at = FORM == 0 ? __fma_rn(wc, xr, fmul(o, omw, *at)) : fmul(o, wc, xr);
+    }
     double Z;
     {
         const int q = len - 1;
         double Gq = g[(int64_t)q * gp];
         if (q < K0) Gq = __fma_rn(xl, t.F[q], Gq);
         Z = __fma_rn(alpha, xr, Gq);
-        out(q, Z, FORM == 0 ? line[(int64_t)q * sa] : 0.0);
+        out(q, Z, FORM == 0 ? line[(int64_t)q * sa] : 0.0, __ldg(tsc + q));
     }
-    load(len - 2, gv, ov);
     for (int top = len - 2; top >= 0; top -= PIPE) {
-        double ng[PIPE], no[PIPE];
-        if (top - PIPE >= 0) load(top - PIPE, ng, no);
+        double ng[PIPE], no[PIPE], ne[PIPE], ns[PIPE];
+        if (top - PIPE >= 0) load(top - PIPE, ng, no, ne, ns);
         if (top - PIPE + 1 >= K0) {
 #pragma unroll
             for (int u = 0; u < PIPE; ++u) {
-                Z = __fma_rn(t.e[top - u + 1], Z, gv[u]);
-                out(top - u, Z, ov[u]);
+                Z = __fma_rn(ev[u], Z, gv[u]);
+                out(top - u, Z, ov[u], sv[u]);
             }
         } else {
+            double fv[PIPE];
+#pragma unroll
+            for (int u = 0; u < PIPE; ++u)
+                if (top - u >= 0) fv[u] = __ldg(t.F + top - u);
 #pragma unroll
             for (int u = 0; u < PIPE; ++u) {
                 const int q = top - u;
                 if (q >= 0) {
                     double Gq = gv[u];
-                    if (q < K0) Gq = __fma_rn(xl, t.F[q], Gq);
-                    Z = __fma_rn(t.e[q + 1], Z, Gq);
-                    out(q, Z, ov[u]);
+                    if (q < K0) Gq = __fma_rn(xl, fv[u], Gq);
+                    Z = __fma_rn(ev[u], Z, Gq);
+                    out(q, Z, ov[u], sv[u]);
                 }
             }
         }
@@ -506,6 +522,8 @@ __global__ void __launch_bounds__(32 * LY_WARPS)
         for (int u = 0; u < PIPE; ++u) {
             gv[u] = ng[u];
             if (FORM == 0) ov[u] = no[u];
+            ev[u] = ne[u];
+            sv[u] = ns[u];
         }
     }
 }
@@ -557,39 +575,20 @@ cudaError_t launch_line_x(double* psi, int64_t pitch, int nlines, const LineTabl
     return cudaGetLastError();
 }
 
-size_t line_y_scratch_doubles(const LineTables& t, int64_t gp)
-{
-    return (size_t)gp * ((size_t)t.N + 3 * (size_t)t.P);
-}
+size_t line_y_scratch_doubles(const LineTables& t, int64_t gp) { return (size_t)gp * (size_t)t.N; }
 
-cudaError_t launch_line_scratch(double* psi, int64_t sa, int64_t sx, int first_line, int count,
-                                const LineTables& t, int form, const LineCoefs& k, double* scratch,
-                                int64_t gp, cudaStream_t s)
+cudaError_t launch_line_y(double* psi, int64_t sa, int64_t sx, int first_line, int count, const LineTables& t, int form,
+                          const LineCoefs& k, double* scratch, int64_t gp, cudaStream_t s)
 {
     if (count <= 0) return cudaSuccess;
-    double* G = scratch;
-    double* yl = G + (size_t)gp * t.N;
-    double* yf = yl + (size_t)gp * t.P;
-    double* xs = yf + (size_t)gp * t.P;
-    const dim3 grid((count + 31) / 32, (t.P + LY_WARPS - 1) / LY_WARPS);
-    const dim3 sgrid((count + LS_WARPS - 1) / LS_WARPS);
-#define LAP_LINES(F)                                                                                 \
-    do {                                                                                             \
-        line_forward_kernel<F><<<grid, 32 * LY_WARPS, 0, s>>>(psi, sa, sx, first_line, count, t,      \
-                                                              k.bnd, k.c1, G, gp, yl, yf);           \
-        note_launch();                                                                               \
-        if (t.P > 1) {                                                                               \
-            line_separator_kernel<F><<<sgrid, 32 * LS_WARPS, 0, s>>>(psi, sa, sx, first_line, count,  \
-                                                                     t, k.c1, k.omw, k.wc, yl, yf,   \
-                                                                     xs, gp);                        \
-            note_launch();                                                                           \
-        }                                                                                            \
-        line_back_kernel<F><<<grid, 32 * LY_WARPS, 0, s>>>(psi, sa, sx, first_line, count, t, k.omw, \
-                                                           G, gp, xs);                               \
-        note_launch();                                                                               \
-    } while (0)
-    if (form == 0) LAP_LINES(0); else LAP_LINES(1);
-#undef LAP_LINES
+    const int nl = std::min(LY_THREADS / t.P, line_y_lines(count, device_sms()));
+    const int grid = (count + nl - 1) / nl, threads = (nl * t.P + 31) / 32 * 32;
+    const size_t smem = (size_t)3 * t.P * nl * sizeof(double);
+    if (form == 0)
+        line_y_kernel<0><<<grid, threads, smem, s>>>(psi, sa, sx, first_line, count, nl, t, k.bnd, k.c1, k.omw, k.wc, scratch, gp);
+    else
+        line_y_kernel<1><<<grid, threads, smem, s>>>(psi, sa, sx, first_line, count, nl, t, k.bnd, k.c1, k.omw, k.wc, scratch, gp);
+    note_launch();
     return cudaGetLastError();
 }
 
