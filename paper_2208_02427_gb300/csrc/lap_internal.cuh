@@ -82,7 +82,7 @@ cudaError_t launch_rb_colour(const Field& f, const double* q, const Coef& c, boo
 // RD_K; the widest strip of an m-wide field has rb_diag_starts(m) walks, and the launch takes
 // rb_diag_walks(m, n) in all, numbered with 32-bit ints: at most RB_DIAG_MAX_WALKS (a field of
 // about 2.5e10 points). The launcher returns cudaErrorInvalidValue above that.
-constexpr int RD_BX = 128, RD_K = 6;
+constexpr int RD_BX = 64, RD_K = 6;
 constexpr int64_t RB_DIAG_MAX_WALKS = 2147483647 - RD_BX;
 inline int rb_diag_starts(int m) { return (m - 2 - (2 - RD_K)) / 2 + 1; }
 inline int64_t rb_diag_walks(int m, int n)
