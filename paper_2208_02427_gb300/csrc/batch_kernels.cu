@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(BT)
     b_rb_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim, const BatchLevel<T>* __restrict__ lv,
                 const int* __restrict__ active, int colour, int gs, T w, T omw)
 {
+    after_prior();
     const Arith<T> A = arith<T>();
     const ItemClaim ic{claim, count};
     for (int b = ic.take(-1); b < count; b = ic.take(b)) {
@@ -209,6 +210,7 @@ __device__ __forceinline__ void sweep_steps(const FmaOps& o, const SweepItem& it
 __global__ void __launch_bounds__(BT)
     b_sweep_kernel(const SweepItem* __restrict__ items, const int* __restrict__ active, int colour)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     const SweepItem it = items[blockIdx.x];
     const int run = active[it.problem];
@@ -223,6 +225,7 @@ __global__ void __launch_bounds__(BT)
     b_defect_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim,
                     const BatchLevel<T>* __restrict__ lv, const int* __restrict__ active, int gs)
 {
+    after_prior();
     const Arith<T> A = arith<T>();
     const ItemClaim ic{claim, count};
     for (int b = ic.take(-1); b < count; b = ic.take(b)) {
@@ -248,6 +251,7 @@ __global__ void __launch_bounds__(BT, 4)
     b_restrict_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim,
                       const BatchLevel<T>* __restrict__ lv, const int* __restrict__ active, int gs)
 {
+    after_prior();
     const Arith<T> A = arith<T>();
     const ItemClaim ic{claim, count};
     for (int b = ic.take(-1); b < count; b = ic.take(b)) {
@@ -283,6 +287,7 @@ __global__ void __launch_bounds__(BT)
     b_prolong_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim,
                      const BatchLevel<T>* __restrict__ lv, const int* __restrict__ active, int gs)
 {
+    after_prior();
     const Arith<T> A = arith<T>();
     const ItemClaim ic{claim, count};
     for (int b = ic.take(-1); b < count; b = ic.take(b)) {
@@ -330,6 +335,7 @@ __global__ void __launch_bounds__(1024)
     b_coarse_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim,
                     const BatchLevel<T>* __restrict__ lv, const int* __restrict__ active)
 {
+    after_prior();
     extern __shared__ double b[];
     const ItemClaim ic{claim, count};
     for (int k = ic.take(-1); k < count; k = ic.take(k)) {
@@ -615,6 +621,7 @@ __global__ void __launch_bounds__(BT, 3)
                         double* __restrict__ partials, const BatchLevel<float>* __restrict__ lv32,
                         const double* __restrict__ r0, int clear_e)
 {
+    after_prior();
     if (!CLAIM) {
         residual32_block(items, blockIdx.x, lv, active, partials, lv32, r0, clear_e);
         return;
@@ -634,6 +641,7 @@ __global__ void __launch_bounds__(BT, 5)
                    double* __restrict__ partials, const BatchLevel<float>* __restrict__ lv32,
                    int skip32, int gs)
 {
+    after_prior();
     if (!CLAIM) {
         sumsq_block(items, blockIdx.x, lv, active, partials, lv32, skip32, gs != 0);
         return;
@@ -680,6 +688,7 @@ __global__ void b_converge_kernel(const double* __restrict__ partials,
                                   const long long* __restrict__ maxit, Completion* __restrict__ done,
                                   int* __restrict__ ndone)
 {
+    after_prior();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= count || !active[p]) return;
     if (first_item[p] == first_item[p + 1]) return;  // not in this list
@@ -723,7 +732,7 @@ cudaError_t launch_b_rb(const BatchList& l, const BatchLevel<T>* lv, const int* 
 {
     if (l.count == 0) return cudaSuccess;
     const int grid = batch_grid((const void*)b_rb_kernel<T>, BT, 0, l.count, l.claim != nullptr);
-    b_rb_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, colour, gs ? 1 : 0, (T)w,
+    launch_after(b_rb_kernel<T>, grid, BT, 0, s, l.items, l.count, l.claim, lv, active, colour, gs ? 1 : 0, (T)w,
                                        (T)(1.0 - w));
     note_launch();
     return cudaGetLastError();
@@ -731,7 +740,7 @@ cudaError_t launch_b_rb(const BatchList& l, const BatchLevel<T>* lv, const int* 
 cudaError_t launch_b_sweep(const SweepItem* items, int count, const int* active, int colour, cudaStream_t s)
 {
     if (count == 0) return cudaSuccess;
-    b_sweep_kernel<<<count, BT, 0, s>>>(items, active, colour);
+    launch_after(b_sweep_kernel, count, BT, 0, s, items, active, colour);
     note_launch();
     return cudaGetLastError();
 }
@@ -742,7 +751,7 @@ cudaError_t launch_b_defect(const BatchList& l, const BatchLevel<T>* lv, const i
 {
     if (l.count == 0) return cudaSuccess;
     const int grid = batch_grid((const void*)b_defect_kernel<T>, BT, 0, l.count, l.claim != nullptr);
-    b_defect_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, gs ? 1 : 0);
+    launch_after(b_defect_kernel<T>, grid, BT, 0, s, l.items, l.count, l.claim, lv, active, gs ? 1 : 0);
     note_launch();
     return cudaGetLastError();
 }
@@ -752,7 +761,7 @@ cudaError_t launch_b_restrict(const BatchList& l, const BatchLevel<T>* lv, const
 {
     if (l.count == 0) return cudaSuccess;
     const int grid = batch_grid((const void*)b_restrict_kernel<T>, BT, 0, l.count, l.claim != nullptr);
-    b_restrict_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, gs ? 1 : 0);
+    launch_after(b_restrict_kernel<T>, grid, BT, 0, s, l.items, l.count, l.claim, lv, active, gs ? 1 : 0);
     note_launch();
     return cudaGetLastError();
 }
@@ -762,7 +771,7 @@ cudaError_t launch_b_prolong(const BatchList& l, const BatchLevel<T>* lv, const 
 {
     if (l.count == 0) return cudaSuccess;
     const int grid = batch_grid((const void*)b_prolong_kernel<T>, BT, 0, l.count, l.claim != nullptr);
-    b_prolong_kernel<T><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, gs ? 1 : 0);
+    launch_after(b_prolong_kernel<T>, grid, BT, 0, s, l.items, l.count, l.claim, lv, active, gs ? 1 : 0);
     note_launch();
     return cudaGetLastError();
 }
@@ -775,7 +784,7 @@ cudaError_t launch_b_coarse(const BatchList& l, const BatchLevel<T>* lv, const i
     threads = threads < 32 ? 32 : (threads > 1024 ? 1024 : threads);
     const size_t smem = sizeof(double) * max_unknowns;
     const int grid = batch_grid((const void*)b_coarse_kernel<T>, threads, smem, l.count, l.claim != nullptr);
-    b_coarse_kernel<T><<<grid, threads, smem, s>>>(l.items, l.count, l.claim, lv, active);
+    launch_after(b_coarse_kernel<T>, grid, threads, smem, s, l.items, l.count, l.claim, lv, active);
     note_launch();
     return cudaGetLastError();
 }
@@ -814,9 +823,9 @@ cudaError_t launch_b_sumsq(const BatchList& l, const BatchLevel<double>* lv, con
     if (l.count == 0) return cudaSuccess;
     if (l.claim) {
         const int grid = batch_grid((const void*)b_sumsq_kernel<true>, BT, 0, l.count, true);
-        b_sumsq_kernel<true><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, partials, lv32, skip32 ? 1 : 0, gs ? 1 : 0);
+        launch_after(b_sumsq_kernel<true>, grid, BT, 0, s, l.items, l.count, l.claim, lv, active, partials, lv32, skip32 ? 1 : 0, gs ? 1 : 0);
     } else {
-        b_sumsq_kernel<false><<<l.count, BT, 0, s>>>(l.items, l.count, nullptr, lv, active, partials, lv32,
+        launch_after(b_sumsq_kernel<false>, l.count, BT, 0, s, l.items, l.count, nullptr, lv, active, partials, lv32,
                                                      skip32 ? 1 : 0, gs ? 1 : 0);
     }
     note_launch();
@@ -830,9 +839,9 @@ cudaError_t launch_b_residual32(const BatchList& l, const BatchLevel<double>* lv
     if (l.count == 0) return cudaSuccess;
     if (l.claim) {
         const int grid = batch_grid((const void*)b_residual32_kernel<true>, BT, 0, l.count, true);
-        b_residual32_kernel<true><<<grid, BT, 0, s>>>(l.items, l.count, l.claim, lv, active, partials, lv32, r0, clear_e ? 1 : 0);
+        launch_after(b_residual32_kernel<true>, grid, BT, 0, s, l.items, l.count, l.claim, lv, active, partials, lv32, r0, clear_e ? 1 : 0);
     } else {
-        b_residual32_kernel<false><<<l.count, BT, 0, s>>>(l.items, l.count, nullptr, lv, active, partials, lv32, r0, clear_e ? 1 : 0);
+        launch_after(b_residual32_kernel<false>, l.count, BT, 0, s, l.items, l.count, nullptr, lv, active, partials, lv32, r0, clear_e ? 1 : 0);
     }
     note_launch();
     return cudaGetLastError();
@@ -854,7 +863,7 @@ cudaError_t launch_b_converge(const double* partials, const int* first_item, int
                               const double* tolv, const long long* maxit, Completion* done,
                               int* ndone)
 {
-    b_converge_kernel<<<(count + 127) / 128, 128, 0, s>>>(partials, first_item, count, active, r0,
+    launch_after(b_converge_kernel, (count + 127) / 128, 128, 0, s, partials, first_item, count, active, r0,
                                                           rnow, iters, status, remaining, mode,
                                                           rel ? 1 : 0, tol, tolv, maxit, done, ndone);
     note_launch();

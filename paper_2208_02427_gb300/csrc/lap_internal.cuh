@@ -68,6 +68,29 @@ cudaError_t prepare_sweep_tiles(const Coef& c, int kind, bool diag);
 cudaError_t launch_sweep_tiles(const Field& in, double* out, const Coef& c, const SweepTiles& t, int kind, bool diag,
                                int sweeps, const double* wslot, cudaStream_t s);
 
+// A launch whose set-up may run before the kernels ahead of it on the stream are through; the kernel calls
+// after_prior() before anything else. 0.2 to 0.35 us a launch in a graph, where small levels and small grids are
+// chains of launches of a few microseconds (measured per sweep: Jacobi 1531 x 1021 9.52 -> 9.27 us, SOR
+// 1000^2 11.7 -> 11.0). Letting the next kernel's CTAs in early as well takes the slots of this kernel's own
+// last wave: 9.5 -> 13.1 us.
+template <class... P, class... A>
+inline void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+// Waits until the kernels ahead on the stream are through and their writes visible.
+__device__ __forceinline__ void after_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---- point kernels (point_kernels.cu) -------------------------------------------
 // One colour of a red-black sweep, in place: Gauss-Seidel (Eq. 6) when gs is true,
 // SOR (Eq. 7) otherwise; q may be null. maxd (nullable) accumulates max|new - old| as

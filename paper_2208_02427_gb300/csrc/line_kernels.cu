@@ -337,6 +337,7 @@ __global__ void __launch_bounds__(LY_THREADS)
     line_y_kernel(double* __restrict__ psi, int64_t sa, int64_t sx, int first_line, int count, int nl, const LineTables t,
                   double bnd, double c1, double omw, double wc, double* __restrict__ G, int64_t gp)
 {
+    after_prior();
     extern __shared__ double sm[];
     const FmaOps o = load_fma_ops();
     const int l0 = blockIdx.x * nl, lines = min(nl, count - l0);
@@ -585,9 +586,9 @@ cudaError_t launch_line_y(double* psi, int64_t sa, int64_t sx, int first_line, i
     const int grid = (count + nl - 1) / nl, threads = (nl * t.P + 31) / 32 * 32;
     const size_t smem = (size_t)3 * t.P * nl * sizeof(double);
     if (form == 0)
-        line_y_kernel<0><<<grid, threads, smem, s>>>(psi, sa, sx, first_line, count, nl, t, k.bnd, k.c1, k.omw, k.wc, scratch, gp);
+        launch_after(line_y_kernel<0>, grid, threads, smem, s, psi, sa, sx, first_line, count, nl, t, k.bnd, k.c1, k.omw, k.wc, scratch, gp);
     else
-        line_y_kernel<1><<<grid, threads, smem, s>>>(psi, sa, sx, first_line, count, nl, t, k.bnd, k.c1, k.omw, k.wc, scratch, gp);
+        launch_after(line_y_kernel<1>, grid, threads, smem, s, psi, sa, sx, first_line, count, nl, t, k.bnd, k.c1, k.omw, k.wc, scratch, gp);
     note_launch();
     return cudaGetLastError();
 }

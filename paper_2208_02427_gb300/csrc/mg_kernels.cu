@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(MG_BX* MG_BY)
     restrict_kernel(const double* __restrict__ r, int mf, int nf, int64_t pf,
                     double* __restrict__ qc, double* __restrict__ ec, int64_t pc, int red, double inv_d, int shift)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     const int mc = (mf - 1) / 2 + 1, nc = (nf - 1) / 2 + 1;
     const int I = 1 + blockIdx.x * MG_BX + threadIdx.x;
@@ -54,6 +55,7 @@ __global__ void __launch_bounds__(32 * GR_WARPS)
     gs_restrict_kernel(const double* __restrict__ u, const double* __restrict__ q, int mf, int nf, int64_t pf,
                        double* __restrict__ qc, double* __restrict__ ec, int64_t pc, int rows, int red)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     const int nc = (nf - 1) / 2 + 1, J0 = 1 + rows * (blockIdx.y * GR_WARPS + (threadIdx.x >> 5));
     gs_restrict_run<HQ>(o, u, q, mf, pf, qc, ec, pc, blockIdx.x, J0, min(J0 + rows, nc - 1), red != 0);
@@ -67,6 +69,7 @@ __global__ void __launch_bounds__(MG_BX* MG_BY)
     prolong_black_kernel(double* __restrict__ u, int mf, int nf, int64_t pf,
                          const double* __restrict__ ec, int64_t pc)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     const int I = blockIdx.x * MG_BX + threadIdx.x;  // coarse column 0 .. mc-2
     const int j = 1 + blockIdx.y * MG_BY + threadIdx.y;
@@ -84,6 +87,7 @@ __global__ void __launch_bounds__(MG_BX* MG_BY)
     prolong_add_kernel(double* __restrict__ u, int mf, int nf, int64_t pf,
                        const double* __restrict__ ec, int64_t pc)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     const int I = blockIdx.x * MG_BX + threadIdx.x;  // coarse column 0 .. mc-2
     const int j = 1 + blockIdx.y * MG_BY + threadIdx.y;
@@ -140,7 +144,7 @@ cudaError_t launch_restrict(const Field& fine_r, double* qc, double* ec, int64_t
 {
     const int mc = (fine_r.m - 1) / 2 + 1, nc = (fine_r.n - 1) / 2 + 1;
     const dim3 grid((mc - 2 + MG_BX - 1) / MG_BX, (nc - 2 + MG_BY - 1) / MG_BY);
-    restrict_kernel<<<grid, dim3(MG_BX, MG_BY), 0, s>>>(fine_r.p, fine_r.m, fine_r.n, fine_r.pitch, qc, ec, pitch_c,
+    launch_after(restrict_kernel, grid, dim3(MG_BX, MG_BY), 0, s, fine_r.p, fine_r.m, fine_r.n, fine_r.pitch, qc, ec, pitch_c,
                                                          red ? 1 : 0, red ? red->inv_d : 0.0,
                                                          red ? red->inv_d_shift : 0);
     note_launch();
@@ -156,9 +160,9 @@ cudaError_t launch_gs_restrict(const Field& f, const double* q, double* qc, doub
     while (rows > 1 && (int64_t)cols * ((nc - 2 + rows - 1) / rows) < 40 * (int64_t)device_sms()) rows /= 2;
     const dim3 grid(cols, (nc - 2 + rows * GR_WARPS - 1) / (rows * GR_WARPS));
     if (q)
-        gs_restrict_kernel<true><<<grid, 32 * GR_WARPS, 0, s>>>(f.p, q, f.m, f.n, f.pitch, qc, ec, pitch_c, rows, red ? 1 : 0);
+        launch_after(gs_restrict_kernel<true>, grid, 32 * GR_WARPS, 0, s, f.p, q, f.m, f.n, f.pitch, qc, ec, pitch_c, rows, red ? 1 : 0);
     else
-        gs_restrict_kernel<false><<<grid, 32 * GR_WARPS, 0, s>>>(f.p, q, f.m, f.n, f.pitch, qc, ec, pitch_c, rows, red ? 1 : 0);
+        launch_after(gs_restrict_kernel<false>, grid, 32 * GR_WARPS, 0, s, f.p, q, f.m, f.n, f.pitch, qc, ec, pitch_c, rows, red ? 1 : 0);
     note_launch();
     return cudaGetLastError();
 }
@@ -167,7 +171,7 @@ cudaError_t launch_prolong_black(const Field& fine_u, const double* ec, int64_t 
 {
     const int mc = (fine_u.m - 1) / 2 + 1;
     const dim3 grid((mc - 1 + MG_BX - 1) / MG_BX, (fine_u.n - 2 + MG_BY - 1) / MG_BY);
-    prolong_black_kernel<<<grid, dim3(MG_BX, MG_BY), 0, s>>>(fine_u.p, fine_u.m, fine_u.n, fine_u.pitch, ec, pitch_c);
+    launch_after(prolong_black_kernel, grid, dim3(MG_BX, MG_BY), 0, s, fine_u.p, fine_u.m, fine_u.n, fine_u.pitch, ec, pitch_c);
     note_launch();
     return cudaGetLastError();
 }
@@ -177,7 +181,7 @@ cudaError_t launch_prolong_add(const Field& fine_u, const double* ec, int64_t pi
 {
     const int mc = (fine_u.m - 1) / 2 + 1;
     const dim3 grid((mc - 1 + MG_BX - 1) / MG_BX, (fine_u.n - 2 + MG_BY - 1) / MG_BY);
-    prolong_add_kernel<<<grid, dim3(MG_BX, MG_BY), 0, s>>>(fine_u.p, fine_u.m, fine_u.n,
+    launch_after(prolong_add_kernel, grid, dim3(MG_BX, MG_BY), 0, s, fine_u.p, fine_u.m, fine_u.n,
                                                             fine_u.pitch, ec, pitch_c);
     note_launch();
     return cudaGetLastError();

@@ -144,6 +144,7 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
                          int64_t pitch32, double* __restrict__ partials,
                          const float* __restrict__ sc, const NormEnd end)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     if (!UNIT) b2 = in_reg(o, b2);
     d = in_reg(o, d);
@@ -192,6 +193,7 @@ constexpr int RUN_BLOCKS_PER_SM = 3;  // 80 registers; with two blocks of 102, 1
 __global__ void __launch_bounds__(NORM_THREADS, RUN_BLOCKS_PER_SM)
     residual32_kernel(const ResidualRuns R, double* __restrict__ partials, const float* __restrict__ sc, const NormEnd end)
 {
+    after_prior();
     const float scale = *sc;
     const int strips = run_strips(R.m), warps = gridDim.x * (NORM_THREADS / 32);
     const int64_t runs = (int64_t)strips * run_blocks(R.n);
@@ -372,14 +374,14 @@ cudaError_t launch_defect64_to32(const Field& psi, const Coef& c, float* r32, fl
         const int grid = (int)std::min<int64_t>((runs + NORM_THREADS / 32 - 1) / (NORM_THREADS / 32),
                                                 std::min(RUN_BLOCKS_PER_SM * device_sms(), NORM_PARTIALS_MAX));
         const bool vec = (psi.pitch & 1) == 0 && ((uintptr_t)psi.p & 15) == 0;
-        residual32_kernel<<<grid, NORM_THREADS, 0, s>>>(
+        launch_after(residual32_kernel, grid, NORM_THREADS, 0, s, 
             ResidualRuns{psi.p, psi.pitch, r32, e32, pitch32, psi.m, psi.n, vec}, partials, norm_scale, end);
         note_launch();
         return cudaGetLastError();
     }
     const int blocks = mixed_norm_blocks(psi.m, psi.n);
 #define LAP_D64(U, F)                                                                            \
-    defect64_to32_kernel<U, F><<<blocks, NORM_THREADS, 0, s>>>(psi.p, psi.m, psi.n, psi.pitch, c.b2, \
+    launch_after(defect64_to32_kernel<U, F>, blocks, NORM_THREADS, 0, s, psi.p, psi.m, psi.n, psi.pitch, c.b2, \
                                                                c.d, r32, e32, pitch32, partials, \
                                                                norm_scale, end)
     if (c.unit_beta) {

@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(RB_BX* RB_BY)
                      double one_minus_w, unsigned long long* __restrict__ maxd,
                      const double* __restrict__ wslot)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     if (!GS && wslot) {  // w and 1 - w from device memory: register operands for the blend
         w = wslot[0];
@@ -98,6 +99,7 @@ __global__ void __launch_bounds__(RD_BX)
                    int64_t pitch, int colour, int starts, double w, double one_minus_w,
                    unsigned long long* __restrict__ maxd, const double* __restrict__ wslot)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     if (!GS && wslot) {
         w = wslot[0];
@@ -188,6 +190,7 @@ __global__ void __launch_bounds__(JA_BX* JA_BY)
                   int64_t pitch, double b2, double inv_d, int shift,
                   unsigned long long* __restrict__ maxd)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     if (!UNIT_BETA) b2 = in_reg(o, b2);
     if (!POW2) inv_d = in_reg(o, inv_d);
@@ -250,6 +253,7 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
                         int64_t pitch, double b2, double d, double* __restrict__ partials,
                         const NormEnd end)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     if (!UNIT_BETA) b2 = in_reg(o, b2);
     d = in_reg(o, d);
@@ -289,6 +293,7 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
     gs_norm_kernel(const double* __restrict__ u, int m, int n, int64_t pitch, double* __restrict__ partials,
                    const NormEnd end)
 {
+    after_prior();
     const FmaOps o = load_fma_ops();
     const double d = in_reg(o, 4.0);
     double acc = 0.0;
@@ -393,7 +398,7 @@ cudaError_t launch_rb_colour(const Field& f, const double* q, const Coef& c, boo
     const double omw = 1.0 - w;
     LAP_DISPATCH_BOOL(c.unit_beta, UB, LAP_DISPATCH_BOOL(c.inv_d_shift > 0, P2,
         LAP_DISPATCH_BOOL(q != nullptr, HQ, LAP_DISPATCH_BOOL(gs, GS, LAP_DISPATCH_BOOL(maxd != nullptr, MD,
-            rb_colour_kernel<UB, P2, HQ, GS, MD><<<grid, block, 0, s>>>(
+            launch_after(rb_colour_kernel<UB, P2, HQ, GS, MD>, grid, block, 0, s, 
                 f.p, q, f.m, f.n, f.pitch, colour, c.b2, c.inv_d, c.inv_d_shift, w, omw, maxd,
                 wslot))))));
     note_launch();
@@ -409,7 +414,7 @@ cudaError_t launch_rb_diag(const Field& f, const double* q, bool gs, double w, i
     const int grid = (int)((walks + RD_BX - 1) / RD_BX);
     const double omw = 1.0 - w;
     LAP_DISPATCH_BOOL(q != nullptr, HQ, LAP_DISPATCH_BOOL(gs, GS, LAP_DISPATCH_BOOL(maxd != nullptr, MD,
-        rb_diag_kernel<HQ, GS, MD><<<grid, RD_BX, 0, s>>>(f.p, q, f.m, f.n, f.pitch, colour, starts,
+        launch_after(rb_diag_kernel<HQ, GS, MD>, grid, RD_BX, 0, s, f.p, q, f.m, f.n, f.pitch, colour, starts,
                                                            w, omw, maxd, wslot))));
     note_launch();
     return cudaGetLastError();
@@ -421,7 +426,7 @@ cudaError_t launch_jacobi(const Field& in, double* out, const Coef& c, unsigned 
     const dim3 grid = point_grid(in.m, in.n), block(JA_BX, JA_BY);
     LAP_DISPATCH_BOOL(c.unit_beta, UB, LAP_DISPATCH_BOOL(c.inv_d_shift > 0, P2,
         LAP_DISPATCH_BOOL(maxd != nullptr, MD,
-            jacobi_kernel<UB, P2, MD><<<grid, block, 0, s>>>(in.p, out, in.m, in.n, in.pitch, c.b2,
+            launch_after(jacobi_kernel<UB, P2, MD>, grid, block, 0, s, in.p, out, in.m, in.n, in.pitch, c.b2,
                                                              c.inv_d, c.inv_d_shift, maxd))));
     note_launch();
     return cudaGetLastError();
@@ -444,7 +449,7 @@ cudaError_t launch_defect_sumsq(const Field& f, const double* q, const Coef& c, 
 {
     const int blocks = norm_blocks(f);
     LAP_DISPATCH_BOOL(c.unit_beta, UB, LAP_DISPATCH_BOOL(q != nullptr, HQ,
-        defect_sumsq_kernel<UB, HQ><<<blocks, NORM_THREADS, 0, s>>>(f.p, q, f.m, f.n, f.pitch, c.b2,
+        launch_after(defect_sumsq_kernel<UB, HQ>, blocks, NORM_THREADS, 0, s, f.p, q, f.m, f.n, f.pitch, c.b2,
                                                                     c.d, partials, end)));
     note_launch();
     return cudaGetLastError();
@@ -453,7 +458,7 @@ cudaError_t launch_defect_sumsq(const Field& f, const double* q, const Coef& c, 
 cudaError_t launch_gs_norm(const Field& f, double* partials, cudaStream_t s, const NormEnd& end)
 {
     const int blocks = norm_blocks_for((f.m - 1) / 2 + 2, f.n);
-    gs_norm_kernel<<<blocks, NORM_THREADS, 0, s>>>(f.p, f.m, f.n, f.pitch, partials, end);
+    launch_after(gs_norm_kernel, blocks, NORM_THREADS, 0, s, f.p, f.m, f.n, f.pitch, partials, end);
     note_launch();
     return cudaGetLastError();
 }

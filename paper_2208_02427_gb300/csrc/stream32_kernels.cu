@@ -507,6 +507,7 @@ __global__ void __launch_bounds__(32 * ST_WARPS, down_ctas(NU, GS))
                        const BatchLevel<float>* __restrict__ lv, const int* __restrict__ active, float w,
                        float omw, int zero_c)
 {
+    after_prior();
     extern __shared__ float4 smem4[];
     const int wid = threadIdx.x >> 5;
     float* smem = reinterpret_cast<float*>(smem4) + wid * down_ring(NU);
@@ -525,6 +526,7 @@ __global__ void __launch_bounds__(32 * ST_WARPS, up_ctas(NU, GS, PSI))
                      const BatchLevel<float>* __restrict__ lv, const int* __restrict__ active, float w,
                      float omw, double* psi, int64_t psi_pitch, const BatchLevel<double>* __restrict__ lv64)
 {
+    after_prior();
     extern __shared__ float4 smem4[];
     const int wid = threadIdx.x >> 5;
     float* smem = reinterpret_cast<float*>(smem4) + wid * up_ring(NU, PSI);
@@ -585,8 +587,7 @@ template <int NU, bool GS>
 cudaError_t down_launch(const StreamItem* items, int count, const StreamCut& cut, const BatchLevel<float>* lv,
                         const int* active, float w, float omw, bool zero_c, cudaStream_t s)
 {
-    stream_down_kernel<NU, GS><<<(count + ST_WARPS - 1) / ST_WARPS, 32 * ST_WARPS,
-                                 ST_WARPS * down_ring(NU) * sizeof(float), s>>>(items, count, cut, lv, active, w,
+    launch_after(stream_down_kernel<NU, GS>, (count + ST_WARPS - 1) / ST_WARPS, 32 * ST_WARPS, ST_WARPS * down_ring(NU) * sizeof(float), s, items, count, cut, lv, active, w,
                                                                                 omw, zero_c ? 1 : 0);
     note_launch();
     return cudaGetLastError();
@@ -606,7 +607,7 @@ cudaError_t up_launch(const StreamItem* items, int count, const StreamCut& cut, 
         if (e != cudaSuccess) return e;
         attr_record(set, dev, smem);
     }
-    kern<<<(count + ST_WARPS - 1) / ST_WARPS, 32 * ST_WARPS, smem, s>>>(items, count, cut, lv, active, w, omw, psi,
+    launch_after(kern, (count + ST_WARPS - 1) / ST_WARPS, 32 * ST_WARPS, smem, s, items, count, cut, lv, active, w, omw, psi,
                                                                          psi_pitch, lv64);
     note_launch();
     return cudaGetLastError();

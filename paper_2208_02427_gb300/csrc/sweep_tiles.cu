@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(ST_THREADS)
     sweep_tiles_kernel(const double* __restrict__ in, double* __restrict__ out, int m, int n, int64_t pitch,
                        int passes, SweepCoef k, const double* __restrict__ wslot)
 {
+    after_prior();
     extern __shared__ double sm[];
     const FmaOps o = load_fma_ops();
     if (KIND == SWEEP_SOR) {
@@ -158,6 +159,7 @@ __global__ void __launch_bounds__(ST_THREADS)
 __global__ void __launch_bounds__(ST_THREADS, 3)
     b_sweep_tiles_kernel(const SweepTileItem* __restrict__ items, const int* __restrict__ active, int k, int launches)
 {
+    after_prior();
     extern __shared__ double sm[];
     const FmaOps o = load_fma_ops();
     const SweepTileItem it = items[blockIdx.x];
@@ -254,7 +256,7 @@ cudaError_t launch_sweep_tiles(const Field& in, double* out, const Coef& c, cons
     const size_t bytes = (size_t)(tw + 2 * h) * (th + 2 * h) * 8 * (kind == SWEEP_JACOBI ? 2 : 1);
     const SweepCoef k{c.b2, c.inv_d, c.inv_d_shift, 1.0, 0.0};
     const cudaError_t e = on_sweep_kernel(c, kind, diag, [&](auto* kernel) {
-        kernel<<<dim3(t.tx, t.ty), ST_THREADS, bytes, s>>>(in.p, out, in.m, in.n, in.pitch, h, k, wslot);
+        launch_after(kernel, dim3(t.tx, t.ty), ST_THREADS, bytes, s, in.p, out, in.m, in.n, in.pitch, h, k, wslot);
         return cudaGetLastError();
     });
     note_launch();
@@ -334,7 +336,7 @@ cudaError_t launch_b_sweep_tiles(const SweepTileItem* items, int count, const Ba
                                                    (int)ST_SMEM_MAX);
         if (e != cudaSuccess) return e;
     }
-    b_sweep_tiles_kernel<<<count, ST_THREADS, bytes, s>>>(items, active, k, launches);
+    launch_after(b_sweep_tiles_kernel, count, ST_THREADS, bytes, s, items, active, k, launches);
     note_launch();
     return cudaGetLastError();
 }

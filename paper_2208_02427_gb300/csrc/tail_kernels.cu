@@ -542,6 +542,7 @@ __global__ void __launch_bounds__(SMEM_TAIL_THREADS, 1)
                      const int* __restrict__ active, int nu1, int nu2, int gs, T w_arg, T omw_arg, int per_level_w,
                      int nc, int ncl)
 {
+    after_prior();
     if (CL) {
         tail_dispatch<T, true>(jobs[0], lv, nu1, nu2, gs != 0, w_arg, omw_arg, nc, ncl);
         return;
@@ -677,12 +678,14 @@ cudaError_t launch_smem_tail(const TailJob* jobs, int count, const BatchLevel<T>
         cfg.blockDim = SMEM_TAIL_THREADS;
         cfg.dynamicSmemBytes = plan.bytes;
         cfg.stream = s;
-        cudaLaunchAttribute at;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = plan.nc;
-        at.val.clusterDim.y = at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
+        cudaLaunchAttribute at[2];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = plan.nc;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_after
+        at[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 2;
         e = cudaLaunchKernelEx(&cfg, smem_tail_kernel<T, true>, jobs, count, (unsigned*)nullptr, lv, active, nu1, nu2,
                                g, wt, omw, pl, plan.nc, plan.ncl);
         note_launch();
@@ -692,7 +695,7 @@ cudaError_t launch_smem_tail(const TailJob* jobs, int count, const BatchLevel<T>
     if (e != cudaSuccess) return e;
     const int grid = batch_grid((const void*)smem_tail_kernel<T, false>, SMEM_TAIL_THREADS, plan.bytes, count,
                                 claim != nullptr);
-    smem_tail_kernel<T, false><<<grid, SMEM_TAIL_THREADS, plan.bytes, s>>>(jobs, count, claim, lv, active, nu1, nu2, g,
+    launch_after(smem_tail_kernel<T, false>, grid, SMEM_TAIL_THREADS, plan.bytes, s, jobs, count, claim, lv, active, nu1, nu2, g,
                                                                            wt, omw, pl, 1, 0);
     note_launch();
     return cudaGetLastError();
