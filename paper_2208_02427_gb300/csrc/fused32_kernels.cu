@@ -421,11 +421,11 @@ __device__ __forceinline__ void up_tile(const BatchLevel<float>& F, const BatchL
         store_owned<NT>(F.u, F.pitch, su, R, x0, x1, y0, y1);
         return;
     }
-    // column pairs (gx even: 16-byte aligned double2 when the pitch is even), two per lane,
-    // so that each thread has four FP64 loads in flight per row
+    // column pairs (gx even: 16-byte aligned double2 when the pitch is even and the field starts on
+    // one), two per lane, so that each thread has four FP64 loads in flight per row
     const FmaOps o = load_fma_ops();
     const int p_lo = (x0 - R.gx0) >> 1, p_hi = (x1 - 1 - R.gx0) >> 1;
-    const bool even_pitch = (psi_pitch & 1) == 0;
+    const bool pairs = (psi_pitch & 1) == 0 && (reinterpret_cast<uintptr_t>(psi) & 15) == 0;
     for (int gy = y0 + wid; gy < y1; gy += NW) {
         const float* row = su + (gy - R.gy0) * FT_RS;
         double* prow = psi + (int64_t)gy * psi_pitch;
@@ -437,7 +437,7 @@ __device__ __forceinline__ void up_tile(const BatchLevel<float>& F, const BatchL
             const int gx = R.gx0 + 2 * p;
             lo[s2] = p <= p_hi && gx >= x0;
             hi[s2] = p <= p_hi && gx + 1 < x1;
-            if (lo[s2] && hi[s2] && even_pitch) {
+            if (lo[s2] && hi[s2] && pairs) {
                 v[s2] = *reinterpret_cast<const double2*>(prow + gx);
             } else {
                 v[s2].x = lo[s2] ? prow[gx] : 0.0;
@@ -451,7 +451,7 @@ __device__ __forceinline__ void up_tile(const BatchLevel<float>& F, const BatchL
             if (!lo[s2] && !hi[s2]) continue;
             const double a = fadd(o, v[s2].x, to_double_exact(row[p]));
             const double b = fadd(o, v[s2].y, to_double_exact(row[FT_HS + p]));
-            if (lo[s2] && hi[s2] && even_pitch) {
+            if (lo[s2] && hi[s2] && pairs) {
                 *reinterpret_cast<double2*>(prow + gx) = make_double2(a, b);
             } else {
                 if (lo[s2]) prow[gx] = a;

@@ -72,3 +72,24 @@ def test_batched_streams(b, inner):
         for k in range(len(inputs)):
             assert np.array_equal(got[0][k], out[0][0][k]), SHAPES[k]
     lap.close()
+
+
+@pytest.mark.parametrize("tiling", [1, 2, 3])
+@pytest.mark.parametrize("offset,extra", [(1, 4), (1, 3), (2, 4)])
+def test_tiles_update_fields_off_16_byte_boundaries(b, tiling, offset, extra):
+    """The tiled level-0 ascent writes psi in pairs of columns: a field that starts 8 bytes past a 16-byte
+    boundary, with an even pitch and an odd one, gives what one kernel per pass gives."""
+    m, n = 193, 129
+    psi = wl.random_ring(m, n, 8)
+    lap = b.Laplace()
+    outs = []
+    for t in (tiling, -1):
+        pitch = m + extra + (m + extra) % 2 - (extra % 2)
+        buf = torch.zeros(n, pitch, dtype=torch.float64, device="cuda")
+        f = buf[:, offset:offset + m]
+        f.copy_(torch.as_tensor(psi))
+        r = lap.solve(f, method="mg_mixed", tol=1e-10, tiling=t, tail_size=-1)
+        outs.append((f.cpu().numpy(), r["iters"], r["status"]))
+    lap.close()
+    assert outs[0][1:] == outs[1][1:] and outs[0][2] == "converged"
+    assert np.array_equal(outs[0][0], outs[1][0])
