@@ -664,8 +664,7 @@ def main():
                "shapes": "m, n in {33, 65, 129, 257, 513}, aspect <= 4, ring U[0,1], interior 0"}
 
         def time_batch(method, warm, reps, **extra):
-            # warm-ups: the plan, the candidates' graphs and the choice by timing (each call's
-            # cycles with every problem running time one candidate configuration)
+            # warm-ups: the plan and the loop's graph
             times, res = [], None
             for rep in range(warm + reps):
                 for f, g in zip(work, pristine):
@@ -687,15 +686,15 @@ def main():
             out[name] = {"ms": ms, "solves_per_s": count / (ms / 1e3),
                          "max_cycles": max(r["iters"] for r in res),
                          "configuration": lap.last_batch_config()}
-        # the FP32 tilings one by one (tail and item size still chosen by timing): what the
-        # choice between them is worth
+        # the FP32 tilings one by one (tail and item size as the batch's size gives them): what
+        # the choice between them is worth
         out["mixed_by_tiling"] = {}
         for tiling, label in ((1, "tiles_512x128x64"), (2, "tiles_1024x128x64"),
                               (3, "tiles_512x128x32"), (-1, "one_kernel_per_pass")):
             ms, _ = time_batch("mg_mixed", 6, 3, tiling=tiling)
             out["mixed_by_tiling"][label] = {"ms": ms, "configuration": lap.last_batch_config()}
         # one CTA per work item against persistent launches (resident CTAs looping over the
-        # items), the other knobs still chosen by timing
+        # items)
         out["by_launch"] = {}
         for name, method in (("fp64", "mg"), ("mixed", "mg_mixed")):
             for persistent, label in ((-1, "one_cta_per_item"), (1, "persistent")):

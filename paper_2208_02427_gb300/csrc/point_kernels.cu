@@ -82,12 +82,13 @@ __global__ void __launch_bounds__(RB_BX* RB_BY)
 // Strip s of rows j0 = 1 + s RD_K .. j0 + RD_K - 1: walk x of the strip starts on row j0 at
 // column lo + 2x, lo the first column >= 2 - RD_K of the colour, and visits (lo + 2x + k,
 // j0 + k). Thread g of the launch takes walk g % starts of strip g / starts (no CTA is left
-// nearly empty at the end of a strip). Walks of RD_K = 6 points: measured per colour pass inside the solve's graphs at 4097^2, (walk, CTA) =
+// nearly empty at the end of a strip). Walks of RD_K = 6 points: measured per colour pass inside the
+// solve's graphs at 4097^2, (walk, CTA) =
 // (4, 128) 63.2 us, (6, 128) 62.9, (8, 128) 64.7, (8, 256) 68.3, (16, 128) 66.0 with the
 // loads one point ahead and 73.4 for walks of 32 (a longer walk adds registers, a shorter one
 // pair adds), against 71.0 us for the paper-order kernel. Since the edge walks below are as quick as the
-// others: CTAs of 64 threads 61.0 us, 128 61.1, walks of 8 61.8, of 5 61.8; at 1000^2 5.7, 5.9, 6.2, 6.0. Within a walk, taking every pair sum
-// first or every (1 - w) C product first gave 63.1 and 62.9 us against 62.7 for the order
+// others: CTAs of 64 threads 61.0 us, 128 61.1, walks of 8 61.8, of 5 61.8; at 1000^2 5.7, 5.9, 6.2, 6.0.
+// Within a walk, taking every pair sum first or every (1 - w) C product first gave 63.1 and 62.9 us against 62.7 for the order
 // below (a pair, then its point).
 // A warp with a walk that leaves the interior takes its points by predicate, their loads in flight together as
 // well: a loop over them, a load's latency a point, kept the last strip's CTAs of every pass running for
