@@ -96,7 +96,7 @@ __device__ __forceinline__ void line_recurrences(const FmaOps& o, const LineTabl
         const double* __restrict__ te = t.e;
         if (act) {
             // operands of a step are loaded in the step before, ahead of its store, which waits for the
-            // fma (half sweeps at 3001 x 2050 113 -> 102 us)
+            // fma (a half sweep at 3001 x 2050 105 -> 93 us)
             const int kb = min(len, K0);
             G = y[0];
             D = fmul(o, __ldg(gl), G);
@@ -324,8 +324,8 @@ __global__ void __launch_bounds__(LX_THREADS, 6)
 // pitch, sx = 1: neighbouring lines share the sectors of a row). With two warps' lines and chunks in CTAs of
 // their own the separators took a launch between forward and back, three launches a colour; one
 // launch gives every multiprocessor the same number of lines and no waits between them. Half sweeps, three
-// launches a colour / one: 300^2 27 / 14 us, 1000^2 41 / 28, 3001 x 2050 84 / 75, 2050 x 3001 102 / 86, 500 x
-// 4000 99 / 72, 4097^2 195 / 203.
+// launches a colour / one: 300^2 27 / 14 us, 1000^2 41 / 28, 2050 x 3001 102 / 86, 500 x 4000 99 / 72, 4097^2
+// 195 / 203 (ADI less SLOR iterations), 3001 x 2050 92 / 77 (launch times).
 // What bounds it is the recurrence: a dependent fma takes 71 clocks, one warp on each scheduler nearly
 // fills the FP64 pipe, and everything else has to be out of the way: a step's field values and table
 // entries are loaded PIPE positions ahead, into registers (a table entry loaded in its step waited for the
