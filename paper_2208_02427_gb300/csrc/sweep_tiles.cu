@@ -1,13 +1,13 @@
 // sweep_tiles.cu -- several point sweeps in one launch, on tiles in shared memory.
 //
 // A small grid is bound by launches, not by its sweeps: a colour pass over 513 x 385 points is 0.8 us of
-// FP64 arithmetic in a launch of 2.3 us. Here a CTA loads its tile with a halo of one
+// FP64 arithmetic in a launch of 2.0 us. Here a CTA loads its tile with a halo of one
 // point per pass, runs the passes of `sweeps` sweeps in shared memory with a CTA barrier between them,
 // and writes its own points to the other buffer. Each pass covers one halo point less than the one
 // before, so every value is the one that the passes over the whole grid would have left: the same
 // expression of the same operands, bit for bit. The halo costs arithmetic (a 37 x 39 tile does 1.3 times its
 // own points over three red-black sweeps), so the number of sweeps and the tile follow from the grid
-// (plan_sweep_tiles). What is left beside the FP64 work: a launch and the window's load and store, 1.7 us
+// (plan_sweep_tiles). What is left beside the FP64 work: a launch and the window's load and store, 1.4 us
 // or more, and about 0.4 us a pass (a point's chain of FP64 operations of 71 cycles each, the barrier, the
 // warps' uneven last round).
 #include <algorithm>
@@ -26,8 +26,8 @@ constexpr size_t ST_SMEM_MAX = 224 * 1024;
 // The cost model of plan_sweep_tiles, in SM cycles beside the FP64 work: a one-pass launch (the walks along
 // diagonals take longer to drain), a tile launch, a window point's load and store, and a pass's latency,
 // barrier and uneven last round. Fitted to times per sweep from 65^2 to 4097^2 points.
-constexpr double PASS_CYCLES = 2900, DIAG_PASS_CYCLES = 5000;
-constexpr double TILE_CYCLES = 3500, TILE_POINT_CYCLES = 0.4, TILE_PASS_CYCLES = 900;
+constexpr double PASS_CYCLES = 2600, DIAG_PASS_CYCLES = 3600;
+constexpr double TILE_CYCLES = 2900, TILE_POINT_CYCLES = 0.4, TILE_PASS_CYCLES = 900;
 
 __device__ __forceinline__ void copy8(double* smem, const double* global)
 {
@@ -206,11 +206,12 @@ int halo(int kind, int sweeps) { return kind == SWEEP_JACOBI ? sweeps : 2 * swee
 }  // namespace
 
 // At most one tile per multiprocessor, nearly square, and as many sweeps per launch as cost least; none
-// where the one-pass kernels are within 5%. Measured per sweep (one pass per launch / tiles), SOR in the
-// paper's order: 65^2 3.06 / 1.8 us, 257^2 3.44 / 2.5, 513 x 385 4.8 / 4.0, 700^2 7.4 / 6.8, 1000^2 equal;
-// paired along diagonals 5.4 / 1.8, 5.9 / 2.5, 6.2 / 4.0, 8.4 / 6.8, equal; Jacobi 1.60 / 1.02, 1.91 / 1.57,
-// from 513 x 385 on equal. Two or three smaller tiles per multiprocessor hide a tile's load but have more
-// halo: equal or slower.
+// where the one-pass kernels are within 2%. Measured per sweep (one pass per launch / tiles), SOR in the
+// paper's order: 129^2 2.66 / 1.79 us, 257^2 2.98 / 2.40, 513 x 385 4.02 / 3.87, 700^2 6.92 / 6.64, 850^2
+// 8.93 / 9.07, 1000^2 11.1 / 11.7; paired along diagonals 5.20 / 1.78, 5.33 / 2.38, 5.68 / 3.88, 7.40 / 6.64, 9.01 /
+// 9.06, 10.8 / 11.7; Gauss-Seidel 700^2 5.02 / 4.84, 850^2 6.25 / 6.40; Jacobi 129^2 1.42 / 0.96, 257^2 1.64 / 1.38,
+// 513 x 385 2.26 / 2.22, 850^2 5.07 / 5.25. Two or three smaller tiles per multiprocessor hide a tile's load but
+// have more halo: equal or slower.
 SweepTiles plan_sweep_tiles(int m, int n, const Coef& c, int kind, bool diag, int sms)
 {
     SweepTiles best;
@@ -219,7 +220,7 @@ SweepTiles plan_sweep_tiles(int m, int n, const Coef& c, int kind, bool diag, in
     // per sweep; an FP64 operation takes half a cycle of an SM
     double least = colours * (diag ? DIAG_PASS_CYCLES : PASS_CYCLES) +
                    1.07 * (m - 2) * (double)(n - 2) * (ops - (diag ? 1 : 0)) / 2 / sms;
-    least *= 0.95;
+    least *= 0.98;
     const int near = (int)std::min(std::sqrt((double)sms * (m - 2) / (n - 2)), (double)sms);
     for (int sweeps = 1; sweeps <= 8; ++sweeps) {
         const int h = halo(kind, sweeps);
