@@ -244,7 +244,10 @@ BatchKey make_key(int count, const lap_grid* grids, double* const* psi_devs, con
 // batch is below about 10M points (whole solves without / with it: 24 grids up to 129^2 1650 / 1400 us, 256 up
 // to 257^2 3680 / 3500, 64 up to 513^2 3420 / 3440); above, and for the row streams of the mixed solver, whose
 // small levels are two launches each, it gains nothing (1024 grids up to 513^2: 22.6 / 23.1 ms, mixed 8.0 /
-// 8.6 ms). FP32 levels: row streams where they cover the smoothing counts, else the first tile variant. Work items: about 16 per
+// 8.6 ms). FP32 levels as tiles or one kernel per pass: up to 129 points in a large batch (none / 65 / 129 on 4096
+// grids 44.0 / 44.4 / 41.1 ms for tile variant 1, 58.2 / 58.6 / 55.3 per pass; 1024 grids 12.4 / 12.6 / 12.4, 16.7 / 16.5 /
+// 16.2), in a small one none with tiles (64 grids 1.82 / 2.10 / 2.79) and 65 without (2.88 / 2.60 / 3.12). FP32 levels: row
+// streams where they cover the smoothing counts, else the first tile variant. Work items: about 16 per
 // multiprocessor, so that the last wave is a small part of a pass, between 1024 points (below, a CTA's
 // start outweighs its work) and 4096 (above, nothing is gained). One CTA per item: the block
 // scheduler hands out uniform items as well as a claim counter does.
@@ -252,12 +255,16 @@ BatchConfig batch_config(const lap_params* p, int64_t points)
 {
     BatchConfig c;
     const int64_t per = points / (16 * (int64_t)device_sms());
-    c.tail = p->tail_size != 0 ? p->tail_size : p->method == LAP_MG && per < 4096 ? 33 : -1;
     c.tiles = 0;
     if (p->method == LAP_MG_MIXED && !p->unfused && p->tiling >= 0 && fused32_supported(p->nu1, p->nu2)) {
         if (p->tiling == 0 && stream32_supported(p->nu1, p->nu2)) c.tiles = FUSED32_STREAMS;
         else c.tiles = fused32_variant_supported(std::max(1, p->tiling), p->nu1, p->nu2) ? std::max(1, p->tiling) : 0;
     }
+    const bool small = per < 4096;
+    if (p->tail_size != 0) c.tail = p->tail_size;
+    else if (p->method == LAP_MG) c.tail = small ? 33 : -1;
+    else if (c.tiles == FUSED32_STREAMS) c.tail = -1;
+    else c.tail = !small ? 129 : c.tiles ? -1 : 65;
     c.item = p->item_points > 0 ? p->item_points : (int)std::min<int64_t>(4096, std::max<int64_t>(1024, per));
     c.persist = p->persistent > 0 ? 1 : 0;
     return c;
