@@ -129,8 +129,14 @@ void srv_levels(lap_server S, SrvRequest& r, C& cv)
 constexpr int SERVER_TAIL_FP64 = 33;
 constexpr int SERVER_TAIL_FP32 = 129;
 
-// Points of a colour per work item of a step's SOR passes (of fields without a second buffer), for `points` of them in all: SWEEP_STEP, or as many
-// steps as leave about 48 items per multiprocessor (more would only cost memory).
+// A step's SOR fields go on tiles up to this many points in all. Per colour pass, pass by pass / tiles: 4.2
+// million points 24.2 / 22.9 us, 15.8 million (60 fields of 513^2) 81.8 / 87.6, 16.8 million 87 / 91, 67 million
+// 332 / 352 (the passes cost their first and last waves once a launch, the tiles their halos at any size).
+constexpr int64_t SERVER_TILE_POINTS = 8000000;
+
+// Points of a colour per work item of a step's SOR passes (of fields not on tiles), for `points` of them in
+// all: SWEEP_STEP, or as many steps as leave about 48 items per multiprocessor (24: 340 against 333 us a
+// pass at 67 million points; 96: equal, for more memory).
 // No effect on the values.
 int sor_item_points(int64_t points)
 {
@@ -155,7 +161,7 @@ struct SrvPlan {
     std::vector<TileItem> tiles;
     std::vector<StreamItem> streams;
     LevelLists mg64, mg32;
-    std::vector<SweepItem> sweeps;  // SOR pass by pass, for the fields without a second buffer
+    std::vector<SweepItem> sweeps;  // SOR pass by pass, for the fields not on tiles
     std::vector<SweepTileItem> tiled;
     BatchSweepPlan tile_plan;
     int tile_launches = 0;
@@ -371,7 +377,11 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
                 if (run[q]->method == LAP_SOR_RB) sor_q.push_back(q);
             std::stable_sort(sor_q.begin(), sor_q.end(),
                              [&](int a, int c) { return sweeps_now(a) > sweeps_now(c); });
-            // a second buffer for a field from the pool's free space, until the step's end
+            // a second buffer for a field from the pool's free space, until the step's end; none for a
+            // set that fills the device pass by pass
+            int64_t sor_total = 0;
+            for (int q : sor_q) sor_total += (int64_t)(run[q]->g.m - 2) * (run[q]->g.n - 2);
+            const bool tiles = S->sor_sweeps >= 2 && sor_total <= SERVER_TILE_POINTS;
             std::vector<std::pair<int, int>> shapes;
             std::vector<SweepTileItem> tiled;
             std::vector<int> rest;
@@ -380,7 +390,7 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
                 const int64_t pitch = round_up(L.m, 32);
                 const size_t bytes = (size_t)(pitch * L.n) * sizeof(double);
                 size_t off = 0;
-                if (S->sor_sweeps < 2 || !pool_alloc(S, bytes, &off)) {
+                if (!tiles || !pool_alloc(S, bytes, &off)) {
                     rest.push_back(q);
                     continue;
                 }

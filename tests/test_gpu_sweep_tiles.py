@@ -93,3 +93,25 @@ def test_server_sweeps_equal_single_solves(b, sweeps, room):
     for f, i, (psi, iters, status) in zip(fields, ids, want):
         assert np.array_equal(f.cpu().numpy(), psi)
         assert (res[i]["iters"], res[i]["status"]) == (iters, status)
+
+
+def test_large_sets_go_pass_by_pass(b):
+    """Past the line where the server's sweeps leave the tiles: three fields of over 8 million points in all,
+    then two of them alone once the third is done."""
+    shapes, caps = [(2049, 2049), (1025, 2049), (2049, 1025)], [4, 9, 9]
+    lap = b.Laplace()
+    srv = b.Server(lap, hbm_budget=256 << 20, max_running=3, sor_sweeps=4)
+    fields, ids, want = [], [], []
+    for k, ((m, n), cap) in enumerate(zip(shapes, caps)):
+        psi = wl.random_ring(m, n, 50 + k)
+        t = b.to_field(psi)
+        r = lap.solve(t, method="sor", w=1.9, tol=1e-13, check_every=4, max_iter=cap)
+        want.append((t.cpu().numpy(), r["iters"], r["status"]))
+        fields.append(b.to_field(psi))
+        ids.append(srv.submit(fields[-1], method="sor", w=1.9, tol=1e-13, max_iter=cap))
+    while sum(srv.step()):
+        pass
+    res = dict(srv.drain())
+    for f, i, (psi, iters, status) in zip(fields, ids, want):
+        assert np.array_equal(f.cpu().numpy(), psi)
+        assert (res[i]["iters"], res[i]["status"]) == (iters, status)
