@@ -51,16 +51,20 @@ __device__ __forceinline__ double swept(const FmaOps& o, const double* c, int W,
     return KIND == SWEEP_SOR ? __fma_rn(k.w, g, fmul(o, k.omw, *c)) : g;
 }
 
+// Points that a tile's window reaches past its own in a launch of `passes` passes. No pass is a copy: the ring
+// beside the tile all the same.
+__host__ __device__ constexpr int window_halo(int passes) { return passes > 1 ? passes : 1; }
+
 // The tile of interior columns [x0, x1) and rows [y0, y1) through `passes` passes (two colours a sweep, or
 // one for Jacobi), in -> out. The ring points beside the tile are copied along, so that `out` needs no
-// preparation. sm: (x1 - x0 + 2 passes) (y1 - y0 + 2 passes) doubles, twice that for Jacobi.
+// preparation. sm: (x1 - x0 + 2 h) (y1 - y0 + 2 h) doubles, h = window_halo(passes), twice that for Jacobi.
 template <int KIND, bool UNIT, bool POW2, bool DIAG>
 __device__ __forceinline__ void sweep_tile(const FmaOps& o, const double* __restrict__ in, double* __restrict__ out,
                                            int m, int n, int64_t pitch, int64_t pitch_out, int x0, int x1, int y0,
                                            int y1, int passes, const SweepCoef& k, double* sm)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int h = max(1, passes);  // no pass, a copy: the ring beside the tile all the same
+    const int h = window_halo(passes);
     const int X0 = max(0, x0 - h), X1 = min(m, x1 + h);
     const int Y0 = max(0, y0 - h), Y1 = min(n, y1 + h);
     const int W = X1 - X0, H = Y1 - Y0;
@@ -252,12 +256,12 @@ cudaError_t prepare_sweep_tiles(const Coef& c, int kind, bool diag)
 cudaError_t launch_sweep_tiles(const Field& in, double* out, const Coef& c, const SweepTiles& t, int kind, bool diag,
                                int sweeps, const double* wslot, cudaStream_t s)
 {
-    const int h = halo(kind, sweeps);
+    const int passes = halo(kind, sweeps), h = window_halo(passes);
     const int tw = (in.m - 2 + t.tx - 1) / t.tx, th = (in.n - 2 + t.ty - 1) / t.ty;
     const size_t bytes = (size_t)(tw + 2 * h) * (th + 2 * h) * 8 * (kind == SWEEP_JACOBI ? 2 : 1);
     const SweepCoef k{c.b2, c.inv_d, c.inv_d_shift, 1.0, 0.0};
     const cudaError_t e = on_sweep_kernel(c, kind, diag, [&](auto* kernel) {
-        launch_after(kernel, dim3(t.tx, t.ty), ST_THREADS, bytes, s, in.p, out, in.m, in.n, in.pitch, h, k, wslot);
+        launch_after(kernel, dim3(t.tx, t.ty), ST_THREADS, bytes, s, in.p, out, in.m, in.n, in.pitch, passes, k, wslot);
         return cudaGetLastError();
     });
     note_launch();
