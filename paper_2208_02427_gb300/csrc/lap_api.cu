@@ -1373,8 +1373,10 @@ struct Solver {
                 ck(cudaGraphAddNode(&node, g, first ? &head : nullptr, nullptr, first ? 1 : 0, np),
                    "conditional node");
                 captured(np->conditional.phGraph_out[0], [&] {
+                    // one stopping test a period: on the largest change it is loop_decide's, and the mixed
+                    // iteration's closing residual only sums
                     end.scale = scaled ? w.nscale : nullptr;
-                    period(steps, maxdelta, fused_maxd, end);
+                    period(steps, maxdelta, fused_maxd, maxdelta ? sum_only() : end);
                     if (maxdelta) {
                         if (!fused_maxd) ck(launch_maxdelta(f, w.aux, w.maxd, s), "max delta kernel");
                         ck(launch_loop_decide(w.loop, w.maxd, hnd, s), "loop test kernel");
