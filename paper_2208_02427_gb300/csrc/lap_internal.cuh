@@ -28,6 +28,10 @@ inline void attr_record(std::atomic<size_t>* table, int d, size_t v)
     while (cur < v && !table[d].compare_exchange_weak(cur, v)) {}
 }
 
+// Dynamic shared memory that a launch may have unasked: the 48 KB hold a kernel's static arrays too (1184 bytes in
+// the one-CTA solves, which have the most of those that go by this line).
+constexpr size_t SMEM_UNASKED = 48 * 1024 - 2048;
+
 // Coefficients of the 5-point equation (E+W) + b2 (N+S) - d psi (+ q) = 0, Eq. 5.
 struct Coef {
     double b2;      // beta^2, beta = dx/dy

@@ -146,7 +146,7 @@ static std::atomic<size_t> g_lex_smem_set[ATTR_DEVICES];
 cudaError_t prepare_lex_kernels(size_t smem)
 {
     const int dev = attr_slot();
-    if (smem <= 48 * 1024 || (dev >= 0 && smem <= g_lex_smem_set[dev].load()))
+    if (smem <= SMEM_UNASKED || (dev >= 0 && smem <= g_lex_smem_set[dev].load()))
         return cudaSuccess;
     const int v = (int)smem;
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;

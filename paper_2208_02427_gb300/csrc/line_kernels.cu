@@ -534,14 +534,14 @@ __global__ void __launch_bounds__(LY_THREADS)
 size_t line_smem_bytes(const LineTables& t) { return sizeof(double) * (size_t)t.P * t.stride; }
 
 // Raise the dynamic shared-memory limit of the x-line kernels to `smem` on the current device
-// (done outside stream capture; later launches only repeat it when a longer line comes). The 48 KB that need
-// no call hold the kernels' static arrays too: lines of 5952 .. 6079 unknowns pass them by those.
+// (done outside stream capture; later launches only repeat it when a longer line comes). Lines of 5952 .. 6079
+// unknowns pass 48 KB by the kernels' static arrays.
 static std::atomic<size_t> g_line_smem_set[ATTR_DEVICES];
 
 cudaError_t prepare_line_kernels(size_t smem)
 {
     const int dev = attr_slot();
-    if (smem + 1024 <= 48 * 1024 || (dev >= 0 && smem <= g_line_smem_set[dev].load()))
+    if (smem <= SMEM_UNASKED || (dev >= 0 && smem <= g_line_smem_set[dev].load()))
         return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(line_x_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);

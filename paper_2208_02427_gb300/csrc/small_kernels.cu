@@ -485,7 +485,7 @@ template <class F>
 cudaError_t raise_smem(F* f, std::atomic<size_t>* set, size_t smem)
 {
     const int dev = attr_slot();
-    if (smem <= 48 * 1024 || (dev >= 0 && smem <= set[dev].load())) return cudaSuccess;
+    if (smem <= SMEM_UNASKED || (dev >= 0 && smem <= set[dev].load())) return cudaSuccess;
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) attr_record(set, dev, smem);
     return e;
