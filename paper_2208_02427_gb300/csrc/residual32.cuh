@@ -73,7 +73,12 @@ __device__ __forceinline__ Fixed to_fixed(double x, int E)
 __device__ __forceinline__ float from_fixed(const Fixed& w, const Fixed& e, const Fixed& s, const Fixed& n, const Fixed& c,
                                             float scale)
 {
-    const int vh = w.h + e.h + n.h + (s.h - 4 * c.h), vl = w.l + e.l + n.l + (s.l - 4 * c.l);
+    int vh = w.h + e.h + n.h + (s.h - 4 * c.h), vl = w.l + e.l + n.l + (s.l - 4 * c.l);
+    // balanced, |vl| <= 2^27: parts that nearly cancel (vl up to 2^31, rounded to FP32) would lose a sum of up to
+    // 64 units in its estimate, and with it the whole residual of a field close to its solution
+    const int carry = (vl + (1 << 27)) >> 28;
+    vh += carry;
+    vl -= carry * (1 << 28);
     const long long v = (long long)vh * (1 << 28) + vl;
     // |v| < 2^(k + 2), k the exponent of its FP32 estimate: shifted by 61 - k it fills 29 bits or more of the
     // upper word, and what is below only has to break ties
