@@ -22,7 +22,8 @@
  *    whatever CUDA reported; the handle stays valid for lap_destroy.
  *  - A lap_handle is not thread-safe: use one handle per host thread.
  *
- * Arithmetic: FP64 throughout. Jacobi, Gauss-Seidel, SOR, the multigrid smoother,
+ * Arithmetic: FP64 throughout, but for the FP32 cycles of LAP_MG_MIXED and LAP_MG_FP32
+ * and the exact residual sums of the former. Jacobi, Gauss-Seidel, SOR, the multigrid smoother,
  * residual, restriction and interpolation evaluate exactly the expressions written in
  * each entry's comment, with every multiply-add fused where the comment says fma and
  * nowhere else, so their results do not depend on the launch configuration. lap_solve's
@@ -59,7 +60,10 @@ typedef enum {
     LAP_MG_MIXED = 5, /* the V-cycle's correction equation (Eqs. 13-15) solved by FP32
                         V-cycles inside FP64 defect correction: per iteration,
                         inner_cycles FP32 V(nu1,nu2) cycles on L e = -R, then psi += e
-                        and R = L(psi) in FP64 */
+                        and R = L(psi): with beta = 1 the exact sum, rounded once to the
+                        FP32 that the cycles take (runs of 62 x 8 points whose values span
+                        more than 31 binades, or leave about 1e-18 .. 1e35: the FP64
+                        expression), else the FP64 expression */
     LAP_SLOR = 6,    /* line SOR by rows alone (SLOR subsection, Eqs. 8-10): one zebra
                         x-line sweep per iteration, form line_form (A = SLORA, B = SLORB) */
     LAP_GS_LEX = 7,  /* Eq. 6 in the paper's lexicographic order (i-1, j-1 already new), as

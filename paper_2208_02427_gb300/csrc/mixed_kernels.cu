@@ -3,9 +3,10 @@
 // The correction equation of the V-cycle (Eqs. 13-15: L dpsi = -R) is solved
 // approximately in FP32 while the fine-grid residual R = L(psi) and the update
 // psi <- psi + dpsi stay FP64:
-//   1. r = dx^2 L(psi) in FP64 (the same expression as the FP64 residual), stored as
-//      FP32 for the inner cycle, its sum of squares accumulated in FP64 for the stopping
-//      test; the inner correction e is zeroed in the same pass;
+//   1. r = dx^2 L(psi) in FP64 (the same expression as the FP64 residual; with beta = 1, after
+//      the first, as an exact sum of integers: residual32.cuh), stored as FP32 for the inner cycle,
+//      its sum of squares taken for the stopping test; the inner correction e is zeroed in the
+//      same pass;
 //   2. one or more V-cycles in FP32 on (E+W) + b2 (N+S) - d e + r = 0, e = 0 on the ring;
 //   3. psi += e in FP64.
 // FP32 runs 62x faster than FP64 on GB300, so the inner cycle is bound by memory, not
@@ -137,7 +138,7 @@ __global__ void __launch_bounds__(1024)
 // (sc r)^2: the norm needs a few digits, not FP64's sixteen, and this takes one of the
 // five FP64 operations per point off the FP64 pipe. sc is a power of two near 1 / ||r0||,
 // so the scaled squares stay within FP32's normal range down to 1e-13 ||r0||. (With beta = 1 and a
-// scale residual32_kernel takes its place: 524 -> 180 us at 8193^2.)
+// scale residual32_kernel takes its place: 524 -> 190 us at 8193^2.)
 template <bool UNIT, bool F32NORM>
 __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
     defect64_to32_kernel(const double* __restrict__ psi, int m, int n, int64_t pitch, double b2,
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_BLOCKS_PER_SM)
 }
 
 // The same with beta = 1 and a norm scale, on the integer pipe (residual32.cuh), a warp per run.
-constexpr int RUN_BLOCKS_PER_SM = 3;  // 80 registers; with two blocks of 102, 194 us at 8193^2 against 178
+constexpr int RUN_BLOCKS_PER_SM = 3;  // 76 registers; with two blocks of 102 a 56-bit form took 194 us at 8193^2 against 178
 __global__ void __launch_bounds__(NORM_THREADS, RUN_BLOCKS_PER_SM)
     residual32_kernel(const ResidualRuns R, double* __restrict__ partials, const float* __restrict__ sc, const NormEnd end)
 {
