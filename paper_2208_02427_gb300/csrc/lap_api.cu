@@ -781,6 +781,15 @@ struct Solver {
            "copy field");
     }
 
+    // psi's interior := src's (the ring is never written)
+    void copy_interior(const double* src)
+    {
+        const int64_t at = f.pitch + 1;
+        ck(cudaMemcpy2DAsync(f.p + at, f.pitch * 8, src + at, f.pitch * 8, (size_t)(f.m - 2) * 8, f.n - 2,
+                             cudaMemcpyDeviceToDevice, s),
+           "copy field");
+    }
+
     // ---- one iteration of each method ----
     double* jac_cur = nullptr;  // Jacobi: buffer holding the current iterate
     double* jac_other = nullptr;
@@ -831,7 +840,9 @@ struct Solver {
         double* b = p->method == LAP_JACOBI ? jac_other : tiles_other;
         for (int64_t k = 0; k < launches; ++k) {
             const int sweeps = (int)(count / launches + (k < count % launches ? 1 : 0));
-            ck(launch_sweep_tiles(Field{a, f.m, f.n, f.pitch}, b, c, tiles, sweep_kind(), tiles_diag(), sweeps, w.wslot, s),
+            // the red-black methods' second field takes its ring from the first; Jacobi's buffers both have one
+            ck(launch_sweep_tiles(Field{a, f.m, f.n, f.pitch}, b, c, tiles, sweep_kind(), tiles_diag(), sweeps,
+                                  b == tiles_other && p->method != LAP_JACOBI, w.wslot, s),
                "tile sweeps");
             std::swap(a, b);
         }
@@ -1595,7 +1606,7 @@ struct Solver {
                 out->status = LAP_CONVERGED;
         }
         out->iters = k;
-        if (p->method == LAP_JACOBI && jac_cur != f.p) copy_field(f.p, jac_cur);
+        if (p->method == LAP_JACOBI && jac_cur != f.p) copy_interior(jac_cur);
         if (p->method == LAP_MG_FP32)
             ck(launch_to64(f, w.levels32[0].u.p, w.levels32[0].u.pitch, s), "conversion kernel");
         // the last stopping test already took the final iterate's norm (no second pass)

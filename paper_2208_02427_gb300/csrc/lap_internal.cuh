@@ -60,8 +60,8 @@ struct Field32 {
 void note_launch();
 
 // Several sweeps in one launch, on tiles in shared memory (sweep_tiles.cu): in -> out, the same values
-// as as many one-pass sweeps leave. diag: neighbour sums paired along diagonals (beta = 1). sweeps = 0 in the
-// plan: the one-pass kernels are as fast.
+// as as many one-pass sweeps leave. diag: neighbour sums paired along diagonals (beta = 1). ring: the ring goes
+// along (out is no field of the caller's). sweeps = 0 in the plan: the one-pass kernels are as fast.
 enum { SWEEP_JACOBI = 0, SWEEP_SOR = 1, SWEEP_GS = 2 };
 struct SweepTiles {
     int sweeps = 0;  // at most this many in a launch
@@ -70,7 +70,7 @@ struct SweepTiles {
 SweepTiles plan_sweep_tiles(int m, int n, const Coef& c, int kind, bool diag, int sms);
 cudaError_t prepare_sweep_tiles(const Coef& c, int kind, bool diag);
 cudaError_t launch_sweep_tiles(const Field& in, double* out, const Coef& c, const SweepTiles& t, int kind, bool diag,
-                               int sweeps, const double* wslot, cudaStream_t s);
+                               int sweeps, bool ring, const double* wslot, cudaStream_t s);
 
 // A launch whose set-up may run before the kernels ahead of it on the stream are through; the kernel calls
 // after_prior() before anything else. 0.2 to 0.35 us a launch in a graph, where small levels and small grids are

@@ -56,12 +56,12 @@ __device__ __forceinline__ double swept(const FmaOps& o, const double* c, int W,
 __host__ __device__ constexpr int window_halo(int passes) { return passes > 1 ? passes : 1; }
 
 // The tile of interior columns [x0, x1) and rows [y0, y1) through `passes` passes (two colours a sweep, or
-// one for Jacobi), in -> out. The ring points beside the tile are copied along, so that `out` needs no
-// preparation. sm: (x1 - x0 + 2 h) (y1 - y0 + 2 h) doubles, h = window_halo(passes), twice that for Jacobi.
+// one for Jacobi), in -> out. ring: the ring points beside the tile are copied along, so that a second buffer
+// needs no preparation (the caller's ring is never written). sm: (x1 - x0 + 2 h) (y1 - y0 + 2 h) doubles, h = window_halo(passes), twice that for Jacobi.
 template <int KIND, bool UNIT, bool POW2, bool DIAG>
 __device__ __forceinline__ void sweep_tile(const FmaOps& o, const double* __restrict__ in, double* __restrict__ out,
                                            int m, int n, int64_t pitch, int64_t pitch_out, int x0, int x1, int y0,
-                                           int y1, int passes, const SweepCoef& k, double* sm)
+                                           int y1, int passes, bool ring, const SweepCoef& k, double* sm)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int h = window_halo(passes);
@@ -128,8 +128,8 @@ __device__ __forceinline__ void sweep_tile(const FmaOps& o, const double* __rest
             b = t;
         }
     }
-    const int sx0 = x0 == 1 ? 0 : x0, sx1 = x1 == m - 1 ? m : x1;
-    const int sy0 = y0 == 1 ? 0 : y0, sy1 = y1 == n - 1 ? n : y1;
+    const int sx0 = ring && x0 == 1 ? 0 : x0, sx1 = ring && x1 == m - 1 ? m : x1;
+    const int sy0 = ring && y0 == 1 ? 0 : y0, sy1 = ring && y1 == n - 1 ? n : y1;
     for (int j = sy0 + wid; j < sy1; j += nw)
         for (int i = sx0 + lane; i < sx1; i += 32) out[(int64_t)j * pitch_out + i] = a[(j - Y0) * W + (i - X0)];
 }
@@ -138,7 +138,7 @@ __device__ __forceinline__ void sweep_tile(const FmaOps& o, const double* __rest
 template <int KIND, bool UNIT, bool POW2, bool DIAG>
 __global__ void __launch_bounds__(ST_THREADS)
     sweep_tiles_kernel(const double* __restrict__ in, double* __restrict__ out, int m, int n, int64_t pitch,
-                       int passes, SweepCoef k, const double* __restrict__ wslot)
+                       int passes, int ring, SweepCoef k, const double* __restrict__ wslot)
 {
     after_prior();
     extern __shared__ double sm[];
@@ -153,7 +153,8 @@ __global__ void __launch_bounds__(ST_THREADS)
     const int x1 = 1 + (int)((int64_t)(blockIdx.x + 1) * (m - 2) / gridDim.x);
     const int y0 = 1 + (int)((int64_t)blockIdx.y * (n - 2) / gridDim.y);
     const int y1 = 1 + (int)((int64_t)(blockIdx.y + 1) * (n - 2) / gridDim.y);
-    sweep_tile<KIND, UNIT, POW2, DIAG>(o, in, out, m, n, pitch, pitch, x0, x1, y0, y1, passes, k, sm);
+    sweep_tile<KIND, UNIT, POW2, DIAG>(o, in, out, m, n, pitch, pitch, x0, x1, y0, y1, passes, ring != 0, k,
+                                       sm);
 }
 
 // Launch `k` of `launches` over the tiles of many fields (SOR, each field's own factor and spacing): an even
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(ST_THREADS, 3)
         if (!decltype(P)::value) c.inv_d = in_reg(o, c.inv_d);
         sweep_tile<SWEEP_SOR, decltype(U)::value, decltype(P)::value, false>(
             o, back ? it.other : it.u, back ? it.u : it.other, it.m, it.n, back ? it.pitch_other : it.pitch,
-            back ? it.pitch : it.pitch_other, it.x0, it.x1, it.y0, it.y1, passes, c, sm);
+            back ? it.pitch : it.pitch_other, it.x0, it.x1, it.y0, it.y1, passes, !back, c, sm);
     };
     on_flag(it.unit_beta != 0, [&](auto U) { on_flag(it.inv_d_shift > 0, [&](auto P) { run(U, P); }); });
 }
@@ -254,14 +255,15 @@ cudaError_t prepare_sweep_tiles(const Coef& c, int kind, bool diag)
 }
 
 cudaError_t launch_sweep_tiles(const Field& in, double* out, const Coef& c, const SweepTiles& t, int kind, bool diag,
-                               int sweeps, const double* wslot, cudaStream_t s)
+                               int sweeps, bool ring, const double* wslot, cudaStream_t s)
 {
     const int passes = halo(kind, sweeps), h = window_halo(passes);
     const int tw = (in.m - 2 + t.tx - 1) / t.tx, th = (in.n - 2 + t.ty - 1) / t.ty;
     const size_t bytes = (size_t)(tw + 2 * h) * (th + 2 * h) * 8 * (kind == SWEEP_JACOBI ? 2 : 1);
     const SweepCoef k{c.b2, c.inv_d, c.inv_d_shift, 1.0, 0.0};
     const cudaError_t e = on_sweep_kernel(c, kind, diag, [&](auto* kernel) {
-        launch_after(kernel, dim3(t.tx, t.ty), ST_THREADS, bytes, s, in.p, out, in.m, in.n, in.pitch, passes, k, wslot);
+        launch_after(kernel, dim3(t.tx, t.ty), ST_THREADS, bytes, s, in.p, out, in.m, in.n, in.pitch, passes,
+                     ring ? 1 : 0, k, wslot);
         return cudaGetLastError();
     });
     note_launch();
