@@ -183,7 +183,12 @@ void lap_destroy(lap_handle h);
 /* Scratch bytes lap_solve needs for this grid and method (admission against a budget).
  * Host arithmetic: no allocation and no launch (it reads the current device's multiprocessor
  * count, 152 when there is no device). Gives the refusals lap_solve would give for the shape
- * and parameters (LAP_EINVAL, LAP_EUNSUPPORTED: the size limits above). */
+ * and parameters (LAP_EINVAL, LAP_EUNSUPPORTED: the size limits above).
+ * Beside it a handle holds tables, and for line methods the scratch of their columns (half the
+ * field). Point and line solves of small and medium grids also keep one spare buffer of at most
+ * 64 MiB (a second field, or the scratch of their rows) where budget and device have room for
+ * it; it is given back when another allocation of the handle is short, and without it they take
+ * another path to the same values (rows: to rounding). */
 int lap_workspace_bytes(const lap_grid* g, const lap_params* p, size_t* bytes);
 
 /* Iterate p->method on psi_dev until the stopping rule (p->norm, p->tol) holds or

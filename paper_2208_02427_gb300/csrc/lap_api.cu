@@ -136,6 +136,7 @@ double* arena(lap_handle h, size_t bytes)
 double* spare(lap_handle h, size_t bytes)
 {
     bytes = (size_t)round_up((int64_t)bytes, 1 << 20);
+    if (bytes > SPARE_MAX) return nullptr;
     if (bytes > h->spare_bytes) {
         drop_spare(h);
         if (h->budget && h->held + bytes > h->budget) return nullptr;
@@ -803,6 +804,7 @@ struct Solver {
     {
         return p->method == LAP_JACOBI ? SWEEP_JACOBI : p->method == LAP_GS_RB ? SWEEP_GS : SWEEP_SOR;
     }
+    int64_t tiles_pitch() const { return round_up(f.m, 32); }  // of the second field (Jacobi: psi's)
     bool tiles_diag() const { return p->method != LAP_JACOBI && p->sum_order == LAP_SUM_DIAGONAL; }
 
     // Takes the tiles where they pay and their second field is to be had.
@@ -813,7 +815,7 @@ struct Solver {
         if (p->check_every < 2 || p->max_iter < 2) return;
         tiles = plan_sweep_tiles(f.m, f.n, c, sweep_kind(), tiles_diag(), device_sms());
         if (!tiles.sweeps) return;
-        tiles_other = p->method == LAP_JACOBI ? w.aux : spare(h, (size_t)f.n * f.pitch * sizeof(double));
+        tiles_other = p->method == LAP_JACOBI ? w.aux : spare(h, (size_t)f.n * tiles_pitch() * sizeof(double));
         if (!tiles_other) tiles = SweepTiles{};
         else ck(prepare_sweep_tiles(c, sweep_kind(), tiles_diag()), "tile sweep attributes");
     }
@@ -836,13 +838,14 @@ struct Solver {
     void tiled_sweeps(int64_t count)
     {
         const int64_t launches = 2 * ((count + 2 * tiles.sweeps - 1) / (2 * tiles.sweeps));
-        double* a = p->method == LAP_JACOBI ? jac_cur : f.p;
-        double* b = p->method == LAP_JACOBI ? jac_other : tiles_other;
+        const bool jacobi = p->method == LAP_JACOBI;
+        Field a{jacobi ? jac_cur : f.p, f.m, f.n, f.pitch};
+        Field b{jacobi ? jac_other : tiles_other, f.m, f.n, jacobi ? f.pitch : tiles_pitch()};
         for (int64_t k = 0; k < launches; ++k) {
             const int sweeps = (int)(count / launches + (k < count % launches ? 1 : 0));
             // the red-black methods' second field takes its ring from the first; Jacobi's buffers both have one
-            ck(launch_sweep_tiles(Field{a, f.m, f.n, f.pitch}, b, c, tiles, sweep_kind(), tiles_diag(), sweeps,
-                                  b == tiles_other && p->method != LAP_JACOBI, w.wslot, s),
+            ck(launch_sweep_tiles(a, b.p, b.pitch, c, tiles, sweep_kind(), tiles_diag(), sweeps,
+                                  !jacobi && b.p == tiles_other, w.wslot, s),
                "tile sweeps");
             std::swap(a, b);
         }

@@ -136,7 +136,9 @@ void drop_graphs(lap_handle h);
 // Scratch for one call: grows (never shrinks) the handle's arena.
 double* arena(lap_handle h, size_t bytes);
 // The handle's spare buffer of at least `bytes`, or null where the budget or the device has no room for
-// it: a call that can do without takes its other path.
+// it, or it would be more than SPARE_MAX: a call that can do without takes its other path. (The rows of the
+// tallest grid of lines, 1024 unknowns to a row and 16383 rows, come to SPARE_MAX; tiles pay up to about a million points.)
+constexpr size_t SPARE_MAX = (size_t)64 << 20;
 double* spare(lap_handle h, size_t bytes);
 
 // Carves aligned sub-buffers out of a byte range.

@@ -69,8 +69,8 @@ struct SweepTiles {
 };
 SweepTiles plan_sweep_tiles(int m, int n, const Coef& c, int kind, bool diag, int sms);
 cudaError_t prepare_sweep_tiles(const Coef& c, int kind, bool diag);
-cudaError_t launch_sweep_tiles(const Field& in, double* out, const Coef& c, const SweepTiles& t, int kind, bool diag,
-                               int sweeps, bool ring, const double* wslot, cudaStream_t s);
+cudaError_t launch_sweep_tiles(const Field& in, double* out, int64_t pitch_out, const Coef& c, const SweepTiles& t,
+                               int kind, bool diag, int sweeps, bool ring, const double* wslot, cudaStream_t s);
 
 // A launch whose set-up may run before the kernels ahead of it on the stream are through; the kernel calls
 // after_prior() before anything else. 0.2 to 0.35 us a launch in a graph, where small levels and small grids are

@@ -138,7 +138,7 @@ __device__ __forceinline__ void sweep_tile(const FmaOps& o, const double* __rest
 template <int KIND, bool UNIT, bool POW2, bool DIAG>
 __global__ void __launch_bounds__(ST_THREADS)
     sweep_tiles_kernel(const double* __restrict__ in, double* __restrict__ out, int m, int n, int64_t pitch,
-                       int passes, int ring, SweepCoef k, const double* __restrict__ wslot)
+                       int64_t pitch_out, int passes, int ring, SweepCoef k, const double* __restrict__ wslot)
 {
     after_prior();
     extern __shared__ double sm[];
@@ -153,8 +153,8 @@ __global__ void __launch_bounds__(ST_THREADS)
     const int x1 = 1 + (int)((int64_t)(blockIdx.x + 1) * (m - 2) / gridDim.x);
     const int y0 = 1 + (int)((int64_t)blockIdx.y * (n - 2) / gridDim.y);
     const int y1 = 1 + (int)((int64_t)(blockIdx.y + 1) * (n - 2) / gridDim.y);
-    sweep_tile<KIND, UNIT, POW2, DIAG>(o, in, out, m, n, pitch, pitch, x0, x1, y0, y1, passes, ring != 0, k,
-                                       sm);
+    sweep_tile<KIND, UNIT, POW2, DIAG>(o, in, out, m, n, pitch, pitch_out, x0, x1, y0, y1, passes,
+                                       ring != 0, k, sm);
 }
 
 // Launch `k` of `launches` over the tiles of many fields (SOR, each field's own factor and spacing): an even
@@ -254,16 +254,16 @@ cudaError_t prepare_sweep_tiles(const Coef& c, int kind, bool diag)
     });
 }
 
-cudaError_t launch_sweep_tiles(const Field& in, double* out, const Coef& c, const SweepTiles& t, int kind, bool diag,
-                               int sweeps, bool ring, const double* wslot, cudaStream_t s)
+cudaError_t launch_sweep_tiles(const Field& in, double* out, int64_t pitch_out, const Coef& c, const SweepTiles& t,
+                               int kind, bool diag, int sweeps, bool ring, const double* wslot, cudaStream_t s)
 {
     const int passes = halo(kind, sweeps), h = window_halo(passes);
     const int tw = (in.m - 2 + t.tx - 1) / t.tx, th = (in.n - 2 + t.ty - 1) / t.ty;
     const size_t bytes = (size_t)(tw + 2 * h) * (th + 2 * h) * 8 * (kind == SWEEP_JACOBI ? 2 : 1);
     const SweepCoef k{c.b2, c.inv_d, c.inv_d_shift, 1.0, 0.0};
     const cudaError_t e = on_sweep_kernel(c, kind, diag, [&](auto* kernel) {
-        launch_after(kernel, dim3(t.tx, t.ty), ST_THREADS, bytes, s, in.p, out, in.m, in.n, in.pitch, passes,
-                     ring ? 1 : 0, k, wslot);
+        launch_after(kernel, dim3(t.tx, t.ty), ST_THREADS, bytes, s, in.p, out, in.m, in.n, in.pitch, pitch_out,
+                     passes, ring ? 1 : 0, k, wslot);
         return cudaGetLastError();
     });
     note_launch();

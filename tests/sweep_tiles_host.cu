@@ -56,7 +56,7 @@ int main()
                 if (!t.sweeps) continue;
                 single += t.sweeps == 1;
                 for (int s = t.sweeps == 1 ? 0 : 1; s <= t.sweeps; ++s) {
-                    launch_sweep_tiles(Field{nullptr, m, n, m}, nullptr, c, t, kind, diag, s, true, nullptr, nullptr);
+                    launch_sweep_tiles(Field{nullptr, m, n, m}, nullptr, m, c, t, kind, diag, s, true, nullptr, nullptr);
                     const int64_t need = window_bytes(m, n, t, kind, s);
                     ++launches;
                     if ((int64_t)g_bytes >= need && g_bytes <= 227 * 1024) continue;
