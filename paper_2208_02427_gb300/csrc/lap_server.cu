@@ -42,6 +42,9 @@ struct lap_server_s {
     char* stage = nullptr;
     size_t stage_bytes = 0;
     std::deque<int64_t> completed;  // finished requests, in the order their steps ended
+    // the tile plan of the last step's fields, for the steps until they change
+    std::vector<std::pair<int, int>> planned;
+    BatchSweepPlan tile_plan;
 };
 
 namespace {
@@ -400,7 +403,11 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
                                  0, 0, 0, 0, L.problem, L.unit_beta, L.inv_d_shift, sweeps_now(q)});
             }
             if (!tiled.empty()) {
-                P.tile_plan = plan_batch_sweeps(shapes, device_sms());
+                if (shapes != S->planned) {
+                    S->tile_plan = plan_batch_sweeps(shapes, device_sms());
+                    S->planned = shapes;
+                }
+                P.tile_plan = S->tile_plan;
                 for (const SweepTileItem& t : tiled) add_sweep_tiles(P.tiled, t, P.tile_plan);
                 const int most = tiled.front().sweeps;  // sor_q is in falling order
                 P.tile_launches = 2 * ((most + 2 * P.tile_plan.sweeps - 1) / (2 * P.tile_plan.sweeps));
