@@ -140,11 +140,12 @@ __device__ __forceinline__ void prolong_black(const Arith<T>& A, const BatchLeve
     *x = A.add(*x, A.half(A.add(a[0], a[odd ? C.pitch : 1])));
 }
 
-// One smoother colour pass (Eq. 6 when gs, Eq. 7 otherwise) over the rows of each item.
+// One smoother colour pass (Eq. 6 when gs, Eq. 7 otherwise) over the rows of each item. per_level_w: each level's own
+// factor in place of w.
 template <class T>
 __global__ void __launch_bounds__(BT)
     b_rb_kernel(const BatchItem* __restrict__ items, int count, unsigned* claim, const BatchLevel<T>* __restrict__ lv,
-                const int* __restrict__ active, int colour, int gs, T w, T omw)
+                const int* __restrict__ active, int colour, int gs, T w_arg, T omw_arg, int per_level_w)
 {
     after_prior();
     const Arith<T> A = arith<T>();
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(BT)
         const BatchItem it = items[b];
         const BatchLevel<T> L = lv[it.level];
         if (!active[L.problem]) continue;
+        const T w = per_level_w ? (T)L.w : w_arg, omw = per_level_w ? (T)L.omw : omw_arg;
         const int half_w = (L.m - 2 + 1) / 2;
         on_rb_flags(L, gs != 0, [&](auto U, auto P, auto Q, auto G) {
             for (Walk k(half_w); k.r < it.rows; k.next()) {
@@ -728,12 +730,12 @@ __global__ void b_converge_kernel(const double* __restrict__ partials,
 
 template <class T>
 cudaError_t launch_b_rb(const BatchList& l, const BatchLevel<T>* lv, const int* active, int colour,
-                        bool gs, double w, cudaStream_t s)
+                        bool gs, double w, cudaStream_t s, bool per_level_w)
 {
     if (l.count == 0) return cudaSuccess;
     const int grid = batch_grid((const void*)b_rb_kernel<T>, BT, 0, l.count, l.claim != nullptr);
     launch_after(b_rb_kernel<T>, grid, BT, 0, s, l.items, l.count, l.claim, lv, active, colour, gs ? 1 : 0, (T)w,
-                                       (T)(1.0 - w));
+                                       (T)(1.0 - w), per_level_w ? 1 : 0);
     note_launch();
     return cudaGetLastError();
 }
@@ -789,8 +791,8 @@ cudaError_t launch_b_coarse(const BatchList& l, const BatchLevel<T>* lv, const i
     return cudaGetLastError();
 }
 
-template cudaError_t launch_b_rb<double>(const BatchList&, const BatchLevel<double>*, const int*, int, bool, double, cudaStream_t);
-template cudaError_t launch_b_rb<float>(const BatchList&, const BatchLevel<float>*, const int*, int, bool, double, cudaStream_t);
+template cudaError_t launch_b_rb<double>(const BatchList&, const BatchLevel<double>*, const int*, int, bool, double, cudaStream_t, bool);
+template cudaError_t launch_b_rb<float>(const BatchList&, const BatchLevel<float>*, const int*, int, bool, double, cudaStream_t, bool);
 template cudaError_t launch_b_defect<double>(const BatchList&, const BatchLevel<double>*, const int*, cudaStream_t, bool);
 template cudaError_t launch_b_defect<float>(const BatchList&, const BatchLevel<float>*, const int*, cudaStream_t, bool);
 template cudaError_t launch_b_restrict<double>(const BatchList&, const BatchLevel<double>*, const int*, cudaStream_t, bool);

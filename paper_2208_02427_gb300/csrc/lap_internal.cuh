@@ -320,7 +320,7 @@ template <class T>
 cudaError_t launch_zero_rings(const BatchLevel<T>* lv, int count, cudaStream_t s);
 template <class T>
 cudaError_t launch_b_rb(const BatchList& l, const BatchLevel<T>* lv, const int* active, int colour,
-                        bool gs, double w, cudaStream_t s);
+                        bool gs, double w, cudaStream_t s, bool per_level_w = false);
 // SOR sweeps over many fields (the server's), several per launch on tiles (sweep_tiles.cu): one tile of
 // a field that takes `sweeps` sweeps in all, with a second buffer for it.
 struct alignas(16) SweepTileItem {

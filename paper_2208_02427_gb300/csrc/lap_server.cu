@@ -136,6 +136,10 @@ constexpr int SERVER_TAIL_FP32 = 129;
 // million points 24.2 / 22.9 us, 15.8 million (60 fields of 513^2) 81.8 / 87.6, 16.8 million 87 / 91, 67 million
 // 332 / 352 (the passes cost their first and last waves once a launch, the tiles their halos at any size).
 constexpr int64_t SERVER_TILE_POINTS = 8000000;
+// And above this many the passes go by rows (b_rb_kernel, BATCH_ITEM_POINTS to an item): the fields then stream from
+// memory, where its 64 warps a multiprocessor hold more loads in flight than the 40 of b_sweep_kernel. By points / by
+// rows, a colour pass of 33.6 million points 169.1 / 164.8 us, 67 million 332.6 / 322.5.
+constexpr int64_t SERVER_ROWS_POINTS = 32000000;
 
 // Points of a colour per work item of a step's SOR passes (of fields not on tiles), for `points` of them in
 // all: SWEEP_STEP, or as many steps as leave about 48 items per multiprocessor (24: 340 against 333 us a
@@ -165,12 +169,13 @@ struct SrvPlan {
     std::vector<StreamItem> streams;
     LevelLists mg64, mg32;
     std::vector<SweepItem> sweeps;  // SOR pass by pass, for the fields not on tiles
+    std::pair<int, int> rows{0, 0};  // the same by rows (items)
     std::vector<SweepTileItem> tiled;
     BatchSweepPlan tile_plan;
     int tile_launches = 0;
     std::pair<int, int> update, init, norm;
     std::vector<int> first_init, first_norm;
-    std::vector<int> sor_upto;  // items of `sweeps` (a prefix) swept in the step's k-th sweep
+    std::vector<int> sor_upto;  // items of `sweeps` or `rows` (a prefix) swept in the step's k-th sweep
 };
 
 }  // namespace
@@ -416,11 +421,15 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
             int64_t sor_points = 0;
             for (int q : rest) sor_points += (int64_t)((run[q]->g.m - 1) / 2) * (run[q]->g.n - 2);
             const int per_item = sor_item_points(sor_points);
+            const bool by_rows = 2 * sor_points > SERVER_ROWS_POINTS;
+            P.rows.first = (int)P.items.size();
             for (int q : rest) {
-                add_sweep_items(P.sweeps, P.lv64[base[q]], per_item);
-                const int upto = (int)P.sweeps.size();
+                if (by_rows) add_items(P.items, base[q], run[q]->g.m, run[q]->g.n);
+                else add_sweep_items(P.sweeps, P.lv64[base[q]], per_item);
+                const int upto = by_rows ? (int)P.items.size() - P.rows.first : (int)P.sweeps.size();
                 for (int k = 0; k < sweeps_now(q); ++k) P.sor_upto[k] = upto;
             }
+            P.rows.second = (int)P.items.size() - P.rows.first;
         }
         P.update = level0([](const SrvRequest& r) { return r.method == LAP_MG_MIXED; }, nullptr);
         P.init = level0([](const SrvRequest& r) { return r.fresh; }, &P.first_init);
@@ -531,7 +540,11 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
             ck(launch_b_sweep_tiles(tiled, (int)P.tiled.size(), P.tile_plan, active, k, P.tile_launches, st), "server sweeps");
         for (int k = 0; k < S->sor_sweeps && P.sor_upto[k]; ++k)
             for (int colour = 0; colour < 2; ++colour)
-                ck(launch_b_sweep(sweeps, P.sor_upto[k], active, colour, st), "server sweep");
+                if (P.rows.second)
+                    ck(launch_b_rb(list({P.rows.first, P.sor_upto[k]}), lv64, active, colour, false, 1.0, st, true),
+                       "server sweep");
+                else
+                    ck(launch_b_sweep(sweeps, P.sor_upto[k], active, colour, st), "server sweep");
         int mixed = 0;
         for (const SrvRequest* r : run) mixed += r->method == LAP_MG_MIXED;
         if (mixed)
