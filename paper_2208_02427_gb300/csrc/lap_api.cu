@@ -418,7 +418,11 @@ double line_coefs(const Coef& c, double w, int form, int direction, LineCoefs* k
 // ends' reach; separators closer than that need the reduction, about 250 clocks a level. One warp alone takes
 // about 900 clocks a position (loads, addresses and stores between the 320 of FP64). Half sweeps of 4 / 12 / 16
 // warps to a multiprocessor at 3001 x 2050: 106 / 85 / 75 us.
-int line_y_chunks(int N, double alpha, double delta, int nl)
+// streams: the lines come from memory (in form A, which reads the old values as well, past the L2's size): then fewer
+// than 16 warps wait for it, and count for a twelfth more. Form A by that rule, ADI iterations: 4097^2 453.2 -> 440.5 us,
+// 4097 x 8193 876 -> 849, 8193^2 1894 -> 1848; below the line 2050 x 3001 would lose (form B 186 -> 193), and form B
+// gains nothing on the largest fields.
+int line_y_chunks(int N, double alpha, double delta, int nl, bool streams)
 {
     const double x = alpha / delta, e = 2.0 * x / (1.0 + std::sqrt(std::max(0.0, 1.0 - 4.0 * x * x)));
     const double K0 = 64.0 * std::log(2.0) / -std::log(std::min(e, 0.999));
@@ -432,7 +436,8 @@ int line_y_chunks(int N, double alpha, double delta, int nl)
         if (P > 1 && L < shortest) break;
         const int rounds = (nl * P + 127) / 128;
         const double levels = P > 2 && L <= K0 ? std::ceil(std::log2(P - 1.0)) : 0.0;
-        const double cost = std::max(rounds * 64.0 * (5.0 * L + 2.0 * std::min<double>(L, K0)), 900.0 * L) + 250.0 * levels;
+        const double work = rounds * 64.0 * (5.0 * L + 2.0 * std::min<double>(L, K0)) * (streams && rounds < 4 ? 1.08 : 1.0);
+        const double cost = std::max(work, 900.0 * L) + 250.0 * levels;
         if (cost < least) {
             least = cost;
             best = P;
@@ -452,7 +457,9 @@ const LineTables& line_setup(lap_handle h, const Field& f, const Coef& c, double
     const double alpha = line_coefs(c, w, form, direction, k);
     *scratch = nullptr;
     if (!x || threads) {
-        const int cut = line_y_chunks(N, alpha, c.d, line_y_lines(((x ? f.n : f.m) - 1) / 2, device_sms()));
+        // field and scratch against the L2's 129 MB
+        const bool streams = !x && form == LAP_FORM_A && 12.0 * f.m * f.n > 129e6;
+        const int cut = line_y_chunks(N, alpha, c.d, line_y_lines(((x ? f.n : f.m) - 1) / 2, device_sms()), streams);
         const LineTables& t = line_tables(h, N, alpha, c.d, k->wc, cut, LINE_Y_MIN_CHUNK);
         if (!x) *scratch = line_scratch(h, t, line_scratch_pitch(f, direction));
         return t;

@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(LX_THREADS, 6)
 // their own the separators took a launch between forward and back, three launches a colour; one
 // launch gives every multiprocessor the same number of lines and no waits between them. Half sweeps, three
 // launches a colour / one: 300^2 27 / 14 us, 1000^2 41 / 28, 2050 x 3001 102 / 86, 500 x 4000 99 / 72, 4097^2
-// 195 / 203 (ADI less SLOR iterations), 3001 x 2050 92 / 77 (launch times).
+// 197 / 193 (ADI less SLOR iterations), 3001 x 2050 92 / 77 (launch times).
 // What bounds it is the recurrence: a dependent fma takes 71 clocks, one warp on each scheduler nearly
 // fills the FP64 pipe, and everything else has to be out of the way: a step's field values and table
 // entries are loaded PIPE positions ahead, into registers (a table entry loaded in its step waited for the
