@@ -221,10 +221,10 @@ int lap_solve_host(lap_handle h, const lap_grid* g, double* psi_host, int64_t ho
  * graph that stops itself when no problem is left or p->max_iter cycles are done, and the host
  * waits once; without, the host polls the number of problems still running every
  * p->check_every cycles. Synchronises `stream` before returning.
- * Where a parameter leaves the launch configuration open (0) it follows from the batch: a
- * small-level tail for small FP64 batches and for FP32 levels that are not streams, the FP32 levels as row streams (tiling 4 in lap_last_batch_config; as tiles
- * of variant 1 where the smoothing counts are outside 1..3), work items of 1024 to 4096 points,
- * one CTA per item. No choice changes a value.
+ * Where a parameter leaves the launch configuration open (0) it follows from the batch's count,
+ * widest side and points: the small-level tail (none for many or wide grids), the FP32 levels as
+ * row streams (tiling 4 in lap_last_batch_config; as tiles where the smoothing counts are outside
+ * 1..3), work items of 1024 to 4096 points, one CTA per item. No choice changes a value.
  * The plan of a call (level descriptors, work lists, the captured cycle graphs) stays in the
  * handle: a following call with the same grids, field addresses and multigrid parameters
  * reuses it, unless another call of the handle has used its scratch memory in between. */

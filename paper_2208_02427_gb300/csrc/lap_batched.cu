@@ -127,7 +127,10 @@ void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJ
         }
         L.tail[l] = {j0, (int)jobs.size() - j0};
         if (!fits64) L.tail64[l] = 0;
-        if (!fits32) L.tail32[l] = 0;
+        // more small FP32 tails than multiprocessors: b_tail_kernel, four of whose CTAs share one (sides up to
+        // 65, in shared memory / there: 256 grids 756 / 728 us a solve, 512 1136 / 1046, 2048 3837 / 2992; up to 129 the
+        // same within 1%; FP64 is faster in shared memory at any number)
+        if (!fits32 || L.tail[l].second > device_sms()) L.tail32[l] = 0;
     }
     if (tiles) {
         const int u0 = (int)items.size();
@@ -239,31 +242,43 @@ BatchKey make_key(int count, const lap_grid* grids, double* const* psi_devs, con
     return k;
 }
 
-// The configuration of a batched solve where its parameters leave it open, for `points` level-0 points
-// in all: none changes a value. Tail: FP64 levels up to 33 points wide as one CTA per problem while the
-// batch is below about 10M points (whole solves without / with it: 24 grids up to 129^2 1650 / 1400 us, 256 up
-// to 257^2 3680 / 3500, 64 up to 513^2 3420 / 3440); above, and for the row streams of the mixed solver, whose
-// small levels are two launches each, it gains nothing (1024 grids up to 513^2: 22.6 / 23.1 ms, mixed 8.0 /
-// 8.6 ms). FP32 levels as tiles or one kernel per pass: up to 129 points in a large batch (none / 65 / 129 on 4096
-// grids 44.0 / 44.4 / 41.1 ms for tile variant 1, 58.2 / 58.6 / 55.3 per pass; 1024 grids 12.4 / 12.6 / 12.4, 16.7 / 16.5 /
-// 16.2), in a small one none with tiles (64 grids 1.82 / 2.10 / 2.79) and 65 without (2.88 / 2.60 / 3.12). FP32 levels: row
-// streams where they cover the smoothing counts, else the first tile variant. Work items: about 16 per
-// multiprocessor, so that the last wave is a small part of a pass, between 1024 points (below, a CTA's
-// start outweighs its work) and 4096 (above, nothing is gained). One CTA per item: the block
+// The configuration of a batched solve where its parameters leave it open, for `count` grids with sides up to `side`
+// and `points` level-0 points in all: none changes a value.
+// Tail: the small levels of a problem in one launch save their launches, and cost the others of the batch the wait
+// for it. Whole solves in us, without a tail / with tails of 33 / 65 / 129 points:
+//   FP64, 16 grids up to 65: 1079 / 784 / 530 / 523; 2048: 4534 / 4824 / 4377 / 4357; 4096 of 33: 5835 / 6095;
+//         4 up to 129: 1148 / 1024 / 908 / 865; 24: 1432 / 1279 / 1216 / 1311; 1024: 4699 / 4658 / 4466 / 4796; 2048: 7962 / 8439 / 8239 / 8163;
+//         16 up to 257: 1699 / 1670 / 1857; 256: 3415 / 3284 / 3235;
+//         24 up to 513: 1920 / 2141 / 2367; 64: 3086 / 3180 / 3480
+//   mixed by row streams, 2 grids up to 65: 477 / 520 / 361; 64: 640 / 596 / 491; 256: 783 / 819 / 742; 2048: 2506 /
+//         3523 / 3873; wider ones gain nothing (24 up to 129: 758 / 795 / 769 / 853)
+//   FP32 levels as tiles, 64 grids up to 65: 642 / 612 / 484; 24 up to 129: 821 / 845 / 799 / 854; 512: 2081 / 2139 / 1937 /
+//         1735; 16 up to 257: 982 / 1077 / 1081; one kernel per pass, 24 up to 129: 1320 / 1089 / 913 / 855; 16 up to 257: 1533 /
+//         1366 / 1259; large batches 129 (4096 grids up to 513, none / 65 / 129: tiles 44.0 / 44.4 / 41.1 ms, per pass 58.2 /
+//         58.6 / 55.3)
+// FP32 levels: row streams where they cover the smoothing counts, else tiles: of variant 3 (smaller regions) below
+// 1.5 million points (variant 1 / 3 with V(4,4): 16 grids up to 257 955 / 835, 24 up to 513 1064 / 992, 64 up to 513 1652 / 1962).
+// Work items: about 16 per multiprocessor, so that the last wave is a small part of a pass, between 1024 points
+// (below, a CTA's start outweighs its work) and 4096 (above, nothing is gained). One CTA per item: the block
 // scheduler hands out uniform items as well as a claim counter does.
-BatchConfig batch_config(const lap_params* p, int64_t points)
+BatchConfig batch_config(const lap_params* p, int count, int side, int64_t points)
 {
     BatchConfig c;
-    const int64_t per = points / (16 * (int64_t)device_sms());
+    const int64_t sms = device_sms(), per = points / (16 * sms);
     c.tiles = 0;
     if (p->method == LAP_MG_MIXED && !p->unfused && p->tiling >= 0 && fused32_supported(p->nu1, p->nu2)) {
+        const int variant = p->tiling > 0 ? p->tiling : points < 1500000 && fused32_variant_supported(3, p->nu1, p->nu2) ? 3 : 1;
         if (p->tiling == 0 && stream32_supported(p->nu1, p->nu2)) c.tiles = FUSED32_STREAMS;
-        else c.tiles = fused32_variant_supported(std::max(1, p->tiling), p->nu1, p->nu2) ? std::max(1, p->tiling) : 0;
+        else c.tiles = fused32_variant_supported(variant, p->nu1, p->nu2) ? variant : 0;
     }
     const bool small = per < 4096;
     if (p->tail_size != 0) c.tail = p->tail_size;
-    else if (p->method == LAP_MG) c.tail = small ? 33 : -1;
-    else if (c.tiles == FUSED32_STREAMS) c.tail = -1;
+    else if (p->method == LAP_MG)
+        c.tail = side <= 129 && points < 8000000 && count <= 16 * sms ? (side > 65 && count <= 8 ? 129 : 65)
+                 : side > 129 && side <= 257 && small ? 33 : -1;
+    else if (c.tiles == FUSED32_STREAMS) c.tail = side <= 65 && count <= 2 * sms ? 65 : -1;
+    else if (side <= 65) c.tail = 65;
+    else if (side <= 129) c.tail = c.tiles && count <= sms / 2 ? 65 : 129;
     else c.tail = !small ? 129 : c.tiles ? -1 : 65;
     c.item = p->item_points > 0 ? p->item_points : (int)std::min<int64_t>(4096, std::max<int64_t>(1024, per));
     c.persist = p->persistent > 0 ? 1 : 0;
@@ -441,8 +456,12 @@ extern "C" int lap_solve_batched(lap_handle h, int count, const lap_grid* grids,
         const bool mixed = p->method == LAP_MG_MIXED;
         cudaStream_t s = (cudaStream_t)stream;
         int64_t points = 0;
-        for (int q = 0; q < count; ++q) points += (int64_t)grids[q].m * grids[q].n;
-        const BatchConfig cfg = batch_config(p, points);
+        int side = 0;
+        for (int q = 0; q < count; ++q) {
+            points += (int64_t)grids[q].m * grids[q].n;
+            side = std::max({side, grids[q].m, grids[q].n});
+        }
+        const BatchConfig cfg = batch_config(p, count, side, points);
         if (mixed && !p->unfused && fused32_supported(p->nu1, p->nu2))
             ck(prepare_fused32(), "tile kernel attributes");
         // the plan of the previous call, if it was this batch and nothing has carved the arena
