@@ -110,16 +110,22 @@ void build_lists(LevelLists& L, std::vector<BatchItem>& items, std::vector<TailJ
         L.coarse[l] = {c0, (int)items.size() - c0};
         const int j0 = (int)jobs.size();
         bool fits64 = true, fits32 = true;
+        std::vector<std::pair<int, int>> planned;  // the sides whose plans are in the sums below
         for (size_t k = 0; k < who.size(); ++k) {
             const int q = who[k];
             if (t[k] == l && l < nlev[q]) {
                 const BatchLevel<double>& f = lv[base[q] + l];
-                const size_t b64 = plan_smem_tail<double>(f.m, f.n, nlev[q] - l, false).bytes;
-                const size_t b32 = plan_smem_tail<float>(f.m, f.n, nlev[q] - l, false).bytes;
-                fits64 = fits64 && b64;
-                fits32 = fits32 && b32;
-                L.tail64[l] = std::max(L.tail64[l], b64);
-                L.tail32[l] = std::max(L.tail32[l], b32);
+                // (the sides give the levels: one list has one coarsest_min and max_levels)
+                const std::pair<int, int> sides{f.m, f.n};
+                if (std::find(planned.begin(), planned.end(), sides) == planned.end()) {
+                    const size_t b64 = plan_smem_tail<double>(f.m, f.n, nlev[q] - l, false).bytes;
+                    const size_t b32 = plan_smem_tail<float>(f.m, f.n, nlev[q] - l, false).bytes;
+                    fits64 = fits64 && b64;
+                    fits32 = fits32 && b32;
+                    L.tail64[l] = std::max(L.tail64[l], b64);
+                    L.tail32[l] = std::max(L.tail32[l], b32);
+                    if (planned.size() < 32) planned.push_back(sides);
+                }
                 jobs.push_back(TailJob{base[q] + l, base[q] + nlev[q] - 1});
                 const BatchLevel<double>& d = lv[base[q] + nlev[q] - 1];
                 L.max_coarse = std::max(L.max_coarse, (d.m - 2) * (d.n - 2));

@@ -128,9 +128,12 @@ void srv_levels(lap_server S, SrvRequest& r, C& cv)
 }
 
 // Small-level tail sizes of the server's V-cycles (one CTA per request runs its levels at
-// or below the size).
+// or below the size): FP64, FP32, and FP32 beside requests wider than the latter, whose levels' launches the other tails
+// would wait for. Mixed steps in us with 129 / 65: 24 requests up to 513 points a side 332 / 246, 64 up to 257 305 / 257, 200
+// up to 257 445 / 399, 64 of 513 and 1025 1160 / 1094; 8 up to 129 119 / 142, 24 175 / 165.
 constexpr int SERVER_TAIL_FP64 = 33;
 constexpr int SERVER_TAIL_FP32 = 129;
+constexpr int SERVER_TAIL_WIDE = 65;
 
 // A step's SOR fields go on tiles up to this many points in all. Per colour pass, pass by pass / tiles: 4.2
 // million points 24.2 / 22.9 us, 15.8 million (60 fields of 513^2) 81.8 / 87.6, 16.8 million 87 / 91, 67 million
@@ -349,16 +352,23 @@ extern "C" int lap_server_step(lap_server S, void* stream, int* running, int* qu
         for (int q = 0; q < R; ++q) nlev[q] = run[q]->nlev;
         auto mg_lists = [&](int method, LevelLists& L) {
             std::vector<int> who;
+            int side = 0;
             for (int q = 0; q < R; ++q)
-                if (run[q]->method == method) who.push_back(q);
+                if (run[q]->method == method) {
+                    who.push_back(q);
+                    side = std::max({side, run[q]->g.m, run[q]->g.n});
+                }
             // no timing across steps (the running set changes): fixed tail sizes
-            const int ts = S->mg.tail_size != 0 ? S->mg.tail_size
-                                                : (method == LAP_MG_MIXED ? SERVER_TAIL_FP32 : SERVER_TAIL_FP64);
             const bool fused = method == LAP_MG_MIXED && !S->mg.unfused &&
                                fused32_supported(S->mg.nu1, S->mg.nu2);
+            const bool streams = fused && stream32_supported(S->mg.nu1, S->mg.nu2);
+            const int ts = S->mg.tail_size != 0                  ? S->mg.tail_size
+                           : method == LAP_MG                    ? SERVER_TAIL_FP64
+                           : streams && side > SERVER_TAIL_FP32 ? SERVER_TAIL_WIDE
+                                                                 : SERVER_TAIL_FP32;
             build_lists(L, P.items, P.jobs, who, base, nlev, P.lv64, ts, fused ? &P.tiles : nullptr,
                         &P.streams, S->mg.nu1, S->mg.nu2,
-                        stream32_supported(S->mg.nu1, S->mg.nu2) ? FUSED32_STREAMS : 1, S->mg.inner_cycles > 1);
+                        streams ? FUSED32_STREAMS : 1, S->mg.inner_cycles > 1);
         };
         mg_lists(LAP_MG, P.mg64);
         mg_lists(LAP_MG_MIXED, P.mg32);
