@@ -423,16 +423,13 @@ __device__ __forceinline__ void tail_job(const TailJob& jb, const BatchLevel<T>*
 template <class T>
 __global__ void __launch_bounds__(TAIL_THREADS, (sizeof(T) == 4 ? 4 : 2))
     b_tail_kernel(const TailJob* __restrict__ jobs, int count, unsigned* claim, const BatchLevel<T>* __restrict__ lv,
-                  const int* __restrict__ active, int nu1, int nu2, int gs, T w_arg, T omw_arg,
-                  int per_level_w)
+                  const int* __restrict__ active, int nu1, int nu2, int gs, T w, T omw)
 {
     extern __shared__ double b[];
     const ItemClaim ic{claim, count};
     for (int k = ic.take(-1); k < count; k = ic.take(k)) {
         const TailJob jb = jobs[k];
         if (active && !active[lv[jb.first].problem]) continue;
-        const T w = per_level_w ? (T)lv[jb.first].w : w_arg;
-        const T omw = per_level_w ? (T)lv[jb.first].omw : omw_arg;
         tail_job(jb, lv, nu1, nu2, gs != 0, w, omw, b);
         __syncthreads();  // shared memory and the job's levels are reused by the next job
     }
@@ -805,18 +802,18 @@ template cudaError_t launch_b_coarse<float>(const BatchList&, const BatchLevel<f
 template <class T>
 cudaError_t launch_b_tail(const TailJob* jobs, int count, const BatchLevel<T>* lv, const int* active,
                           int nu1, int nu2, bool gs, double w, int max_unknowns, cudaStream_t s,
-                          bool per_level_w, unsigned* claim)
+                          unsigned* claim)
 {
     if (count == 0) return cudaSuccess;
     const size_t smem = sizeof(double) * (max_unknowns > 0 ? max_unknowns : 1);
     const int grid = batch_grid((const void*)b_tail_kernel<T>, TAIL_THREADS, smem, count, claim != nullptr);
     b_tail_kernel<T><<<grid, TAIL_THREADS, smem, s>>>(jobs, count, claim, lv, active, nu1, nu2, gs ? 1 : 0,
-                                                      (T)w, (T)(1.0 - w), per_level_w ? 1 : 0);
+                                                      (T)w, (T)(1.0 - w));
     note_launch();
     return cudaGetLastError();
 }
-template cudaError_t launch_b_tail<double>(const TailJob*, int, const BatchLevel<double>*, const int*, int, int, bool, double, int, cudaStream_t, bool, unsigned*);
-template cudaError_t launch_b_tail<float>(const TailJob*, int, const BatchLevel<float>*, const int*, int, int, bool, double, int, cudaStream_t, bool, unsigned*);
+template cudaError_t launch_b_tail<double>(const TailJob*, int, const BatchLevel<double>*, const int*, int, int, bool, double, int, cudaStream_t, unsigned*);
+template cudaError_t launch_b_tail<float>(const TailJob*, int, const BatchLevel<float>*, const int*, int, int, bool, double, int, cudaStream_t, unsigned*);
 
 cudaError_t launch_b_sumsq(const BatchList& l, const BatchLevel<double>* lv, const int* active,
                            double* partials, const BatchLevel<float>* lv32, cudaStream_t s,

@@ -189,9 +189,10 @@ int mg_level_count(int m, int n, int coarsest_min, int max_levels);
 
 
 // ---- V-cycles over many problems (lap_batched.cu, lap_server.cu) ----
-// Interior points per work item (rows are not split). Measured on the 4096-grid batch (sides
-// 33..513, V(2,2) to 1e-10): FP64 145 / 140 / 140 / 145 ms at 2048 / 8192 / 16384 / 32768
-// points, the mixed solver 74 / 71 / 69 / 68 ms; 8192 for both.
+// Interior points per work item (rows are not split) of the norm, update and server lists. A batch's
+// level passes have items by its size (batch_config). Measured on the 4096-grid batch (sides
+// 33..513, V(2,2) to 1e-10) with all lists alike: FP64 145 / 140 / 140 / 145 ms at 2048 / 8192 / 16384 /
+// 32768 points, the mixed solver 74 / 71 / 69 / 68 ms.
 constexpr int BATCH_ITEM_POINTS = 8192;
 void add_items(std::vector<BatchItem>& items, int level_index, int m, int n,
                int points = BATCH_ITEM_POINTS, bool red = false, int unit = 1);
@@ -239,11 +240,11 @@ void enqueue_tail(const LevelLists& L, int l, const BatchLevel<T>* lv, const int
     plan.bytes = (sizeof(T) == 8 ? L.tail64 : L.tail32)[l];
     if (plan.bytes)
         ck(launch_smem_tail(jobs + L.tail[l].first, L.tail[l].second, lv, active, p.nu1, p.nu2, gs, smoother_w, plan,
-                            st, false, L.claim),
+                            st, L.claim),
            "batched tail");
     else
         ck(launch_b_tail(jobs + L.tail[l].first, L.tail[l].second, lv, active, p.nu1, p.nu2, gs, smoother_w,
-                         L.max_coarse, st, false, L.claim),
+                         L.max_coarse, st, L.claim),
            "batched tail");
 }
 

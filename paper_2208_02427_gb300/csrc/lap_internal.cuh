@@ -371,13 +371,13 @@ template <class T>
 cudaError_t launch_b_coarse(const BatchList& l, const BatchLevel<T>* lv, const int* active,
                             int max_unknowns, cudaStream_t s);
 // One CTA per job runs the V-cycle from level `first` down to the coarsest and back (nu1/nu2
-// smoothing sweeps, gs or SOR with w, or each level's own w); active may be null (all run).
+// smoothing sweeps, gs or SOR with w); active may be null (all run).
 // max_unknowns: the largest coarsest level among the jobs.
 // claim (nullable): a persistent launch over the jobs (see BatchList).
 template <class T>
 cudaError_t launch_b_tail(const TailJob* jobs, int count, const BatchLevel<T>* lv, const int* active,
                           int nu1, int nu2, bool gs, double w, int max_unknowns, cudaStream_t s,
-                          bool per_level_w = false, unsigned* claim = nullptr);
+                          unsigned* claim = nullptr);
 // The same with every level's u and q in shared memory (tail_kernels.cu): nc = 1 one CTA per job, or
 // one job on a cluster of nc CTAs that split its first ncl levels by rows. bytes = 0: the levels do
 // not fit.
@@ -392,7 +392,7 @@ SmemTail plan_smem_tail(int m, int n, int nl, bool cluster);
 template <class T>
 cudaError_t launch_smem_tail(const TailJob* jobs, int count, const BatchLevel<T>* lv, const int* active, int nu1,
                              int nu2, bool gs, double w, const SmemTail& plan, cudaStream_t s,
-                             bool per_level_w = false, unsigned* claim = nullptr);
+                             unsigned* claim = nullptr);
 // per-item FP64 sum of squares of the residual; with lv32 also r32 := residual, e32 := 0;
 // skip32: the mixed problems are left to launch_b_residual32
 // gs: FP64 multigrid problems come from Gauss-Seidel smoothing (with beta = 1 only their red points

@@ -30,9 +30,7 @@ namespace {
 
 constexpr unsigned ALL = 0xffffffffu;
 constexpr int ST_WARPS = 4;  // warps per CTA
-#ifndef STREAM_WARPS_PER_SM
-#define STREAM_WARPS_PER_SM 16
-#endif
+constexpr int STREAM_WARPS_PER_SM = 16;
 
 // Row pipelines are unrolled over their D rows in flight in registers; rows come from memory R
 // ahead (R divides D, so that a row's slot is known at compile time).

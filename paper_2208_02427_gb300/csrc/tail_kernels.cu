@@ -539,20 +539,17 @@ __device__ __forceinline__ void tail_dispatch(const TailJob& jb, const BatchLeve
 template <class T, bool CL>
 __global__ void __launch_bounds__(SMEM_TAIL_THREADS, 1)
     smem_tail_kernel(const TailJob* __restrict__ jobs, int count, unsigned* claim, const BatchLevel<T>* __restrict__ lv,
-                     const int* __restrict__ active, int nu1, int nu2, int gs, T w_arg, T omw_arg, int per_level_w,
-                     int nc, int ncl)
+                     const int* __restrict__ active, int nu1, int nu2, int gs, T w, T omw, int nc, int ncl)
 {
     after_prior();
     if (CL) {
-        tail_dispatch<T, true>(jobs[0], lv, nu1, nu2, gs != 0, w_arg, omw_arg, nc, ncl);
+        tail_dispatch<T, true>(jobs[0], lv, nu1, nu2, gs != 0, w, omw, nc, ncl);
         return;
     }
     const ItemClaim ic{claim, count};
     for (int k = ic.take(-1); k < count; k = ic.take(k)) {
         const TailJob jb = jobs[k];
         if (active && !active[lv[jb.first].problem]) continue;
-        const T w = per_level_w ? (T)lv[jb.first].w : w_arg;
-        const T omw = per_level_w ? (T)lv[jb.first].omw : omw_arg;
         tail_dispatch<T, false>(jb, lv, nu1, nu2, gs != 0, w, omw, 1, 0);
         __syncthreads();  // shared memory is reused by the next job
     }
@@ -664,11 +661,10 @@ template SmemTail plan_smem_tail<float>(int, int, int, bool);
 
 template <class T>
 cudaError_t launch_smem_tail(const TailJob* jobs, int count, const BatchLevel<T>* lv, const int* active, int nu1,
-                             int nu2, bool gs, double w, const SmemTail& plan, cudaStream_t s, bool per_level_w,
-                             unsigned* claim)
+                             int nu2, bool gs, double w, const SmemTail& plan, cudaStream_t s, unsigned* claim)
 {
     if (count == 0) return cudaSuccess;
-    const int g = gs ? 1 : 0, pl = per_level_w ? 1 : 0;
+    const int g = gs ? 1 : 0;
     const T wt = (T)w, omw = (T)(1.0 - w);
     if (plan.nc > 1) {
         cudaError_t e = tail_attributes<T, true>(SMEM_MAX);
@@ -687,7 +683,7 @@ cudaError_t launch_smem_tail(const TailJob* jobs, int count, const BatchLevel<T>
         cfg.attrs = at;
         cfg.numAttrs = 2;
         e = cudaLaunchKernelEx(&cfg, smem_tail_kernel<T, true>, jobs, count, (unsigned*)nullptr, lv, active, nu1, nu2,
-                               g, wt, omw, pl, plan.nc, plan.ncl);
+                               g, wt, omw, plan.nc, plan.ncl);
         note_launch();
         return e != cudaSuccess ? e : cudaGetLastError();
     }
@@ -696,11 +692,11 @@ cudaError_t launch_smem_tail(const TailJob* jobs, int count, const BatchLevel<T>
     const int grid = batch_grid((const void*)smem_tail_kernel<T, false>, SMEM_TAIL_THREADS, plan.bytes, count,
                                 claim != nullptr);
     launch_after(smem_tail_kernel<T, false>, grid, SMEM_TAIL_THREADS, plan.bytes, s, jobs, count, claim, lv, active, nu1, nu2, g,
-                                                                           wt, omw, pl, 1, 0);
+                                                                           wt, omw, 1, 0);
     note_launch();
     return cudaGetLastError();
 }
-template cudaError_t launch_smem_tail<double>(const TailJob*, int, const BatchLevel<double>*, const int*, int, int, bool, double, const SmemTail&, cudaStream_t, bool, unsigned*);
-template cudaError_t launch_smem_tail<float>(const TailJob*, int, const BatchLevel<float>*, const int*, int, int, bool, double, const SmemTail&, cudaStream_t, bool, unsigned*);
+template cudaError_t launch_smem_tail<double>(const TailJob*, int, const BatchLevel<double>*, const int*, int, int, bool, double, const SmemTail&, cudaStream_t, unsigned*);
+template cudaError_t launch_smem_tail<float>(const TailJob*, int, const BatchLevel<float>*, const int*, int, int, bool, double, const SmemTail&, cudaStream_t, unsigned*);
 
 }  // namespace lap
