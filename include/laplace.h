@@ -60,10 +60,10 @@ typedef enum {
     LAP_MG_MIXED = 5, /* the V-cycle's correction equation (Eqs. 13-15) solved by FP32
                         V-cycles inside FP64 defect correction: per iteration,
                         inner_cycles FP32 V(nu1,nu2) cycles on L e = -R, then psi += e
-                        and R = L(psi): with beta = 1 the exact sum, rounded once to the
-                        FP32 that the cycles take (runs of 62 x 8 points whose values span
-                        more than 31 binades, or leave about 1e-18 .. 1e35: the FP64
-                        expression), else the FP64 expression */
+                        and R = L(psi): the FP64 expression rounded to the cycles' FP32, or
+                        after the first one, with beta = 1, the exact sum rounded once to it
+                        (but for runs of 62 x 8 points whose values span more than 31
+                        binades or leave about 1e-18 .. 1e35) */
     LAP_SLOR = 6,    /* line SOR by rows alone (SLOR subsection, Eqs. 8-10): one zebra
                         x-line sweep per iteration, form line_form (A = SLORA, B = SLORB) */
     LAP_GS_LEX = 7,  /* Eq. 6 in the paper's lexicographic order (i-1, j-1 already new), as
