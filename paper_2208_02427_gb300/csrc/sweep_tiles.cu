@@ -279,7 +279,7 @@ cudaError_t launch_sweep_tiles(const Field& in, double* out, int64_t pitch_out, 
 // Fields of one size count once, sides past the widest field's are as good as its own, and a pair of sides is
 // only worked out where a lower bound of its cost (no partial tiles, no partial last round) beats the best
 // cost so far: a step plans on the host with the device idle. 1000 fields of different sizes take 0.28 ms, every pair
-// of sides over every field 1.16 (on the build machine).
+// of sides over every field 1.16 (one host core).
 BatchSweepPlan plan_batch_sweeps(const std::vector<std::pair<int, int>>& fields, int sms)
 {
     BatchSweepPlan best;

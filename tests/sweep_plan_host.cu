@@ -76,7 +76,7 @@ int main()
     for (int c = 0; c < 1000; ++c) many.push_back({sides(33, 97), sides(33, 97)});
     auto least_time = [&](auto&& run) {
         double t = 1e300;
-        for (int k = 0; k < 5; ++k) {
+        for (int k = 0; k < 25; ++k) {
             const auto a = std::chrono::steady_clock::now();
             run();
             t = std::min(t, std::chrono::duration<double, std::micro>(std::chrono::steady_clock::now() - a).count());

@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 
 
 @pytest.fixture(scope="module")
-def checker(tmp_path_factory):
+def host_side(tmp_path_factory):
     try:
         cc = build.nvcc()
     except RuntimeError as exc:
@@ -38,9 +38,9 @@ def sizes():
     return out
 
 
-def test_windows_fit(checker):
+def test_windows_fit(host_side):
     text = "".join(f"{m} {n} {sms}\n" for m, n in sizes() for sms in (152, 148))
-    r = subprocess.run([checker], input=text, capture_output=True, text=True, check=True)
+    r = subprocess.run([host_side], input=text, capture_output=True, text=True, check=True)
     launches, bad, single = map(int, r.stdout.split())
     assert launches > 10000 and single > 100
     assert bad == 0, r.stderr
