@@ -56,6 +56,14 @@ struct StreamCoef {
 
 __device__ __forceinline__ float2 pair2(float v) { return make_float2(v, v); }
 
+// f v, for a product that is added next: the compiler joins a packed product and a packed sum to
+// one multiply-add (also under --fmad=false), which halves and quarters show below FP32's normal
+// range, where they round. Scalar products stay separate.
+__device__ __forceinline__ float2 times2(float f, float2 v)
+{
+    return make_float2(__fmul_rn(f, v.x), __fmul_rn(f, v.y));
+}
+
 __device__ __forceinline__ void cp16(unsigned dst, const void* src, int bytes)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
@@ -390,16 +398,16 @@ __device__ __forceinline__ void stream_up(const StreamItem& it, const BatchLevel
                     float rt = __shfl_down_sync(ALL, cur.v.x, 1, a.sw);
                     rt = a.last ? cur.right : rt;
                     if (!GS) pe = cur.v;
-                    po = __fmul2_rn(pair2(0.5f), __fadd2_rn(cur.v, make_float2(cur.v.y, rt)));
+                    po = times2(0.5f, __fadd2_rn(cur.v, make_float2(cur.v.y, rt)));
                 } else {
-                    pe = __fmul2_rn(pair2(0.5f), __fadd2_rn(cur.v, nxt.v));
+                    pe = times2(0.5f, __fadd2_rn(cur.v, nxt.v));
                     if (!GS) {
                         float r0 = __shfl_down_sync(ALL, cur.v.x, 1, a.sw);
                         float r1 = __shfl_down_sync(ALL, nxt.v.x, 1, a.sw);
                         r0 = a.last ? cur.right : r0;
                         r1 = a.last ? nxt.right : r1;
-                        po = __fmul2_rn(pair2(0.25f), __fadd2_rn(__fadd2_rn(cur.v, make_float2(cur.v.y, r0)),
-                                                                 __fadd2_rn(nxt.v, make_float2(nxt.v.y, r1))));
+                        po = times2(0.25f, __fadd2_rn(__fadd2_rn(cur.v, make_float2(cur.v.y, r0)),
+                                                      __fadd2_rn(nxt.v, make_float2(nxt.v.y, r1))));
                     }
                 }
                 // the ring and the columns outside stay as they are (a zero 1/d marks them)
